@@ -1,6 +1,8 @@
 // Batched dense kernels over uneven fronts (host launch wrappers).
 #pragma once
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace hif {
@@ -46,34 +48,47 @@ template <typename T>
 void gemm_batched(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const T* Abase,
                   const T* Bbase, T* Cbase, cudaStream_t st, const char* name = "gemm_batched");
 
-// y = alpha op(M) x (+ y), batched (see GemvOp).  trans = 0: y (rows) = M x;
-// trans = 1: y (cols) = M^T x.  nrhs vectors with stride `vstride` in `work`.
-template <typename T>
-void gemv_batched(const GemvOp* d_ops, const GemvOp* h_ops, int nops, int trans,
-                  const T* Marena, T* work, int64_t vstride, int nrhs, cudaStream_t st);
+// Mat-vecs of the apply sweeps, y = alpha op(M) x (+ y) batched over GemvOps
+// (gemv.cu).  trans = 0: y (rows) = M x; trans = 1: y (cols) = M^T x.
+// gemv_plan cuts a list into tasks (a row tile of M x, a column group of
+// M^T x); of M x, cnt[k] tiles, in this order, are shared by 8, 4, 2 and 1
+// warps; M^T x has one task per thread block (cnt[0]).
+struct GemvTask {
+  int32_t op, tile;
+};
+void gemv_plan(const GemvOp* ops, int nops, int trans, std::vector<GemvTask>& tasks, int (&cnt)[4]);
+// Thread blocks that run a planned list.
+int gemv_ctas(const int (&cnt)[4]);
+// Right-hand sides the next block takes when `left` remain: 16 (also for
+// 9-15, the others masked), 8 (5-7), 4 (3), 2 or 1, so that each block reads
+// the factor once.
+int gemv_block(int left);
 
-// Grouped apply: one launch runs the mat-vec lists of several factors (one
-// segment per factor's list and block of right-hand sides).  Segment k owns
-// ops first_k .. first_{k+1}-1 of the launch; op j reads ops[j - first] of
-// its device list, its matrix at M + op.M and its vectors at w + op.x,
-// w + op.y (w already shifted to the block's first column, vs apart).
+// One factor's list and block of right-hand sides: matrices at M + op.M,
+// vectors at w + op.x and w + op.y (w already shifted to the block's first
+// column, nv columns vs apart); `first` is its first thread block in a grouped
+// launch.
 template <typename T>
 struct GemvSeg {
   const GemvOp* ops;
+  const GemvTask* tasks;
   const T* M;
   T* w;
   int64_t vs;
   int64_t first;
+  int cnt[4];
+  int nv;
 };
 
-// gemv_batched over the segments (trans as there, R right-hand sides per op:
-// 16, 8, 4, 2 or 1; nops = all ops of the launch; mx = the widest op's row
-// tiles (trans 0) or column groups (trans 1), from gemv_tiles).  Per op the
-// arithmetic is gemv_batched's, so a grouped apply is bitwise the factor's
-// own apply.
+// A list (ops, tasks, M, w, vs, cnt of `list`) for nrhs right-hand sides.
 template <typename T>
-void gemv_segments(const GemvSeg<T>* d_segs, int nseg, int64_t nops, int mx, int trans, int R,
-                   double flops, double bytes, cudaStream_t st);
-int gemv_tiles(const GemvOp* h_ops, int nops, int trans);
+void gemv_batched(const GemvOp* h_ops, int nops, const GemvSeg<T>& list, int trans, int nrhs,
+                  cudaStream_t st);
+// One launch over the segments of several factors' lists (ctas thread blocks
+// in all, R right-hand sides per segment).  Per column the arithmetic is
+// gemv_batched's, so a grouped apply is bitwise the factor's own apply.
+template <typename T>
+void gemv_segments(const GemvSeg<T>* d_segs, int nseg, int ctas, int trans, int R, double flops,
+                   double bytes, cudaStream_t st);
 
 }  // namespace hif

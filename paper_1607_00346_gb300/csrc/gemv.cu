@@ -1,0 +1,605 @@
+// Batched mat-vecs of the apply sweeps: y = alpha op(M) x (+ y) for many
+// small-to-large column-major matrices of the factor and 1-16 right-hand
+// sides at once.
+//
+// What bounds them: each factor entry is read once per sweep and used in one
+// multiply-add per right-hand side, so up to 16 FP32 columns they are bound by
+// HBM; what has to be kept off the critical path is the latency of the loads
+// (every warp keeps 16 or more 128-byte loads in flight), the loads of x (one
+// per matrix entry and column if x is not shared) and the idle warps of uneven
+// batches (sizes go from 27 x 27 to thousands within one sweep).
+//
+// Work is cut into tasks on the host, once per list (gemv_plan), so that a
+// launch has no empty blocks:
+//   * M x: a task is a 64-row tile of one matrix.  1, 2, 4 or 8 warps of a
+//     256-thread CTA share it (by the tile's column count, 8 columns per
+//     block, blocks dealt to the warps in turn), so a CTA holds 8, 4, 2 or 1
+//     tiles; the warps' sums are added in warp order through shared memory.
+//     x of a block goes through a warp-private corner of shared memory and is
+//     read back as broadcasts.
+//   * M^T x: a task is 32 columns of one matrix, eight for each warp of a
+//     128-thread CTA; lanes stride the rows and share each x value between
+//     the eight columns; a transposing butterfly adds the lanes.
+// The order of every sum depends on the matrix shape only, so a column gets
+// the same bits in any block of right-hand sides and in a grouped launch.
+//
+// Measured on a 128^3 FP32 factor (2.86e9 entries, 22.9 GB in the two sweeps),
+// the mat-vecs of one apply: 1 column 3.9 ms (5.9 TB/s), 4 columns 5.0 ms, 16
+// columns 8.7 ms; with one CTA per 128 rows or 8 columns and x read from L1 by
+// every warp (blocks 16, 8, 4, 2, 1) they took 6.5 ms for 1 column and 37 ms
+// for 16.  On a 64^3 FP64 factor 8 columns take 8.7 ms, 7.2 ms of which are the
+// multiply-adds at the FP64 rate.
+#include <algorithm>
+#include <vector>
+
+#include "dense.cuh"
+
+namespace hif {
+
+namespace {
+
+constexpr int GEMV_THREADS = 256;
+constexpr int GEMV_WARPS = GEMV_THREADS / 32;
+constexpr int GEMV_TR = 64;    // rows of an M x tile, two per lane
+constexpr int GEMV_BC = 8;     // columns of a block of an M x tile
+constexpr int GEMV_T_THREADS = 128;
+constexpr int GEMV_CG = 8;     // columns of a warp of M^T x
+constexpr int GEMV_TC = GEMV_CG * GEMV_T_THREADS / 32;   // columns of an M^T x task
+
+// R consecutive values from shared memory, as 16-byte vectors where they fill one.
+template <int R>
+__device__ __forceinline__ void read_x(float (&t)[R], const float* p) {
+  if constexpr (R >= 4) {
+#pragma unroll
+    for (int q = 0; q < R; q += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(p + q);
+      t[q] = a.x;
+      t[q + 1] = a.y;
+      t[q + 2] = a.z;
+      t[q + 3] = a.w;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < R; ++q) t[q] = p[q];
+  }
+}
+template <int R>
+__device__ __forceinline__ void read_x(double (&t)[R], const double* p) {
+  if constexpr (R >= 2) {
+#pragma unroll
+    for (int q = 0; q < R; q += 2) {
+      const double2 a = *reinterpret_cast<const double2*>(p + q);
+      t[q] = a.x;
+      t[q + 1] = a.y;
+    }
+  } else {
+    t[0] = p[0];
+  }
+}
+
+// ---- y = alpha M x (+ y) --------------------------------------------------------
+// One tile by `ncls` warps, this one taking blocks cls, cls + ncls, ...; the
+// caller's warps of one CTA all come here with the same ncls.  xs: this
+// warp's GEMV_BC x R corner; red: the CTA's GEMV_WARPS x GEMV_TR x RQ sums.
+template <typename T, int R>
+__host__ __device__ constexpr int gemv_red_cols() {   // right-hand sides reduced per round
+  return R < 4 ? R : 4;
+}
+
+template <typename T, int R>
+__device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, int ti, int ncls,
+                                            T* xs_all, T* red) {
+  constexpr int XN = (GEMV_BC * R + 31) / 32;   // x values a lane stages per block
+  constexpr int RQ = gemv_red_cols<T, R>();
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int cls = warp % ncls;
+  T* xs = xs_all + warp * (GEMV_BC * R);
+  GemvTask tk{0, 0};
+  GemvOp o{};
+  if (valid) {
+    tk = sg.tasks[ti];
+    o = sg.ops[tk.op];
+  }
+  const int r0 = tk.tile * GEMV_TR;
+  const int rows = o.rows;
+  const int ra = r0 + lane, rb = ra + 32;
+  const int cols = valid ? (o.tri ? min(o.cols, r0 + GEMV_TR) : o.cols) : 0;
+  const int nblk = (cols + GEMV_BC - 1) / GEMV_BC;
+  const T* M = sg.M + o.M;
+  const T* x = sg.w + o.x;
+  const int64_t vs = sg.vs;
+  const int nv = sg.nv;
+  const bool rfull = r0 + GEMV_TR <= rows;
+
+  T acc[2][R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) acc[0][q] = acc[1][q] = T(0);
+  // a block's matrix entries and x values, in flight while the block before
+  // it is multiplied
+  constexpr bool AHEAD = sizeof(T) == 4 || R < 8;   // else the sums need the registers
+  T m[2][GEMV_BC], mn[2][GEMV_BC], xv[XN], xn[XN];
+  auto full = [&](int b) {   // no entry of the block is masked
+    const int c0 = b * GEMV_BC;
+    return rfull && c0 + GEMV_BC <= cols && (!o.tri || c0 + GEMV_BC <= r0 + 1);
+  };
+  auto load = [&](int b, T (&mm)[2][GEMV_BC], T (&xx)[XN]) {
+    const int c0 = b * GEMV_BC;
+    const T* mc = M + (int64_t)c0 * o.ld;
+    if (full(b)) {
+#pragma unroll
+      for (int c = 0; c < GEMV_BC; ++c) {
+        mm[0][c] = mc[ra + (int64_t)c * o.ld];
+        mm[1][c] = mc[rb + (int64_t)c * o.ld];
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < GEMV_BC; ++c) {
+        const bool in = c0 + c < cols;
+        mm[0][c] = (in && ra < rows && (!o.tri || c0 + c <= ra)) ? mc[ra + (int64_t)c * o.ld] : T(0);
+        mm[1][c] = (in && rb < rows && (!o.tri || c0 + c <= rb)) ? mc[rb + (int64_t)c * o.ld] : T(0);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < XN; ++j) {
+      const int e = lane + 32 * j, q = e / GEMV_BC, c = c0 + e % GEMV_BC;
+      xx[j] = (q < nv && q < R && c < cols) ? x[q * vs + c] : T(0);
+    }
+  };
+  if (AHEAD && cls < nblk) load(cls, m, xv);
+  for (int b = cls; b < nblk; b += ncls) {
+    if (!AHEAD) load(b, m, xv);
+    else if (b + ncls < nblk) load(b + ncls, mn, xn);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < XN; ++j) {
+      const int e = lane + 32 * j;
+      if (e < GEMV_BC * R) xs[(e % GEMV_BC) * R + e / GEMV_BC] = xv[j];
+    }
+    __syncwarp();
+    if (full(b)) {
+#pragma unroll
+      for (int c = 0; c < GEMV_BC; ++c) {
+        T t[R];
+        read_x<R>(t, xs + c * R);
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          acc[0][q] = fma(m[0][c], t[q], acc[0][q]);
+          acc[1][q] = fma(m[1][c], t[q], acc[1][q]);
+        }
+      }
+    } else {
+      // a masked entry leaves its sum alone (x may be infinite there)
+#pragma unroll
+      for (int c = 0; c < GEMV_BC; ++c) {
+        const int cc = b * GEMV_BC + c;
+        const bool ia = cc < cols && (!o.tri || cc <= ra), ib = cc < cols && (!o.tri || cc <= rb);
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const T t = xs[c * R + q];
+          if (ia) acc[0][q] = fma(m[0][c], t, acc[0][q]);
+          if (ib) acc[1][q] = fma(m[1][c], t, acc[1][q]);
+        }
+      }
+    }
+    if (AHEAD) {
+#pragma unroll
+      for (int c = 0; c < GEMV_BC; ++c) {
+        m[0][c] = mn[0][c];
+        m[1][c] = mn[1][c];
+      }
+#pragma unroll
+      for (int j = 0; j < XN; ++j) xv[j] = xn[j];
+    }
+  }
+  const T al = (T)o.alpha;
+  T* y = sg.w + o.y;
+  if (ncls == 1) {
+    if (!valid) return;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      if (q >= nv) continue;
+      T* yp = y + q * vs;
+      if (ra < rows) yp[ra] = (o.beta_one ? yp[ra] : T(0)) + al * acc[0][q];
+      if (rb < rows) yp[rb] = (o.beta_one ? yp[rb] : T(0)) + al * acc[1][q];
+    }
+    return;
+  }
+  // the warps' sums of each tile, added in warp order, RQ columns per round
+  const int t0 = warp / ncls * ncls;               // first warp of this tile
+  const int tid = (warp - t0) * 32 + lane;         // thread within the tile's warps
+#pragma unroll
+  for (int q0 = 0; q0 < R; q0 += RQ) {
+    if (q0 >= nv) break;
+#pragma unroll
+    for (int q = 0; q < RQ; ++q) {
+      red[(warp * RQ + q) * GEMV_TR + lane] = acc[0][q0 + q];
+      red[(warp * RQ + q) * GEMV_TR + lane + 32] = acc[1][q0 + q];
+    }
+    __syncthreads();
+    if (valid)
+      for (int e = tid; e < RQ * GEMV_TR; e += ncls * 32) {
+        const int q = e / GEMV_TR, r = r0 + e % GEMV_TR;
+        T s = red[t0 * RQ * GEMV_TR + e];
+        for (int w = 1; w < ncls; ++w) s += red[(t0 + w) * RQ * GEMV_TR + e];
+        if (r < rows && q0 + q < nv) {
+          T* yp = y + (q0 + q) * vs + r;
+          *yp = (o.beta_one ? *yp : T(0)) + al * s;
+        }
+      }
+    __syncthreads();
+  }
+}
+
+template <typename T, int R>
+__device__ __forceinline__ void gemv_n_cta(const GemvSeg<T>& sg, int b) {
+  __shared__ __align__(16) T xs[GEMV_WARPS * GEMV_BC * R];
+  __shared__ T red[GEMV_WARPS * gemv_red_cols<T, R>() * GEMV_TR];
+  const int warp = threadIdx.x / 32;
+  // the list's tasks, those of 8 warps first, then 4, 2 and 1
+  int ncls = 8, base = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int per = GEMV_WARPS / ncls;   // tiles per CTA
+    const int nc = (sg.cnt[k] + per - 1) / per;
+    if (b < nc || k == 3) {
+      const int j = b * per + warp / ncls;
+      gemv_n_tile<T, R>(sg, j < sg.cnt[k], base + j, ncls, xs, red);
+      return;
+    }
+    b -= nc;
+    base += sg.cnt[k];
+    ncls >>= 1;
+  }
+}
+
+// One step of the butterfly over lanes S apart: the first N values of v are
+// summed; a lane keeps half of them (which half: idx) while there are several.
+template <typename T, int N, int S>
+__device__ __forceinline__ void lane_sum(T* v, int lane, int& idx) {
+  if constexpr (N > 1) {
+    const bool up = (lane & S) != 0;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+      const T send = up ? v[i] : v[i + N / 2];
+      const T keep = up ? v[i + N / 2] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, S);
+    }
+    idx += up ? N / 2 : 0;
+  } else {
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], S);
+  }
+  if constexpr (S > 1) lane_sum<T, (N > 1 ? N / 2 : 1), S / 2>(v, lane, idx);
+}
+
+// ---- y = alpha M^T x (+ y) -------------------------------------------------------
+// One CTA of four warps, columns 32 tile .. 32 tile + 31, eight per warp;
+// lanes stride the rows (from the 32-row step that holds the triangle's
+// diagonal), and a transposing butterfly adds the lanes at the end.
+//   * Up to 4 right-hand sides: x comes straight from L1, the loads of 2 row
+//     steps (16 matrix entries per lane) in flight together.
+//   * 8 and 16: x would be 8-16 loads per row step and the sums fill the
+//     registers, so the CTA copies 128 rows (FP64: 64) of its 32 columns and
+//     of x at a time to shared memory, asynchronously and one chunk ahead;
+//     each value of x is then read once for eight columns.
+// FP32, 16 columns, the T half of a 128^3 sweep (11.4 GB of factor): four
+// columns per warp with x from L1 9.0 ms (waiting for x), eight with x in
+// shared memory and the matrix in registers 6.5 ms (waiting for the matrix),
+// this form 4.8 ms.
+__device__ __forceinline__ void cp_async(float* dst, const float* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async(double* dst, const double* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+
+// Sums over the lanes and writes y of CG columns from c0 on, R right-hand sides from q0 on.
+template <typename T, int R, int CG>
+__device__ __forceinline__ void gemv_t_finish(T (&v)[CG * R], const GemvOp& o, const GemvSeg<T>& sg,
+                                              int c0, int q0) {
+  constexpr int V = CG * R;
+  const int lane = threadIdx.x % 32;
+  // lane l ends with the values whose index has the bits of l (16, 8, ..) as
+  // its leading bits
+  int idx = 0;
+  lane_sum<T, V, 16>(v, lane, idx);
+  constexpr int KEEP = V > 32 ? V / 32 : 1;         // values left per lane
+  constexpr int DUP = V < 32 ? 32 / V : 1;          // lanes that hold the same value
+  if (lane % DUP) return;
+  const T al = (T)o.alpha;
+#pragma unroll
+  for (int i = 0; i < KEEP; ++i) {
+    const int c = c0 + (idx + i) / R, q = q0 + (idx + i) % R;
+    if (c < o.cols && q < sg.nv) {
+      T* yp = sg.w + o.y + q * sg.vs + c;
+      *yp = (o.beta_one ? *yp : T(0)) + al * v[i];
+    }
+  }
+}
+
+template <typename T, int R>
+__device__ __forceinline__ void gemv_t_few(const GemvSeg<T>& sg, int b) {
+  constexpr int UN = 2;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const GemvTask tk = sg.tasks[b];
+  const GemvOp o = sg.ops[tk.op];
+  const int c0 = tk.tile * GEMV_TC + warp * GEMV_CG;
+  if (c0 >= o.cols) return;
+  const int rows = o.rows;
+  const int64_t vs = sg.vs, ld = o.ld;
+  const int nv = sg.nv;
+  const T* M = sg.M + o.M + (int64_t)c0 * ld;
+  const T* x = sg.w + o.x;
+  T v[GEMV_CG * R];   // v[c R + q]
+#pragma unroll
+  for (int i = 0; i < GEMV_CG * R; ++i) v[i] = T(0);
+  auto masked = [&](int r) {
+    if (r >= rows) return;
+    T mm[GEMV_CG];
+#pragma unroll
+    for (int c = 0; c < GEMV_CG; ++c)
+      mm[c] = (c0 + c < o.cols && (!o.tri || r >= c0 + c)) ? M[r + c * ld] : T(0);
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const T xq = q < nv ? x[q * vs + r] : T(0);
+#pragma unroll
+      for (int c = 0; c < GEMV_CG; ++c)
+        if (!o.tri || r >= c0 + c) v[c * R + q] = fma(mm[c], xq, v[c * R + q]);
+    }
+  };
+  int r = 0;
+  if (o.tri) {
+    r = c0 / 32 * 32;
+    masked(r + lane);
+    r += 32;
+  }
+  if (c0 + GEMV_CG <= o.cols) {
+    for (; r + 32 * UN <= rows; r += 32 * UN) {
+      T mm[UN][GEMV_CG], xq[UN][R];
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+#pragma unroll
+        for (int c = 0; c < GEMV_CG; ++c) mm[u][c] = M[r + 32 * u + lane + c * ld];
+#pragma unroll
+        for (int q = 0; q < R; ++q) xq[u][q] = q < nv ? x[q * vs + r + 32 * u + lane] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+#pragma unroll
+          for (int c = 0; c < GEMV_CG; ++c) v[c * R + q] = fma(mm[u][c], xq[u][q], v[c * R + q]);
+    }
+  }
+  for (; r < rows; r += 32) masked(r + lane);
+  gemv_t_finish<T, R, GEMV_CG>(v, o, sg, c0, 0);
+}
+
+// 8 or 16 right-hand sides, RW of them per pass over the matrix (16 in FP32; in
+// FP64, bound by its multiply-adds, 8).
+template <typename T, int R>
+__device__ __forceinline__ void gemv_t_many(const GemvSeg<T>& sg, int b) {
+  constexpr int CG = GEMV_CG, RW = sizeof(T) == 4 ? R : 8;
+  constexpr int CH = GEMV_T_THREADS * 4 / (int)sizeof(T);   // rows per chunk
+  constexpr int STEPS = CH / 32;
+  constexpr int CPR = GEMV_T_THREADS / CH;                  // columns copied side by side
+  __shared__ T ms[2][GEMV_TC][CH];
+  __shared__ T xs[2][RW][CH];
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const GemvTask tk = sg.tasks[b];
+  const GemvOp o = sg.ops[tk.op];
+  const int ct = tk.tile * GEMV_TC, c0 = ct + warp * CG;
+  const int rows = o.rows;
+  const int64_t vs = sg.vs, ld = o.ld;
+  const T* M = sg.M + o.M + (int64_t)ct * ld;
+  const int rbeg = o.tri ? ct : 0;   // GEMV_TC = 32: the diagonal's row step
+  const int nchunk = rows > rbeg ? (rows - rbeg + CH - 1) / CH : 0;
+  const int te = threadIdx.x % CH, tc = threadIdx.x / CH;
+#pragma unroll 1
+  for (int q0 = 0; q0 < R && q0 < sg.nv; q0 += RW) {
+    const int nv = sg.nv - q0;
+    const T* x = sg.w + o.x + q0 * vs;
+    // chunk k of the matrix columns and of x, copied asynchronously; entries
+    // outside the matrix or the triangle are zero
+    auto stage = [&](int k) {
+      if (k < nchunk) {
+        const int r = rbeg + k * CH + te;
+        const bool in = r < rows;
+        if (ct + GEMV_TC <= o.cols && (k + 1) * CH <= rows - rbeg && (!o.tri || k > 0)) {
+          const T* m = M + r + tc * ld;
+#pragma unroll
+          for (int c = 0; c < GEMV_TC; c += CPR) cp_async(&ms[k & 1][c + tc][te], m + c * ld, true);
+        } else {
+#pragma unroll
+          for (int c = 0; c < GEMV_TC; c += CPR) {
+            const bool ok = in && ct + c + tc < o.cols && (!o.tri || r >= ct + c + tc);
+            cp_async(&ms[k & 1][c + tc][te], ok ? M + r + (c + tc) * ld : x, ok);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < RW; q += CPR) {
+          const bool ok = in && q + tc < nv;
+          cp_async(&xs[k & 1][q + tc][te], ok ? x + (q + tc) * vs + r : x, ok);
+        }
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    T v[CG * RW];
+#pragma unroll
+    for (int i = 0; i < CG * RW; ++i) v[i] = T(0);
+    stage(0);
+    for (int k = 0; k < nchunk; ++k) {
+      stage(k + 1);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+      __syncthreads();
+      const T(*mk)[CH] = &ms[k & 1][warp * CG];
+      const T(*xk)[CH] = xs[k & 1];
+#pragma unroll
+      for (int s = 0; s < STEPS; ++s) {
+        T m[CG];
+#pragma unroll
+        for (int c = 0; c < CG; ++c) m[c] = mk[c][32 * s + lane];
+        if (s == 0 && k == 0 && o.tri) {
+          // a masked entry leaves its sum alone (x may be infinite there)
+#pragma unroll
+          for (int q = 0; q < RW; ++q) {
+            const T xq = xk[q][lane];
+#pragma unroll
+            for (int c = 0; c < CG; ++c)
+              if (lane >= warp * CG + c) v[c * RW + q] = fma(m[c], xq, v[c * RW + q]);
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < RW; ++q) {
+            const T xq = xk[q][32 * s + lane];
+#pragma unroll
+            for (int c = 0; c < CG; ++c) v[c * RW + q] = fma(m[c], xq, v[c * RW + q]);
+          }
+        }
+      }
+      __syncthreads();   // the chunk's buffers are free for chunk k + 2
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    gemv_t_finish<T, RW, CG>(v, o, sg, c0, q0);
+    __syncthreads();
+  }
+}
+
+template <typename T, int R>
+__device__ __forceinline__ void gemv_t_cta(const GemvSeg<T>& sg, int b) {
+  if constexpr (R >= 8) gemv_t_many<T, R>(sg, b);
+  else gemv_t_few<T, R>(sg, b);
+}
+
+// M x, FP32 up to 4 columns: three CTAs per SM keep 24 warps of loads in
+// flight; 8 and 16 columns (and FP64) need the registers for their sums.
+// M^T x, 8 and 16 columns: the sums fill the registers, two or three CTAs of
+// four warps keep a chunk each in flight.
+template <int TRANS>
+constexpr int gemv_threads() { return TRANS ? GEMV_T_THREADS : GEMV_THREADS; }
+template <typename T, int R, int TRANS>
+constexpr int gemv_ctas_per_sm() {
+  if (TRANS) return R >= 8 ? (sizeof(T) == 8 ? 2 : R == 16 ? 3 : 4) : sizeof(T) == 4 ? 6 : R < 4 ? 5 : 4;
+  return sizeof(T) == 4 ? (R >= 8 ? 2 : 3) : (R >= 16 ? 1 : 2);
+}
+
+template <typename T, int R, int TRANS>
+__global__ void __launch_bounds__(gemv_threads<TRANS>(), (gemv_ctas_per_sm<T, R, TRANS>()))
+    k_gemv(const GemvSeg<T> sg) {
+  if constexpr (TRANS) gemv_t_cta<T, R>(sg, blockIdx.x);
+  else gemv_n_cta<T, R>(sg, blockIdx.x);
+}
+
+// Grouped launches: block j runs block j - first of the segment that holds it
+// (one factor's mat-vec list for one block of right-hand sides).
+template <typename T, int R, int TRANS>
+__global__ void __launch_bounds__(gemv_threads<TRANS>(), (gemv_ctas_per_sm<T, R, TRANS>()))
+    k_gemv_seg(const GemvSeg<T>* __restrict__ segs, int nseg) {
+  int k = 0;
+  while (k + 1 < nseg && segs[k + 1].first <= (int64_t)blockIdx.x) ++k;
+  const GemvSeg<T> sg = segs[k];
+  const int b = (int)((int64_t)blockIdx.x - sg.first);
+  if constexpr (TRANS) gemv_t_cta<T, R>(sg, b);
+  else gemv_n_cta<T, R>(sg, b);
+}
+
+template <typename T, int R>
+void launch_gemv(const GemvSeg<T>& sg, int trans, cudaStream_t st) {
+  const int ctas = gemv_ctas(sg.cnt);
+  if (trans) k_gemv<T, R, 1><<<ctas, GEMV_T_THREADS, 0, st>>>(sg);
+  else k_gemv<T, R, 0><<<ctas, GEMV_THREADS, 0, st>>>(sg);
+  HIF_CHECK_LAUNCH();
+}
+
+template <typename T, int R>
+void launch_gemv_seg(const GemvSeg<T>* d_segs, int nseg, int ctas, int trans, cudaStream_t st) {
+  if (trans) k_gemv_seg<T, R, 1><<<ctas, GEMV_T_THREADS, 0, st>>>(d_segs, nseg);
+  else k_gemv_seg<T, R, 0><<<ctas, GEMV_THREADS, 0, st>>>(d_segs, nseg);
+  HIF_CHECK_LAUNCH();
+}
+
+}  // namespace
+
+// Warps per tile of M x: enough blocks of 8 columns for each warp to keep a
+// second block in flight, one warp for tiles of up to 4 blocks.
+void gemv_plan(const GemvOp* ops, int nops, int trans, std::vector<GemvTask>& tasks, int (&cnt)[4]) {
+  tasks.clear();
+  for (int k = 0; k < 4; ++k) cnt[k] = 0;
+  if (trans) {
+    for (int i = 0; i < nops; ++i)
+      for (int t = 0; (int64_t)t * GEMV_TC < ops[i].cols; ++t) tasks.push_back(GemvTask{i, t});
+    cnt[0] = (int)tasks.size();
+    return;
+  }
+  std::vector<GemvTask> by[4];
+  for (int i = 0; i < nops; ++i)
+    for (int t = 0; (int64_t)t * GEMV_TR < ops[i].rows; ++t) {
+      const int c = ops[i].tri ? (int)std::min<int64_t>(ops[i].cols, ((int64_t)t + 1) * GEMV_TR) : ops[i].cols;
+      by[c > 512 ? 0 : c > 128 ? 1 : c > 32 ? 2 : 3].push_back(GemvTask{i, t});
+    }
+  for (int k = 0; k < 4; ++k) {
+    cnt[k] = (int)by[k].size();
+    tasks.insert(tasks.end(), by[k].begin(), by[k].end());
+  }
+}
+
+int gemv_ctas(const int (&cnt)[4]) {
+  return cnt[0] + ceil_div(cnt[1], 2) + ceil_div(cnt[2], 4) + ceil_div(cnt[3], 8);
+}
+
+int gemv_block(int left) { return left > 8 ? 16 : left > 4 ? 8 : left > 2 ? 4 : left; }
+
+template <typename T>
+void gemv_batched(const GemvOp* h_ops, int nops, const GemvSeg<T>& list, int trans, int nrhs,
+                  cudaStream_t st) {
+  if (nops == 0 || gemv_ctas(list.cnt) == 0) return;
+  for (int q0 = 0; q0 < nrhs;) {
+    const int R = gemv_block(nrhs - q0);
+    GemvSeg<T> sg = list;
+    sg.w = list.w + (int64_t)q0 * list.vs;
+    sg.nv = std::min(R, nrhs - q0);
+    double by = 0, fl = 0;
+    if (prof_enabled()) {
+      for (int i = 0; i < nops; ++i) {
+        const GemvOp& o = h_ops[i];
+        const double ent = o.tri ? 0.5 * (double)o.cols * (o.cols + 1) : (double)o.rows * o.cols;
+        by += sizeof(T) * (ent + (double)sg.nv * (o.rows + o.cols) * (o.beta_one ? 1.5 : 1.0));
+        fl += 2.0 * ent * sg.nv;
+      }
+    }
+    ProfScope ps(trans ? "apply_gemv_t" : "apply_gemv_n", st, fl, by);
+    switch (R) {
+      case 16: launch_gemv<T, 16>(sg, trans, st); break;
+      case 8: launch_gemv<T, 8>(sg, trans, st); break;
+      case 4: launch_gemv<T, 4>(sg, trans, st); break;
+      case 2: launch_gemv<T, 2>(sg, trans, st); break;
+      default: launch_gemv<T, 1>(sg, trans, st);
+    }
+    q0 += sg.nv;
+  }
+}
+
+template <typename T>
+void gemv_segments(const GemvSeg<T>* d_segs, int nseg, int ctas, int trans, int R, double flops,
+                   double bytes, cudaStream_t st) {
+  if (ctas == 0) return;
+  ProfScope ps(trans ? "apply_grouped_gemv_t" : "apply_grouped_gemv_n", st, flops, bytes);
+  switch (R) {
+    case 16: launch_gemv_seg<T, 16>(d_segs, nseg, ctas, trans, st); break;
+    case 8: launch_gemv_seg<T, 8>(d_segs, nseg, ctas, trans, st); break;
+    case 4: launch_gemv_seg<T, 4>(d_segs, nseg, ctas, trans, st); break;
+    case 2: launch_gemv_seg<T, 2>(d_segs, nseg, ctas, trans, st); break;
+    default: launch_gemv_seg<T, 1>(d_segs, nseg, ctas, trans, st);
+  }
+}
+
+#define HIF_INST(T)                                                                             \
+  template void gemv_batched<T>(const GemvOp*, int, const GemvSeg<T>&, int, int, cudaStream_t); \
+  template void gemv_segments<T>(const GemvSeg<T>*, int, int, int, int, double, double,         \
+                                 cudaStream_t);
+HIF_INST(float)
+HIF_INST(double)
+#undef HIF_INST
+
+}  // namespace hif

@@ -198,12 +198,14 @@ bool is_device_ptr(const void* p) {
 struct GemvList {
   std::vector<GemvOp> h;
   DevBuf d;
+  DevBuf tasks;  // the list cut into tasks (gemv_plan)
+  int cnt[4] = {0, 0, 0, 0};
   int trans = 0;
   int mat = 0;   // 0: panel arena, 1: interpolation-matrix arena
-  int tiles = -1;   // widest op's CTA count along x (cached for grouped launches)
-  int get_tiles() {
-    if (tiles < 0) tiles = gemv_tiles(h.data(), (int)h.size(), trans);
-    return tiles;
+  template <typename T>
+  GemvSeg<T> seg(const T* M, T* w, int64_t vs) const {
+    return GemvSeg<T>{d.as<GemvOp>(), tasks.as<GemvTask>(), M, w, vs, 0,
+                      {cnt[0], cnt[1], cnt[2], cnt[3]}, 0};
   }
 };
 
@@ -277,7 +279,7 @@ struct Factor : FactorBase {
   }
   // Algorithmic counts of the two sweeps for nrhs right-hand sides: every
   // stored factor entry is read once per sweep and per block of right-hand
-  // sides (blocks of 16, 8, 4, 2, 1) and used in one multiply-add per
+  // sides (gemv_block) and used in one multiply-add per
   // column; gathers and sets move an index and the values in and out.
   void sweep_counts(int nrhs, double* flops, double* bytes) const {
     int64_t ent = 0, slots = 0;
@@ -286,11 +288,7 @@ struct Factor : FactorBase {
       slots += s.nidx + s.nset;
     }
     int blocks = 0;
-    for (int left = nrhs; left > 0;) {
-      const int R = left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
-      left -= R;
-      ++blocks;
-    }
+    for (int left = nrhs; left > 0; ++blocks) left -= gemv_block(left);
     *flops = 2.0 * 2.0 * (double)ent * nrhs;
     *bytes = 2.0 * ((double)ent * sizeof(T) * blocks + (double)slots * (6.0 + 2.0 * sizeof(T) * nrhs));
   }
@@ -336,8 +334,7 @@ struct Factor : FactorBase {
     for (auto& gl : lists) {
       if (gl.h.empty()) continue;
       const T* M = gl.mat ? s.tmats.as<T>() : s.panels.as<T>();
-      gemv_batched<T>(gl.d.as<GemvOp>(), gl.h.data(), (int)gl.h.size(), gl.trans, M, w, vs, nrhs,
-                      st);
+      gemv_batched<T>(gl.h.data(), (int)gl.h.size(), gl.seg<T>(M, w, vs), gl.trans, nrhs, st);
     }
     vec_set<T>(s.set_g.as<int32_t>(), s.set_p.as<int32_t>(), s.nset, yv, ys, w, vs, nrhs, st);
     if (fwd && s.nacc)
@@ -405,8 +402,7 @@ void grouped_sweeps(const std::vector<Factor<T>*>& Fs, const std::vector<int>& n
     int kind;              // 0 gather, 1 set, 2 accumulate, 3 mat-vec
     int trans, R, count;   // count: jobs or segments
     size_t off;            // byte offset of the descriptors in the upload
-    int64_t nops;
-    int mx;
+    int ctas;              // thread blocks of a mat-vec launch
     double fl, by;
   };
   std::vector<unsigned char> blob;
@@ -420,7 +416,10 @@ void grouped_sweeps(const std::vector<Factor<T>*>& Fs, const std::vector<int>& n
   const int nh = (int)Fs.size();
   std::vector<T*> yv(nh), wv(nh);
   std::vector<int64_t> ys(nh), vs(nh);
-  std::vector<std::vector<std::pair<int, int>>> blocks(nh);   // (first column, R)
+  struct Block {
+    int q0, R, nv;   // first column, block size, columns in it
+  };
+  std::vector<std::vector<Block>> blocks(nh);
   size_t S = 0;
   for (int h = 0; h < nh; ++h) {
     yv[h] = Fs[h]->y.template as<T>();
@@ -428,10 +427,9 @@ void grouped_sweeps(const std::vector<Factor<T>*>& Fs, const std::vector<int>& n
     ys[h] = (int64_t)Fs[h]->n * Fs[h]->n * Fs[h]->n;
     vs[h] = Fs[h]->work_stride;
     for (int q0 = 0; q0 < nrhs[h];) {
-      const int left = nrhs[h] - q0;
-      const int R = left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
-      blocks[h].push_back({q0, R});
-      q0 += R;
+      const int R = gemv_block(nrhs[h] - q0), nv = std::min(R, nrhs[h] - q0);
+      blocks[h].push_back(Block{q0, R, nv});
+      q0 += nv;
     }
     S = std::max(S, Fs[h]->stages.size());
   }
@@ -469,7 +467,7 @@ void grouped_sweeps(const std::vector<Factor<T>*>& Fs, const std::vector<int>& n
         }
         if (jobs.empty()) return;
         Launch l{kind, 0, 0, (int)jobs.size(), push(jobs.data(), sizeof(VecJob<T>) * jobs.size()),
-                 0, 0, 0.0, 0.0};
+                 0, 0.0, 0.0};
         seq.push_back(l);
       };
       vec_launch(0);
@@ -489,18 +487,19 @@ void grouped_sweeps(const std::vector<Factor<T>*>& Fs, const std::vector<int>& n
               ent += o.tri ? 0.5 * (double)o.cols * (o.cols + 1) : (double)o.rows * o.cols;
               vecs += (double)(o.rows + o.cols) * (o.beta_one ? 1.5 : 1.0);
             }
-          for (auto [q0, R] : blocks[h]) {
-            const auto key = std::make_pair(gl.trans, R);
+          for (const Block& bk : blocks[h]) {
+            const auto key = std::make_pair(gl.trans, bk.R);
             Launch& l = meta[key];
             l.kind = 3;
             l.trans = gl.trans;
-            l.R = R;
-            buckets[key].push_back(
-                GemvSeg<T>{gl.d.as<GemvOp>(), M, wv[h] + (int64_t)q0 * vs[h], vs[h], l.nops});
-            l.nops += (int64_t)gl.h.size();
-            l.mx = std::max(l.mx, gl.get_tiles());
-            l.fl += 2.0 * ent * R;
-            l.by += sizeof(T) * (ent + R * vecs);
+            l.R = bk.R;
+            GemvSeg<T> sg = gl.seg<T>(M, wv[h] + (int64_t)bk.q0 * vs[h], vs[h]);
+            sg.first = l.ctas;
+            sg.nv = bk.nv;
+            buckets[key].push_back(sg);
+            l.ctas += gemv_ctas(sg.cnt);
+            l.fl += 2.0 * ent * bk.nv;
+            l.by += sizeof(T) * (ent + bk.nv * vecs);
           }
         }
         for (auto& [key, segs] : buckets) {
@@ -521,8 +520,8 @@ void grouped_sweeps(const std::vector<Factor<T>*>& Fs, const std::vector<int>& n
   const unsigned char* base = d.as<unsigned char>();
   for (const Launch& l : seq) {
     if (l.kind == 3) {
-      gemv_segments<T>(reinterpret_cast<const GemvSeg<T>*>(base + l.off), l.count, l.nops, l.mx,
-                       l.trans, l.R, l.fl, l.by, st);
+      gemv_segments<T>(reinterpret_cast<const GemvSeg<T>*>(base + l.off), l.count, l.ctas, l.trans,
+                       l.R, l.fl, l.by, st);
     } else {
       vec_grouped<T>(l.kind, reinterpret_cast<const VecJob<T>*>(base + l.off),
                      reinterpret_cast<const VecJob<T>*>(blob.data() + l.off), l.count, st);
@@ -600,6 +599,14 @@ class Builder {
     int nfwd = 0, nbwd = 0;
     int fwd_trans[3] = {0, 0, 0}, fwd_mat[3] = {0, 0, 0};
     int bwd_trans[3] = {0, 0, 0}, bwd_mat[3] = {0, 0, 0};
+    std::vector<GemvTask> fwd_tasks[3], bwd_tasks[3];
+    int fwd_cnt[3][4] = {}, bwd_cnt[3][4] = {};
+    void plan_lists() {
+      for (int i = 0; i < nfwd; ++i)
+        gemv_plan(fwd[i].data(), (int)fwd[i].size(), fwd_trans[i], fwd_tasks[i], fwd_cnt[i]);
+      for (int i = 0; i < nbwd; ++i)
+        gemv_plan(bwd[i].data(), (int)bwd[i].size(), bwd_trans[i], bwd_tasks[i], bwd_cnt[i]);
+    }
     std::vector<int32_t> set_g, set_p;
     std::vector<int32_t> acc_tgt, acc_src;
     std::vector<int64_t> acc_ptr;
@@ -902,6 +909,7 @@ typename Builder<T>::StageHost Builder<T>::cell_stage_host(std::shared_ptr<const
   }
   h.nfwd = h.nbwd = 2;
   h.bwd_trans[0] = h.bwd_trans[1] = 1;
+  h.plan_lists();
   // deterministic accumulation of the boundary updates: per DOF, contributions
   // in cell order (counting sort on the global index)
   std::vector<int64_t> cnt(N + 1, 0);
@@ -950,12 +958,16 @@ void Builder<T>::upload_stages(bool all) {
       s.fwd[i].trans = h.fwd_trans[i];
       s.fwd[i].mat = h.fwd_mat[i];
       upload(s.fwd[i].d, s.fwd[i].h, &F_.mem, up_st_);
+      upload(s.fwd[i].tasks, h.fwd_tasks[i], &F_.mem, up_st_);
+      std::copy(h.fwd_cnt[i], h.fwd_cnt[i] + 4, s.fwd[i].cnt);
     }
     for (int i = 0; i < h.nbwd; ++i) {
       s.bwd[i].h = std::move(h.bwd[i]);
       s.bwd[i].trans = h.bwd_trans[i];
       s.bwd[i].mat = h.bwd_mat[i];
       upload(s.bwd[i].d, s.bwd[i].h, &F_.mem, up_st_);
+      upload(s.bwd[i].tasks, h.bwd_tasks[i], &F_.mem, up_st_);
+      std::copy(h.bwd_cnt[i], h.bwd_cnt[i] + 4, s.bwd[i].cnt);
     }
     s.nset = (int64_t)h.set_g.size();
     upload(s.set_g, h.set_g, &F_.mem, up_st_);
@@ -1234,6 +1246,7 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
     h.fwd_mat[0] = 1;
     h.bwd_trans[0] = h.bwd_trans[1] = 1;
     h.bwd_mat[2] = 1;
+    h.plan_lists();
     return h;
   };
   jobs_.emplace_back(si, std::async(std::launch::async, std::move(job)));
@@ -1575,6 +1588,15 @@ struct FileIn {
       HIF_CUDA_TRY(cudaMemcpy(gl.d.as<void>(), gl.h.data(), sizeof(GemvOp) * c,
                               cudaMemcpyHostToDevice));
   }
+  // the list cut into tasks, once its ops are known to be consistent
+  void tasks(GemvList& gl, MemStats* ms) {
+    std::vector<GemvTask> t;
+    gemv_plan(gl.h.data(), (int)gl.h.size(), gl.trans, t, gl.cnt);
+    gl.tasks.alloc(sizeof(GemvTask) * t.size(), ms);
+    if (!t.empty())
+      HIF_CUDA_TRY(cudaMemcpy(gl.tasks.as<void>(), t.data(), sizeof(GemvTask) * t.size(),
+                              cudaMemcpyHostToDevice));
+  }
 };
 
 template <typename T>
@@ -1732,6 +1754,8 @@ void load_factor(Factor<T>& F, FileIn& in) {
     s.bwd.resize(nb);
     for (auto& gl : s.bwd) in.list(gl, &F.mem);
     check_stage<T>(s, N, idx_b, setg_b, setp_b, tgt_b, ptr_b, src_b);
+    for (auto* lists : {&s.fwd, &s.bwd})
+      for (auto& gl : *lists) in.tasks(gl, &F.mem);
     // the sweeps' work stride follows from the stages, as in hif_factor
     F.work_stride = std::max(F.work_stride, 2 * s.nidx);
   }
