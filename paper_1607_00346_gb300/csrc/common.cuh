@@ -97,6 +97,10 @@ struct DFront {
 };
 
 // Batched matrix product C (m x n) = beta C + alpha op(A) op(B) with k inner.
+// kzero: a triangular operand, whose zeros the kernels leave out tile by tile
+// (half of the product): KZ_B_UP op(B)[k][c] = 0 for k > c, KZ_B_LOW
+// op(B)[k][c] = 0 for k < c, KZ_A_LOW op(A)[r][k] = 0 for k > r.
+enum : int { KZ_NONE = 0, KZ_B_UP = 1, KZ_B_LOW = 2, KZ_A_LOW = 3 };
 struct GemmOp {
   int64_t A, B, C;   // element offsets from the A, B and C base pointers of the launch
   int m, n, k;
@@ -104,8 +108,21 @@ struct GemmOp {
   int transA, transB;
   float alpha, beta;
   int lower;         // 1: C is symmetric, only tiles touching its lower triangle are computed
-  int pad;
+  int kzero;
 };
+
+// The tile a block computes (longest sums first: with a triangular operand the
+// tiles of the last columns or rows have them) and the k it has to visit.
+__host__ __device__ inline int gemm_tile(const GemmOp& o, int block, int tiles) {
+  return o.kzero == KZ_B_UP || o.kzero == KZ_A_LOW ? tiles - 1 - block : block;
+}
+__host__ __device__ inline void gemm_k_range(const GemmOp& o, int rb, int tr, int cb, int tc,
+                                             int* kbeg, int* kend) {
+  *kbeg = o.kzero == KZ_B_LOW ? cb : 0;
+  const int e = o.kzero == KZ_B_UP ? cb + tc : o.kzero == KZ_A_LOW ? rb + tr : o.k;
+  *kend = e < o.k ? e : o.k;
+  if (*kbeg > *kend) *kbeg = *kend;
+}
 
 // Batched matrix-vector product on a front of the apply (see apply kernels).
 struct GemvOp {

@@ -360,8 +360,11 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmOp* __restrict__ ops, co
   const GemmOp o = ops[blockIdx.y];
   const int tm = (o.m + TILE - 1) / TILE, tn = (o.n + TILE - 1) / TILE;
   if ((int)blockIdx.x >= tm * tn) return;
-  const int rb = (blockIdx.x % tm) * TILE, cb = (blockIdx.x / tm) * TILE;
+  const int tile = gemm_tile(o, blockIdx.x, tm * tn);
+  const int rb = (tile % tm) * TILE, cb = (tile / tm) * TILE;
   if (o.lower && cb >= rb + TILE) return;
+  int kbeg, kend;
+  gemm_k_range(o, rb, TILE, cb, TILE, &kbeg, &kend);
   const T* A = Ab + o.A;
   const T* B = Bb + o.B;
   T* C = Cb + o.C;
@@ -369,7 +372,7 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmOp* __restrict__ ops, co
   __shared__ T Bs[KC][TILE + 4];
   TileAcc<T> acc;
   acc.zero();
-  for (int k0 = 0; k0 < o.k; k0 += KC) {
+  for (int k0 = kbeg; k0 < kend; k0 += KC) {
     for (int e = threadIdx.x; e < KC * TILE; e += 256) {
       int rr, kk;
       // choose the thread mapping that reads memory contiguously
@@ -658,8 +661,8 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
         const int64_t boff = (i0 + s) + (int64_t)i0 * ld;
         const int64_t aoff = i0 + (int64_t)i0 * ld;
         const int64_t coff = (i0 + s) + (int64_t)(i0 + s) * ld;
-        tops.push_back(GemmOp{h.K + boff, h.P + aoff, scr, rs, s, s, ld, ld, rs, 0, 0, 1.f, 0.f, 0, 0});
-        rops.push_back(GemmOp{h.P + coff, scr, h.P + boff, rs, s, rs, ld, rs, ld, 0, 0, -1.f, 0.f, 0, 0});
+        tops.push_back(GemmOp{h.K + boff, h.P + aoff, scr, rs, s, s, ld, ld, rs, 0, 0, 1.f, 0.f, 0, KZ_B_LOW});
+        rops.push_back(GemmOp{h.P + coff, scr, h.P + boff, rs, s, rs, ld, rs, ld, 0, 0, -1.f, 0.f, 0, KZ_A_LOW});
         scr += (int64_t)rs * s;
       }
     }
@@ -696,7 +699,7 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
     const int nb = h.n - h.p;
     if (nb <= 0 || h.p <= 0) continue;
     const int ld = h.ld;
-    GemmOp x{h.K + h.p, h.P, h.P + h.p, nb, h.p, h.p, ld, ld, ld, 0, 1, 1.f, 0.f, 0, 0};
+    GemmOp x{h.K + h.p, h.P, h.P + h.p, nb, h.p, h.p, ld, ld, ld, 0, 1, 1.f, 0.f, 0, KZ_B_UP};
     GemmOp s{h.P + h.p, h.P + h.p, h.K + h.p + (int64_t)h.p * ld, nb, nb, h.p, ld, ld, ld, 0, 1,
              -1.f, 1.f, 1, 0};
     xo.push_back(x);
@@ -734,7 +737,7 @@ void gemm_batched(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const T* A
     const int nb = std::min(MAX_GRID_Y, nops - f0);
     double fl = 0;
     if (prof_enabled())
-      for (int i = f0; i < f0 + nb; ++i) fl += 2.0 * h_ops[i].m * (double)h_ops[i].n * h_ops[i].k;
+      for (int i = f0; i < f0 + nb; ++i) fl += 2.0 * h_ops[i].m * (double)h_ops[i].n * h_ops[i].k * (h_ops[i].kzero ? 0.5 : 1.0);
     ProfScope ps(name, st, fl, 0.0);
     k_gemm<T><<<dim3(mt, nb), 256, 0, st>>>(d_ops + f0, Abase, Bbase, Cbase);
     HIF_CHECK_LAUNCH();

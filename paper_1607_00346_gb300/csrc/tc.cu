@@ -77,7 +77,8 @@ __global__ void __launch_bounds__(TC_M + TN, KC == 16 ? (TN == 128 ? 3 : 2) : 1)
   const GemmOp o = ops[blockIdx.y];
   const int tm_n = (o.m + TC_M - 1) / TC_M, tn_n = (o.n + TN - 1) / TN;
   if ((int)blockIdx.x >= tm_n * tn_n) return;
-  const int rb = (blockIdx.x % tm_n) * TC_M, cb = (blockIdx.x / tm_n) * TN;
+  const int tile = gemm_tile(o, blockIdx.x, tm_n * tn_n);
+  const int rb = (tile % tm_n) * TC_M, cb = (tile / tm_n) * TN;
   if (o.lower && cb >= rb + TC_M) return;
   const float* A = Ab + o.A;
   const float* B = Bb + o.B;
@@ -108,9 +109,13 @@ __global__ void __launch_bounds__(TC_M + TN, KC == 16 ? (TN == 128 ? 3 : 2) : 1)
   const uint32_t idesc = idesc_tf32(TC_M, TN);
   // split K (gridDim.z > 1): this CTA takes chunks [cbeg, cbeg + nchunk) of
   // the product and leaves its partial tile in the work space Wk
+  // (shares of the whole K, so that they do not depend on the tile's shape)
+  int kbeg, kend;
+  gemm_k_range(o, rb, TC_M, cb, TN, &kbeg, &kend);   // kbeg: a multiple of TN
   const int nch_all = (o.k + KC - 1) / KC;
-  const int cbeg = (int)(((int64_t)nch_all * blockIdx.z) / gridDim.z);
-  const int nchunk = (int)(((int64_t)nch_all * (blockIdx.z + 1)) / gridDim.z) - cbeg;
+  const int cbeg = max(kbeg / KC, (int)(((int64_t)nch_all * blockIdx.z) / gridDim.z));
+  const int nchunk = max(0, min((kend + KC - 1) / KC,
+                                (int)(((int64_t)nch_all * (blockIdx.z + 1)) / gridDim.z)) - cbeg);
   uint32_t phase[2] = {0u, 0u};
   // outstanding[s]: products committed on buffer s whose completion this
   // thread has not yet seen (at most one commit per buffer is in flight)
@@ -418,7 +423,8 @@ void gemm_tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const float* Ab
     mmax = std::max(mmax, h_ops[i].m);
     nmax = std::max(nmax, h_ops[i].n);
     kmax = std::max(kmax, h_ops[i].k);
-    fl += 2.0 * h_ops[i].m * (double)h_ops[i].n * h_ops[i].k * (h_ops[i].lower ? 0.5 : 1.0);
+    fl += 2.0 * h_ops[i].m * (double)h_ops[i].n * h_ops[i].k *
+          (h_ops[i].lower || h_ops[i].kzero ? 0.5 : 1.0);
   }
   // built-in rule: few rows (one tile, mostly padding): fewer, longer
   // chunks; wide products: 128 x 256 tiles (half the A staging per product)
