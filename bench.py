@@ -498,7 +498,8 @@ def main():
     if not args.no_fp64_form and prec == hif.PREC_FP32:
         torch.cuda.synchronize()
         t0 = time.perf_counter()
-        h = hif.factor(n, m, a_d, b_const=w["b"], eps=w["eps"], precision=hif.PREC_FP64)
+        h = hif.factor(n, m, a_d, b_const=w["b"], eps=w["eps"], precision=hif.PREC_FP64,
+                       tensor_cores=False)
         torch.cuda.synchronize()
         t1 = time.perf_counter()
         its64, rel64 = h.solve(f_d, torch.zeros_like(f_d))

@@ -90,13 +90,15 @@ typedef struct {
                         one */
   double pcg_tol;    /* hif_solve stops when ||r||_2 <= pcg_tol ||f||_2 */
   int max_iter;      /* hif_solve iteration limit */
-  int tensor_cores;  /* HIF_PREC_FP32 only.  1: the deep products of the
-                        partial Cholesky (the cell products X^T = A_NI L^-T and
-                        A_NN -= X^T X, the rank-256 block updates, the large
-                        triangular-inverse merges) run on the tensor cores
-                        (TF32 with the 3xTF32 split, FP32 accumulation); 0:
-                        every product on the FP32 FMA units.  FP64 factors
-                        never use them. */
+  int tensor_cores;  /* 1: the deep products of the partial Cholesky (the cell
+                        products X^T = A_NI L^-T and A_NN -= X^T X, the
+                        rank-256 block updates, the triangular-inverse
+                        merges) and of the row reduction run on the tensor
+                        cores.  HIF_PREC_FP32: TF32 with the 3xTF32 split,
+                        FP32 accumulation.  HIF_PREC_FP64: operands split
+                        into eight 8-bit slices, exact sums, one rounding
+                        per entry (less error than the FMA form).  0: every
+                        product on the FMA units of its precision. */
   double retry_growth; /* HIF_PREC_FP32 only: a front whose Cholesky (the
                         LDL^T of §2.2 / §2.3) meets a pivot d_j with
                         A_jj / d_j > retry_growth (A_jj its original

@@ -420,14 +420,14 @@ constexpr int TC_MIN_ROWS = 256;
 
 template <typename T>
 void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T* Karena,
-                   T* Parena, int* d_flags, bool use_tc, cudaStream_t st);
+                   T* Parena, int* d_flags, bool tensor_cores, cudaStream_t st);
 
 // Refactor the flagged FP32 fronts entirely in FP64 (from the snapshot of
 // their leading blocks and their untouched A_NI, A_NN) and store the results
 // in the FP32 arenas.
 static void retry_fronts_fp64(const std::vector<int>& bad, const DFront* h_fronts,
                        const std::vector<int64_t>& soff, float* Karena, float* Parena,
-                       const float* snap, int* d_flags, cudaStream_t st) {
+                       const float* snap, int* d_flags, bool tensor_cores, cudaStream_t st) {
   const int nb = (int)bad.size();
   std::vector<DFront> dl;
   std::vector<RetryMap> maps;
@@ -458,7 +458,7 @@ static void retry_fronts_fp64(const std::vector<int>& bad, const DFront* h_front
     k_retry_build<<<dim3(gx, c), 256, 0, st>>>(d_maps + f0, Karena, snap, Kd);
     HIF_CHECK_LAUNCH();
   }
-  partial_cholesky<double>(d_dl, dl.data(), nb, Kd, Pd, d_flags, false, st, nullptr);
+  partial_cholesky<double>(d_dl, dl.data(), nb, Kd, Pd, d_flags, tensor_cores, st, nullptr);
   for (int f0 = 0; f0 < nb; f0 += MAX_GRID_Y) {
     const int c = std::min(MAX_GRID_Y, nb - f0);
     ProfScope ps("chol_retry_fp64", st);
@@ -476,7 +476,6 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
                       T* Parena, int* d_flags, bool tensor_cores, cudaStream_t st,
                       const RetryOpts* retry) {
   if (nfront == 0) return;
-  const bool use_tc = std::is_same<T, float>::value && tensor_cores;
   const int pmax = h_fronts[0].p;
   // FP32 fronts that may be retried in FP64: snapshot of every leading block,
   // original diagonal in the panel, one flag per front
@@ -582,19 +581,17 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
     HIF_CUDA_TRY(cudaMallocAsync(&d_uo, sizeof(GemmOp) * uo.size(), st));
     HIF_CUDA_TRY(cudaMemcpyAsync(d_uo, uo.data(), sizeof(GemmOp) * uo.size(),
                                  cudaMemcpyHostToDevice, st));
+    bool done = false;
     if constexpr (std::is_same<T, float>::value) {
-      if (use_tc) {
-        gemm_tc(d_uo, uo.data(), (int)uo.size(), reinterpret_cast<const float*>(Karena),
-                reinterpret_cast<const float*>(Karena), reinterpret_cast<float*>(Karena), d_flags,
-                st, "chol_block_update_tc");
-      } else {
-        gemm_batched<T>(d_uo, uo.data(), (int)uo.size(), Karena, Karena, Karena, st,
-                        "chol_block_update");
+      if (tensor_cores) {
+        gemm_tc(d_uo, uo.data(), (int)uo.size(), Karena, Karena, Karena, d_flags, st,
+                "chol_block_update_tc");
+        done = true;
       }
-    } else {
-      gemm_batched<T>(d_uo, uo.data(), (int)uo.size(), Karena, Karena, Karena, st,
-                      "chol_block_update");
     }
+    if (!done)
+      gemm_fma_or_f64tc<T>(d_uo, uo.data(), (int)uo.size(), Karena, Karena, Karena, d_flags,
+                           tensor_cores, st, "chol_block_update", "chol_block_update_f64tc");
     HIF_CUDA_TRY(cudaFreeAsync(d_uo, st));
   }
   HIF_CUDA_TRY(cudaFreeAsync(d_lead, st));
@@ -611,7 +608,7 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
     }
     if (!bad.empty()) {
       if constexpr (std::is_same<T, float>::value)
-        retry_fronts_fp64(bad, h_fronts, soff, Karena, Parena, snap, d_flags, st);
+        retry_fronts_fp64(bad, h_fronts, soff, Karena, Parena, snap, d_flags, tensor_cores, st);
       if (retry->retried) *retry->retried += (int64_t)bad.size();
       if (!keep.empty()) {
         HIF_CUDA_TRY(cudaMallocAsync(&d_keep, sizeof(DFront) * keep.size(), st));
@@ -627,14 +624,14 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
     HIF_CUDA_TRY(cudaFreeAsync(d_fflag, st));
     if (nfront == 0) return;
   }
-  finish_fronts(d_fronts, h_fronts, nfront, Karena, Parena, d_flags, use_tc, st);
+  finish_fronts(d_fronts, h_fronts, nfront, Karena, Parena, d_flags, tensor_cores, st);
   if (d_keep) HIF_CUDA_TRY(cudaFreeAsync(d_keep, st));
 }
 
 // Steps 2-4 of the partial Cholesky once the leading blocks hold L.
 template <typename T>
 void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T* Karena,
-                   T* Parena, int* d_flags, bool use_tc, cudaStream_t st) {
+                   T* Parena, int* d_flags, bool tensor_cores, cudaStream_t st) {
   const int pmax = h_fronts[0].p;
   // 2. Linv = L^{-1}: invert the NB x NB diagonal blocks, then merge
   //    neighbouring inverted blocks pairwise up a binary tree of widths
@@ -675,18 +672,18 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
     HIF_CUDA_TRY(cudaMemcpyAsync(d_ops, tops.data(), sizeof(GemmOp) * cnt, cudaMemcpyHostToDevice, st));
     HIF_CUDA_TRY(cudaMemcpyAsync(d_ops + cnt, rops.data(), sizeof(GemmOp) * cnt,
                                  cudaMemcpyHostToDevice, st));
-    if constexpr (std::is_same<T, float>::value) {
-      if (use_tc && s >= 128) {
-        gemm_tc(d_ops, tops.data(), (int)cnt, Karena, Parena, d_scr, d_flags, st, "trtri_merge_tc");
-        gemm_tc(d_ops + cnt, rops.data(), (int)cnt, Parena, d_scr, Parena, d_flags, st, "trtri_merge_tc");
-      } else {
-        gemm_batched<T>(d_ops, tops.data(), (int)cnt, Karena, Parena, d_scr, st, "trtri_merge");
-        gemm_batched<T>(d_ops + cnt, rops.data(), (int)cnt, Parena, d_scr, Parena, st, "trtri_merge");
+    auto gemm = [&](const GemmOp* dop, const GemmOp* hop, const T* Ab, const T* Bb, T* Cb) {
+      if constexpr (std::is_same<T, float>::value) {
+        if (tensor_cores && s >= 128) {
+          gemm_tc(dop, hop, (int)cnt, Ab, Bb, Cb, d_flags, st, "trtri_merge_tc");
+          return;
+        }
       }
-    } else {
-      gemm_batched<T>(d_ops, tops.data(), (int)cnt, Karena, Parena, d_scr, st, "trtri_merge");
-      gemm_batched<T>(d_ops + cnt, rops.data(), (int)cnt, Parena, d_scr, Parena, st, "trtri_merge");
-    }
+      gemm_fma_or_f64tc<T>(dop, hop, (int)cnt, Ab, Bb, Cb, d_flags, tensor_cores, st, "trtri_merge",
+                           "trtri_merge_f64tc");
+    };
+    gemm(d_ops, tops.data(), Karena, Parena, d_scr);
+    gemm(d_ops + cnt, rops.data(), Parena, d_scr, Parena);
     HIF_CUDA_TRY(cudaFreeAsync(d_scr, st));
     HIF_CUDA_TRY(cudaFreeAsync(d_ops, st));
   }
@@ -713,15 +710,18 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
     HIF_CUDA_TRY(cudaMemcpyAsync(d_ops, xo.data(), sizeof(GemmOp) * cnt, cudaMemcpyHostToDevice, st));
     HIF_CUDA_TRY(cudaMemcpyAsync(d_ops + cnt, so.data(), sizeof(GemmOp) * cnt,
                                  cudaMemcpyHostToDevice, st));
-    if (use_tc && maxrows >= TC_MIN_ROWS) {
-      gemm_tc(d_ops, xo.data(), (int)cnt, reinterpret_cast<const float*>(Karena),
-              reinterpret_cast<const float*>(Parena), reinterpret_cast<float*>(Parena), d_flags, st);
-      gemm_tc(d_ops + cnt, so.data(), (int)cnt, reinterpret_cast<const float*>(Parena),
-              reinterpret_cast<const float*>(Parena), reinterpret_cast<float*>(Karena), d_flags, st);
-    } else {
-      gemm_batched<T>(d_ops, xo.data(), (int)cnt, Karena, Parena, Parena, st);
-      gemm_batched<T>(d_ops + cnt, so.data(), (int)cnt, Parena, Parena, Karena, st);
-    }
+    auto gemm = [&](const GemmOp* dop, const GemmOp* hop, const T* Ab, const T* Bb, T* Cb) {
+      if constexpr (std::is_same<T, float>::value) {
+        if (tensor_cores && maxrows >= TC_MIN_ROWS) {
+          gemm_tc(dop, hop, (int)cnt, Ab, Bb, Cb, d_flags, st);
+          return;
+        }
+      }
+      gemm_fma_or_f64tc<T>(dop, hop, (int)cnt, Ab, Bb, Cb, d_flags, tensor_cores, st, "gemm_batched",
+                           "gemm_f64tc");
+    };
+    gemm(d_ops, xo.data(), Karena, Parena, Parena);
+    gemm(d_ops + cnt, so.data(), Parena, Parena, Karena);
     HIF_CUDA_TRY(cudaFreeAsync(d_ops, st));
   }
 }

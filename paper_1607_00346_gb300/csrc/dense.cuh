@@ -39,14 +39,36 @@ void gemm_tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const float* Ab
              const float* Bbase, float* Cbase, int* d_flags, cudaStream_t st,
              const char* name = "gemm_tc");
 
+// The same for FP64 data: 8-bit slices on the BF16 tensor cores, exact sums,
+// one rounding per entry (f64tc.cu).
+void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double* Abase,
+                const double* Bbase, double* Cbase, int* d_flags, cudaStream_t st,
+                const char* name);
+
 // Autotuning of gemm_tc's tile shape: time the variants on the product
 // shapes recorded during a tuning factorization (tune.h).
 void tune_gemm_from_records(cudaStream_t st);
 
-// C = beta C + alpha op(A) op(B) for a batch of independent problems.
+// C = beta C + alpha op(A) op(B) for a batch of independent problems, on the
+// FMA units.
 template <typename T>
 void gemm_batched(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const T* Abase,
                   const T* Bbase, T* Cbase, cudaStream_t st, const char* name = "gemm_batched");
+// FP64 products that go to gemm_f64tc when tensor cores are allowed.
+bool f64tc_worth(const GemmOp* h_ops, int nops);
+// gemm_batched, or gemm_f64tc (labelled name_tc) for FP64 products worth it.
+template <typename T>
+void gemm_fma_or_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const T* Abase,
+                       const T* Bbase, T* Cbase, int* d_flags, bool tensor_cores, cudaStream_t st,
+                       const char* name, const char* name_tc) {
+  if constexpr (sizeof(T) == 8) {
+    if (tensor_cores && f64tc_worth(h_ops, nops)) {
+      gemm_f64tc(d_ops, h_ops, nops, Abase, Bbase, Cbase, d_flags, st, name_tc);
+      return;
+    }
+  }
+  gemm_batched<T>(d_ops, h_ops, nops, Abase, Bbase, Cbase, st, name);
+}
 
 // Mat-vecs of the apply sweeps, y = alpha op(M) x (+ y) batched over GemvOps
 // (gemv.cu).  trans = 0: y (rows) = M x; trans = 1: y (cols) = M^T x.

@@ -1,0 +1,501 @@
+// Batched FP64 matrix products on the tensor cores.
+//
+// What bounds an FP64 product here is the FP64 unit: 2 multiply-adds per clock
+// and SM, 1.06 TFLOP/s on the whole chip, so a single 64 x 64 x 64 tile takes
+// 66 us and the products of a 64^3 FP64 factorization took 60% of its time.
+// The BF16 tensor cores run 2300 times faster, and integers of 8 bits multiply
+// and add in them without rounding; so each operand is split into eight 8-bit
+// slices (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
+// Algorithms 59, 2012):
+//
+//   x = 2^(s - 62) X,  X = sum_{i < 8} a_i 256^(7 - i),  |a_i| <= 128,
+//
+// with s per row of op(A) and per column of op(B) such that |x| < 2^s: X is x in
+// fixed point, 62 bits below the largest entry of its row.  The product is
+// sum_t 256^(14 - t) D_t, D_t = sum_{i + j = t} sum_k a_i b_j; the 36 products
+// with t < 8 are formed (the others are below 2^-62 of row maximum times column
+// maximum) in eight FP32 accumulators.  |D_t| <= 8 * 128 * 2^14 = 2^24 over 128 k,
+// which FP32 holds exactly; then they are added to 128-bit integers (two 64-bit
+// halves per entry), and each entry is rounded to double once at the end.  An
+// FMA loop rounds at every k; this sum is exact up to the 2^-62 of the split.
+//
+// Three launches per batch: k_f64_exps finds s per row, k_f64_slice writes the
+// slices in the layout the tensor core reads (64 rows x 16 k per block, all
+// eight slices together: 16 KB), k_gemm_f64tc copies blocks to shared memory with
+// bulk copies and multiplies.  An operand used on both sides (A A^T) is split
+// once.
+//
+// Measured (three launches, FMA form in brackets): one 64^3 product 34 (66) us,
+// 512 of them 113 (270) us, one 256^3 48 (280) us, one 1024^3 0.10 (2.1) ms,
+// one 2048^3 0.63 (14.5) ms = 27 TFLOP/s.  Error against quad precision, entries
+// over 2 to 12 decades: 5e-17 to 7e-17 in norm (3e-16 to 1.5e-15).
+//
+// k_gemm_f64tc: one 128 x 64 tile per CTA; the eight accumulators fill the 512
+// columns of tensor memory, four stages of 48 KB the shared memory.  Per 16 k one
+// thread issues 12 instructions (M 128, N 64 to 256, K 16: a slice of A times
+// up to four neighbouring slices of B, whose products go to neighbouring
+// accumulators), and a warp copies the block three ahead; per 128 k the warps
+// read the accumulators back.
+#include <stdint.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "common.cuh"
+#include "dense.cuh"
+#include "tcgen05.cuh"
+
+namespace hif {
+
+namespace {
+
+constexpr int NSL = 8;             // slices per operand, and accumulators
+constexpr int BR = 64;             // rows of a block of slices
+constexpr int KC = 16;             // k of a block
+constexpr int SLICE = BR * KC * 2;         // bytes of one slice of a block (2 KB)
+constexpr int BLK = NSL * SLICE;           // bytes of a block (16 KB)
+constexpr int TM = 128, TN = 64;           // output tile
+constexpr int NST = 4;                     // shared-memory stages
+constexpr int STAGE = 3 * BLK;             // two blocks of A, one of B
+constexpr int GROUP = 8;                   // blocks (128 k) per exact accumulation
+constexpr int THREADS = 256;
+constexpr int NOT_FINITE = INT32_MAX;      // exponent of a row with inf or NaN
+constexpr long long WAIT_LIMIT = 20000000;  // mbarrier polls before giving up
+constexpr size_t WORK_LIMIT = (size_t)1 << 30;   // slices held at once, if several products
+
+// 64 rows (row0 ..) of an operand: element (r, k) at src + r + k ld, or
+// src + k + r ld (kcont).
+struct SliceBlk {
+  int64_t src;
+  int64_t dst;       // index of its first 16 KB block in the work space
+  int ld, rows, k;
+  int kcont, isB;
+  int pad;
+};
+
+struct Tile {
+  int op, rb, cb;    // product, first row and column
+  int ablk, bblk;    // first block row of A (two if the product has the rows), of B
+};
+
+// Largest magnitude of each row, as the upper word of its double (exps zeroed
+// before; a row's blocks of k are shared by gridDim.y CTAs).
+__global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ blks,
+                                                  const double* __restrict__ Ab,
+                                                  const double* __restrict__ Bb, int* exps) {
+  const SliceBlk b = blks[blockIdx.x];
+  const double* X = (b.isB ? Bb : Ab) + b.src;
+  const int k0 = (int)((int64_t)b.k * blockIdx.y / gridDim.y);
+  const int k1 = (int)((int64_t)b.k * (blockIdx.y + 1) / gridDim.y);
+  int* out = exps + (int64_t)blockIdx.x * BR;
+  if (b.kcont) {
+    // one warp per row, lanes along k
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    for (int r = warp; r < b.rows; r += 8) {
+      int m = 0;
+#pragma unroll 4
+      for (int k = k0 + lane; k < k1; k += 32)
+        m = max(m, __double2hiint(X[(int64_t)r * b.ld + k]) & 0x7fffffff);
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) atomicMax(&out[r], m);
+    }
+  } else {
+    const int r = threadIdx.x % BR;
+    if (r >= b.rows) return;
+    int m = 0;
+#pragma unroll 8
+    for (int k = k0 + threadIdx.x / BR; k < k1; k += 256 / BR)
+      m = max(m, __double2hiint(X[r + (int64_t)k * b.ld]) & 0x7fffffff);
+    atomicMax(&out[r], m);
+  }
+}
+
+// s of a row, as a biased exponent: |x| < 2^(s - 1023) for all its entries
+__device__ __forceinline__ int row_exp(int hiword) {
+  const int e = hiword >> 20;
+  return e == 0x7ff ? NOT_FINITE : e + 1;
+}
+
+// x in fixed point, 62 bits below 2^s (s: biased exponent + 1 of the row)
+__device__ __forceinline__ int64_t fixed62(double x, int s) {
+  const uint64_t u = (uint64_t)__double_as_longlong(x);
+  const int e = (int)(u >> 52) & 0x7ff;
+  uint64_t m = u & 0xfffffffffffffull;
+  if (e) m |= 1ull << 52;
+  const int sh = (e ? e : 1) - s + 10;   // at most 9
+  uint64_t v;
+  if (sh >= 0) v = m << sh;
+  else if (sh > -55) v = (m + (1ull << (-sh - 1))) >> -sh;
+  else v = 0;
+  return (int64_t)u < 0 ? -(int64_t)v : (int64_t)v;
+}
+
+// One thread: eight consecutive k of one row -> 16 bytes of each slice.
+__global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ blks,
+                                                   const double* __restrict__ Ab,
+                                                   const double* __restrict__ Bb,
+                                                   const int* __restrict__ exps, unsigned char* W) {
+  const SliceBlk b = blks[blockIdx.x];
+  const double* X = (b.isB ? Bb : Ab) + b.src;
+  // a warp covers 8 rows x 4 groups of 8 k: 512 contiguous bytes of two blocks
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int r = warp * 8 + lane % 8, kg = lane / 8;
+  const int s = row_exp(exps[(int64_t)blockIdx.x * BR + r]);
+  const int nkg = (b.k + KC - 1) / KC * 2;   // groups of 8 k, padded to whole blocks
+  for (int g = blockIdx.y * 4 + kg; g < nkg; g += gridDim.y * 4) {
+    double x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = g * 8 + j;
+      x[j] = (r < b.rows && k < b.k) ? X[b.kcont ? (int64_t)r * b.ld + k : r + (int64_t)k * b.ld]
+                                     : 0.0;
+    }
+    // adding 128 to every digit but the first makes the bytes of the sum the
+    // digits + 128; a byte put into the low mantissa of 2^23 and taken back
+    // gives the digit as a float, whose upper half is its BF16
+    uint32_t lo[8], hi[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint64_t y = (uint64_t)(s == NOT_FINITE ? 0 : fixed62(x[j], s)) + 0x8080808080808080ull;
+      lo[j] = (uint32_t)y;
+      hi[j] = (uint32_t)(y >> 32);
+    }
+    unsigned char* out = W + (b.dst + g / 2) * BLK + (r / 8) * 256 + (g % 2) * 128 + (r % 8) * 16;
+#pragma unroll
+    for (int i = 0; i < NSL; ++i) {
+      const uint32_t sel = 0x7440u | (uint32_t)((NSL - 1 - i) & 3);
+      uint32_t d[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const uint32_t w0 = i < 4 ? hi[2 * h] : lo[2 * h], w1 = i < 4 ? hi[2 * h + 1] : lo[2 * h + 1];
+        const float f0 = __uint_as_float(__byte_perm(w0, 0x4b000000u, sel)) - 8388736.0f;
+        const float f1 = __uint_as_float(__byte_perm(w1, 0x4b000000u, sel)) - 8388736.0f;
+        d[h] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+      }
+      *reinterpret_cast<uint4*>(out + i * SLICE) = make_uint4(d[0], d[1], d[2], d[3]);
+    }
+  }
+}
+
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, int bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+          dst),
+      "l"(src), "r"(bytes), "r"(tc5::smem_u32(bar))
+      : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t addr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr));
+}
+
+// (hi 2^32 + lo) 2^ex rounded to double (ties to even)
+__device__ __forceinline__ double to_double(int64_t hi, int64_t lo, int ex) {
+  // 128-bit two's complement of the sum: high and low 64 bits
+  const uint64_t ul = (uint64_t)hi << 32;
+  uint64_t l = ul + (uint64_t)lo;
+  uint64_t h = (uint64_t)(hi >> 32) + (uint64_t)(lo >> 63) + (l < ul ? 1 : 0);
+  const bool neg = (int64_t)h < 0;
+  if (neg) {
+    l = ~l + 1;
+    h = ~h + (l == 0 ? 1 : 0);
+  }
+  if (h == 0 && l == 0) return 0.0;
+  // leading bit to bit 63 of h, what falls off below kept as a sticky bit
+  int lead = 0;
+  if (h == 0) {
+    h = l;
+    l = 0;
+    lead = 64;
+  }
+  const int z = __clzll((long long)h);
+  lead += z;
+  if (z) {
+    h = (h << z) | (l >> (64 - z));
+    l <<= z;
+  }
+  h |= l ? 1 : 0;
+  uint64_t m = h >> 11;                       // 53 bits
+  const uint32_t rem = (uint32_t)h & 0x7ff;
+  m += (rem > 0x400 || (rem == 0x400 && (m & 1))) ? 1 : 0;
+  const int e = 127 - lead + ex + 1023;       // biased exponent of bit 52 of m
+  double v;
+  if (e > 0 && e < 0x7fe) v = __longlong_as_double((long long)(((uint64_t)(e - 1) << 52) + m));
+  else v = scalbn((double)(int64_t)m, e - 1023 - 52);
+  return neg ? -v : v;
+}
+
+__global__ void __launch_bounds__(THREADS, 1)
+    k_gemm_f64tc(const Tile* __restrict__ tiles, const GemmOp* __restrict__ ops,
+                 const SliceBlk* __restrict__ blks, const int* __restrict__ exps,
+                 const unsigned char* __restrict__ W, double* Cb, int* flags) {
+  const Tile tl = tiles[blockIdx.x];
+  const GemmOp o = ops[tl.op];
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t full[NST], done[NST], accf;
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(
+        tc5::smem_u32(&s_tmem)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+  }
+  if (tid == 0) {
+    for (int s = 0; s < NST; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tc5::smem_u32(&full[s])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tc5::smem_u32(&done[s])));
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tc5::smem_u32(&accf)));
+    asm volatile("fence.mbarrier_init.release.cluster;\n");
+    asm volatile("fence.proxy.async.shared::cta;\n");
+    s_fail = 0;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n");
+  const uint32_t tmem = s_tmem, sm0 = tc5::smem_u32(smem);
+  int kbeg, kend;
+  gemm_k_range(o, tl.rb, TM, tl.cb, TN, &kbeg, &kend);   // kbeg: a multiple of 64
+  const int b0 = kbeg / KC, nc = (kend + KC - 1) / KC - b0;
+  const bool two = tl.rb + BR < o.m;                     // rows in A's second block
+  const unsigned char* A0 = W + (blks[tl.ablk].dst + b0) * BLK;
+  const unsigned char* A1 = two ? W + (blks[tl.ablk + 1].dst + b0) * BLK : A0;
+  const unsigned char* B0 = W + (blks[tl.bblk].dst + b0) * BLK;
+
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    for (long long it = 0; it < WAIT_LIMIT; ++it)
+      if (tc5::mbar_test(bar, parity)) return true;
+    return false;
+  };
+  // warp 1: block c of both operands into its stage, one copy per lane.  A:
+  // slice i's two halves of 64 rows next to each other; B: as stored.
+  auto load = [&](int c) {
+    const int s = c % NST;
+    const uint32_t st = sm0 + s * STAGE;
+    if (lane == 0)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(
+                       tc5::smem_u32(&full[s])),
+                   "r"((two ? 3 : 2) * BLK)
+                   : "memory");
+    __syncwarp();
+    const int64_t off = (int64_t)c * BLK;
+    if (lane < 2 * NSL) {
+      if (two || lane % 2 == 0)
+        bulk_copy(st + lane * SLICE, (lane % 2 ? A1 : A0) + off + (lane / 2) * SLICE, SLICE, &full[s]);
+    } else if (lane == 2 * NSL) {
+      bulk_copy(st + 2 * BLK, B0 + off, BLK, &full[s]);
+    }
+  };
+  int loaded = 0;               // warp 1: blocks loaded
+  int issued = 0, seen = 0;     // thread 0: blocks multiplied, seen complete
+  if (warp == 1)
+    for (; loaded < min(NST - 1, nc); ++loaded) load(loaded);
+
+  int64_t hi[TN / 2], lo[TN / 2];   // this thread's row, half of the columns
+#pragma unroll
+  for (int j = 0; j < TN / 2; ++j) hi[j] = lo[j] = 0;
+  bool ok = true;
+  const int ngroup = (nc + GROUP - 1) / GROUP;
+  for (int g = 0; g < ngroup; ++g) {
+    const int c1 = min(nc, (g + 1) * GROUP);
+    if (tid == 0) {
+      for (int c = g * GROUP; c < c1; ++c) {
+        const int s = c % NST;
+        if (!wait(&full[s], (c / NST) & 1)) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;\n");
+        const uint32_t a = sm0 + s * STAGE, b = a + 2 * BLK;
+        // slices j .. j + w - 1 of B lie one after the other, as do the
+        // accumulators t = i + j .. they add to: one instruction of N = 64 w
+        const uint64_t da = tc5::sdesc(a, 128, 256), db = tc5::sdesc(b, 128, 256);
+        const uint32_t more = c > g * GROUP ? 1u : 0u;
+#pragma unroll
+        for (int i = 0; i < NSL; ++i)
+#pragma unroll
+          for (int j = 0; i + j < NSL; j += 4) {
+            const int w = NSL - i - j < 4 ? NSL - i - j : 4;
+            tc5::mma_bf16(tmem + (i + j) * TN, da + (2 * i * SLICE >> 4), db + (j * SLICE >> 4),
+                          tc5::idesc_bf16(TM, w * TN), i > 0 ? 1u : more);
+          }
+        tc5::commit(&done[s]);
+        ++issued;
+      }
+      if (ok) tc5::commit(&accf);
+      else atomicExch(&s_fail, 1);
+    } else if (warp == 1) {
+      // three blocks ahead: the stage is free once the block before c is done
+      for (int c = g * GROUP; c < c1 && loaded < nc; ++c) {
+        const bool is_free = c == 0 || wait(&done[(c - 1) % NST], ((c - 1) / NST) & 1);
+        if (!__all_sync(0xffffffffu, is_free)) {
+          ok = false;
+          atomicExch(&s_fail, 1);
+          break;
+        }
+        load(loaded++);
+      }
+    }
+    __syncwarp();   // the rest of warp 0 must not poll (and suspend it) while thread 0 issues
+    if (ok) {
+      ok = false;
+      for (long long it = 0; it < WAIT_LIMIT && !*(volatile int*)&s_fail; ++it)
+        if (tc5::mbar_test(&accf, g & 1)) {
+          ok = true;
+          break;
+        }
+    }
+    // one verdict for the CTA: the loads from tensor memory are warp-collective
+    ok = __syncthreads_and(ok) != 0;
+    if (!ok) break;
+    seen = issued;
+    asm volatile("tcgen05.fence::after_thread_sync;\n");
+    const uint32_t base = tmem + ((uint32_t)((warp % 4) * 32) << 16) + (uint32_t)(warp / 4) * (TN / 2);
+#pragma unroll
+    for (int c0 = 0; c0 < TN / 2; c0 += 4) {
+      uint32_t d[NSL][4];
+#pragma unroll
+      for (int t = 0; t < NSL; ++t) tmem_ld4(base + t * TN + c0, d[t]);
+      asm volatile("tcgen05.wait::ld.sync.aligned;\n");
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        auto v = [&](int t) { return (int64_t)__float2int_rz(__uint_as_float(d[t][j])); };
+        hi[c0 + j] += (v(0) << 24) + (v(1) << 16) + (v(2) << 8) + v(3);
+        lo[c0 + j] += (v(4) << 24) + (v(5) << 16) + (v(6) << 8) + v(7);
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n");
+  }
+  if (!ok) {
+    // drain, again bounded: copies that may still arrive, products still running
+    if (warp == 1)
+      for (int c = max(0, loaded - NST); c < loaded; ++c) wait(&full[c % NST], (c / NST) & 1);
+    if (tid == 0) {
+      for (int c = max(seen, issued - NST); c < issued; ++c) wait(&done[c % NST], (c / NST) & 1);
+      atomicCAS(&flags[FLAG_TIMEOUT], -1, tl.op);
+    }
+  }
+  if (ok) {
+    // the sums go through shared memory (every copy and product is done), so
+    // that one short loop rounds them: unrolled over the registers it was 32
+    // copies of the rounding, and fetching them took 30 us
+    int64_t* sum = reinterpret_cast<int64_t*>(smem) + tid;
+#pragma unroll
+    for (int j = 0; j < TN / 2; ++j) {
+      sum[(2 * j) * THREADS] = hi[j];
+      sum[(2 * j + 1) * THREADS] = lo[j];
+    }
+    const int r = tl.rb + (warp % 4) * 32 + lane, cb = tl.cb + (warp / 4) * (TN / 2);
+    if (r < o.m) {
+      const int ea = row_exp(exps[(int64_t)tl.ablk * BR + r - tl.rb]);
+      double* C = Cb + o.C + r + (int64_t)cb * o.ldc;
+      const double al = (double)o.alpha;
+      const int nj = min(TN / 2, o.n - cb);
+      const int* ebp = exps + (int64_t)tl.bblk * BR + (cb - tl.cb);
+#pragma unroll 2
+      for (int j = 0; j < nj; ++j) {
+        const int eb = row_exp(ebp[j]);
+        // 2^(sA - 62) 2^(sB - 62) 256^7, the biased exponents' offset 2 * 1023 taken out
+        const double v = ea == NOT_FINITE || eb == NOT_FINITE
+                             ? __longlong_as_double(0x7ff8000000000000ll)
+                             : to_double(sum[(2 * j) * THREADS], sum[(2 * j + 1) * THREADS],
+                                         ea + eb - 2 * 1023 - 124 + 56);
+        double* cp = C + (int64_t)j * o.ldc;
+        *cp = o.beta != 0.f ? fma(al, v, *cp) : al * v;
+      }
+    }
+  }
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+}
+
+}  // namespace
+
+// One 64 x 64 tile of the FMA form takes 1.2 us per k on its SM; the three
+// launches and one tile here take about 30 us, whatever the k up to 100.
+bool f64tc_worth(const GemmOp* h_ops, int nops) {
+  for (int i = 0; i < nops; ++i)
+    if (h_ops[i].k >= 24 && (int64_t)h_ops[i].m * h_ops[i].n >= 1024) return true;
+  return false;
+}
+
+void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double* Abase,
+                const double* Bbase, double* Cbase, int* d_flags, cudaStream_t st,
+                const char* name) {
+  static const bool attr = [] {   // initialised once, also under concurrent factorizations
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_gemm_f64tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      NST * STAGE));
+    return true;
+  }();
+  (void)attr;
+  for (int f0 = 0; f0 < nops;) {
+    // the products whose slices fit the work space together (at least one)
+    std::vector<SliceBlk> blks;
+    std::vector<Tile> tiles;
+    int64_t nblk = 0;
+    double fl = 0;
+    int f = f0, kmax = 0;
+    for (; f < nops; ++f) {
+      const GemmOp& o = h_ops[f];
+      const int nk = ceil_div(o.k, KC);
+      const bool same = Abase == Bbase && o.A == o.B && o.lda == o.ldb && o.transA != o.transB;
+      const int na = ceil_div(o.m, BR), nb = ceil_div(o.n, BR);
+      const int64_t need = (int64_t)(same ? std::max(na, nb) : na + nb) * nk;
+      if (f > f0 && (size_t)(nblk + need) * BLK > WORK_LIMIT) break;
+      auto add = [&](int64_t src, int rows, int ld, bool kcont, bool isB) {
+        const int first = (int)blks.size();
+        for (int r0 = 0; r0 < rows; r0 += BR) {
+          blks.push_back(SliceBlk{src + (kcont ? (int64_t)r0 * ld : r0), nblk, ld,
+                                  std::min(BR, rows - r0), o.k, kcont ? 1 : 0, isB ? 1 : 0, 0});
+          nblk += nk;
+        }
+        return first;
+      };
+      const int fa = add(o.A, same ? std::max(o.m, o.n) : o.m, o.lda, o.transA != 0, false);
+      const int fb = same ? fa : add(o.B, o.n, o.ldb, o.transB == 0, true);
+      const int tm = ceil_div(o.m, TM), tn = ceil_div(o.n, TN);
+      for (int t = 0; t < tm * tn; ++t) {
+        const int q = gemm_tile(o, t, tm * tn);
+        const int rb = (q % tm) * TM, cb = (q / tm) * TN;
+        if (o.lower && cb >= rb + TM) continue;
+        tiles.push_back(Tile{f, rb, cb, fa + rb / BR, fb + cb / BR});
+      }
+      kmax = std::max(kmax, o.k);
+      fl += 2.0 * o.m * (double)o.n * o.k * (o.lower || o.kzero ? 0.5 : 1.0);
+    }
+    ProfScope ps(name, st, fl, 0.0);
+    const size_t bb = sizeof(SliceBlk) * blks.size(), tb = sizeof(Tile) * tiles.size();
+    unsigned char *d_tab = nullptr, *W = nullptr;
+    int* d_exps = nullptr;
+    HIF_CUDA_TRY(cudaMallocAsync(&d_tab, bb + tb, st));
+    HIF_CUDA_TRY(cudaMallocAsync(&W, (size_t)std::max<int64_t>(1, nblk) * BLK, st));
+    HIF_CUDA_TRY(cudaMallocAsync(&d_exps, sizeof(int) * BR * blks.size(), st));
+    std::vector<unsigned char> tab(bb + tb);
+    std::copy_n(reinterpret_cast<const unsigned char*>(blks.data()), bb, tab.data());
+    std::copy_n(reinterpret_cast<const unsigned char*>(tiles.data()), tb, tab.data() + bb);
+    HIF_CUDA_TRY(cudaMemcpyAsync(d_tab, tab.data(), bb + tb, cudaMemcpyHostToDevice, st));
+    const SliceBlk* d_blks = reinterpret_cast<const SliceBlk*>(d_tab);
+    const Tile* d_tiles = reinterpret_cast<const Tile*>(d_tab + bb);
+    HIF_CUDA_TRY(cudaMemsetAsync(d_exps, 0, sizeof(int) * BR * blks.size(), st));
+    const int gy = std::max(1, std::min({ceil_div(kmax, 64), 64, ceil_div(4096, (int64_t)blks.size())}));
+    k_f64_exps<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_exps);
+    HIF_CHECK_LAUNCH();
+    k_f64_slice<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_exps, W);
+    HIF_CHECK_LAUNCH();
+    k_gemm_f64tc<<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(d_tiles, d_ops, d_blks, d_exps,
+                                                                       W, Cbase, d_flags);
+    HIF_CHECK_LAUNCH();
+    HIF_CUDA_TRY(cudaFreeAsync(d_exps, st));
+    HIF_CUDA_TRY(cudaFreeAsync(W, st));
+    HIF_CUDA_TRY(cudaFreeAsync(d_tab, st));
+    f0 = f;
+  }
+}
+
+}  // namespace hif

@@ -954,16 +954,17 @@ void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garen
     HIF_CUDA_TRY(cudaMemcpyAsync(d_ops + 2 * nb, o2.data(), sizeof(GemmOp) * nb, cudaMemcpyHostToDevice, st));
     HIF_CUDA_TRY(cudaMemcpyAsync(d_ops + 3 * nb, ou.data(), sizeof(GemmOp) * nb, cudaMemcpyHostToDevice, st));
     auto gemm = [&](const GemmOp* dop, const GemmOp* hop, const T* Ab, const T* Bb, T* Cb,
-                    const char* tc_name, const char* name) {
+                    const char* tc_name, const char* name, const char* f64_name) {
       if constexpr (std::is_same<T, float>::value) {
         if (tensor_cores) {
           gemm_tc(dop, hop, nb, Ab, Bb, Cb, d_flags, st, tc_name);
           return;
         }
       }
-      gemm_batched<T>(dop, hop, nb, Ab, Bb, Cb, st, name);
+      gemm_fma_or_f64tc<T>(dop, hop, nb, Ab, Bb, Cb, d_flags, tensor_cores, st, name, f64_name);
     };
-    gemm(d_ops, og.data(), Var, Var, Gb, "id_rowreduce_gram_tc", "id_rowreduce_gram");
+    gemm(d_ops, og.data(), Var, Var, Gb, "id_rowreduce_gram_tc", "id_rowreduce_gram",
+         "id_rowreduce_gram_f64tc");
     {
       static const bool tb_attr = [] {
         HIF_CUDA_TRY(cudaFuncSetAttribute(k_qr_tblk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -975,9 +976,12 @@ void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garen
       k_qr_tblk<T><<<nb, QB2, sizeof(T) * QB2 * (QB2 + 1), st>>>(d_qd, Gb, Tar, Tb);
       HIF_CHECK_LAUNCH();
     }
-    gemm(d_ops + nb, o1.data(), Var, Garena, W1b, "id_rowreduce_vta_tc", "id_rowreduce_vta");
-    gemm(d_ops + 2 * nb, o2.data(), Tb, W1b, W2b, "id_rowreduce_tw_tc", "id_rowreduce_tw");
-    gemm(d_ops + 3 * nb, ou.data(), Var, W2b, Garena, "id_rowreduce_block_tc", "id_rowreduce_block");
+    gemm(d_ops + nb, o1.data(), Var, Garena, W1b, "id_rowreduce_vta_tc", "id_rowreduce_vta",
+         "id_rowreduce_vta_f64tc");
+    gemm(d_ops + 2 * nb, o2.data(), Tb, W1b, W2b, "id_rowreduce_tw_tc", "id_rowreduce_tw",
+         "id_rowreduce_tw_f64tc");
+    gemm(d_ops + 3 * nb, ou.data(), Var, W2b, Garena, "id_rowreduce_block_tc", "id_rowreduce_block",
+         "id_rowreduce_block_f64tc");
     HIF_CUDA_TRY(cudaFreeAsync(d_ops, st));
   }
   if (blocks) {
