@@ -18,7 +18,6 @@ namespace hif {
 
 namespace {
 
-constexpr int PANEL_ROWS = 128;   // rows solved per CTA in the panel kernel
 constexpr int KC = 16;            // inner-dimension chunk of the tile products
 constexpr int MAX_GRID_Y = 65535;
 
@@ -54,21 +53,48 @@ struct TileAcc {
   }
 };
 
-// ---- panel: Cholesky of the diagonal block, then triangular solve of the rows below
-// k_chol_diag: one CTA per front factors the jb x jb diagonal block (jb <= 64)
-// right-looking with the block in registers: thread (ty, tx) of a 16 x 16 grid
-// holds rows ty + 16 i and columns tx + 16 j (i, j < 4).  Per column c the
-// threads holding column c scale it by the pivot and publish it to shared
-// memory; every thread then updates its entries right of c, and the holder
-// of entry (c+1, c+1) publishes the next pivot.  L goes to the factor panel
-// (zeros above the diagonal); a non-positive or non-finite pivot flags the
-// front and continues with 1.
+// ---- one step of the leading-block Cholesky: diagonal block, panel, update -----
+// What bounds a step is its chain: the fronts of the upper levels are few, so
+// the three kernels run one after the other with most of the chip idle.
 //
-// With growth > 0 (FP32 fronts that may be retried in FP64), the panel's
-// diagonal holds the front's original diagonal A_jj on entry, and a pivot
-// d_j with A_jj / d_j > growth (cancellation has eaten all but a few bits of
-// it), or one that is not positive or not finite, marks the front in
-// fflag[blockIdx.x] instead of failing it.
+// k_chol_diag: one CTA per front factors the jb x jb diagonal block (jb <= 64) in
+// shared memory, 16 columns at a time: one warp factors the 16 x 16 block in
+// registers (rows across lanes, pivot column by shuffles), one thread per row
+// solves the rows below, all threads update the rest; three CTA barriers per 16
+// columns.  Then it inverts L in the same pass (16 x 16 blocks by substitution,
+// merged pairwise to 32 and 64) and leaves L^{-1} in the factor panel, zeros above
+// the diagonal: the panel below becomes a product, and the triangular inverse of
+// the whole front needs these blocks anyway.  64 columns, FP32 25 us, FP64 100 us:
+// with one column per barrier pair and no inverse 62 and 112 us; the panel below
+// 8 us (by substitution 30-37, FP64 117), the 64-deep update of one tile 11 us
+// (18, FP64 49), and the separate inverse took 25-95 us.
+//
+// A non-positive or non-finite pivot flags the front and continues with 1.  With
+// growth > 0 (FP32 fronts that may be retried in FP64), the panel's diagonal
+// holds the front's original diagonal A_jj on entry, and a pivot d_j with
+// A_jj / d_j > growth (cancellation has eaten all but a few bits of it), or one
+// that is not positive or not finite, marks the front in fflag[blockIdx.x]
+// instead of failing it.
+constexpr int CB = 16;             // columns factored per step of the diagonal block
+constexpr int DP = NB + 1;         // row pitch of the shared-memory blocks
+
+template <typename T>
+constexpr size_t chol_diag_smem() {
+  return sizeof(T) * 2 * NB * DP;
+}
+
+// sqrt(d) and its reciprocal in one chain (a reciprocal square root and, in
+// FP32, one Newton step on it): every column of the block waits for it.
+__device__ __forceinline__ void sqrt_and_inverse(float d, float& piv, float& inv) {
+  const float y = rsqrtf(d);
+  inv = fmaf(0.5f * y, fmaf(-d * y, y, 1.0f), y);
+  piv = d * inv;
+}
+__device__ __forceinline__ void sqrt_and_inverse(double d, double& piv, double& inv) {
+  inv = rsqrt(d);
+  piv = d * inv;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_chol_diag(const DFront* __restrict__ fr, const T* Kar,
                                                    T* Par, int j0, int* flags, float growth,
@@ -79,120 +105,231 @@ __global__ void __launch_bounds__(256) k_chol_diag(const DFront* __restrict__ fr
   const int64_t ld = d.ld;
   const T* K = Kar + d.K + (int64_t)j0 + (int64_t)j0 * ld;
   T* P = Par + d.P + (int64_t)j0 + (int64_t)j0 * ld;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  __shared__ T colv[2][NB];
-  __shared__ T diagv[NB];
-  __shared__ T origv[NB];
-  if (growth > 0.f && threadIdx.x < jb) origv[threadIdx.x] = P[threadIdx.x + (int64_t)threadIdx.x * ld];
-  T a[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = ty + 16 * i, c = tx + 16 * j;
-      a[i][j] = (r < jb && c < jb && r >= c) ? K[r + (int64_t)c * ld] : T(0);
-      if (r == c && r == 0) diagv[0] = a[i][j];
-    }
+  extern __shared__ __align__(16) unsigned char dsm[];
+  T(*S)[DP] = reinterpret_cast<T(*)[DP]>(dsm);                       // A, then L
+  T(*V)[DP] = reinterpret_cast<T(*)[DP]>(dsm + sizeof(T) * NB * DP);  // L^{-1}
+  __shared__ T s_inv[NB], s_orig[NB];
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const int nb16 = (jb + CB - 1) / CB, je = nb16 * CB;
+  // lower triangle, padded to whole 16-blocks with the identity
+  for (int e = tid; e < NB * je; e += 256) {
+    const int r = e % NB, c = e / NB;
+    if (r < je) S[r][c] = (r < jb && c < jb && r >= c) ? K[r + (int64_t)c * ld] : T(r == c ? 1 : 0);
+  }
+  if (growth > 0.f && tid < jb) s_orig[tid] = P[tid + (int64_t)tid * ld];
   __syncthreads();
-  for (int c = 0; c < jb; ++c) {
-    const int par = c & 1;
-    if (tx == c % 16) {
-      const int j = c / 16;
-      T dv = diagv[c];
-      if (growth > 0.f) {
-        if (!(dv > T(0)) || !isfinite(dv) || dv * (T)growth < origv[c]) {
-          if (ty == 0) fflag[blockIdx.x] = 1;
-          if (!(dv > T(0)) || !isfinite(dv)) dv = T(1);
-        }
-      } else if (!(dv > T(0)) || !isfinite(dv)) {
-        if (ty == 0) flag_front(flags, FLAG_NOT_SPD, d.id);
-        dv = T(1);
-      }
-      const T piv = sqrt(dv), inv = T(1) / piv;
+  for (int o = 0; o < je; o += CB) {
+    if (warp == 0) {
+      // lane (r, h): the entries of row r in columns 2 u + h
+      const int r = lane % CB, h = lane / CB;
+      T a[CB / 2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = ty + 16 * i;
-        if (r > c) {
-          a[i][j] *= inv;
-          colv[par][r] = a[i][j];
-        } else if (r == c) {
-          a[i][j] = piv;
+      for (int u = 0; u < CB / 2; ++u) a[u] = 2 * u + h <= r ? S[o + r][o + 2 * u + h] : T(0);
+      bool bad = false, weak = false;
+      T myinv = T(0);
+#pragma unroll
+      for (int c = 0; c < CB; ++c) {
+        T dv = __shfl_sync(0xffffffffu, a[c / 2], c + (c % 2) * CB);
+        const bool ok = dv > T(0) && isfinite(dv);
+        if (o + c < jb) {
+          bad = bad || !ok;
+          if (growth > 0.f) weak = weak || !ok || dv * (T)growth < s_orig[o + c];
+        }
+        if (!ok) dv = T(1);
+        T piv, inv;
+        sqrt_and_inverse(dv, piv, inv);
+        // column c of L, in every lane of row r
+        const T ac = __shfl_sync(0xffffffffu, a[c / 2], r + (c % 2) * CB);
+        const T l = r > c ? ac * inv : (r == c ? piv : T(0));
+        if (h == c % 2) a[c / 2] = l;
+        if (r == c) myinv = inv;
+#pragma unroll
+        for (int u = (c + 1) / 2; u < CB / 2; ++u) {
+          const T lj = __shfl_sync(0xffffffffu, l, 2 * u + h);
+          if (2 * u + h > c) a[u] = fma(-l, lj, a[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < CB / 2; ++u) S[o + r][o + 2 * u + h] = 2 * u + h <= r ? a[u] : T(0);
+      if (h == 0) s_inv[o + r] = myinv;
+      if (lane == 0) {
+        if (growth > 0.f) {
+          if (weak) fflag[blockIdx.x] = 1;
+        } else if (bad) {
+          flag_front(flags, FLAG_NOT_SPD, d.id);
         }
       }
     }
     __syncthreads();
+    const int below = je - o - CB;
+    if (below == 0) break;
+    if (tid < below) {
+      T x[CB];
+      T* row = &S[o + CB + tid][o];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = ty + 16 * i;
-      if (r <= c) continue;
-      const T lr = colv[par][r];
+      for (int j = 0; j < CB; ++j) x[j] = row[j];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int cc = tx + 16 * j;
-        if (cc > c && cc <= r) {
-          a[i][j] = fma(-lr, colv[par][cc], a[i][j]);
-          if (r == cc && r == c + 1) diagv[r] = a[i][j];
-        }
+      for (int c = 0; c < CB; ++c) {
+        x[c] *= s_inv[o + c];
+#pragma unroll
+        for (int j = c + 1; j < CB; ++j) x[j] = fma(-x[c], S[o + j][o + c], x[j]);
       }
+#pragma unroll
+      for (int j = 0; j < CB; ++j) row[j] = x[j];
+    }
+    __syncthreads();
+    // rank-16 update of the lower triangle of the rest: thread (ty, tx) of a
+    // 16 x 16 grid takes one entry of each 16 x 16 block
+    const int tx = tid % 16, ty = tid / 16, nbl = below / CB;
+    T u[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+#pragma unroll
+    for (int l = 0; l < CB; ++l) {
+      T xr[3], xc[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        if (i < nbl) {
+          xr[i] = S[o + CB + ty + 16 * i][o + l];
+          xc[i] = S[o + CB + tx + 16 * i][o + l];
+        }
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j <= i; ++j)
+          if (i < nbl) u[i * (i + 1) / 2 + j] = fma(xr[i], xc[j], u[i * (i + 1) / 2 + j]);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j <= i; ++j)
+        if (i < nbl) S[o + CB + ty + 16 * i][o + CB + tx + 16 * j] -= u[i * (i + 1) / 2 + j];
+    __syncthreads();
+  }
+  // inverses of the 16 x 16 diagonal blocks: one warp each, one lane per column
+  if (warp < nb16 && lane < CB) {
+    const int o = warp * CB, c = lane;
+    T z[CB];
+#pragma unroll
+    for (int r = 0; r < CB; ++r) {
+      T t = T(0);
+#pragma unroll
+      for (int l = 0; l < r; ++l) t = fma(S[o + r][o + l], z[l], t);
+      z[r] = r == c ? s_inv[o + r] : (r > c ? -t * s_inv[o + r] : T(0));
+    }
+#pragma unroll
+    for (int r = 0; r < CB; ++r) V[o + r][o + c] = z[r];
+  }
+  __syncthreads();
+  // pairs of blocks of w: [A 0; B C]^-1 = [A^-1 0; -C^-1 B A^-1  C^-1].  B A^-1 is
+  // kept transposed in the free block above the diagonal.
+  for (int w = CB; w < je; w *= 2) {
+    // 2 x 2 entries per thread: w = 16 has up to two pairs (128 threads), w = 32
+    // one (256); rows past je (a shorter right block) are computed and unused
+    const int per = w * w / 4, q = tid / per, r = tid % per % (w / 2) * 2, c = tid % per / (w / 2) * 2;
+    const int o = 2 * w * q;
+    const bool in = o + w + r < je;
+    if (in) {
+      T t00 = T(0), t01 = T(0), t10 = T(0), t11 = T(0);
+#pragma unroll 8
+      for (int k = c; k < w; ++k) {   // V[o + k][.] is zero for k < c
+        const T s0 = S[o + w + r][o + k], s1 = S[o + w + r + 1][o + k];
+        const T v0 = V[o + k][o + c], v1 = k > c ? V[o + k][o + c + 1] : T(0);
+        t00 = fma(s0, v0, t00);
+        t01 = fma(s0, v1, t01);
+        t10 = fma(s1, v0, t10);
+        t11 = fma(s1, v1, t11);
+      }
+      V[o + c][o + w + r] = t00;
+      V[o + c + 1][o + w + r] = t01;
+      V[o + c][o + w + r + 1] = t10;
+      V[o + c + 1][o + w + r + 1] = t11;
+    }
+    __syncthreads();
+    if (in) {
+      T t00 = T(0), t01 = T(0), t10 = T(0), t11 = T(0);
+#pragma unroll 8
+      for (int k = 0; k <= r + 1; ++k) {
+        const T v0 = k <= r ? V[o + w + r][o + w + k] : T(0), v1 = V[o + w + r + 1][o + w + k];
+        const T s0 = V[o + c][o + w + k], s1 = V[o + c + 1][o + w + k];
+        t00 = fma(v0, s0, t00);
+        t01 = fma(v0, s1, t01);
+        t10 = fma(v1, s0, t10);
+        t11 = fma(v1, s1, t11);
+      }
+      V[o + w + r][o + c] = -t00;
+      V[o + w + r][o + c + 1] = -t01;
+      V[o + w + r + 1][o + c] = -t10;
+      V[o + w + r + 1][o + c + 1] = -t11;
     }
     __syncthreads();
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = ty + 16 * i, c = tx + 16 * j;
-      if (r < jb && c < jb) P[r + (int64_t)c * ld] = r >= c ? a[i][j] : T(0);
-    }
+  for (int e = tid; e < NB * jb; e += 256) {
+    const int r = e % NB, c = e / NB;
+    if (r < jb) P[r + (int64_t)c * ld] = r >= c ? V[r][c] : T(0);
+  }
 }
 
-// k_panel: the rows below the diagonal block, L21 = A21 L11^{-T}, by forward
-// substitution per row (one thread per row) with L11 read from the factor
-// panel; rows past the leading block also go to the panel.
+// 64 x 64 tiles with the whole depth of 64 in shared memory: one load phase, one
+// barrier, 64 steps.  Xs[k][i], Ys[k][j]; thread t owns rows (t % 16) 4 .. and
+// columns (t / 16) 4 ..
+constexpr int SP = TILE + 4;       // row pitch: 16-byte rows
 template <typename T>
-__global__ void __launch_bounds__(PANEL_ROWS) k_panel(const DFront* __restrict__ fr, T* Kar,
-                                                      T* Par, int j0) {
+constexpr size_t step_smem() {
+  return sizeof(T) * 2 * NB * SP;
+}
+template <typename T>
+__device__ __forceinline__ void step_mma(const T (*Xs)[SP], const T (*Ys)[SP], int depth,
+                                         T (&v)[4][4]) {
+  const int tr = (threadIdx.x % 16) * 4, tc = (threadIdx.x / 16) * 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[i][j] = T(0);
+#pragma unroll 4
+  for (int k = 0; k < depth; ++k) {
+    T x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      x[i] = Xs[k][tr + i];
+      y[i] = Ys[k][tc + i];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[i][j] = fma(x[i], y[j], v[i][j]);
+  }
+}
+
+// k_panel: the rows below the diagonal block, L21 = A21 L11^{-T}, in place (a CTA
+// owns 64 rows of all 64 columns; only fronts with a full block have rows below).
+// L11^{-1} is lower triangular: column c sums k <= c.
+template <typename T>
+__global__ void __launch_bounds__(256) k_panel(const DFront* __restrict__ fr, T* Kar,
+                                               const T* __restrict__ Par, int j0) {
   const DFront d = fr[blockIdx.y];
-  if (j0 >= d.p) return;
-  const int jb = min(NB, d.p - j0);
-  const int j1 = j0 + jb;
-  const int n = d.n;
+  const int j1 = j0 + NB;
+  const int r0 = j1 + blockIdx.x * TILE;
+  if (r0 >= d.n) return;
   const int64_t ld = d.ld;
-  const int r0 = j1 + blockIdx.x * PANEL_ROWS;
-  if (r0 >= n) return;
-  T* K = Kar + d.K;
-  T* P = Par + d.P;
-  __shared__ T D[NB][NB + 1];
-  const int tid = threadIdx.x;
-  for (int e = tid; e < NB * NB; e += PANEL_ROWS) {
-    int r = e % NB, c = e / NB;
-    D[r][c] = (r < jb && c < jb && r >= c) ? P[(int64_t)(j0 + r) + (int64_t)(j0 + c) * ld] : T(0);
+  T* K = Kar + d.K + (int64_t)j0 * ld;
+  const T* P = Par + d.P + (int64_t)j0 + (int64_t)j0 * ld;
+  extern __shared__ __align__(16) unsigned char ssm[];
+  T(*Xs)[SP] = reinterpret_cast<T(*)[SP]>(ssm);
+  T(*Ys)[SP] = Xs + NB;
+#pragma unroll 8
+  for (int e = threadIdx.x; e < NB * TILE; e += 256) {
+    const int r = e % TILE, k = e / TILE;
+    Xs[k][r] = r0 + r < d.n ? K[r0 + r + (int64_t)k * ld] : T(0);
+    Ys[k][r] = P[r + (int64_t)k * ld];
   }
   __syncthreads();
-  const int r = r0 + tid;
-  if (r >= n) return;
-  T x[NB];
+  T v[4][4];
+  step_mma<T>(Xs, Ys, (threadIdx.x / 16) * 4 + 4, v);
+  const int tr = (threadIdx.x % 16) * 4, tc = (threadIdx.x / 16) * 4;
 #pragma unroll
-  for (int c = 0; c < NB; ++c) x[c] = c < jb ? K[(int64_t)r + (int64_t)(j0 + c) * ld] : T(0);
-  // four partial sums per dot product shorten the dependent chains
+  for (int j = 0; j < 4; ++j)
 #pragma unroll
-  for (int c = 0; c < NB; ++c) {
-    if (c < jb) {
-      T s[4] = {x[c], T(0), T(0), T(0)};
-#pragma unroll
-      for (int l = 0; l < c; ++l) s[l & 3] = fma(-x[l], D[c][l], s[l & 3]);
-      x[c] = ((s[0] + s[1]) + (s[2] + s[3])) / D[c][c];
-    }
-  }
-  const bool toP = r >= d.p;
-#pragma unroll
-  for (int c = 0; c < NB; ++c) {
-    if (c < jb) {
-      const int64_t o = (int64_t)r + (int64_t)(j0 + c) * ld;
-      K[o] = x[c];
-      if (toP) P[o] = x[c];
-    }
-  }
+    for (int i = 0; i < 4; ++i)
+      if (r0 + tr + i < d.n) K[r0 + tr + i + (int64_t)(tc + j) * ld] = v[i][j];
 }
 
 __device__ __forceinline__ void tri_index(int t, int& ti, int& tj) {
@@ -210,10 +347,9 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_syrk(const DFront* __restrict__ fr, T* Kar, int j0,
                                               int jmax) {
   const DFront d = fr[blockIdx.y];
-  if (j0 >= d.p) return;
-  const int jb = min(NB, d.p - j0);
-  const int j1 = j0 + jb;
+  const int j1 = j0 + NB;   // a front with rows below has a full block
   const int n = d.n;
+  if (j1 >= n) return;
   const int64_t ld = d.ld;
   const int nt = (n - j1 + TILE - 1) / TILE;
   int ti, tj;
@@ -229,68 +365,37 @@ __global__ void __launch_bounds__(256) k_syrk(const DFront* __restrict__ fr, T* 
   }
   const int rb = j1 + ti * TILE, cb = j1 + tj * TILE;
   T* K = Kar + d.K;
-  __shared__ T As[KC][TILE + 4];
-  __shared__ T Bs[KC][TILE + 4];
-  TileAcc<T> acc;
-  acc.zero();
-  for (int k0 = 0; k0 < jb; k0 += KC) {
-    for (int e = threadIdx.x; e < KC * TILE; e += 256) {
-      int rr = e % TILE, kk = e / TILE;
-      int col = j0 + k0 + kk;
-      bool kin = k0 + kk < jb;
-      As[kk][rr] = (kin && rb + rr < n) ? K[(int64_t)(rb + rr) + (int64_t)col * ld] : T(0);
-      Bs[kk][rr] = (kin && cb + rr < n) ? K[(int64_t)(cb + rr) + (int64_t)col * ld] : T(0);
-    }
-    __syncthreads();
-    acc.mma(As, Bs, KC);
-    __syncthreads();
+  extern __shared__ __align__(16) unsigned char ssm[];
+  T(*Xs)[SP] = reinterpret_cast<T(*)[SP]>(ssm);
+  T(*Ys)[SP] = Xs + NB;
+#pragma unroll 8
+  for (int e = threadIdx.x; e < NB * TILE; e += 256) {
+    const int r = e % TILE, k = e / TILE;
+    const int64_t o = (int64_t)(j0 + k) * ld;
+    Xs[k][r] = rb + r < n ? K[rb + r + o] : T(0);
+    Ys[k][r] = cb + r < n ? K[cb + r + o] : T(0);
   }
+  // this thread's entries of the tile, loaded before the barrier
   const int tr = (threadIdx.x % 16) * 4, tc = (threadIdx.x / 16) * 4;
+  T u[4][4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int c = cb + tc + j;
-    if (c >= n || c >= jmax) continue;
+  for (int j = 0; j < 4; ++j)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = rb + tr + i;
-      if (r < n && r >= c) K[(int64_t)r + (int64_t)c * ld] -= acc.v[i][j];
+      const int r = rb + tr + i, c = cb + tc + j;
+      u[i][j] = r < n && r >= c && c < jmax ? K[(int64_t)r + (int64_t)c * ld] : T(0);
     }
-  }
-}
-
-// ---- inverse of the diagonal NB x NB blocks of L (held in P) in place ----------
-template <typename T>
-__global__ void __launch_bounds__(NB) k_trtri_diag(const DFront* __restrict__ fr, T* Par) {
-  const DFront d = fr[blockIdx.y];
-  const int i0 = blockIdx.x * NB;
-  if (i0 >= d.p) return;
-  const int ib = min(NB, d.p - i0);
-  const int64_t n = d.ld;
-  T* P = Par + d.P;
-  __shared__ T Ls[NB][NB + 1];
-  __shared__ T Zs[NB][NB + 1];
-  for (int e = threadIdx.x; e < NB * NB; e += NB) {
-    int r = e % NB, c = e / NB;
-    Ls[r][c] = (r < ib && c < ib && r >= c) ? P[(int64_t)(i0 + r) + (int64_t)(i0 + c) * n] : T(0);
-  }
   __syncthreads();
-  const int c = threadIdx.x;   // one column of the inverse per thread
-  if (c < ib) {
-    for (int r = 0; r < c; ++r) Zs[r][c] = T(0);
-    Zs[c][c] = T(1) / Ls[c][c];
-    for (int r = c + 1; r < ib; ++r) {
-      T s = T(0);
-      for (int l = c; l < r; ++l) s = fma(Ls[r][l], Zs[l][c], s);
-      Zs[r][c] = -s / Ls[r][r];
+  T v[4][4];
+  step_mma<T>(Xs, Ys, NB, v);
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = rb + tr + i, c = cb + tc + j;
+      if (r < n && r >= c && c < jmax) K[(int64_t)r + (int64_t)c * ld] = u[i][j] - v[i][j];
     }
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < ib * ib; e += NB) {
-    int r = e % ib, cc = e / ib;
-    P[(int64_t)(i0 + r) + (int64_t)(i0 + cc) * n] = Zs[r][cc];
-  }
 }
-
 
 // ---- FP64 retry of FP32 fronts flagged by the leading-block Cholesky ----------
 // Before the leading block is factored: its p x p entries are copied to a
@@ -517,20 +622,34 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
   // two levels: inner panels of NB factor an outer block of NB2 columns and
   // update only its remaining columns; the rows and columns right of the
   // outer block then get one rank-NB2 update A22 -= L21 L21^T as a batched
-  // product (tensor cores for FP32)
+  // product (tensor cores for FP32).  FP64 on the tensor cores: a product
+  // costs its three launches (about 35 us) up to several waves of tiles, so
+  // panel and update are one product each over all that is left.
   constexpr int NB2 = 256;
-  const bool outer = pmax > NB2;
+  const bool f64tc = sizeof(T) == 8 && tensor_cores;
+  const bool outer = pmax > NB2 && !f64tc;
+  static const bool attr = [] {   // initialised once, also under concurrent factorizations
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_chol_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)chol_diag_smem<T>()));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)step_smem<T>()));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_syrk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)step_smem<T>()));
+    return true;
+  }();
+  (void)attr;
   for (int J0 = 0; J0 < pmax; J0 += NB2) {
     const int jend = outer ? J0 + NB2 : INT_MAX;
     for (int j0 = J0; j0 < std::min(pmax, J0 + NB2); j0 += NB) {
-      int nact = 0;
+      // active fronts, and those with rows below the block (sorted by p,
+      // largest first)
+      int nact = 0, nbelow = 0;
       while (nact < nfront && lead[nact].p > j0) ++nact;
-      const int nm = lead[0].p;   // fronts are sorted by p, largest first
-      const int j1min = j0 + 1;   // smallest possible j1 among active fronts
-      const int chunks = ceil_div(std::max(0, nm - j1min), PANEL_ROWS);
-      const int ntile = ceil_div(std::max(0, nm - j1min), TILE);
-      const int nctile = outer ? std::max(1, ceil_div(std::max(0, jend - j1min), TILE)) : 0;
-      const int grid = outer ? std::max(1, ntile * nctile) : std::max(1, ntile * (ntile + 1) / 2);
+      while (nbelow < nact && lead[nbelow].p > j0 + NB) ++nbelow;
+      const int rest = std::max(0, lead[0].p - j0 - NB);
+      const int ntile = ceil_div(rest, TILE);
+      const int nctile = outer ? ceil_div(std::min(rest, jend - j0 - NB), TILE) : 0;
+      const int grid = outer ? ntile * nctile : ntile * (ntile + 1) / 2;
       // algorithmic counts of this step (only while profiling)
       double pf = 0, pb = 0, sf = 0, sb = 0;
       if (prof_enabled()) {
@@ -538,34 +657,60 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
           const double jb = std::min(NB, lead[f].p - j0);
           const double rest = lead[f].p - j0 - jb;
           const double cols = std::min<double>(rest, (double)std::min(jend, lead[f].p) - j0 - jb);
-          pf += jb * jb * jb / 3.0 + rest * jb * jb;
-          pb += sizeof(T) * (jb * jb / 2.0 + 2.0 * rest * jb);
+          pf += 2.0 * jb * jb * jb / 3.0 + rest * jb * jb;
+          pb += sizeof(T) * (jb * jb + 2.0 * rest * jb);
           sf += (2.0 * rest - cols + 1.0) * cols * jb;
           sb += sizeof(T) * (rest * jb + (2.0 * rest - cols + 1.0) * cols);
         }
       }
       for (int f0 = 0; f0 < nact; f0 += MAX_GRID_Y) {
         const int nb = std::min(MAX_GRID_Y, nact - f0);
-        {
-          ProfScope ps("chol_panel", st, pf, pb);
-          k_chol_diag<T><<<nb, 256, 0, st>>>(d_lead + f0, Karena, Parena, j0, d_flags,
-                                             growth_on ? (float)retry->growth : 0.f,
-                                             growth_on ? d_fflag + f0 : nullptr);
-          HIF_CHECK_LAUNCH();
-          if (chunks > 0) {
-            k_panel<T><<<dim3(chunks, nb), PANEL_ROWS, 0, st>>>(d_lead + f0, Karena, Parena, j0);
-            HIF_CHECK_LAUNCH();
+        ProfScope ps("chol_panel", st, pf, pb);
+        k_chol_diag<T><<<nb, 256, chol_diag_smem<T>(), st>>>(d_lead + f0, Karena, Parena, j0,
+                                                            d_flags,
+                                                            growth_on ? (float)retry->growth : 0.f,
+                                                            growth_on ? d_fflag + f0 : nullptr);
+        HIF_CHECK_LAUNCH();
+      }
+      if (nbelow == 0) continue;
+      if constexpr (sizeof(T) == 8) {
+        if (f64tc) {
+          std::vector<GemmOp> po(nbelow), uo(nbelow);
+          for (int f = 0; f < nbelow; ++f) {
+            const DFront& h = lead[f];
+            const int ld = h.ld, r = h.p - j0 - NB;
+            const int64_t a21 = h.K + j0 + NB + (int64_t)j0 * ld;
+            po[f] = GemmOp{a21, h.P + j0 + (int64_t)j0 * ld, a21, r, NB, NB, ld, ld, ld, 0, 1, 1.f, 0.f,
+                           0, KZ_B_UP};
+            uo[f] = GemmOp{a21, a21, a21 + (int64_t)NB * ld, r, r, NB, ld, ld, ld, 0, 1, -1.f, 1.f, 1, 0};
           }
-        }
-        {
-          ProfScope ps("chol_trailing_update", st, sf, sb);
-          k_syrk<T><<<dim3(grid, nb), 256, 0, st>>>(d_lead + f0, Karena, j0,
-                                                     outer ? jend : INT_MAX);
-          HIF_CHECK_LAUNCH();
+          GemmOp* d_step = nullptr;
+          HIF_CUDA_TRY(cudaMallocAsync(&d_step, sizeof(GemmOp) * 2 * nbelow, st));
+          po.insert(po.end(), uo.begin(), uo.end());
+          HIF_CUDA_TRY(cudaMemcpyAsync(d_step, po.data(), sizeof(GemmOp) * 2 * nbelow,
+                                       cudaMemcpyHostToDevice, st));
+          gemm_f64tc(d_step, po.data(), nbelow, Karena, Parena, Karena, d_flags, st, "chol_panel_f64tc");
+          gemm_f64tc(d_step + nbelow, uo.data(), nbelow, Karena, Karena, Karena, d_flags, st,
+                     "chol_trailing_update_f64tc");
+          HIF_CUDA_TRY(cudaFreeAsync(d_step, st));
+          continue;
         }
       }
+      for (int f0 = 0; f0 < nbelow; f0 += MAX_GRID_Y) {
+        const int nb = std::min(MAX_GRID_Y, nbelow - f0);
+        {
+          ProfScope ps("chol_panel", st);
+          k_panel<T><<<dim3(ntile, nb), 256, step_smem<T>(), st>>>(d_lead + f0, Karena, Parena, j0);
+          HIF_CHECK_LAUNCH();
+        }
+        if (grid == 0) continue;
+        ProfScope ps("chol_trailing_update", st, sf, sb);
+        k_syrk<T><<<dim3(grid, nb), 256, step_smem<T>(), st>>>(d_lead + f0, Karena, j0,
+                                                              outer ? jend : INT_MAX);
+        HIF_CHECK_LAUNCH();
+      }
     }
-    if (!outer) break;
+    if (!outer) continue;
     // A22 -= L21 L21^T for the fronts that extend past the outer block
     std::vector<GemmOp> uo;
     for (int f = 0; f < nfront && lead[f].p > jend; ++f) {
@@ -633,20 +778,10 @@ template <typename T>
 void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T* Karena,
                    T* Parena, int* d_flags, bool tensor_cores, cudaStream_t st) {
   const int pmax = h_fronts[0].p;
-  // 2. Linv = L^{-1}: invert the NB x NB diagonal blocks, then merge
+  // 2. Linv = L^{-1}: the diagonal blocks are inverted already; merge
   //    neighbouring inverted blocks pairwise up a binary tree of widths
   //    s = NB, 2 NB, 4 NB, ...:  inv([A 0; B C]) = [A^-1 0; -C^-1 B A^-1  C^-1]
   //    (two batched products per width: T = B A^-1, then -C^-1 T)
-  const int nblk = ceil_div(pmax, NB);
-  for (int f0 = 0; f0 < nfront; f0 += MAX_GRID_Y) {
-    const int nb = std::min(MAX_GRID_Y, nfront - f0);
-    double fl = 0;
-    if (prof_enabled())
-      for (int f = f0; f < f0 + nb; ++f) fl += (double)h_fronts[f].p * NB * NB / 3.0;
-    ProfScope ps("trtri_diag", st, fl, 0.0);
-    k_trtri_diag<T><<<dim3(nblk, nb), NB, 0, st>>>(d_fronts + f0, Parena);
-    HIF_CHECK_LAUNCH();
-  }
   for (int s = NB; s < pmax; s *= 2) {
     std::vector<GemmOp> tops, rops;
     int64_t scr = 0;
