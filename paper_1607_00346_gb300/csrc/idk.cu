@@ -1048,6 +1048,18 @@ bool launch_cpqr_dsm(const std::vector<int>& fronts, const SkelDesc* h_f, SkelDe
                      int32_t* perm, double eps, int cs_min, cudaStream_t st) {
   if (fronts.empty()) return true;
   int CS = std::max(1, cs_min);
+  if (sizeof(T) == 8) {
+    // FP64 columns are bound by their CTA's FP64 unit: a few fronts spread
+    // over the SMs they leave free, at least 8 columns per CTA (12 fronts of
+    // 56 x 256: 2.1 ms on one CTA each, 1.0 ms on 7; 4 columns per CTA 1.3 ms).
+    // FP32 steps are bound by the exchange, which grows with the cluster
+    // (9 fronts of 81 x 240: 1.0 ms on one CTA, 1.2 ms on 10).
+    int nfm = 0, dev = 0, nsm = 0;
+    for (int f : fronts) nfm = std::max(nfm, h_f[f].nF);
+    HIF_CUDA_TRY(cudaGetDevice(&dev));
+    HIF_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    CS = std::max(CS, std::min({DSM_MAX_CS, nsm / (int)fronts.size(), nfm / 8}));
+  }
   for (int f : fronts)
     CS = std::max(CS, dsm_min_cluster(h_f[f].idm, h_f[f].nF, (int)sizeof(T), std::max(1, cs_min)));
   for (; CS <= DSM_MAX_CS; ++CS) {
@@ -1278,13 +1290,17 @@ void interpolative_decomposition(SkelDesc* d_f, const SkelDesc* h_f, int nf, T* 
       HIF_CUDA_TRY(cudaFreeAsync(d_list, st));
     }
   };
-  // built-in rule: small fronts get one CTA; large fronts (work per step
-  // nF x nR above ~1e6) spread their columns over as many SMs as the batch
-  // leaves free (two CTAs per SM), up to 16, at least 8 columns per CTA
+  // built-in rule: large fronts (work per step nF x nR above ~1e6) spread
+  // their columns over as many SMs as they leave free (two CTAs per SM), up
+  // to 16, at least 8 columns per CTA; the other fronts over as many as the
+  // whole batch leaves free, so that a few medium fronts do not run on one SM
+  // each (12 FP64 fronts of 600 x 600: 89 ms on one CTA each, 17 ms on
+  // 16)
   int nbig = 0;
   for (int f : rest)
     if ((double)h_f[f].nF * (h_f[f].nF + h_f[f].idm) > 1.0e6) ++nbig;
   const int cs_big = std::max(1, std::min(16, 2 * nsm / std::max(1, nbig)));
+  const int cs_other = std::max(1, std::min(16, 2 * nsm / (int)rest.size()));
   // one bucket per call: the width class of its widest cluster front and the
   // count class of its cluster fronts; one shape (cluster size, fronts per
   // launch) for all of them, the cluster size capped per front at nF / 8
@@ -1303,7 +1319,7 @@ void interpolative_decomposition(SkelDesc* d_f, const SkelDesc* h_f, int nf, T* 
       int cs = cs_choice;
       if (cs <= 0) {   // built-in rule
         const double work = (double)h_f[f].nF * (h_f[f].nF + h_f[f].idm);
-        cs = work > 1.0e6 ? cs_big : 1;
+        cs = work > 1.0e6 ? cs_big : cs_other;
       }
       by_cs[std::min(cs, std::max(1, h_f[f].nF / 8))].push_back(f);
     }
