@@ -11,7 +11,13 @@
 //   x = 2^(s - 62) X,  X = sum_{i < 8} a_i 256^(7 - i),  |a_i| <= 128,
 //
 // with s per row of op(A) and per column of op(B) such that |x| < 2^s: X is x in
-// fixed point, 62 bits below the largest entry of its row.  The product is
+// fixed point, 62 bits below the largest entry of its row.  Before that, k is
+// balanced: column k of op(A) is scaled by 2^t_k and row k of op(B) by 2^-t_k, with
+// t_k half the difference of their largest exponents, so that neither hides the
+// other's entries (A_NI = D^ A D and L^-T = D^-1 L^ have opposite scales in k, as
+// have the factors of every product with an inverse or an interpolation matrix;
+// coefficients over eight decades lost two decimal digits without it).  The
+// product is
 // sum_t 256^(14 - t) D_t, D_t = sum_{i + j = t} sum_k a_i b_j; the 36 products
 // with t < 8 are formed (the others are below 2^-62 of row maximum times column
 // maximum) in eight FP32 accumulators.  |D_t| <= 8 * 128 * 2^14 = 2^24 over 128 k,
@@ -19,16 +25,18 @@
 // halves per entry), and each entry is rounded to double once at the end.  An
 // FMA loop rounds at every k; this sum is exact up to the 2^-62 of the split.
 //
-// Three launches per batch: k_f64_exps finds s per row, k_f64_slice writes the
-// slices in the layout the tensor core reads (64 rows x 16 k per block, all
-// eight slices together: 16 KB), k_gemm_f64tc copies blocks to shared memory with
-// bulk copies and multiplies.  An operand used on both sides (A A^T) is split
-// once.
+// Four launches per batch: k_f64_kmax finds t_k (not for A A^T), k_f64_exps s per
+// row, k_f64_slice writes the slices in the layout the tensor core reads (64 rows
+// x 16 k per block, all eight slices together: 16 KB), k_gemm_f64tc copies blocks
+// to shared memory with bulk copies and multiplies.  An operand used on both
+// sides (A A^T) is split once.
 //
-// Measured (three launches, FMA form in brackets): one 64^3 product 34 (66) us,
-// 512 of them 113 (270) us, one 256^3 48 (280) us, one 1024^3 0.10 (2.1) ms,
-// one 2048^3 0.63 (14.5) ms = 27 TFLOP/s.  Error against quad precision, entries
-// over 2 to 12 decades: 5e-17 to 7e-17 in norm (3e-16 to 1.5e-15).
+// Measured (all launches, FMA form in brackets): one 64^3 product 40 (66) us, 512
+// of them 125 (270) us, one 256^3 55 (280) us, one 1024^3 0.11 (2.1) ms, one 2048^3
+// 0.65 (14.5) ms = 26 TFLOP/s.  Error against quad precision, entries over 2 to
+// 12 decades: 5e-17 to 7e-17 in norm (3e-16 to 1.5e-15).  Solve error of an exact
+// factorization, coefficients over 2, 4, 6, 8 decades: 1.0, 1.0, 0.9, 1.5 to 2 times
+// the FMA form's.
 //
 // k_gemm_f64tc: one 128 x 64 tile per CTA; the eight accumulators fill the 512
 // columns of tensor memory, four stages of 48 KB the shared memory.  Per 16 k one
@@ -68,6 +76,8 @@ constexpr size_t WORK_LIMIT = (size_t)1 << 30;   // slices held at once, if seve
 struct SliceBlk {
   int64_t src;
   int64_t dst;       // index of its first 16 KB block in the work space
+  int64_t kx;        // index of the largest magnitudes of its product's columns of
+                     // op(A), then rows of op(B) (k each); -1: not balanced
   int ld, rows, k;
   int kcont, isB;
   int pad;
@@ -78,11 +88,61 @@ struct Tile {
   int ablk, bblk;    // first block row of A (two if the product has the rows), of B
 };
 
-// Largest magnitude of each row, as the upper word of its double (exps zeroed
-// before; a row's blocks of k are shared by gridDim.y CTAs).
+// Largest magnitude over a block's rows for each k, as the upper word of its
+// double (kx zeroed before; gridDim.y CTAs share the block's k).
+__global__ void __launch_bounds__(256) k_f64_kmax(const SliceBlk* __restrict__ blks,
+                                                  const double* __restrict__ Ab,
+                                                  const double* __restrict__ Bb, int* kx) {
+  const SliceBlk b = blks[blockIdx.x];
+  if (b.kx < 0) return;
+  const double* X = (b.isB ? Bb : Ab) + b.src;
+  int* out = kx + b.kx + (b.isB ? b.k : 0);
+  const int k0 = (int)((int64_t)b.k * blockIdx.y / gridDim.y);
+  const int k1 = (int)((int64_t)b.k * (blockIdx.y + 1) / gridDim.y);
+  if (b.kcont) {
+    for (int k = k0 + threadIdx.x; k < k1; k += 256) {
+      int m = 0;
+#pragma unroll 8
+      for (int r = 0; r < b.rows; ++r)
+        m = max(m, __double2hiint(X[(int64_t)r * b.ld + k]) & 0x7fffffff);
+      atomicMax(&out[k], m);
+    }
+  } else {
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+#pragma unroll 4
+    for (int k = k0 + warp; k < k1; k += 8) {
+      int m = 0;
+      for (int r = lane; r < b.rows; r += 32)
+        m = max(m, __double2hiint(X[r + (int64_t)k * b.ld]) & 0x7fffffff);
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) atomicMax(&out[k], m);
+    }
+  }
+}
+
+// The exponent added to this operand's entries at k.
+__device__ __forceinline__ int balance(const SliceBlk& b, const int* kx, int k) {
+  if (b.kx < 0) return 0;
+  const int ea = kx[b.kx + k] >> 20, eb = kx[b.kx + b.k + k] >> 20;
+  if (ea == 0 || eb == 0 || ea == 0x7ff || eb == 0x7ff) return 0;
+  const int t = (eb - ea) >> 1;
+  return b.isB ? -t : t;
+}
+
+// Largest balanced exponent of each row, biased by ROW_BIAS on top of the
+// double's own bias so that a zero row is 0 (exps zeroed before; gridDim.y CTAs
+// share the block's k).
+constexpr int ROW_BIAS = 4096;
+__device__ __forceinline__ int entry_exp(double x, int t) {
+  const int h = __double2hiint(x) & 0x7fffffff, e = h >> 20;
+  if (e == 0x7ff) return NOT_FINITE;
+  if (h == 0 && __double2loint(x) == 0) return 0;
+  return max(e, 1) + t + ROW_BIAS;
+}
 __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ blks,
                                                   const double* __restrict__ Ab,
-                                                  const double* __restrict__ Bb, int* exps) {
+                                                  const double* __restrict__ Bb,
+                                                  const int* __restrict__ kx, int* exps) {
   const SliceBlk b = blks[blockIdx.x];
   const double* X = (b.isB ? Bb : Ab) + b.src;
   const int k0 = (int)((int64_t)b.k * blockIdx.y / gridDim.y);
@@ -95,7 +155,7 @@ __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ b
       int m = 0;
 #pragma unroll 4
       for (int k = k0 + lane; k < k1; k += 32)
-        m = max(m, __double2hiint(X[(int64_t)r * b.ld + k]) & 0x7fffffff);
+        m = max(m, entry_exp(X[(int64_t)r * b.ld + k], balance(b, kx, k)));
       m = __reduce_max_sync(0xffffffffu, m);
       if (lane == 0) atomicMax(&out[r], m);
     }
@@ -105,15 +165,14 @@ __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ b
     int m = 0;
 #pragma unroll 8
     for (int k = k0 + threadIdx.x / BR; k < k1; k += 256 / BR)
-      m = max(m, __double2hiint(X[r + (int64_t)k * b.ld]) & 0x7fffffff);
+      m = max(m, entry_exp(X[r + (int64_t)k * b.ld], balance(b, kx, k)));
     atomicMax(&out[r], m);
   }
 }
 
 // s of a row, as a biased exponent: |x| < 2^(s - 1023) for all its entries
-__device__ __forceinline__ int row_exp(int hiword) {
-  const int e = hiword >> 20;
-  return e == 0x7ff ? NOT_FINITE : e + 1;
+__device__ __forceinline__ int row_exp(int v) {
+  return v == NOT_FINITE ? NOT_FINITE : v == 0 ? 1 : v - ROW_BIAS + 1;
 }
 
 // x in fixed point, 62 bits below 2^s (s: biased exponent + 1 of the row)
@@ -134,6 +193,7 @@ __device__ __forceinline__ int64_t fixed62(double x, int s) {
 __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ blks,
                                                    const double* __restrict__ Ab,
                                                    const double* __restrict__ Bb,
+                                                   const int* __restrict__ kx,
                                                    const int* __restrict__ exps, unsigned char* W) {
   const SliceBlk b = blks[blockIdx.x];
   const double* X = (b.isB ? Bb : Ab) + b.src;
@@ -144,9 +204,11 @@ __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ 
   const int nkg = (b.k + KC - 1) / KC * 2;   // groups of 8 k, padded to whole blocks
   for (int g = blockIdx.y * 4 + kg; g < nkg; g += gridDim.y * 4) {
     double x[8];
+    int t[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int k = g * 8 + j;
+      t[j] = k < b.k ? balance(b, kx, k) : 0;
       x[j] = (r < b.rows && k < b.k) ? X[b.kcont ? (int64_t)r * b.ld + k : r + (int64_t)k * b.ld]
                                      : 0.0;
     }
@@ -156,7 +218,7 @@ __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ 
     uint32_t lo[8], hi[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const uint64_t y = (uint64_t)(s == NOT_FINITE ? 0 : fixed62(x[j], s)) + 0x8080808080808080ull;
+      const uint64_t y = (uint64_t)(s == NOT_FINITE ? 0 : fixed62(x[j], s - t[j])) + 0x8080808080808080ull;
       lo[j] = (uint32_t)y;
       hi[j] = (uint32_t)(y >> 32);
     }
@@ -417,8 +479,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 }  // namespace
 
-// One 64 x 64 tile of the FMA form takes 1.2 us per k on its SM; the three
-// launches and one tile here take about 30 us, whatever the k up to 100.
+// One 64 x 64 tile of the FMA form takes 1.2 us per k on its SM; the four
+// launches and one tile here take about 40 us, whatever the k up to 100.
 bool f64tc_worth(const GemmOp* h_ops, int nops) {
   for (int i = 0; i < nops; ++i)
     if (h_ops[i].k >= 24 && (int64_t)h_ops[i].m * h_ops[i].n >= 1024) return true;
@@ -438,7 +500,7 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double
     // the products whose slices fit the work space together (at least one)
     std::vector<SliceBlk> blks;
     std::vector<Tile> tiles;
-    int64_t nblk = 0;
+    int64_t nblk = 0, nkx = 0;
     double fl = 0;
     int f = f0, kmax = 0;
     for (; f < nops; ++f) {
@@ -451,7 +513,7 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double
       auto add = [&](int64_t src, int rows, int ld, bool kcont, bool isB) {
         const int first = (int)blks.size();
         for (int r0 = 0; r0 < rows; r0 += BR) {
-          blks.push_back(SliceBlk{src + (kcont ? (int64_t)r0 * ld : r0), nblk, ld,
+          blks.push_back(SliceBlk{src + (kcont ? (int64_t)r0 * ld : r0), nblk, same ? -1 : nkx, ld,
                                   std::min(BR, rows - r0), o.k, kcont ? 1 : 0, isB ? 1 : 0, 0});
           nblk += nk;
         }
@@ -459,6 +521,7 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double
       };
       const int fa = add(o.A, same ? std::max(o.m, o.n) : o.m, o.lda, o.transA != 0, false);
       const int fb = same ? fa : add(o.B, o.n, o.ldb, o.transB == 0, true);
+      if (!same) nkx += 2 * (int64_t)o.k;
       const int tm = ceil_div(o.m, TM), tn = ceil_div(o.n, TN);
       for (int t = 0; t < tm * tn; ++t) {
         const int q = gemm_tile(o, t, tm * tn);
@@ -475,18 +538,24 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double
     int* d_exps = nullptr;
     HIF_CUDA_TRY(cudaMallocAsync(&d_tab, bb + tb, st));
     HIF_CUDA_TRY(cudaMallocAsync(&W, (size_t)std::max<int64_t>(1, nblk) * BLK, st));
-    HIF_CUDA_TRY(cudaMallocAsync(&d_exps, sizeof(int) * BR * blks.size(), st));
+    const size_t eb = sizeof(int) * (BR * blks.size() + (size_t)nkx);   // exps, then kx
+    HIF_CUDA_TRY(cudaMallocAsync(&d_exps, eb, st));
+    int* d_kx = d_exps + BR * blks.size();
     std::vector<unsigned char> tab(bb + tb);
     std::copy_n(reinterpret_cast<const unsigned char*>(blks.data()), bb, tab.data());
     std::copy_n(reinterpret_cast<const unsigned char*>(tiles.data()), tb, tab.data() + bb);
     HIF_CUDA_TRY(cudaMemcpyAsync(d_tab, tab.data(), bb + tb, cudaMemcpyHostToDevice, st));
     const SliceBlk* d_blks = reinterpret_cast<const SliceBlk*>(d_tab);
     const Tile* d_tiles = reinterpret_cast<const Tile*>(d_tab + bb);
-    HIF_CUDA_TRY(cudaMemsetAsync(d_exps, 0, sizeof(int) * BR * blks.size(), st));
+    HIF_CUDA_TRY(cudaMemsetAsync(d_exps, 0, eb, st));
     const int gy = std::max(1, std::min({ceil_div(kmax, 64), 64, ceil_div(4096, (int64_t)blks.size())}));
-    k_f64_exps<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_exps);
+    if (nkx) {
+      k_f64_kmax<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx);
+      HIF_CHECK_LAUNCH();
+    }
+    k_f64_exps<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps);
     HIF_CHECK_LAUNCH();
-    k_f64_slice<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_exps, W);
+    k_f64_slice<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps, W);
     HIF_CHECK_LAUNCH();
     k_gemm_f64tc<<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(d_tiles, d_ops, d_blks, d_exps,
                                                                        W, Cbase, d_flags);

@@ -9,6 +9,14 @@
 // Householder QR, whose work is in batched matrix products, and the pivoted QR
 // then runs on the small square R.
 //
+// The reflectors go to V scaled by powers of two to norms in [1, 2), and T by
+// the inverse squares, both exactly: the columns of A_RF, and with them the
+// reflectors, shrink by ten decades and more (it is numerically of low rank), and
+// the FP64 products split their operands into slices below the largest entry of
+// a row, which V of one scale and T of O(1) keep small.  (Unscaled, the FP64
+// factor of a 64^3 grid moved by 1e-9 to 1e-11 against the FMA form; scaled, by
+// less than 1e-13.)
+//
 // Blocked Householder QR, panel by panel (32 columns):
 //   * the panel: Householder reflectors of its columns, the explicit
 //     reflector matrix V and the triangular T of the compact form
@@ -64,6 +72,14 @@ struct QRDesc {
   int pad;
 };
 
+// 2^-e for the exponent e of the norm of a reflector with square vtv, and 2^e
+template <typename T>
+__device__ __forceinline__ void reflector_scale(T vtv, T& down, T& up) {
+  const int e = vtv > T(0) && isfinite(vtv) ? ilogb(vtv) >> 1 : 0;
+  down = ldexp(T(1), -e);
+  up = ldexp(T(1), e);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(QR_THREADS) k_qr_panel(const QRDesc* __restrict__ ds, T* Gar,
                                                          T* Var, T* Tar, int p, int p0) {
@@ -75,7 +91,7 @@ __global__ void __launch_bounds__(QR_THREADS) k_qr_panel(const QRDesc* __restric
   T* V = Var + d.V + qr_voff(p, p0, m);
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   __shared__ double s_red[QR_WARPS];
-  __shared__ double s_tau[QB], s_v0[QB];
+  __shared__ double s_tau[QB], s_v0[QB], s_dn[QB], s_up[QB];
   __shared__ double s_G[QB][QB + 1];
   __shared__ double s_T[QB][QB + 1];
   for (int j = 0; j < jb; ++j) {
@@ -100,13 +116,14 @@ __global__ void __launch_bounds__(QR_THREADS) k_qr_panel(const QRDesc* __restric
       const double vtv = v0 * v0 + tail;
       s_tau[j] = vtv > 0.0 ? 2.0 / vtv : 0.0;
       s_v0[j] = v0;
+      reflector_scale(vtv, s_dn[j], s_up[j]);
       col[c] = (T)alpha;          // R_cc; v0 lives in shared memory
     }
     __syncthreads();
-    const T v0 = (T)s_v0[j], tau = (T)s_tau[j];
+    const T v0 = (T)s_v0[j], tau = (T)s_tau[j], dn = (T)s_dn[j];
     // explicit reflector column j of V (rows p0..m-1 of the block's V)
     for (int r = p0 + tid; r < m; r += QR_THREADS)
-      V[(r - p) + (int64_t)j * m] = r < c ? T(0) : (r == c ? v0 : col[r]);
+      V[(r - p) + (int64_t)j * m] = r < c ? T(0) : dn * (r == c ? v0 : col[r]);
     // the rest of the panel
     for (int jj = j + 1 + warp; jj < jb; jj += QR_WARPS) {
       T* a = A + (int64_t)(p + jj) * ld;
@@ -135,11 +152,12 @@ __global__ void __launch_bounds__(QR_THREADS) k_qr_panel(const QRDesc* __restric
   if (tid == 0) {
     for (int j = 0; j < jb; ++j) {
       for (int i = 0; i < QB; ++i) s_T[i][j] = 0.0;
-      s_T[j][j] = s_tau[j];
+      const double tau = s_tau[j] * s_up[j] * s_up[j];   // of the scaled reflector
+      s_T[j][j] = tau;
       for (int i = 0; i < j; ++i) {
         double t = 0.0;
         for (int l = i; l < j; ++l) t += s_T[i][l] * s_G[l][j];
-        s_T[i][j] = -s_tau[j] * t;
+        s_T[i][j] = -tau * t;
       }
     }
   }
@@ -205,6 +223,7 @@ __global__ void __launch_bounds__(qrc_threads<T>()) k_qr_panel_cluster(const QRD
   __shared__ T s_tw[QB];                             // tau w_jj of the current column
   __shared__ T s_v0[QB];
   __shared__ T s_tau[QB];
+  __shared__ T s_dn[QB], s_up[QB];
   __shared__ T s_T[QB][QB + 1];                      // V^T V above the diagonal, then T
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const int nr = max(0, r1 - r0);
@@ -291,6 +310,7 @@ __global__ void __launch_bounds__(qrc_threads<T>()) k_qr_panel_cluster(const QRD
       } else if (l == j) {
         s_tau[j] = tau;
         s_v0[j] = v0;
+        reflector_scale(vtv, s_dn[j], s_up[j]);
       }
     }
     __syncthreads();
@@ -345,8 +365,8 @@ __global__ void __launch_bounds__(qrc_threads<T>()) k_qr_panel_cluster(const QRD
     const int i = e % nr, j = e / nr, row = r0 + i;
     T v = T(0);
     if (j < jb) {
-      if (row == j) v = s_v0[j];
-      else if (row > j) v = P[i + j * rb];
+      if (row == j) v = s_dn[j] * s_v0[j];
+      else if (row > j) v = s_dn[j] * P[i + j * rb];
       A[(p + row) + (int64_t)(p + j) * ld] = P[i + j * rb];
     }
     V[row + (int64_t)j * m] = v;
@@ -369,7 +389,7 @@ __global__ void __launch_bounds__(qrc_threads<T>()) k_qr_panel_cluster(const QRD
     T* Tt = Tar + d.Tt + qr_toff(p, p0);
     for (int e = tid; e < QB * QB; e += QRC_THREADS) {
       const int i = e % QB, j = e / QB;
-      Tt[e] = (i < jb && j < jb) ? s_T[i][j] : T(0);
+      Tt[e] = (i < jb && j < jb) ? s_T[i][j] * s_up[i] * s_up[j] : T(0);
     }
   }
 }
