@@ -623,7 +623,7 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
   // update only its remaining columns; the rows and columns right of the
   // outer block then get one rank-NB2 update A22 -= L21 L21^T as a batched
   // product (tensor cores for FP32).  FP64 on the tensor cores: a product
-  // costs its three launches (about 35 us) up to several waves of tiles, so
+  // costs its launches (about 40 us) up to several waves of tiles, so
   // panel and update are one product each over all that is left.
   constexpr int NB2 = 256;
   const bool f64tc = sizeof(T) == 8 && tensor_cores;

@@ -81,10 +81,11 @@ struct GemvTask {
 void gemv_plan(const GemvOp* ops, int nops, int trans, std::vector<GemvTask>& tasks, int (&cnt)[4]);
 // Thread blocks that run a planned list.
 int gemv_ctas(const int (&cnt)[4]);
-// Right-hand sides the next block takes when `left` remain: 16 (also for
-// 9-15, the others masked), 8 (5-7), 4 (3), 2 or 1, so that each block reads
-// the factor once.
-int gemv_block(int left);
+// Right-hand sides the next block takes when `left` remain, for words of 4
+// bytes: 16 (also for 9-15, the others masked), 8 (5-7), 4 (3), 2 or 1, so that
+// each block reads the factor once; of 8 bytes, where the multiply-adds of
+// masked columns would cost more than a second read: 8, 4, 2 or 1.
+int gemv_block(int left, size_t word);
 
 // One factor's list and block of right-hand sides: matrices at M + op.M,
 // vectors at w + op.x and w + op.y (w already shifted to the block's first

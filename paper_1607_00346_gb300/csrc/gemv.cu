@@ -44,6 +44,7 @@ constexpr int GEMV_TR = 64;    // rows of an M x tile, two per lane
 constexpr int GEMV_BC = 8;     // columns of a block of an M x tile
 constexpr int GEMV_T_THREADS = 128;
 constexpr int GEMV_CG = 8;     // columns of a warp of M^T x
+constexpr int GEMV_CG_FINE = 2;   // the same in the fine form
 constexpr int GEMV_TC = GEMV_CG * GEMV_T_THREADS / 32;   // columns of an M^T x task
 
 // R consecutive values from shared memory, as 16-byte vectors where they fill one.
@@ -86,9 +87,11 @@ __host__ __device__ constexpr int gemv_red_cols() {   // right-hand sides reduce
   return R < 4 ? R : 4;
 }
 
-template <typename T, int R>
-__device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, int ti, int ncls,
-                                            T* xs_all, T* red) {
+// RL = 2: the whole tile, two rows per lane; RL = 1: its half `half`.
+template <typename T, int R, int RL>
+__device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, int ti, int half,
+                                            int ncls, T* xs_all, T* red) {
+  constexpr int TR = 32 * RL;
   constexpr int XN = (GEMV_BC * R + 31) / 32;   // x values a lane stages per block
   constexpr int RQ = gemv_red_cols<T, R>();
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -100,44 +103,46 @@ __device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, in
     tk = sg.tasks[ti];
     o = sg.ops[tk.op];
   }
-  const int r0 = tk.tile * GEMV_TR;
+  const int r0 = tk.tile * GEMV_TR + 32 * half;
   const int rows = o.rows;
-  const int ra = r0 + lane, rb = ra + 32;
-  const int cols = valid ? (o.tri ? min(o.cols, r0 + GEMV_TR) : o.cols) : 0;
+  const int cols = valid ? (o.tri ? min(o.cols, r0 + TR) : o.cols) : 0;
   const int nblk = (cols + GEMV_BC - 1) / GEMV_BC;
   const T* M = sg.M + o.M;
   const T* x = sg.w + o.x;
   const int64_t vs = sg.vs;
   const int nv = sg.nv;
-  const bool rfull = r0 + GEMV_TR <= rows;
+  const bool rfull = r0 + TR <= rows;
 
-  T acc[2][R];
+  T acc[RL][R];
 #pragma unroll
-  for (int q = 0; q < R; ++q) acc[0][q] = acc[1][q] = T(0);
+  for (int i = 0; i < RL; ++i)
+#pragma unroll
+    for (int q = 0; q < R; ++q) acc[i][q] = T(0);
   // a block's matrix entries and x values, in flight while the block before
   // it is multiplied
   constexpr bool AHEAD = sizeof(T) == 4 || R < 8;   // else the sums need the registers
-  T m[2][GEMV_BC], mn[2][GEMV_BC], xv[XN], xn[XN];
+  T m[RL][GEMV_BC], mn[RL][GEMV_BC], xv[XN], xn[XN];
   auto full = [&](int b) {   // no entry of the block is masked
     const int c0 = b * GEMV_BC;
     return rfull && c0 + GEMV_BC <= cols && (!o.tri || c0 + GEMV_BC <= r0 + 1);
   };
-  auto load = [&](int b, T (&mm)[2][GEMV_BC], T (&xx)[XN]) {
+  auto load = [&](int b, T (&mm)[RL][GEMV_BC], T (&xx)[XN]) {
     const int c0 = b * GEMV_BC;
     const T* mc = M + (int64_t)c0 * o.ld;
     if (full(b)) {
 #pragma unroll
-      for (int c = 0; c < GEMV_BC; ++c) {
-        mm[0][c] = mc[ra + (int64_t)c * o.ld];
-        mm[1][c] = mc[rb + (int64_t)c * o.ld];
-      }
+      for (int c = 0; c < GEMV_BC; ++c)
+#pragma unroll
+        for (int i = 0; i < RL; ++i) mm[i][c] = mc[r0 + lane + 32 * i + (int64_t)c * o.ld];
     } else {
 #pragma unroll
-      for (int c = 0; c < GEMV_BC; ++c) {
-        const bool in = c0 + c < cols;
-        mm[0][c] = (in && ra < rows && (!o.tri || c0 + c <= ra)) ? mc[ra + (int64_t)c * o.ld] : T(0);
-        mm[1][c] = (in && rb < rows && (!o.tri || c0 + c <= rb)) ? mc[rb + (int64_t)c * o.ld] : T(0);
-      }
+      for (int c = 0; c < GEMV_BC; ++c)
+#pragma unroll
+        for (int i = 0; i < RL; ++i) {
+          const int r = r0 + lane + 32 * i;
+          mm[i][c] = (c0 + c < cols && r < rows && (!o.tri || c0 + c <= r)) ? mc[r + (int64_t)c * o.ld]
+                                                                           : T(0);
+        }
     }
 #pragma unroll
     for (int j = 0; j < XN; ++j) {
@@ -162,31 +167,28 @@ __device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, in
         T t[R];
         read_x<R>(t, xs + c * R);
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-          acc[0][q] = fma(m[0][c], t[q], acc[0][q]);
-          acc[1][q] = fma(m[1][c], t[q], acc[1][q]);
-        }
+        for (int q = 0; q < R; ++q)
+#pragma unroll
+          for (int i = 0; i < RL; ++i) acc[i][q] = fma(m[i][c], t[q], acc[i][q]);
       }
     } else {
       // a masked entry leaves its sum alone (x may be infinite there)
 #pragma unroll
       for (int c = 0; c < GEMV_BC; ++c) {
         const int cc = b * GEMV_BC + c;
-        const bool ia = cc < cols && (!o.tri || cc <= ra), ib = cc < cols && (!o.tri || cc <= rb);
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-          const T t = xs[c * R + q];
-          if (ia) acc[0][q] = fma(m[0][c], t, acc[0][q]);
-          if (ib) acc[1][q] = fma(m[1][c], t, acc[1][q]);
+        for (int i = 0; i < RL; ++i) {
+          if (cc >= cols || (o.tri && cc > r0 + lane + 32 * i)) continue;
+#pragma unroll
+          for (int q = 0; q < R; ++q) acc[i][q] = fma(m[i][c], xs[c * R + q], acc[i][q]);
         }
       }
     }
     if (AHEAD) {
 #pragma unroll
-      for (int c = 0; c < GEMV_BC; ++c) {
-        m[0][c] = mn[0][c];
-        m[1][c] = mn[1][c];
-      }
+      for (int c = 0; c < GEMV_BC; ++c)
+#pragma unroll
+        for (int i = 0; i < RL; ++i) m[i][c] = mn[i][c];
 #pragma unroll
       for (int j = 0; j < XN; ++j) xv[j] = xn[j];
     }
@@ -198,9 +200,13 @@ __device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, in
 #pragma unroll
     for (int q = 0; q < R; ++q) {
       if (q >= nv) continue;
-      T* yp = y + q * vs;
-      if (ra < rows) yp[ra] = (o.beta_one ? yp[ra] : T(0)) + al * acc[0][q];
-      if (rb < rows) yp[rb] = (o.beta_one ? yp[rb] : T(0)) + al * acc[1][q];
+#pragma unroll
+      for (int i = 0; i < RL; ++i) {
+        const int r = r0 + lane + 32 * i;
+        if (r >= rows) continue;
+        T* yp = y + q * vs + r;
+        *yp = (o.beta_one ? *yp : T(0)) + al * acc[i][q];
+      }
     }
     return;
   }
@@ -211,16 +217,15 @@ __device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, in
   for (int q0 = 0; q0 < R; q0 += RQ) {
     if (q0 >= nv) break;
 #pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-      red[(warp * RQ + q) * GEMV_TR + lane] = acc[0][q0 + q];
-      red[(warp * RQ + q) * GEMV_TR + lane + 32] = acc[1][q0 + q];
-    }
+    for (int q = 0; q < RQ; ++q)
+#pragma unroll
+      for (int i = 0; i < RL; ++i) red[(warp * RQ + q) * TR + lane + 32 * i] = acc[i][q0 + q];
     __syncthreads();
     if (valid)
-      for (int e = tid; e < RQ * GEMV_TR; e += ncls * 32) {
-        const int q = e / GEMV_TR, r = r0 + e % GEMV_TR;
-        T s = red[t0 * RQ * GEMV_TR + e];
-        for (int w = 1; w < ncls; ++w) s += red[(t0 + w) * RQ * GEMV_TR + e];
+      for (int e = tid; e < RQ * TR; e += ncls * 32) {
+        const int q = e / TR, r = r0 + e % TR;
+        T s = red[t0 * RQ * TR + e];
+        for (int w = 1; w < ncls; ++w) s += red[(t0 + w) * RQ * TR + e];
         if (r < rows && q0 + q < nv) {
           T* yp = y + (q0 + q) * vs + r;
           *yp = (o.beta_one ? *yp : T(0)) + al * s;
@@ -230,11 +235,14 @@ __device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, in
   }
 }
 
-template <typename T, int R>
+template <typename T, int R, bool FINE>
 __device__ __forceinline__ void gemv_n_cta(const GemvSeg<T>& sg, int b) {
+  constexpr int RL = FINE ? 1 : 2;
   __shared__ __align__(16) T xs[GEMV_WARPS * GEMV_BC * R];
-  __shared__ T red[GEMV_WARPS * gemv_red_cols<T, R>() * GEMV_TR];
+  __shared__ T red[GEMV_WARPS * gemv_red_cols<T, R>() * 32 * RL];
   const int warp = threadIdx.x / 32;
+  const int half = FINE ? b % 2 : 0;
+  if (FINE) b /= 2;
   // the list's tasks, those of 8 warps first, then 4, 2 and 1
   int ncls = 8, base = 0;
 #pragma unroll
@@ -243,7 +251,7 @@ __device__ __forceinline__ void gemv_n_cta(const GemvSeg<T>& sg, int b) {
     const int nc = (sg.cnt[k] + per - 1) / per;
     if (b < nc || k == 3) {
       const int j = b * per + warp / ncls;
-      gemv_n_tile<T, R>(sg, j < sg.cnt[k], base + j, ncls, xs, red);
+      gemv_n_tile<T, R, RL>(sg, j < sg.cnt[k], base + j, half, ncls, xs, red);
       return;
     }
     b -= nc;
@@ -294,10 +302,10 @@ __device__ __forceinline__ void cp_async(double* dst, const double* src, bool ok
                    (uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 8 : 0) : "memory");
 }
 
-// Sums over the lanes and writes y of CG columns from c0 on, R right-hand sides from q0 on.
+// Sums over the lanes and writes y of CG columns from c0 on.
 template <typename T, int R, int CG>
 __device__ __forceinline__ void gemv_t_finish(T (&v)[CG * R], const GemvOp& o, const GemvSeg<T>& sg,
-                                              int c0, int q0) {
+                                              int c0) {
   constexpr int V = CG * R;
   const int lane = threadIdx.x % 32;
   // lane l ends with the values whose index has the bits of l (16, 8, ..) as
@@ -310,7 +318,7 @@ __device__ __forceinline__ void gemv_t_finish(T (&v)[CG * R], const GemvOp& o, c
   const T al = (T)o.alpha;
 #pragma unroll
   for (int i = 0; i < KEEP; ++i) {
-    const int c = c0 + (idx + i) / R, q = q0 + (idx + i) % R;
+    const int c = c0 + (idx + i) / R, q = (idx + i) % R;
     if (c < o.cols && q < sg.nv) {
       T* yp = sg.w + o.y + q * sg.vs + c;
       *yp = (o.beta_one ? *yp : T(0)) + al * v[i];
@@ -318,33 +326,34 @@ __device__ __forceinline__ void gemv_t_finish(T (&v)[CG * R], const GemvOp& o, c
   }
 }
 
-template <typename T, int R>
+template <typename T, int R, int CG>
 __device__ __forceinline__ void gemv_t_few(const GemvSeg<T>& sg, int b) {
-  constexpr int UN = 2;
+  constexpr int UN = 2 * GEMV_CG / CG;   // row steps in flight
+  constexpr int SUB = GEMV_CG / CG;      // CTAs per task
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const GemvTask tk = sg.tasks[b];
+  const GemvTask tk = sg.tasks[b / SUB];
   const GemvOp o = sg.ops[tk.op];
-  const int c0 = tk.tile * GEMV_TC + warp * GEMV_CG;
+  const int c0 = tk.tile * GEMV_TC + (b % SUB * (GEMV_T_THREADS / 32) + warp) * CG;
   if (c0 >= o.cols) return;
   const int rows = o.rows;
   const int64_t vs = sg.vs, ld = o.ld;
   const int nv = sg.nv;
   const T* M = sg.M + o.M + (int64_t)c0 * ld;
   const T* x = sg.w + o.x;
-  T v[GEMV_CG * R];   // v[c R + q]
+  T v[CG * R];   // v[c R + q]
 #pragma unroll
-  for (int i = 0; i < GEMV_CG * R; ++i) v[i] = T(0);
+  for (int i = 0; i < CG * R; ++i) v[i] = T(0);
   auto masked = [&](int r) {
     if (r >= rows) return;
-    T mm[GEMV_CG];
+    T mm[CG];
 #pragma unroll
-    for (int c = 0; c < GEMV_CG; ++c)
+    for (int c = 0; c < CG; ++c)
       mm[c] = (c0 + c < o.cols && (!o.tri || r >= c0 + c)) ? M[r + c * ld] : T(0);
 #pragma unroll
     for (int q = 0; q < R; ++q) {
       const T xq = q < nv ? x[q * vs + r] : T(0);
 #pragma unroll
-      for (int c = 0; c < GEMV_CG; ++c)
+      for (int c = 0; c < CG; ++c)
         if (!o.tri || r >= c0 + c) v[c * R + q] = fma(mm[c], xq, v[c * R + q]);
     }
   };
@@ -354,13 +363,13 @@ __device__ __forceinline__ void gemv_t_few(const GemvSeg<T>& sg, int b) {
     masked(r + lane);
     r += 32;
   }
-  if (c0 + GEMV_CG <= o.cols) {
+  if (c0 + CG <= o.cols) {
     for (; r + 32 * UN <= rows; r += 32 * UN) {
-      T mm[UN][GEMV_CG], xq[UN][R];
+      T mm[UN][CG], xq[UN][R];
 #pragma unroll
       for (int u = 0; u < UN; ++u) {
 #pragma unroll
-        for (int c = 0; c < GEMV_CG; ++c) mm[u][c] = M[r + 32 * u + lane + c * ld];
+        for (int c = 0; c < CG; ++c) mm[u][c] = M[r + 32 * u + lane + c * ld];
 #pragma unroll
         for (int q = 0; q < R; ++q) xq[u][q] = q < nv ? x[q * vs + r + 32 * u + lane] : T(0);
       }
@@ -369,107 +378,105 @@ __device__ __forceinline__ void gemv_t_few(const GemvSeg<T>& sg, int b) {
 #pragma unroll
         for (int q = 0; q < R; ++q)
 #pragma unroll
-          for (int c = 0; c < GEMV_CG; ++c) v[c * R + q] = fma(mm[u][c], xq[u][q], v[c * R + q]);
+          for (int c = 0; c < CG; ++c) v[c * R + q] = fma(mm[u][c], xq[u][q], v[c * R + q]);
     }
   }
   for (; r < rows; r += 32) masked(r + lane);
-  gemv_t_finish<T, R, GEMV_CG>(v, o, sg, c0, 0);
+  gemv_t_finish<T, R, CG>(v, o, sg, c0);
 }
 
-// 8 or 16 right-hand sides, RW of them per pass over the matrix (16 in FP32; in
-// FP64, bound by its multiply-adds, 8).
-template <typename T, int R>
+// 8 or 16 right-hand sides.
+template <typename T, int R, int CG>
 __device__ __forceinline__ void gemv_t_many(const GemvSeg<T>& sg, int b) {
-  constexpr int CG = GEMV_CG, RW = sizeof(T) == 4 ? R : 8;
+  constexpr int SUB = GEMV_CG / CG;                         // CTAs per task
+  constexpr int TC = GEMV_TC / SUB;                         // columns of the CTA
   constexpr int CH = GEMV_T_THREADS * 4 / (int)sizeof(T);   // rows per chunk
   constexpr int STEPS = CH / 32;
   constexpr int CPR = GEMV_T_THREADS / CH;                  // columns copied side by side
-  __shared__ T ms[2][GEMV_TC][CH];
-  __shared__ T xs[2][RW][CH];
+  __shared__ T ms[2][TC][CH];
+  __shared__ T xs[2][R][CH];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const GemvTask tk = sg.tasks[b];
+  const GemvTask tk = sg.tasks[b / SUB];
   const GemvOp o = sg.ops[tk.op];
-  const int ct = tk.tile * GEMV_TC, c0 = ct + warp * CG;
+  const int ct = tk.tile * GEMV_TC + b % SUB * TC, c0 = ct + warp * CG;
+  if (ct >= o.cols) return;
   const int rows = o.rows;
   const int64_t vs = sg.vs, ld = o.ld;
   const T* M = sg.M + o.M + (int64_t)ct * ld;
-  const int rbeg = o.tri ? ct : 0;   // GEMV_TC = 32: the diagonal's row step
+  const int rbeg = o.tri ? tk.tile * GEMV_TC : 0;   // GEMV_TC = 32: the diagonal's row step
   const int nchunk = rows > rbeg ? (rows - rbeg + CH - 1) / CH : 0;
   const int te = threadIdx.x % CH, tc = threadIdx.x / CH;
-#pragma unroll 1
-  for (int q0 = 0; q0 < R && q0 < sg.nv; q0 += RW) {
-    const int nv = sg.nv - q0;
-    const T* x = sg.w + o.x + q0 * vs;
-    // chunk k of the matrix columns and of x, copied asynchronously; entries
-    // outside the matrix or the triangle are zero
-    auto stage = [&](int k) {
-      if (k < nchunk) {
-        const int r = rbeg + k * CH + te;
-        const bool in = r < rows;
-        if (ct + GEMV_TC <= o.cols && (k + 1) * CH <= rows - rbeg && (!o.tri || k > 0)) {
-          const T* m = M + r + tc * ld;
+  const int nv = sg.nv;
+  const T* x = sg.w + o.x;
+  // chunk k of the matrix columns and of x, copied asynchronously; entries
+  // outside the matrix or the triangle are zero
+  auto stage = [&](int k) {
+    if (k < nchunk) {
+      const int r = rbeg + k * CH + te;
+      const bool in = r < rows;
+      if (ct + TC <= o.cols && (k + 1) * CH <= rows - rbeg && (!o.tri || k > 0)) {
+        const T* m = M + r + tc * ld;
 #pragma unroll
-          for (int c = 0; c < GEMV_TC; c += CPR) cp_async(&ms[k & 1][c + tc][te], m + c * ld, true);
-        } else {
+        for (int c = 0; c < TC; c += CPR) cp_async(&ms[k & 1][c + tc][te], m + c * ld, true);
+      } else {
 #pragma unroll
-          for (int c = 0; c < GEMV_TC; c += CPR) {
-            const bool ok = in && ct + c + tc < o.cols && (!o.tri || r >= ct + c + tc);
-            cp_async(&ms[k & 1][c + tc][te], ok ? M + r + (c + tc) * ld : x, ok);
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < RW; q += CPR) {
-          const bool ok = in && q + tc < nv;
-          cp_async(&xs[k & 1][q + tc][te], ok ? x + (q + tc) * vs + r : x, ok);
+        for (int c = 0; c < TC; c += CPR) {
+          const bool ok = in && ct + c + tc < o.cols && (!o.tri || r >= ct + c + tc);
+          cp_async(&ms[k & 1][c + tc][te], ok ? M + r + (c + tc) * ld : x, ok);
         }
       }
-      asm volatile("cp.async.commit_group;\n" ::: "memory");
-    };
-    T v[CG * RW];
 #pragma unroll
-    for (int i = 0; i < CG * RW; ++i) v[i] = T(0);
-    stage(0);
-    for (int k = 0; k < nchunk; ++k) {
-      stage(k + 1);
-      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-      __syncthreads();
-      const T(*mk)[CH] = &ms[k & 1][warp * CG];
-      const T(*xk)[CH] = xs[k & 1];
-#pragma unroll
-      for (int s = 0; s < STEPS; ++s) {
-        T m[CG];
-#pragma unroll
-        for (int c = 0; c < CG; ++c) m[c] = mk[c][32 * s + lane];
-        if (s == 0 && k == 0 && o.tri) {
-          // a masked entry leaves its sum alone (x may be infinite there)
-#pragma unroll
-          for (int q = 0; q < RW; ++q) {
-            const T xq = xk[q][lane];
-#pragma unroll
-            for (int c = 0; c < CG; ++c)
-              if (lane >= warp * CG + c) v[c * RW + q] = fma(m[c], xq, v[c * RW + q]);
-          }
-        } else {
-#pragma unroll
-          for (int q = 0; q < RW; ++q) {
-            const T xq = xk[q][32 * s + lane];
-#pragma unroll
-            for (int c = 0; c < CG; ++c) v[c * RW + q] = fma(m[c], xq, v[c * RW + q]);
-          }
-        }
+      for (int q = 0; q < R; q += CPR) {
+        const bool ok = in && q + tc < nv;
+        cp_async(&xs[k & 1][q + tc][te], ok ? x + (q + tc) * vs + r : x, ok);
       }
-      __syncthreads();   // the chunk's buffers are free for chunk k + 2
     }
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    gemv_t_finish<T, RW, CG>(v, o, sg, c0, q0);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  T v[CG * R];
+#pragma unroll
+  for (int i = 0; i < CG * R; ++i) v[i] = T(0);
+  stage(0);
+  for (int k = 0; k < nchunk; ++k) {
+    stage(k + 1);
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();
+    const T(*mk)[CH] = &ms[k & 1][warp * CG];
+    const T(*xk)[CH] = xs[k & 1];
+#pragma unroll
+    for (int s = 0; s < STEPS; ++s) {
+      T m[CG];
+#pragma unroll
+      for (int c = 0; c < CG; ++c) m[c] = mk[c][32 * s + lane];
+      if (s == 0 && k == 0 && o.tri) {
+        // a masked entry leaves its sum alone (x may be infinite there)
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const T xq = xk[q][lane];
+#pragma unroll
+          for (int c = 0; c < CG; ++c)
+            if (rbeg + lane >= c0 + c) v[c * R + q] = fma(m[c], xq, v[c * R + q]);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const T xq = xk[q][32 * s + lane];
+#pragma unroll
+          for (int c = 0; c < CG; ++c) v[c * R + q] = fma(m[c], xq, v[c * R + q]);
+        }
+      }
+    }
+    __syncthreads();   // the chunk's buffers are free for chunk k + 2
   }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  gemv_t_finish<T, R, CG>(v, o, sg, c0);
 }
 
-template <typename T, int R>
+template <typename T, int R, bool FINE>
 __device__ __forceinline__ void gemv_t_cta(const GemvSeg<T>& sg, int b) {
-  if constexpr (R >= 8) gemv_t_many<T, R>(sg, b);
-  else gemv_t_few<T, R>(sg, b);
+  constexpr int CG = FINE ? GEMV_CG_FINE : GEMV_CG;
+  if constexpr (R >= 8) gemv_t_many<T, R, CG>(sg, b);
+  else gemv_t_few<T, R, CG>(sg, b);
 }
 
 // M x, FP32 up to 4 columns: three CTAs per SM keep 24 warps of loads in
@@ -478,44 +485,69 @@ __device__ __forceinline__ void gemv_t_cta(const GemvSeg<T>& sg, int b) {
 // four warps keep a chunk each in flight.
 template <int TRANS>
 constexpr int gemv_threads() { return TRANS ? GEMV_T_THREADS : GEMV_THREADS; }
+template <int TRANS>   // fine blocks per coarse block
+__host__ __device__ constexpr int gemv_finer() { return TRANS ? GEMV_CG / GEMV_CG_FINE : 2; }
 template <typename T, int R, int TRANS>
 constexpr int gemv_ctas_per_sm() {
   if (TRANS) return R >= 8 ? (sizeof(T) == 8 ? 2 : R == 16 ? 3 : 4) : sizeof(T) == 4 ? 6 : R < 4 ? 5 : 4;
-  return sizeof(T) == 4 ? (R >= 8 ? 2 : 3) : (R >= 16 ? 1 : 2);
+  return sizeof(T) == 4 ? (R >= 8 ? 2 : 3) : 2;
 }
 
-template <typename T, int R, int TRANS>
+template <typename T, int R, int TRANS, bool FINE>
 __global__ void __launch_bounds__(gemv_threads<TRANS>(), (gemv_ctas_per_sm<T, R, TRANS>()))
     k_gemv(const GemvSeg<T> sg) {
-  if constexpr (TRANS) gemv_t_cta<T, R>(sg, blockIdx.x);
-  else gemv_n_cta<T, R>(sg, blockIdx.x);
+  if constexpr (TRANS) gemv_t_cta<T, R, FINE>(sg, blockIdx.x);
+  else gemv_n_cta<T, R, FINE>(sg, blockIdx.x);
 }
 
 // Grouped launches: block j runs block j - first of the segment that holds it
-// (one factor's mat-vec list for one block of right-hand sides).
-template <typename T, int R, int TRANS>
+// (one factor's mat-vec list for one block of right-hand sides; first counts
+// coarse blocks).
+template <typename T, int R, int TRANS, bool FINE>
 __global__ void __launch_bounds__(gemv_threads<TRANS>(), (gemv_ctas_per_sm<T, R, TRANS>()))
     k_gemv_seg(const GemvSeg<T>* __restrict__ segs, int nseg) {
+  constexpr int FINER = FINE ? gemv_finer<TRANS>() : 1;
+  const int64_t j = blockIdx.x / FINER;
   int k = 0;
-  while (k + 1 < nseg && segs[k + 1].first <= (int64_t)blockIdx.x) ++k;
+  while (k + 1 < nseg && segs[k + 1].first <= j) ++k;
   const GemvSeg<T> sg = segs[k];
-  const int b = (int)((int64_t)blockIdx.x - sg.first);
-  if constexpr (TRANS) gemv_t_cta<T, R>(sg, b);
-  else gemv_n_cta<T, R>(sg, b);
+  const int b = (int)((int64_t)blockIdx.x - sg.first * FINER);
+  if constexpr (TRANS) gemv_t_cta<T, R, FINE>(sg, b);
+  else gemv_n_cta<T, R, FINE>(sg, b);
 }
 
-template <typename T, int R>
-void launch_gemv(const GemvSeg<T>& sg, int trans, cudaStream_t st) {
+// A launch with fewer coarse blocks than this takes the fine form: half the
+// rows per CTA (M x) or a quarter of the columns (M^T x), the same sums.  Two
+// blocks per SM: below that SMs idle while others, in FP64 above all, work
+// through their tile (20^3 FP64, 10 columns: 7.6 ms a solve with the coarse
+// form alone, 4.9 ms with one column per warp).
+int gemv_fine_below() {
+  static const int n = [] {
+    int dev = 0, count = 0;
+    HIF_CUDA_TRY(cudaGetDevice(&dev));
+    HIF_CUDA_TRY(cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev));
+    return 2 * count;
+  }();
+  return n;
+}
+
+template <typename T, int R, int TRANS>
+void launch_gemv(const GemvSeg<T>& sg, cudaStream_t st) {
   const int ctas = gemv_ctas(sg.cnt);
-  if (trans) k_gemv<T, R, 1><<<ctas, GEMV_T_THREADS, 0, st>>>(sg);
-  else k_gemv<T, R, 0><<<ctas, GEMV_THREADS, 0, st>>>(sg);
+  if (ctas < gemv_fine_below())
+    k_gemv<T, R, TRANS, true><<<ctas * gemv_finer<TRANS>(), gemv_threads<TRANS>(), 0, st>>>(sg);
+  else
+    k_gemv<T, R, TRANS, false><<<ctas, gemv_threads<TRANS>(), 0, st>>>(sg);
   HIF_CHECK_LAUNCH();
 }
 
-template <typename T, int R>
-void launch_gemv_seg(const GemvSeg<T>* d_segs, int nseg, int ctas, int trans, cudaStream_t st) {
-  if (trans) k_gemv_seg<T, R, 1><<<ctas, GEMV_T_THREADS, 0, st>>>(d_segs, nseg);
-  else k_gemv_seg<T, R, 0><<<ctas, GEMV_THREADS, 0, st>>>(d_segs, nseg);
+template <typename T, int R, int TRANS>
+void launch_gemv_seg(const GemvSeg<T>* d_segs, int nseg, int ctas, cudaStream_t st) {
+  if (ctas < gemv_fine_below())
+    k_gemv_seg<T, R, TRANS, true>
+        <<<ctas * gemv_finer<TRANS>(), gemv_threads<TRANS>(), 0, st>>>(d_segs, nseg);
+  else
+    k_gemv_seg<T, R, TRANS, false><<<ctas, gemv_threads<TRANS>(), 0, st>>>(d_segs, nseg);
   HIF_CHECK_LAUNCH();
 }
 
@@ -548,14 +580,17 @@ int gemv_ctas(const int (&cnt)[4]) {
   return cnt[0] + ceil_div(cnt[1], 2) + ceil_div(cnt[2], 4) + ceil_div(cnt[3], 8);
 }
 
-int gemv_block(int left) { return left > 8 ? 16 : left > 4 ? 8 : left > 2 ? 4 : left; }
+int gemv_block(int left, size_t word) {
+  if (word == 8) return left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
+  return left > 8 ? 16 : left > 4 ? 8 : left > 2 ? 4 : left;
+}
 
 template <typename T>
 void gemv_batched(const GemvOp* h_ops, int nops, const GemvSeg<T>& list, int trans, int nrhs,
                   cudaStream_t st) {
   if (nops == 0 || gemv_ctas(list.cnt) == 0) return;
   for (int q0 = 0; q0 < nrhs;) {
-    const int R = gemv_block(nrhs - q0);
+    const int R = gemv_block(nrhs - q0, sizeof(T));
     GemvSeg<T> sg = list;
     sg.w = list.w + (int64_t)q0 * list.vs;
     sg.nv = std::min(R, nrhs - q0);
@@ -569,12 +604,14 @@ void gemv_batched(const GemvOp* h_ops, int nops, const GemvSeg<T>& list, int tra
       }
     }
     ProfScope ps(trans ? "apply_gemv_t" : "apply_gemv_n", st, fl, by);
+    if constexpr (sizeof(T) == 4)
+      if (R == 16) trans ? launch_gemv<T, 16, 1>(sg, st) : launch_gemv<T, 16, 0>(sg, st);
     switch (R) {
-      case 16: launch_gemv<T, 16>(sg, trans, st); break;
-      case 8: launch_gemv<T, 8>(sg, trans, st); break;
-      case 4: launch_gemv<T, 4>(sg, trans, st); break;
-      case 2: launch_gemv<T, 2>(sg, trans, st); break;
-      default: launch_gemv<T, 1>(sg, trans, st);
+      case 16: break;   // FP32 only (gemv_block)
+      case 8: trans ? launch_gemv<T, 8, 1>(sg, st) : launch_gemv<T, 8, 0>(sg, st); break;
+      case 4: trans ? launch_gemv<T, 4, 1>(sg, st) : launch_gemv<T, 4, 0>(sg, st); break;
+      case 2: trans ? launch_gemv<T, 2, 1>(sg, st) : launch_gemv<T, 2, 0>(sg, st); break;
+      default: trans ? launch_gemv<T, 1, 1>(sg, st) : launch_gemv<T, 1, 0>(sg, st);
     }
     q0 += sg.nv;
   }
@@ -585,12 +622,27 @@ void gemv_segments(const GemvSeg<T>* d_segs, int nseg, int ctas, int trans, int 
                    double bytes, cudaStream_t st) {
   if (ctas == 0) return;
   ProfScope ps(trans ? "apply_grouped_gemv_t" : "apply_grouped_gemv_n", st, flops, bytes);
+  if constexpr (sizeof(T) == 4)
+    if (R == 16)
+      trans ? launch_gemv_seg<T, 16, 1>(d_segs, nseg, ctas, st)
+            : launch_gemv_seg<T, 16, 0>(d_segs, nseg, ctas, st);
   switch (R) {
-    case 16: launch_gemv_seg<T, 16>(d_segs, nseg, ctas, trans, st); break;
-    case 8: launch_gemv_seg<T, 8>(d_segs, nseg, ctas, trans, st); break;
-    case 4: launch_gemv_seg<T, 4>(d_segs, nseg, ctas, trans, st); break;
-    case 2: launch_gemv_seg<T, 2>(d_segs, nseg, ctas, trans, st); break;
-    default: launch_gemv_seg<T, 1>(d_segs, nseg, ctas, trans, st);
+    case 16: break;
+    case 8:
+      trans ? launch_gemv_seg<T, 8, 1>(d_segs, nseg, ctas, st)
+            : launch_gemv_seg<T, 8, 0>(d_segs, nseg, ctas, st);
+      break;
+    case 4:
+      trans ? launch_gemv_seg<T, 4, 1>(d_segs, nseg, ctas, st)
+            : launch_gemv_seg<T, 4, 0>(d_segs, nseg, ctas, st);
+      break;
+    case 2:
+      trans ? launch_gemv_seg<T, 2, 1>(d_segs, nseg, ctas, st)
+            : launch_gemv_seg<T, 2, 0>(d_segs, nseg, ctas, st);
+      break;
+    default:
+      trans ? launch_gemv_seg<T, 1, 1>(d_segs, nseg, ctas, st)
+            : launch_gemv_seg<T, 1, 0>(d_segs, nseg, ctas, st);
   }
 }
 

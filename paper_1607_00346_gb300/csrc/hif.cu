@@ -288,7 +288,7 @@ struct Factor : FactorBase {
       slots += s.nidx + s.nset;
     }
     int blocks = 0;
-    for (int left = nrhs; left > 0; ++blocks) left -= gemv_block(left);
+    for (int left = nrhs; left > 0; ++blocks) left -= gemv_block(left, sizeof(T));
     *flops = 2.0 * 2.0 * (double)ent * nrhs;
     *bytes = 2.0 * ((double)ent * sizeof(T) * blocks + (double)slots * (6.0 + 2.0 * sizeof(T) * nrhs));
   }
@@ -427,7 +427,7 @@ void grouped_sweeps(const std::vector<Factor<T>*>& Fs, const std::vector<int>& n
     ys[h] = (int64_t)Fs[h]->n * Fs[h]->n * Fs[h]->n;
     vs[h] = Fs[h]->work_stride;
     for (int q0 = 0; q0 < nrhs[h];) {
-      const int R = gemv_block(nrhs[h] - q0), nv = std::min(R, nrhs[h] - q0);
+      const int R = gemv_block(nrhs[h] - q0, sizeof(T)), nv = std::min(R, nrhs[h] - q0);
       blocks[h].push_back(Block{q0, R, nv});
       q0 += nv;
     }
