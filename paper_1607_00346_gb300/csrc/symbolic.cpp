@@ -2,54 +2,133 @@
 #include "symbolic.h"
 
 #include <algorithm>
-#include <thread>
+#include <exception>
+#include <system_error>
 
 namespace hif {
 
 namespace {
 
+// f(i) for i in [0, n) in chunks of at least `grain` (about 20 us of work)
 template <class F>
-void parallel_for(int64_t n, F&& f) {
-  unsigned hw = std::thread::hardware_concurrency();
-  if (hw == 0) hw = 1;
-  int64_t nt = std::min<int64_t>(hw, (n + 255) / 256);
-  if (nt <= 1) {
+void parallel_for(Workers& w, int64_t n, int64_t grain, F&& f) {
+  const int64_t nc = std::min<int64_t>(4 * Workers::width(), (n + grain - 1) / grain);
+  if (nc <= 1) {
     for (int64_t i = 0; i < n; ++i) f(i);
     return;
   }
-  std::vector<std::thread> th;
-  th.reserve(nt);
-  for (int64_t t = 0; t < nt; ++t) {
-    th.emplace_back([&, t] {
-      int64_t a = n * t / nt, b = n * (t + 1) / nt;
-      for (int64_t i = a; i < b; ++i) f(i);
-    });
-  }
-  for (auto& x : th) x.join();
+  w.run((int)nc, [&](int c) {
+    for (int64_t i = n * c / nc, e = n * (c + 1) / nc; i < e; ++i) f(i);
+  });
 }
+constexpr int64_t LIGHT = 8192;   // grain of a few instructions per element
+constexpr int64_t FRONT = 16;     // of a cell's or front's rows
 
+// chunks of the two passes of build_cells_from over n DOFs
+int chunk_count(int64_t n) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(Workers::width(), n / 4096));
+}
 // f(t, a, b) on nt contiguous chunks [a, b) of [0, n), in parallel; the
 // chunks are in index order, so per-chunk results combine deterministically
 template <class F>
-int parallel_chunks(int64_t n, F&& f) {
-  unsigned hw = std::thread::hardware_concurrency();
-  if (hw == 0) hw = 1;
-  const int nt = (int)std::max<int64_t>(1, std::min<int64_t>(hw, n / 4096));
-  if (nt == 1) {
-    f(0, (int64_t)0, n);
-    return 1;
-  }
-  std::vector<std::thread> th;
-  th.reserve(nt);
-  for (int t = 0; t < nt; ++t)
-    th.emplace_back([&, t] { f(t, n * t / nt, n * (t + 1) / nt); });
-  for (auto& x : th) x.join();
-  return nt;
+void parallel_chunks(Workers& w, int nt, int64_t n, F&& f) {
+  w.run(nt, [&](int t) { f(t, n * t / nt, n * (t + 1) / nt); });
 }
 
 inline int popc3(int m) { return (m & 1) + ((m >> 1) & 1) + ((m >> 2) & 1); }
 
 }  // namespace
+
+// A loop of fewer chunks than this (0.3 ms of work) does not start the threads,
+// which takes longer: a 16^3 grid never starts them.
+constexpr int START = 16;
+
+struct Workers::Loop {
+  const std::function<void(int)>* f;
+  int chunks, next = 0, left;       // taken, not yet finished (under mu_)
+  std::exception_ptr err;
+  std::condition_variable done;
+};
+
+int Workers::width() {
+  const unsigned hw = std::thread::hardware_concurrency();
+  return hw == 0 ? 1 : (int)hw;
+}
+
+void Workers::start() {
+  started_ = true;
+  try {
+    for (int t = 1; t < width(); ++t) threads_.emplace_back([this] { work(); });
+  } catch (const std::system_error&) {
+    // fewer threads: the callers do the work themselves
+  }
+}
+
+Workers::~Workers() {
+  {
+    std::lock_guard<std::mutex> g(mu_);
+    stop_ = true;
+  }
+  wake_.notify_all();
+  for (auto& t : threads_) t.join();
+}
+
+void Workers::work() {
+  std::unique_lock<std::mutex> g(mu_);
+  for (;;) {
+    wake_.wait(g, [this] { return stop_ || !loops_.empty(); });
+    if (stop_) return;
+    Loop* l = loops_.front();
+    const int c = l->next++;
+    if (l->next == l->chunks) loops_.erase(loops_.begin());
+    g.unlock();
+    std::exception_ptr err;
+    try {
+      (*l->f)(c);
+    } catch (...) {
+      err = std::current_exception();
+    }
+    g.lock();
+    if (err && !l->err) l->err = err;
+    if (--l->left == 0) l->done.notify_one();   // l may be gone once mu_ is free
+  }
+}
+
+void Workers::run(int chunks, const std::function<void(int)>& f) {
+  if (chunks <= 0) return;
+  if (chunks == 1) {
+    f(0);
+    return;
+  }
+  Loop l;
+  l.f = &f;
+  l.chunks = l.left = chunks;
+  std::unique_lock<std::mutex> g(mu_);
+  if (!started_ && chunks < START) {
+    g.unlock();
+    for (int c = 0; c < chunks; ++c) f(c);
+    return;
+  }
+  if (!started_) start();
+  loops_.push_back(&l);
+  wake_.notify_all();
+  while (l.next < l.chunks) {
+    const int c = l.next++;
+    if (l.next == l.chunks) loops_.erase(std::find(loops_.begin(), loops_.end(), &l));
+    g.unlock();
+    std::exception_ptr err;
+    try {
+      f(c);
+    } catch (...) {
+      err = std::current_exception();
+    }
+    g.lock();
+    if (err && !l.err) l.err = err;
+    --l.left;
+  }
+  l.done.wait(g, [&] { return l.left == 0; });
+  if (l.err) std::rethrow_exception(l.err);
+}
 
 int hif_num_levels(int n, int m) {
   if (n <= 0 || m <= 0 || n % m) return -1;
@@ -111,7 +190,7 @@ void Symbolic::filter_rows(const SkelPlan& sp, const std::vector<uint8_t>& alive
   out.nF = sp.nF;
   out.nR.assign(nf, 0);
   std::vector<int64_t> kept(nf, 0);
-  parallel_for(nf, [&](int64_t f) {
+  parallel_for(workers_, nf, FRONT, [&](int64_t f) {
     int64_t k = 0;
     for (int64_t r = sp.rowOff[f]; r < sp.rowOff[f + 1]; ++r)
       if (r < sp.rowOff[f] + sp.nF[f] || alive[sp.rowDof[r]]) ++k;
@@ -121,7 +200,7 @@ void Symbolic::filter_rows(const SkelPlan& sp, const std::vector<uint8_t>& alive
   for (int f = 0; f < nf; ++f) off[f + 1] = off[f] + kept[f];
   PlanVec32 dof(off[nf]);
   PlanVec32 pos(off[nf] * ncp);
-  parallel_for(nf, [&](int64_t f) {
+  parallel_for(workers_, nf, FRONT, [&](int64_t f) {
     int64_t o = off[f];
     for (int64_t r = sp.rowOff[f]; r < sp.rowOff[f + 1]; ++r) {
       if (!(r < sp.rowOff[f] + sp.nF[f] || alive[sp.rowDof[r]])) continue;
@@ -148,9 +227,9 @@ void Symbolic::build_cells_from(int level, const std::vector<int32_t>& active, C
   cp.active = active;
   const int64_t na = (int64_t)cp.active.size();
   cp.slot.resize(N);
-  parallel_for(N, [&](int64_t g) { cp.slot[g] = -1; });
+  parallel_for(workers_, N, LIGHT, [&](int64_t g) { cp.slot[g] = -1; });
   cp.packed.resize(na);
-  parallel_for(na, [&](int64_t i) {
+  parallel_for(workers_, na, LIGHT, [&](int64_t i) {
     int32_t g = cp.active[i];
     cp.slot[g] = (int32_t)i;
     int x[3] = {g % n, (g / n) % n, g / (n * n)};
@@ -175,10 +254,9 @@ void Symbolic::build_cells_from(int level, const std::vector<int32_t>& active, C
   // interior / boundary counts per cell, per chunk of the active list; the
   // chunks then fill the lists at their running offsets, so the lists keep
   // ascending global order within each part, as a sequential pass would
-  unsigned hw = std::thread::hardware_concurrency();
-  const int ntmax = (int)std::max<int64_t>(1, std::min<int64_t>(hw == 0 ? 1 : hw, na / 4096));
-  std::vector<std::vector<int32_t>> cntI(ntmax), cntB(ntmax);
-  const int nt = parallel_chunks(na, [&](int t, int64_t a, int64_t b) {
+  const int nt = chunk_count(na);
+  std::vector<std::vector<int32_t>> cntI(nt), cntB(nt);
+  parallel_chunks(workers_, nt, na, [&](int t, int64_t a, int64_t b) {
     std::vector<int32_t>& ci = cntI[t];
     std::vector<int32_t>& cb = cntB[t];
     ci.assign(cp.ncell, 0);
@@ -212,7 +290,7 @@ void Symbolic::build_cells_from(int level, const std::vector<int32_t>& active, C
   cp.dofSlot.resize(cp.off[cp.ncell]);
   cp.dofPk.resize(cp.off[cp.ncell]);
   cp.posB.resize(na * 8);
-  parallel_chunks(na, [&](int t, int64_t a, int64_t b) {
+  parallel_chunks(workers_, nt, na, [&](int t, int64_t a, int64_t b) {
     std::vector<int32_t>& curI = cntI[t];
     std::vector<int32_t>& curB = cntB[t];
     for (int64_t i = a; i < b; ++i) {
@@ -250,7 +328,7 @@ void Symbolic::merge_maps(const CellPlan& child, const CellPlan& parent,
   for (int c = 0; c < parent.ncell; ++c)
     mapOff[c + 1] = mapOff[c] + 8 * (parent.off[c + 1] - parent.off[c]);
   map.resize(mapOff[parent.ncell]);
-  parallel_for(parent.ncell, [&](int64_t c) {
+  parallel_for(workers_, parent.ncell, FRONT, [&](int64_t c) {
     int px = (int)(c % C), py = (int)((c / C) % C), pz = (int)(c / ((int64_t)C * C));
     int64_t o = parent.off[c];
     int64_t nn = parent.off[c + 1] - o;
@@ -382,7 +460,7 @@ void Symbolic::build_skel(const CellPlan& cp, int kind, const std::vector<uint8_
     }
   };
   std::vector<int64_t> cnt(nf, 0);
-  parallel_for(nf, [&](int64_t f) {
+  parallel_for(workers_, nf, FRONT, [&](int64_t f) {
     int64_t c = 0;
     for_rows((int)f, false, [&](int32_t, const int32_t*) { ++c; });
     cnt[f] = c;
@@ -393,7 +471,7 @@ void Symbolic::build_skel(const CellPlan& cp, int kind, const std::vector<uint8_
   for (int f = 0; f < nf; ++f) sp.rowOff[f + 1] = sp.rowOff[f] + cnt[f];
   sp.rowDof.resize(sp.rowOff[nf]);
   sp.rowPos.resize(sp.rowOff[nf] * ncp);
-  parallel_for(nf, [&](int64_t f) {
+  parallel_for(workers_, nf, FRONT, [&](int64_t f) {
     int64_t r = sp.rowOff[f];
     for_rows((int)f, true, [&](int32_t g, const int32_t* pos) {
       sp.rowDof[r] = g;
