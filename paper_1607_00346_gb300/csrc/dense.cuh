@@ -87,31 +87,22 @@ int gemv_ctas(const int (&cnt)[4]);
 // masked columns would cost more than a second read: 8, 4, 2 or 1.
 int gemv_block(int left, size_t word);
 
-// One factor's list and block of right-hand sides: matrices at M + op.M,
-// vectors at w + op.x and w + op.y (w already shifted to the block's first
-// column, nv columns vs apart); `first` is its first thread block in a grouped
-// launch.
+// A planned list and its block of right-hand sides: matrices at M + op.M,
+// vectors at w + op.x and w + op.y, nv columns vs apart.
 template <typename T>
-struct GemvSeg {
+struct GemvList {
   const GemvOp* ops;
   const GemvTask* tasks;
   const T* M;
   T* w;
   int64_t vs;
-  int64_t first;
   int cnt[4];
   int nv;
 };
 
 // A list (ops, tasks, M, w, vs, cnt of `list`) for nrhs right-hand sides.
 template <typename T>
-void gemv_batched(const GemvOp* h_ops, int nops, const GemvSeg<T>& list, int trans, int nrhs,
+void gemv_batched(const GemvOp* h_ops, int nops, const GemvList<T>& list, int trans, int nrhs,
                   cudaStream_t st);
-// One launch over the segments of several factors' lists (ctas thread blocks
-// in all, R right-hand sides per segment).  Per column the arithmetic is
-// gemv_batched's, so a grouped apply is bitwise the factor's own apply.
-template <typename T>
-void gemv_segments(const GemvSeg<T>* d_segs, int nseg, int ctas, int trans, int R, double flops,
-                   double bytes, cudaStream_t st);
 
 }  // namespace hif

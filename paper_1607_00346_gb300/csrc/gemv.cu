@@ -21,7 +21,7 @@
 //     128-thread CTA; lanes stride the rows and share each x value between
 //     the eight columns; a transposing butterfly adds the lanes.
 // The order of every sum depends on the matrix shape only, so a column gets
-// the same bits in any block of right-hand sides and in a grouped launch.
+// the same bits in any block of right-hand sides.
 //
 // Measured on a 128^3 FP32 factor (2.86e9 entries, 22.9 GB in the two sweeps),
 // the mat-vecs of one apply: 1 column 3.9 ms (5.9 TB/s), 4 columns 5.0 ms, 16
@@ -89,7 +89,7 @@ __host__ __device__ constexpr int gemv_red_cols() {   // right-hand sides reduce
 
 // RL = 2: the whole tile, two rows per lane; RL = 1: its half `half`.
 template <typename T, int R, int RL>
-__device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, int ti, int half,
+__device__ __forceinline__ void gemv_n_tile(const GemvList<T>& sg, bool valid, int ti, int half,
                                             int ncls, T* xs_all, T* red) {
   constexpr int TR = 32 * RL;
   constexpr int XN = (GEMV_BC * R + 31) / 32;   // x values a lane stages per block
@@ -236,7 +236,7 @@ __device__ __forceinline__ void gemv_n_tile(const GemvSeg<T>& sg, bool valid, in
 }
 
 template <typename T, int R, bool FINE>
-__device__ __forceinline__ void gemv_n_cta(const GemvSeg<T>& sg, int b) {
+__device__ __forceinline__ void gemv_n_cta(const GemvList<T>& sg, int b) {
   constexpr int RL = FINE ? 1 : 2;
   __shared__ __align__(16) T xs[GEMV_WARPS * GEMV_BC * R];
   __shared__ T red[GEMV_WARPS * gemv_red_cols<T, R>() * 32 * RL];
@@ -304,7 +304,7 @@ __device__ __forceinline__ void cp_async(double* dst, const double* src, bool ok
 
 // Sums over the lanes and writes y of CG columns from c0 on.
 template <typename T, int R, int CG>
-__device__ __forceinline__ void gemv_t_finish(T (&v)[CG * R], const GemvOp& o, const GemvSeg<T>& sg,
+__device__ __forceinline__ void gemv_t_finish(T (&v)[CG * R], const GemvOp& o, const GemvList<T>& sg,
                                               int c0) {
   constexpr int V = CG * R;
   const int lane = threadIdx.x % 32;
@@ -327,7 +327,7 @@ __device__ __forceinline__ void gemv_t_finish(T (&v)[CG * R], const GemvOp& o, c
 }
 
 template <typename T, int R, int CG>
-__device__ __forceinline__ void gemv_t_few(const GemvSeg<T>& sg, int b) {
+__device__ __forceinline__ void gemv_t_few(const GemvList<T>& sg, int b) {
   constexpr int UN = 2 * GEMV_CG / CG;   // row steps in flight
   constexpr int SUB = GEMV_CG / CG;      // CTAs per task
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -387,7 +387,7 @@ __device__ __forceinline__ void gemv_t_few(const GemvSeg<T>& sg, int b) {
 
 // 8 or 16 right-hand sides.
 template <typename T, int R, int CG>
-__device__ __forceinline__ void gemv_t_many(const GemvSeg<T>& sg, int b) {
+__device__ __forceinline__ void gemv_t_many(const GemvList<T>& sg, int b) {
   constexpr int SUB = GEMV_CG / CG;                         // CTAs per task
   constexpr int TC = GEMV_TC / SUB;                         // columns of the CTA
   constexpr int CH = GEMV_T_THREADS * 4 / (int)sizeof(T);   // rows per chunk
@@ -473,7 +473,7 @@ __device__ __forceinline__ void gemv_t_many(const GemvSeg<T>& sg, int b) {
 }
 
 template <typename T, int R, bool FINE>
-__device__ __forceinline__ void gemv_t_cta(const GemvSeg<T>& sg, int b) {
+__device__ __forceinline__ void gemv_t_cta(const GemvList<T>& sg, int b) {
   constexpr int CG = FINE ? GEMV_CG_FINE : GEMV_CG;
   if constexpr (R >= 8) gemv_t_many<T, R, CG>(sg, b);
   else gemv_t_few<T, R, CG>(sg, b);
@@ -495,25 +495,9 @@ constexpr int gemv_ctas_per_sm() {
 
 template <typename T, int R, int TRANS, bool FINE>
 __global__ void __launch_bounds__(gemv_threads<TRANS>(), (gemv_ctas_per_sm<T, R, TRANS>()))
-    k_gemv(const GemvSeg<T> sg) {
+    k_gemv(const GemvList<T> sg) {
   if constexpr (TRANS) gemv_t_cta<T, R, FINE>(sg, blockIdx.x);
   else gemv_n_cta<T, R, FINE>(sg, blockIdx.x);
-}
-
-// Grouped launches: block j runs block j - first of the segment that holds it
-// (one factor's mat-vec list for one block of right-hand sides; first counts
-// coarse blocks).
-template <typename T, int R, int TRANS, bool FINE>
-__global__ void __launch_bounds__(gemv_threads<TRANS>(), (gemv_ctas_per_sm<T, R, TRANS>()))
-    k_gemv_seg(const GemvSeg<T>* __restrict__ segs, int nseg) {
-  constexpr int FINER = FINE ? gemv_finer<TRANS>() : 1;
-  const int64_t j = blockIdx.x / FINER;
-  int k = 0;
-  while (k + 1 < nseg && segs[k + 1].first <= j) ++k;
-  const GemvSeg<T> sg = segs[k];
-  const int b = (int)((int64_t)blockIdx.x - sg.first * FINER);
-  if constexpr (TRANS) gemv_t_cta<T, R, FINE>(sg, b);
-  else gemv_n_cta<T, R, FINE>(sg, b);
 }
 
 // A launch with fewer coarse blocks than this takes the fine form: half the
@@ -532,22 +516,12 @@ int gemv_fine_below() {
 }
 
 template <typename T, int R, int TRANS>
-void launch_gemv(const GemvSeg<T>& sg, cudaStream_t st) {
+void launch_gemv(const GemvList<T>& sg, cudaStream_t st) {
   const int ctas = gemv_ctas(sg.cnt);
   if (ctas < gemv_fine_below())
     k_gemv<T, R, TRANS, true><<<ctas * gemv_finer<TRANS>(), gemv_threads<TRANS>(), 0, st>>>(sg);
   else
     k_gemv<T, R, TRANS, false><<<ctas, gemv_threads<TRANS>(), 0, st>>>(sg);
-  HIF_CHECK_LAUNCH();
-}
-
-template <typename T, int R, int TRANS>
-void launch_gemv_seg(const GemvSeg<T>* d_segs, int nseg, int ctas, cudaStream_t st) {
-  if (ctas < gemv_fine_below())
-    k_gemv_seg<T, R, TRANS, true>
-        <<<ctas * gemv_finer<TRANS>(), gemv_threads<TRANS>(), 0, st>>>(d_segs, nseg);
-  else
-    k_gemv_seg<T, R, TRANS, false><<<ctas, gemv_threads<TRANS>(), 0, st>>>(d_segs, nseg);
   HIF_CHECK_LAUNCH();
 }
 
@@ -586,12 +560,12 @@ int gemv_block(int left, size_t word) {
 }
 
 template <typename T>
-void gemv_batched(const GemvOp* h_ops, int nops, const GemvSeg<T>& list, int trans, int nrhs,
+void gemv_batched(const GemvOp* h_ops, int nops, const GemvList<T>& list, int trans, int nrhs,
                   cudaStream_t st) {
   if (nops == 0 || gemv_ctas(list.cnt) == 0) return;
   for (int q0 = 0; q0 < nrhs;) {
     const int R = gemv_block(nrhs - q0, sizeof(T));
-    GemvSeg<T> sg = list;
+    GemvList<T> sg = list;
     sg.w = list.w + (int64_t)q0 * list.vs;
     sg.nv = std::min(R, nrhs - q0);
     double by = 0, fl = 0;
@@ -617,39 +591,8 @@ void gemv_batched(const GemvOp* h_ops, int nops, const GemvSeg<T>& list, int tra
   }
 }
 
-template <typename T>
-void gemv_segments(const GemvSeg<T>* d_segs, int nseg, int ctas, int trans, int R, double flops,
-                   double bytes, cudaStream_t st) {
-  if (ctas == 0) return;
-  ProfScope ps(trans ? "apply_grouped_gemv_t" : "apply_grouped_gemv_n", st, flops, bytes);
-  if constexpr (sizeof(T) == 4)
-    if (R == 16)
-      trans ? launch_gemv_seg<T, 16, 1>(d_segs, nseg, ctas, st)
-            : launch_gemv_seg<T, 16, 0>(d_segs, nseg, ctas, st);
-  switch (R) {
-    case 16: break;
-    case 8:
-      trans ? launch_gemv_seg<T, 8, 1>(d_segs, nseg, ctas, st)
-            : launch_gemv_seg<T, 8, 0>(d_segs, nseg, ctas, st);
-      break;
-    case 4:
-      trans ? launch_gemv_seg<T, 4, 1>(d_segs, nseg, ctas, st)
-            : launch_gemv_seg<T, 4, 0>(d_segs, nseg, ctas, st);
-      break;
-    case 2:
-      trans ? launch_gemv_seg<T, 2, 1>(d_segs, nseg, ctas, st)
-            : launch_gemv_seg<T, 2, 0>(d_segs, nseg, ctas, st);
-      break;
-    default:
-      trans ? launch_gemv_seg<T, 1, 1>(d_segs, nseg, ctas, st)
-            : launch_gemv_seg<T, 1, 0>(d_segs, nseg, ctas, st);
-  }
-}
-
-#define HIF_INST(T)                                                                             \
-  template void gemv_batched<T>(const GemvOp*, int, const GemvSeg<T>&, int, int, cudaStream_t); \
-  template void gemv_segments<T>(const GemvSeg<T>*, int, int, int, int, double, double,         \
-                                 cudaStream_t);
+#define HIF_INST(T) \
+  template void gemv_batched<T>(const GemvOp*, int, const GemvList<T>&, int, int, cudaStream_t);
 HIF_INST(float)
 HIF_INST(double)
 #undef HIF_INST

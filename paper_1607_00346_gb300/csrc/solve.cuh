@@ -17,25 +17,6 @@ void vec_set(const int32_t* g, const int32_t* pos, int64_t cnt, T* y, int64_t ys
 template <typename T>
 void vec_accumulate(const int32_t* tgt, const int64_t* ptr, const int32_t* src, int64_t ntgt,
                     T* y, int64_t ys, const T* work, int64_t vs, int nrhs, cudaStream_t st);
-// One factor's part of a grouped gather (kind 0: w[q vs + i] = y[q ys + a[i]]),
-// set (kind 1: y[q ys + a[i]] = w[q vs + b[i]]) or accumulate (kind 2:
-// y[q ys + a[t]] -= sum_{e = ptr[t]}^{ptr[t+1]-1} w[q vs + b[e]]), i < cnt,
-// q < nrhs: the parts of several factors in one launch.
-template <typename T>
-struct VecJob {
-  const int32_t* a;
-  const int32_t* b;
-  const int64_t* ptr;
-  int64_t cnt;
-  T* y;
-  int64_t ys;
-  T* w;
-  int64_t vs;
-  int nrhs;
-};
-template <typename T>
-void vec_grouped(int kind, const VecJob<T>* d_jobs, const VecJob<T>* h_jobs, int njobs,
-                 cudaStream_t st);
 // y = (T) x
 template <typename T>
 void vec_convert_in(const double* x, T* y, int64_t cnt, cudaStream_t st);
@@ -47,17 +28,33 @@ void vec_convert_out(const T* y, double* x, int64_t cnt, cudaStream_t st);
 // periodic: neighbours wrap around).
 void residual(const double* cpl, const double* diag, int n, int periodic, const double* f,
               const double* u, double* r, int nrhs, cudaStream_t st);
-// q = A p
-void matvec(const double* cpl, const double* diag, int n, int periodic, const double* p,
-            double* q, int nrhs, cudaStream_t st);
-// out[c] = sum_i x[c*N + i] * y[c*N + i] for c < ncol; `part` holds
-// ncol * 1024 partial sums.
-void dots(const double* x, const double* y, int64_t N, int ncol, double* part, double* out,
-          cudaStream_t st);
-// y[c] = y[c] + a[c] x[c]   (a: device array of ncol scalars; sign applied)
-void axpy_cols(const double* a, double sign, const double* x, double* y, int64_t N, int ncol,
-               cudaStream_t st);
-// p[c] = z[c] + b[c] p[c]
-void xpby_cols(const double* z, const double* b, double* p, int64_t N, int ncol, cudaStream_t st);
+
+// ---- the vector steps of the conjugate gradients --------------------------------
+// Scalars of nrhs columns on the device: the iteration's coefficients are formed
+// there, so the host waits once per iteration, for rr.
+struct PcgScalars {
+  double* rz;    // r . z
+  double* al;    // r . z / p . q, 0 for a finished column
+  double* be;    // see pcg_next_p, 0 for a finished column
+  double* rr;    // r . r
+  int* done;     // finished columns (kept by the caller, except the start's)
+  double* part;  // pcg_part_elems(N, nrhs) partial sums
+};
+int64_t pcg_part_elems(int64_t N, int nrhs);
+// rr = r . r; done = (rr == 0)
+void pcg_start(const double* r, int64_t N, int nrhs, const PcgScalars& s, cudaStream_t st);
+// p = z, rz = r . z
+void pcg_first_p(const double* r, const double* z, double* p, int64_t N, int nrhs,
+                 const PcgScalars& s, cudaStream_t st);
+// q = A p, al = rz / p . q
+void pcg_matvec(const double* cpl, const double* diag, int n, int periodic, const double* p,
+                double* q, int nrhs, const PcgScalars& s, cudaStream_t st);
+// u += al p, r -= al q, rr = r . r
+void pcg_update(const double* p, const double* q, double* u, double* r, int64_t N, int nrhs,
+                const PcgScalars& s, cudaStream_t st);
+// beta = (r . z - r_old . z) / rz (Polak-Ribiere) with r_old = r + al q, rz = r . z,
+// p = z + beta p (0 for a finished column)
+void pcg_next_p(const double* r, const double* q, const double* z, double* p, int64_t N, int nrhs,
+                const PcgScalars& s, cudaStream_t st);
 
 }  // namespace hif

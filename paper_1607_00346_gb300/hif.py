@@ -337,16 +337,16 @@ def _batch_args(handles, fs, us):
 
 
 def apply_batch(handles, fs, us, stream=None):
-    """hif_apply_batch: us[i] = F_i^{-1} fs[i] with the sweeps of every factor in
-    shared launches (bitwise each handle's own apply)."""
+    """hif_apply_batch: us[i] = F_i^{-1} fs[i] with the factors' sweeps side by
+    side on the GPU (bitwise each handle's own apply)."""
     hp, fp, up, nr, _keep = _batch_args(handles, fs, us)
     _check(load().hif_apply_batch(hp, len(handles), fp, up, nr, _stream(stream)))
     return us
 
 
 def solve_batch(handles, fs, us, stream=None, check=True):
-    """hif_solve_batch: PCG of every system in lockstep, preconditioner applied
-    as one grouped apply; returns per system (iterations, relative residuals)."""
+    """hif_solve_batch: PCG of every system in lockstep, each on its own
+    stream; returns per system (iterations, relative residuals)."""
     hp, fp, up, nr, _keep = _batch_args(handles, fs, us)
     tot = sum(nr)
     its = (ctypes.c_int * tot)()

@@ -15,7 +15,7 @@ right-hand sides.  The server
 * batches waiting requests: those for one operator become one multi-column
   system, and the systems of every resident operator that has waiting
   requests (grids of different sizes included) are solved together by one
-  hif_solve_batch, whose preconditioner applications share their launches;
+  hif_solve_batch, whose systems run side by side on the GPU;
   each request's result is bitwise the one it gets when served alone;
 * runs admitted jobs on several worker threads, each with its own CUDA stream,
   so that requests that arrive while others are on the GPU are taken up as
