@@ -18,7 +18,7 @@ LIB = os.path.join(BUILD, "libhif.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU_SOURCES = ["dense.cu", "gemv.cu", "tc.cu", "f64tc.cu", "front.cu", "idk.cu", "qr.cu", "solve.cu", "prof.cu", "peaks.cu",
+CU_SOURCES = ["dense.cu", "gemv.cu", "tc.cu", "f64tc.cu", "front.cu", "idk.cu", "pchol.cu", "qr.cu", "solve.cu", "prof.cu", "peaks.cu",
               "hif.cu"]
 CXX_SOURCES = ["symbolic.cpp", "tune.cpp"]
 

@@ -689,8 +689,8 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
           po.insert(po.end(), uo.begin(), uo.end());
           HIF_CUDA_TRY(cudaMemcpyAsync(d_step, po.data(), sizeof(GemmOp) * 2 * nbelow,
                                        cudaMemcpyHostToDevice, st));
-          gemm_f64tc(d_step, po.data(), nbelow, Karena, Parena, Karena, d_flags, st, "chol_panel_f64tc");
-          gemm_f64tc(d_step + nbelow, uo.data(), nbelow, Karena, Karena, Karena, d_flags, st,
+          gemm_f64tc<double>(d_step, po.data(), nbelow, Karena, Parena, Karena, d_flags, st, "chol_panel_f64tc");
+          gemm_f64tc<double>(d_step + nbelow, uo.data(), nbelow, Karena, Karena, Karena, d_flags, st,
                      "chol_trailing_update_f64tc");
           HIF_CUDA_TRY(cudaFreeAsync(d_step, st));
           continue;

@@ -39,11 +39,11 @@ void gemm_tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const float* Ab
              const float* Bbase, float* Cbase, int* d_flags, cudaStream_t st,
              const char* name = "gemm_tc");
 
-// The same for FP64 data: 8-bit slices on the BF16 tensor cores, exact sums,
-// one rounding per entry (f64tc.cu).
-void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double* Abase,
-                const double* Bbase, double* Cbase, int* d_flags, cudaStream_t st,
-                const char* name);
+// The same with an FP64 result of FP64 or FP32 operands: 8-bit slices on the
+// BF16 tensor cores, exact sums, one rounding per entry (f64tc.cu).
+template <typename S>
+void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Abase, const S* Bbase,
+                double* Cbase, int* d_flags, cudaStream_t st, const char* name);
 
 // Autotuning of gemm_tc's tile shape: time the variants on the product
 // shapes recorded during a tuning factorization (tune.h).
@@ -63,7 +63,7 @@ void gemm_fma_or_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const
                        const char* name, const char* name_tc) {
   if constexpr (sizeof(T) == 8) {
     if (tensor_cores && f64tc_worth(h_ops, nops)) {
-      gemm_f64tc(d_ops, h_ops, nops, Abase, Bbase, Cbase, d_flags, st, name_tc);
+      gemm_f64tc<double>(d_ops, h_ops, nops, Abase, Bbase, Cbase, d_flags, st, name_tc);
       return;
     }
   }

@@ -90,12 +90,13 @@ struct Tile {
 
 // Largest magnitude over a block's rows for each k, as the upper word of its
 // double (kx zeroed before; gridDim.y CTAs share the block's k).
+template <typename S>
 __global__ void __launch_bounds__(256) k_f64_kmax(const SliceBlk* __restrict__ blks,
-                                                  const double* __restrict__ Ab,
-                                                  const double* __restrict__ Bb, int* kx) {
+                                                  const S* __restrict__ Ab,
+                                                  const S* __restrict__ Bb, int* kx) {
   const SliceBlk b = blks[blockIdx.x];
   if (b.kx < 0) return;
-  const double* X = (b.isB ? Bb : Ab) + b.src;
+  const S* X = (b.isB ? Bb : Ab) + b.src;
   int* out = kx + b.kx + (b.isB ? b.k : 0);
   const int k0 = (int)((int64_t)b.k * blockIdx.y / gridDim.y);
   const int k1 = (int)((int64_t)b.k * (blockIdx.y + 1) / gridDim.y);
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(256) k_f64_kmax(const SliceBlk* __restrict__ b
       int m = 0;
 #pragma unroll 8
       for (int r = 0; r < b.rows; ++r)
-        m = max(m, __double2hiint(X[(int64_t)r * b.ld + k]) & 0x7fffffff);
+        m = max(m, __double2hiint((double)X[(int64_t)r * b.ld + k]) & 0x7fffffff);
       atomicMax(&out[k], m);
     }
   } else {
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(256) k_f64_kmax(const SliceBlk* __restrict__ b
     for (int k = k0 + warp; k < k1; k += 8) {
       int m = 0;
       for (int r = lane; r < b.rows; r += 32)
-        m = max(m, __double2hiint(X[r + (int64_t)k * b.ld]) & 0x7fffffff);
+        m = max(m, __double2hiint((double)X[r + (int64_t)k * b.ld]) & 0x7fffffff);
       m = __reduce_max_sync(0xffffffffu, m);
       if (lane == 0) atomicMax(&out[k], m);
     }
@@ -139,12 +140,13 @@ __device__ __forceinline__ int entry_exp(double x, int t) {
   if (h == 0 && __double2loint(x) == 0) return 0;
   return max(e, 1) + t + ROW_BIAS;
 }
+template <typename S>
 __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ blks,
-                                                  const double* __restrict__ Ab,
-                                                  const double* __restrict__ Bb,
+                                                  const S* __restrict__ Ab,
+                                                  const S* __restrict__ Bb,
                                                   const int* __restrict__ kx, int* exps) {
   const SliceBlk b = blks[blockIdx.x];
-  const double* X = (b.isB ? Bb : Ab) + b.src;
+  const S* X = (b.isB ? Bb : Ab) + b.src;
   const int k0 = (int)((int64_t)b.k * blockIdx.y / gridDim.y);
   const int k1 = (int)((int64_t)b.k * (blockIdx.y + 1) / gridDim.y);
   int* out = exps + (int64_t)blockIdx.x * BR;
@@ -190,13 +192,14 @@ __device__ __forceinline__ int64_t fixed62(double x, int s) {
 }
 
 // One thread: eight consecutive k of one row -> 16 bytes of each slice.
+template <typename S>
 __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ blks,
-                                                   const double* __restrict__ Ab,
-                                                   const double* __restrict__ Bb,
+                                                   const S* __restrict__ Ab,
+                                                   const S* __restrict__ Bb,
                                                    const int* __restrict__ kx,
                                                    const int* __restrict__ exps, unsigned char* W) {
   const SliceBlk b = blks[blockIdx.x];
-  const double* X = (b.isB ? Bb : Ab) + b.src;
+  const S* X = (b.isB ? Bb : Ab) + b.src;
   // a warp covers 8 rows x 4 groups of 8 k: 512 contiguous bytes of two blocks
   const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
   const int r = warp * 8 + lane % 8, kg = lane / 8;
@@ -209,8 +212,9 @@ __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ 
     for (int j = 0; j < 8; ++j) {
       const int k = g * 8 + j;
       t[j] = k < b.k ? balance(b, kx, k) : 0;
-      x[j] = (r < b.rows && k < b.k) ? X[b.kcont ? (int64_t)r * b.ld + k : r + (int64_t)k * b.ld]
-                                     : 0.0;
+      x[j] = (r < b.rows && k < b.k)
+                 ? (double)X[b.kcont ? (int64_t)r * b.ld + k : r + (int64_t)k * b.ld]
+                 : 0.0;
     }
     // adding 128 to every digit but the first makes the bytes of the sum the
     // digits + 128; a byte put into the low mantissa of 2^23 and taken back
@@ -487,9 +491,9 @@ bool f64tc_worth(const GemmOp* h_ops, int nops) {
   return false;
 }
 
-void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double* Abase,
-                const double* Bbase, double* Cbase, int* d_flags, cudaStream_t st,
-                const char* name) {
+template <typename S>
+void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Abase, const S* Bbase,
+                double* Cbase, int* d_flags, cudaStream_t st, const char* name) {
   static const bool attr = [] {   // initialised once, also under concurrent factorizations
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_gemm_f64tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       NST * STAGE));
@@ -550,12 +554,12 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double
     HIF_CUDA_TRY(cudaMemsetAsync(d_exps, 0, eb, st));
     const int gy = std::max(1, std::min({ceil_div(kmax, 64), 64, ceil_div(4096, (int64_t)blks.size())}));
     if (nkx) {
-      k_f64_kmax<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx);
+      k_f64_kmax<S><<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx);
       HIF_CHECK_LAUNCH();
     }
-    k_f64_exps<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps);
+    k_f64_exps<S><<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps);
     HIF_CHECK_LAUNCH();
-    k_f64_slice<<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps, W);
+    k_f64_slice<S><<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps, W);
     HIF_CHECK_LAUNCH();
     k_gemm_f64tc<<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(d_tiles, d_ops, d_blks, d_exps,
                                                                        W, Cbase, d_flags);
@@ -566,5 +570,10 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const double
     f0 = f;
   }
 }
+
+template void gemm_f64tc<double>(const GemmOp*, const GemmOp*, int, const double*, const double*,
+                                 double*, int*, cudaStream_t, const char*);
+template void gemm_f64tc<float>(const GemmOp*, const GemmOp*, int, const float*, const float*,
+                                double*, int*, cudaStream_t, const char*);
 
 }  // namespace hif

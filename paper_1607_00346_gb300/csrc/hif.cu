@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "dense.cuh"
 #include "front.cuh"
+#include "pchol.cuh"
 #include "solve.cuh"
 #include "symbolic.h"
 #include "tune.h"
@@ -919,16 +920,21 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
   for (int f = 0; f < nf; ++f)
     sel[(sd[f].nR > 2 * sd[f].nF && sd[f].nF >= 96) ? 1 : 0].push_back(f);
   DevBuf Rbuf;
+  bool gram = false;   // FP32 with tensor cores: both at once, from the Gram matrix
   if (!sel[1].empty()) {
     std::vector<int64_t> roff(sel[1].size());
     int64_t rtot = 0;
+    int nFmax = 0;
     for (size_t i = 0; i < sel[1].size(); ++i) {
       roff[i] = rtot;
       rtot += (int64_t)sd[sel[1][i]].nF * sd[sel[1][i]].nF;
+      nFmax = std::max(nFmax, sd[sel[1][i]].nF);
     }
     Rbuf.alloc_async(sizeof(T) * rtot, &F_.mem, st_);
-    reduce_rows_qr<T>(sd.data(), sel[1], G.as<T>(), Rbuf.as<T>(), roff, flags_.as<int>(),
-                      F_.opt.tensor_cores != 0, st_);
+    gram = std::is_same<T, float>::value && F_.opt.tensor_cores && gram_id_fits(nFmax);
+    if (!gram)
+      reduce_rows_qr<T>(sd.data(), sel[1], G.as<T>(), Rbuf.as<T>(), roff, flags_.as<int>(),
+                        F_.opt.tensor_cores != 0, st_);
     for (size_t i = 0; i < sel[1].size(); ++i) {
       SkelDesc& d = sd[sel[1][i]];
       d.idoff = roff[i];
@@ -959,13 +965,19 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
   for (int g = 0; g < 2; ++g) {
     if (sel[g].empty()) continue;
     for (int f : sel[g]) sub[g].push_back(sd[f]);
-    route[g].assign(sel[g].size(), ID_ROUTE_STREAM);
+    route[g].assign(sel[g].size(), g == 1 && gram ? ID_ROUTE_GRAM : ID_ROUTE_STREAM);
     upload_async(sub_d[g], sub[g], &F_.mem, st_);
-    interpolative_decomposition<T>(sub_d[g].as<SkelDesc>(), sub[g].data(), (int)sub[g].size(),
+    if (g == 1 && gram) {
+      if constexpr (std::is_same<T, float>::value)
+        gram_id(sub_d[g].as<SkelDesc>(), sub[g].data(), (int)sub[g].size(), G.as<T>(), Rbuf.as<T>(),
+                perm_d.as<int32_t>(), F_.eps, flags_.as<int>(), st_);
+    } else {
+      interpolative_decomposition<T>(sub_d[g].as<SkelDesc>(), sub[g].data(), (int)sub[g].size(),
                                    g == 0 ? G.as<T>() : Rbuf.as<T>(),
                                    (g == 0 ? G.bytes() : Rbuf.bytes()) / sizeof(T),
                                    perm_d.as<int32_t>(), tm.as<T>(), steps.as<int32_t>(), F_.eps,
                                    st_, route[g].data());
+    }
     HIF_CUDA_TRY(cudaMemcpyAsync(sub[g].data(), sub_d[g].as<void>(),
                                  sizeof(SkelDesc) * sub[g].size(), cudaMemcpyDeviceToHost, st_));
   }
@@ -1006,11 +1018,16 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
     // the k steps; in the shared-memory kernel also T = R11^{-1} R12
     // (k^2 (nF - k) flops; id_solve_t counts it for the others); bytes: the
     // matrix read once, T (or R) and the pivots written once
-    double fl[3] = {0.0, 0.0, 0.0}, by[3] = {0.0, 0.0, 0.0};
+    double fl[4] = {0.0, 0.0, 0.0, 0.0}, by[4] = {0.0, 0.0, 0.0, 0.0};
     for (int g = 0; g < 2; ++g)
       for (size_t j = 0; j < sel[g].size(); ++j) {
         const int f = sel[g][j], sm = route[g][j];
         const double k = sd[f].k, nF = sd[f].nF;
+        if (sm == ID_ROUTE_GRAM) {   // pivoted Cholesky: k nF (nF - k) + k^3 / 3 ..
+          fl[sm] += k * nF * (nF - k) + k * k * k / 3.0;
+          by[sm] += 8.0 * 0.5 * nF * nF;
+          continue;
+        }
         for (int i = 0; i < sd[f].k; ++i)
           fl[sm] += 4.0 * (double)(sd[f].idm - i) * (sd[f].nF - i - 1);
         if (sm == ID_ROUTE_SMEM) {
@@ -1023,6 +1040,7 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
     prof_add("id_cpqr", fl[ID_ROUTE_STREAM], by[ID_ROUTE_STREAM]);
     prof_add("id_cpqr_smem", fl[ID_ROUTE_SMEM], by[ID_ROUTE_SMEM]);
     prof_add("id_cpqr_dsm", fl[ID_ROUTE_CLUSTER_SMEM], by[ID_ROUTE_CLUSTER_SMEM]);
+    if (gram) prof_add("id_pchol", fl[ID_ROUTE_GRAM], by[ID_ROUTE_GRAM]);
   }
   // fronts with redundant DOFs are eliminated; the others keep every DOF
   std::vector<int> act;

@@ -1,0 +1,340 @@
+// Interpolative decomposition of FP32 faces with many coupled rows, from their
+// Gram matrix in FP64.
+//
+// The ID of A_RF (§2.3) depends on A_RF only through the norms of combinations of
+// its columns, so the pivots and the R factor of its column-pivoted QR are those
+// of the pivoted Cholesky factorization G = A_RF^T A_RF = P R^T R P^T: each step
+// takes the column with the largest remaining diagonal entry, |R_ii|^2, and
+// subtracts the outer product of its row of R.  Squaring the matrix squares its
+// condition number, so G needs twice the digits: it is formed from the FP32
+// entries with exact sums (f64tc.cu, 2^-62 below column maximum times column
+// maximum) and factored in FP64, which leaves R_ii an error of 1e-8 |R_11| at the
+// worst, where Householder QR in FP32 leaves 6e-8.
+//
+// What it replaces is bound by chains: the unpivoted QR of the tall A_RF column by
+// column (two barriers and a pass over a 32-column panel each), then pivoted QR of
+// R, whose every step reads the trailing matrix once.  Here the tall matrix is
+// read once, by tensor-core products, and a pivot step reads one column of G: 64
+// steps per launch in k_pchol (a cluster per front, one column per thread), then
+// one product per front updates G.  128^3, FP32, eps 1e-6: row reduction and ID of
+// the three upper levels' faces 300 ms, here 115 ms (61 + 28 the products, 26 the
+// steps; 32 steps per launch: 61 + 53 + 18).
+#include <algorithm>
+#include <vector>
+
+#include <cooperative_groups.h>
+
+#include "common.cuh"
+#include "dense.cuh"
+#include "front.cuh"
+#include "pchol.cuh"
+
+namespace hif {
+
+namespace cg = cooperative_groups;
+
+namespace {
+
+constexpr int PC_THREADS = 256;    // columns per CTA
+constexpr int PC_WARPS = PC_THREADS / 32;
+constexpr int PC_STEPS = 64;       // pivots per launch
+constexpr int PC_MAX_CS = 16;
+constexpr size_t PC_SMEM = sizeof(double) * PC_STEPS * PC_THREADS;
+
+struct PcDesc {
+  int64_t G;       // n x n (lower triangle), in the Gram arena
+  int64_t L;       // n x PC_STEPS, in the block arena
+  int64_t R;       // offset in the R arena (leading dimension n)
+  int64_t col;     // first entry of its columns' state
+  int64_t perm;    // offset of its permutation
+  int n, front;    // front: index in the SkelDesc array
+};
+
+struct PcState {
+  double d1;       // the first pivot's diagonal, |R_11|^2
+  int k, done;     // pivots so far; no further ones
+};
+
+__global__ void k_pchol_init(const PcDesc* __restrict__ ds, const double* __restrict__ G,
+                             double* diag, int* step, PcState* stt) {
+  const PcDesc d = ds[blockIdx.x];
+  for (int c = threadIdx.x; c < d.n; c += blockDim.x) {
+    diag[d.col + c] = G[d.G + c + (int64_t)c * d.n];
+    step[d.col + c] = -1;
+  }
+  if (threadIdx.x == 0) stt[blockIdx.x] = PcState{0.0, 0, 0};
+}
+
+// PC_STEPS pivots of each listed front: column c belongs to thread c % 256 of CTA
+// c / 256 of its cluster, which keeps its remaining diagonal in a register and its
+// entries of the block's rows of R in shared memory.  Per step every CTA proposes
+// its largest diagonal, with that column's entries of the block so far, to all
+// CTAs of the cluster; after one cluster barrier all pick the same winner
+// (largest, lowest column on ties) and each thread forms its entry of the new row,
+// (G_cp - sum of the block's products) / R_pp.
+__global__ void __launch_bounds__(PC_THREADS) k_pchol(const PcDesc* __restrict__ ds,
+                                                     const int* __restrict__ list,
+                                                     const double* __restrict__ Gar, double* Lar,
+                                                     float* Rar, double* diag, int* step,
+                                                     PcState* stt, double eps2) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int f = list[blockIdx.x / CS];
+  const PcDesc d = ds[f];
+  const int n = d.n, tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const int c = rank * PC_THREADS + tid;
+  const bool in = c < n;
+  extern __shared__ __align__(16) unsigned char psm[];
+  double(*Lb)[PC_THREADS] = reinterpret_cast<double(*)[PC_THREADS]>(psm);
+  __shared__ double s_bd[2][PC_MAX_CS], s_row[2][PC_MAX_CS][PC_STEPS];
+  __shared__ int s_bc[2][PC_MAX_CS];
+  __shared__ double w_d[PC_WARPS];
+  __shared__ int w_c[PC_WARPS];
+  const double* G = Gar + d.G;
+  double dc = in ? diag[d.col + c] : 0.0;
+  int tk = in ? step[d.col + c] : 0;
+  const PcState s0 = stt[f];
+  double d1 = s0.d1;
+  bool done = false;
+  int j = 0;
+  cl.sync();   // every CTA of the cluster runs before the first push
+  for (; j < PC_STEPS; ++j) {
+    const int par = j & 1;
+    double bd = tk < 0 ? dc : -1.0;
+    int bc = c;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+      const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
+      if (od > bd || (od == bd && oc < bc)) {
+        bd = od;
+        bc = oc;
+      }
+    }
+    if (lane == 0) {
+      w_d[warp] = bd;
+      w_c[warp] = bc;
+    }
+    __syncthreads();   // also: every thread's entry of the last row is in Lb
+    if (warp == 0) {
+      bd = w_d[lane % PC_WARPS];
+      bc = w_c[lane % PC_WARPS];
+#pragma unroll
+      for (int o = PC_WARPS / 2; o > 0; o >>= 1) {
+        const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+        const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
+        if (od > bd || (od == bd && oc < bc)) {
+          bd = od;
+          bc = oc;
+        }
+      }
+      for (int q = 0; q < CS; ++q) {
+        for (int t = lane; t < j; t += 32)
+          *cl.map_shared_rank(&s_row[par][rank][t], q) = Lb[t][bc - rank * PC_THREADS];
+        if (lane == 0) {
+          *cl.map_shared_rank(&s_bd[par][rank], q) = bd;
+          *cl.map_shared_rank(&s_bc[par][rank], q) = bc;
+        }
+      }
+    }
+    cl.sync();
+    double md = -1.0;
+    int mc = 0, mr = 0;
+    for (int q = 0; q < CS; ++q)
+      if (s_bd[par][q] > md || (s_bd[par][q] == md && s_bc[par][q] < mc)) {
+        md = s_bd[par][q];
+        mc = s_bc[par][q];
+        mr = q;
+      }
+    if (s0.k + j == 0) d1 = md;
+    if (!(md > 0.0) || !(md > eps2 * d1) || !isfinite(md)) {
+      done = true;
+      break;
+    }
+    double l = 0.0;
+    if (tk < 0) {
+      const double inv = rsqrt(md);
+      const double g = c >= mc ? G[c + (int64_t)mc * n] : G[mc + (int64_t)c * n];
+      const double* row = s_row[par][mr];
+      double t0 = g, t1 = 0.0, t2 = 0.0, t3 = 0.0;
+      int q = 0;
+      for (; q + 4 <= j; q += 4) {
+        t0 = fma(-Lb[q][tid], row[q], t0);
+        t1 = fma(-Lb[q + 1][tid], row[q + 1], t1);
+        t2 = fma(-Lb[q + 2][tid], row[q + 2], t2);
+        t3 = fma(-Lb[q + 3][tid], row[q + 3], t3);
+      }
+      for (; q < j; ++q) t0 = fma(-Lb[q][tid], row[q], t0);
+      l = ((t0 + t1) + (t2 + t3)) * inv;
+      if (c == mc) {
+        l = md * inv;
+        tk = s0.k + j;
+      } else {
+        dc = fma(-l, l, dc);
+      }
+    }
+    Lb[j][tid] = l;
+  }
+  cl.sync();   // no CTA leaves while another may still read its proposal
+  if (in) {
+    for (int q = 0; q < PC_STEPS; ++q) Lar[d.L + c + (int64_t)q * n] = q < j ? Lb[q][tid] : 0.0;
+    float* R = Rar + d.R + s0.k + (int64_t)c * n;
+    for (int q = 0; q < j; ++q) R[q] = (float)Lb[q][tid];
+    diag[d.col + c] = dc;
+    step[d.col + c] = tk;
+  }
+  if (rank == 0 && tid == 0) stt[f] = PcState{d1, s0.k + j, done || s0.k + j == n ? 1 : 0};
+}
+
+// the pivots in order, then the other columns in increasing order
+__global__ void __launch_bounds__(PC_THREADS) k_pchol_perm(const PcDesc* __restrict__ ds,
+                                                          const int* __restrict__ step,
+                                                          const PcState* __restrict__ stt,
+                                                          int32_t* perm, SkelDesc* fr) {
+  const PcDesc d = ds[blockIdx.x];
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  int32_t* pv = perm + d.perm;
+  __shared__ int s_cnt[PC_WARPS];
+  int base = stt[blockIdx.x].k;
+  if (tid == 0) fr[d.front].k = base;
+  for (int c0 = 0; c0 < d.n; c0 += PC_THREADS) {
+    const int c = c0 + tid;
+    const int t = c < d.n ? step[d.col + c] : 0;
+    const bool left = c < d.n && t < 0;
+    const unsigned m = __ballot_sync(0xffffffffu, left);
+    if (lane == 0) s_cnt[warp] = __popc(m);
+    __syncthreads();
+    int before = base, all = 0;
+    for (int w = 0; w < PC_WARPS; ++w) {
+      before += w < warp ? s_cnt[w] : 0;
+      all += s_cnt[w];
+    }
+    if (left) pv[before + __popc(m & ((1u << lane) - 1u))] = c;
+    else if (c < d.n) pv[t] = c;
+    base += all;
+    __syncthreads();
+  }
+}
+
+struct Pooled {   // stream-ordered scratch
+  void* p = nullptr;
+  cudaStream_t st;
+  Pooled(size_t bytes, cudaStream_t s) : st(s) {
+    HIF_CUDA_TRY(cudaMallocAsync(&p, std::max<size_t>(16, bytes), s));
+  }
+  Pooled(const Pooled&) = delete;
+  Pooled& operator=(const Pooled&) = delete;
+  ~Pooled() { cudaFreeAsync(p, st); }
+  template <typename U>
+  U* as() const { return static_cast<U*>(p); }
+};
+
+}  // namespace
+
+bool gram_id_fits(int nFmax) {
+  const int cs = ceil_div(nFmax, PC_THREADS);
+  if (cs > PC_MAX_CS) return false;
+  static const std::vector<int> placeable = [] {
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_pchol, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_pchol, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)PC_SMEM));
+    std::vector<int> ok(PC_MAX_CS + 1, 0);
+    for (int s = 1; s <= PC_MAX_CS; ++s) {
+      cudaLaunchConfig_t q = {};
+      q.gridDim = dim3((unsigned)s);
+      q.blockDim = dim3(PC_THREADS);
+      q.dynamicSmemBytes = PC_SMEM;
+      cudaLaunchAttribute qa[1];
+      qa[0].id = cudaLaunchAttributeClusterDimension;
+      qa[0].val.clusterDim.x = s;
+      qa[0].val.clusterDim.y = 1;
+      qa[0].val.clusterDim.z = 1;
+      q.attrs = qa;
+      q.numAttrs = 1;
+      int ncl = 0;
+      ok[s] = cudaOccupancyMaxActiveClusters(&ncl, k_pchol, &q) == cudaSuccess && ncl > 0;
+      cudaGetLastError();
+    }
+    return ok;
+  }();
+  return placeable[cs] != 0;
+}
+
+void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, float* Rout,
+             int32_t* perm, double eps, int* d_flags, cudaStream_t st) {
+  if (nf == 0) return;
+  std::vector<PcDesc> ds(nf);
+  std::vector<GemmOp> ops(nf);
+  int64_t gt = 0, lt = 0, ct = 0;
+  int nmax = 1;
+  for (int f = 0; f < nf; ++f) {
+    const SkelDesc& s = h_f[f];
+    ds[f] = PcDesc{gt, lt, s.idoff, ct, s.perm, s.nF, f};
+    ops[f] = GemmOp{s.G + s.nF, s.G + s.nF, gt, s.nF, s.nF, s.nR, s.nF + s.nR, s.nF + s.nR, s.nF, 1, 0,
+                    1.f, 0.f, 1, 0};
+    gt += (int64_t)s.nF * s.nF;
+    lt += (int64_t)s.nF * PC_STEPS;
+    ct += s.nF;
+    nmax = std::max(nmax, s.nF);
+  }
+  const int CS = ceil_div(nmax, PC_THREADS);
+  Pooled G(sizeof(double) * gt, st), L(sizeof(double) * lt, st), diag(sizeof(double) * ct, st),
+      step(sizeof(int) * ct, st), stt(sizeof(PcState) * nf, st), dds(sizeof(PcDesc) * nf, st),
+      dop(sizeof(GemmOp) * nf, st), lst(sizeof(int) * nf, st);
+  HIF_CUDA_TRY(cudaMemcpyAsync(dds.p, ds.data(), sizeof(PcDesc) * nf, cudaMemcpyHostToDevice, st));
+  HIF_CUDA_TRY(cudaMemcpyAsync(dop.p, ops.data(), sizeof(GemmOp) * nf, cudaMemcpyHostToDevice, st));
+  gemm_f64tc<float>(dop.as<GemmOp>(), ops.data(), nf, Garena, Garena, G.as<double>(), d_flags, st,
+                    "id_gram_f64tc");
+  {
+    ProfScope ps("id_pchol", st);
+    k_pchol_init<<<nf, 256, 0, st>>>(dds.as<PcDesc>(), G.as<double>(), diag.as<double>(),
+                                    step.as<int>(), stt.as<PcState>());
+    HIF_CHECK_LAUNCH();
+  }
+  std::vector<int> act(nf);
+  for (int f = 0; f < nf; ++f) act[f] = f;
+  std::vector<PcState> h(nf);
+  while (!act.empty()) {
+    HIF_CUDA_TRY(cudaMemcpyAsync(lst.p, act.data(), sizeof(int) * act.size(), cudaMemcpyHostToDevice, st));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(act.size() * CS));
+    cfg.blockDim = dim3(PC_THREADS);
+    cfg.dynamicSmemBytes = PC_SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CS;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    {
+      ProfScope ps("id_pchol", st);
+      HIF_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_pchol, (const PcDesc*)dds.as<PcDesc>(),
+                                      (const int*)lst.as<int>(), (const double*)G.as<double>(),
+                                      L.as<double>(), Rout, diag.as<double>(), step.as<int>(),
+                                      stt.as<PcState>(), eps * eps));
+      HIF_CHECK_LAUNCH();
+    }
+    HIF_CUDA_TRY(cudaMemcpyAsync(h.data(), stt.p, sizeof(PcState) * nf, cudaMemcpyDeviceToHost, st));
+    HIF_CUDA_TRY(cudaStreamSynchronize(st));
+    std::vector<int> next;
+    for (int f : act)
+      if (!h[f].done) next.push_back(f);
+    act.swap(next);
+    if (act.empty()) break;
+    // G -= L L^T of the fronts that go on
+    std::vector<GemmOp> up(act.size());
+    for (size_t i = 0; i < act.size(); ++i) {
+      const PcDesc& d = ds[act[i]];
+      up[i] = GemmOp{d.L, d.L, d.G, d.n, d.n, PC_STEPS, d.n, d.n, d.n, 0, 1, -1.f, 1.f, 1, 0};
+    }
+    HIF_CUDA_TRY(cudaMemcpyAsync(dop.p, up.data(), sizeof(GemmOp) * up.size(), cudaMemcpyHostToDevice, st));
+    gemm_f64tc<double>(dop.as<GemmOp>(), up.data(), (int)up.size(), L.as<double>(), L.as<double>(),
+                       G.as<double>(), d_flags, st, "id_pchol_update_f64tc");
+  }
+  k_pchol_perm<<<nf, PC_THREADS, 0, st>>>(dds.as<PcDesc>(), step.as<int>(), stt.as<PcState>(), perm, d_f);
+  HIF_CHECK_LAUNCH();
+}
+
+}  // namespace hif
