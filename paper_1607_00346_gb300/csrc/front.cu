@@ -287,7 +287,150 @@ __global__ void __launch_bounds__(256) k_skel_writeback(const SkelDesc* __restri
   }
 }
 
+
+// ---- row lists of faces and edges ------------------------------------------------
+// Listing the rows on the host and uploading them was the longest wait of the
+// level-0 plan (128^3: 15 million rows of 95232 faces, 38 ms); here a front is a
+// block of 32 to 256 threads that walks its cells' lists, bound by the loads of
+// the lists and of posb from L2.
+struct DofGeom {
+  int lc[3], sep;   // lowest cell holding the DOF, separator mask
+};
+__device__ __forceinline__ DofGeom dof_geom(const LevelGeom& geo, int g) {
+  DofGeom d;
+  const int z = g / (geo.n * geo.n), r = g - z * geo.n * geo.n;
+  const int x[3] = {r % geo.n, r / geo.n, z};
+  d.sep = 0;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int q = x[i] / geo.s;
+    const bool sd = x[i] == q * geo.s && (geo.wrap || x[i] != 0);
+    d.lc[i] = sd ? (q == 0 ? geo.C - 1 : q - 1) : q;
+    d.sep |= sd ? 1 << i : 0;
+  }
+  return d;
+}
+// corner of cell c (its three indices) relative to the DOF, -1 if its closure
+// does not hold the DOF
+__device__ __forceinline__ int corner_of(const LevelGeom& geo, const DofGeom& d, int c) {
+  const int cc[3] = {c % geo.C, c / geo.C % geo.C, c / (geo.C * geo.C)};
+  int q = 0;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (cc[i] == d.lc[i]) continue;
+    if (!((d.sep >> i) & 1) || cc[i] != (d.lc[i] + 1 == geo.C ? 0 : d.lc[i] + 1)) return -1;
+    q |= 1 << i;
+  }
+  return q;
+}
+
+__global__ void k_cell_positions(LevelGeom geo, const CellDesc* __restrict__ cells,
+                                 const int32_t* __restrict__ lists, int32_t* posb) {
+  const CellDesc c = cells[blockIdx.x];
+  const int32_t* b = lists + c.list + c.p;
+  for (int t = threadIdx.x; t < c.n - c.p; t += blockDim.x) {
+    const int g = b[t];
+    const int q = corner_of(geo, dof_geom(geo, g), blockIdx.x);
+    if (q >= 0) posb[(int64_t)g * 8 + q] = t;
+  }
+}
+
+template <int NCP, bool FILL>
+__global__ void k_skel_rows(LevelGeom geo, const RowFront* __restrict__ fronts,
+                            const CellDesc* __restrict__ cells, const int32_t* __restrict__ lists,
+                            const int32_t* __restrict__ posb, const uint8_t* __restrict__ alive,
+                            int* nR, const int64_t* __restrict__ rowOff, int32_t* rowPos) {
+  const RowFront f = fronts[blockIdx.x];
+  const int nw = blockDim.x / 32, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  __shared__ int s_cnt[32];
+  int32_t* out = FILL ? rowPos + rowOff[blockIdx.x] * NCP : nullptr;
+  int64_t base = 0;   // rows so far (the same in every thread)
+  const int low[3] = {f.cell[0] % geo.C, f.cell[0] / geo.C % geo.C, f.cell[0] / (geo.C * geo.C)};
+  // pass -1: the front's own DOFs, from its first cell; pass i: the rows its
+  // cell i adds
+  for (int i = FILL ? -1 : 0; i < NCP; ++i) {
+    const CellDesc c = cells[f.cell[max(i, 0)]];
+    const int32_t* b = lists + c.list + c.p;
+    const int nb = c.n - c.p;
+    for (int t0 = 0; t0 < nb; t0 += blockDim.x) {
+      const int t = t0 + threadIdx.x;
+      bool take = false;
+      int g = 0;
+      DofGeom d{};
+      if (t < nb) {
+        g = b[t];
+        d = dof_geom(geo, g);
+        const bool own = d.sep == f.sep && d.lc[0] == low[0] && d.lc[1] == low[1] && d.lc[2] == low[2];
+        if (i < 0) {
+          take = own;
+        } else if (!own && (!alive || alive[g])) {
+          take = true;
+          for (int j = 0; j < i; ++j) take = take && corner_of(geo, d, f.cell[j]) < 0;
+        }
+      }
+      // the taken entries keep their order: place within the block
+      const unsigned m = __ballot_sync(0xffffffffu, take);
+      int before = __popc(m & ((1u << lane) - 1u)), all = __popc(m);
+      if (nw > 1) {
+        __syncthreads();
+        if (lane == 0) s_cnt[warp] = all;
+        __syncthreads();
+        all = 0;
+        for (int w = 0; w < nw; ++w) {
+          before += w < warp ? s_cnt[w] : 0;
+          all += s_cnt[w];
+        }
+      }
+      if (FILL && take) {
+        int32_t* o = out + (base + before) * NCP;
+#pragma unroll
+        for (int j = 0; j < NCP; ++j) {
+          int pos = -1;
+          if (j == max(i, 0)) {
+            pos = t;
+          } else if (j > i) {
+            const int q = corner_of(geo, d, f.cell[j]);
+            if (q >= 0) pos = posb[(int64_t)g * 8 + q];
+          }
+          o[j] = pos;
+        }
+      }
+      base += all;
+    }
+  }
+  if (!FILL && threadIdx.x == 0) nR[blockIdx.x] = (int)base;
+}
+
 }  // namespace
+
+void cell_positions(const LevelGeom& geo, const CellDesc* d_cells, int ncell, const int32_t* lists,
+                    int32_t* posb, cudaStream_t st) {
+  if (ncell == 0) return;
+  ProfScope ps("row_lists", st);
+  k_cell_positions<<<ncell, 128, 0, st>>>(geo, d_cells, lists, posb);
+  HIF_CHECK_LAUNCH();
+}
+
+void skel_rows(const LevelGeom& geo, const RowFront* d_fronts, int nf, int ncp,
+               const CellDesc* d_cells, const int32_t* lists, const int32_t* posb,
+               const uint8_t* alive, int mean_list, int* nR, const int64_t* rowOff, int32_t* rowPos,
+               cudaStream_t st) {
+  if (nf == 0) return;
+  ProfScope ps("row_lists", st);
+  // threads per front: one walk of the list in a few rounds
+  const int th = mean_list <= 256 ? 32 : mean_list <= 1024 ? 128 : 256;
+  auto go = [&](auto kern) {
+    kern<<<nf, th, 0, st>>>(geo, d_fronts, d_cells, lists, posb, alive, nR, rowOff, rowPos);
+    HIF_CHECK_LAUNCH();
+  };
+  if (ncp == 2) {
+    if (rowPos) go(k_skel_rows<2, true>);
+    else go(k_skel_rows<2, false>);
+  } else {
+    if (rowPos) go(k_skel_rows<4, true>);
+    else go(k_skel_rows<4, false>);
+  }
+}
 
 void stencil_coefficients(const double* a, const double* b, double b_const, int n, int periodic,
                           double* cpl, double* diag, int* d_bad, cudaStream_t st) {

@@ -62,6 +62,29 @@ struct SkelDesc {
 // with the matrix spread over its CTAs' shared memory; or pivoted Cholesky of the
 // Gram matrix
 enum : int8_t { ID_ROUTE_STREAM = 0, ID_ROUTE_SMEM = 1, ID_ROUTE_CLUSTER_SMEM = 2, ID_ROUTE_GRAM = 3 };
+
+// The level's geometry (see symbolic.h), for the row lists.
+struct LevelGeom {
+  int n, s, C;
+  int wrap;         // periodic below the top level: every multiple of s separates
+};
+// A front as its rows are listed: its cells, separator mask and DOF count.
+struct RowFront {
+  int cell[4];
+  int sep, nF;
+};
+// posb[8 g + q]: position of DOF g in the boundary list of its corner-q cell, for
+// the cells that hold it (the other entries stay unwritten and are never read).
+void cell_positions(const LevelGeom& geo, const CellDesc* d_cells, int ncell, const int32_t* lists,
+                    int32_t* posb, cudaStream_t st);
+// Rows of each front: its own DOFs, then the boundary DOFs of its ncp cells that
+// are not its own and (with alive) still alive, each once, in the order of its
+// cells and their lists.  Counts (nR, rowPos = nullptr), or each row's position
+// in the front's cells (-1: not in that cell) to rowPos + ncp (rowOff[f] + row).
+void skel_rows(const LevelGeom& geo, const RowFront* d_fronts, int nf, int ncp,
+               const CellDesc* d_cells, const int32_t* lists, const int32_t* posb,
+               const uint8_t* alive, int mean_list, int* nR, const int64_t* rowOff, int32_t* rowPos,
+               cudaStream_t st);
 template <typename T>
 void skel_gather(const SkelDesc* d_f, const SkelDesc* h_f, int nf, int ncp,
                  const int32_t* rowPos, const CellDesc* d_cells, const T* Karena, T* Garena,

@@ -465,10 +465,14 @@ class Builder {
   }
   ~Builder() {
     jobs_.clear();   // waits for the host workers
-    if (up_st_) {
-      cudaStreamSynchronize(up_st_);
-      cudaStreamDestroy(up_st_);
-    }
+    cudaStreamSynchronize(st_);   // the row lists may still be read after an error
+    row_bufs_.clear();
+    for (cudaStream_t s : {up_st_, row_st_})
+      if (s) {
+        cudaStreamSynchronize(s);
+        cudaStreamDestroy(s);
+      }
+    if (row_ev_) cudaEventDestroy(row_ev_);
   }
 
   void run(const double* a_dev, const double* b_dev, double b_const);
@@ -478,8 +482,9 @@ class Builder {
   void cell_step(std::shared_ptr<const CellPlan> cpp, DevBuf& Kar, DevBuf& cdesc_d,
                  std::vector<CellDesc>& cdesc, DevBuf& lists_d);
   // returns the number of DOFs the step eliminated (marked dead in alive)
-  int64_t skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>& alive, DevBuf& Kar,
-                    DevBuf& cdesc_d, std::shared_ptr<const SkelPlan> plan);
+  // (filter: rows that are no longer alive are left out)
+  int64_t skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>& alive, bool filter,
+                    DevBuf& Kar, DevBuf& cdesc_d, std::shared_ptr<const SkelPlan> plan);
 
   // Host side of an apply stage (gather list, mat-vec lists, set and
   // accumulate lists).  It depends only on the plan and, for faces and edges,
@@ -514,6 +519,20 @@ class Builder {
     unstarted_.clear();
   }
   cudaStream_t up_st_ = nullptr;
+  // row lists of a level's faces and edges, made on a stream of their own while
+  // the cells are eliminated; freed at the end of the level
+  cudaStream_t row_st_ = nullptr;
+  cudaEvent_t row_ev_ = nullptr;
+  std::vector<DevBuf> row_bufs_;
+  LevelGeom geo_{};
+  const CellDesc* row_cells_ = nullptr;   // the level's cells and their lists
+  const int32_t* row_lists_ = nullptr;
+  const int32_t* row_posb_ = nullptr;
+  void* row_alloc(size_t bytes) {
+    row_bufs_.emplace_back();
+    row_bufs_.back().alloc_async(std::max<size_t>(16, bytes), &F_.mem, row_st_);
+    return row_bufs_.back().template as<void>();
+  }
   void upload_stages(bool all);
   static StageHost cell_stage_host(std::shared_ptr<const CellPlan> cpp,
                                    std::vector<CellDesc> cdesc, std::vector<int64_t> poff,
@@ -582,6 +601,8 @@ void Builder<T>::run(const double* a_dev, const double* b_dev, double b_const) {
   HIF_CUDA_TRY(cudaMemsetAsync(flags_.as<int>(), 0xff, sizeof(int) * FLAG_COUNT, st_));
 
   HIF_CUDA_TRY(cudaStreamCreateWithFlags(&up_st_, cudaStreamNonBlocking));
+  HIF_CUDA_TRY(cudaStreamCreateWithFlags(&row_st_, cudaStreamNonBlocking));
+  HIF_CUDA_TRY(cudaEventCreateWithFlags(&row_ev_, cudaEventDisableTiming));
   const int L = F_.L;
   std::shared_ptr<const CellPlan> prevp;
   DevBuf prevK, prevDesc;
@@ -619,6 +640,16 @@ void Builder<T>::run(const double* a_dev, const double* b_dev, double b_const) {
     Kar.alloc_async(sizeof(T) * std::max<int64_t>(1, koff), &F_.mem, st_);
     upload_async(cdesc_d, cdesc, &F_.mem, st_);
     upload(lists_d, cp.dofs, &F_.mem, st_);
+    geo_ = LevelGeom{n, cp.s, cp.C, F_.bc == 1 && level < L ? 1 : 0};
+    row_cells_ = cdesc_d.as<CellDesc>();
+    row_lists_ = lists_d.as<int32_t>();
+    if (level < L && F_.eps > 0.0) {
+      HIF_CUDA_TRY(cudaEventRecord(row_ev_, st_));   // cells and lists are on the device
+      HIF_CUDA_TRY(cudaStreamWaitEvent(row_st_, row_ev_, 0));
+      int32_t* posb = static_cast<int32_t*>(row_alloc(sizeof(int32_t) * 8 * N));
+      cell_positions(geo_, row_cells_, cp.ncell, row_lists_, posb, row_st_);
+      row_posb_ = posb;
+    }
     if (level == 0) {
       HIF_CUDA_TRY(cudaMemsetAsync(Kar.as<T>(), 0, sizeof(T) * koff, st_));
       const int maxbox = (cp.s + 1) * (cp.s + 1) * (cp.s + 1);
@@ -646,10 +677,10 @@ void Builder<T>::run(const double* a_dev, const double* b_dev, double b_const) {
       prevDesc.release();
     }
     tr_.mark(level, "frontal matrices");
-    // after the cell step the interiors are gone; the face and edge plans
-    // depend only on that set, so two host threads build them while the
-    // cells are eliminated on the GPU (the edge rows are filtered again once
-    // the faces have dropped their redundant DOFs)
+    // after the cell step the interiors are gone; the faces and edges depend
+    // only on that set, so two host threads find them while the cells are
+    // eliminated on the GPU (their rows are listed there, the edges' after the
+    // faces have dropped their redundant DOFs)
     std::vector<uint8_t> alive(N, 0);
     for (int32_t g : cp.active) alive[g] = 1;
     for (int c = 0; c < cp.ncell; ++c)
@@ -663,8 +694,8 @@ void Builder<T>::run(const double* a_dev, const double* b_dev, double b_const) {
     std::future<void> face_plan, edge_plan;
     if (level < L && F_.eps > 0.0) {
       alive_plan = alive;
-      face_plan = std::async(std::launch::async, [&]() { sym_.build_skel(cp, 1, alive_plan, *fbuild); });
-      edge_plan = std::async(std::launch::async, [&]() { sym_.build_skel(cp, 2, alive_plan, *ebuild); });
+      face_plan = std::async(std::launch::async, [&]() { sym_.build_fronts(cp, 1, alive_plan, *fbuild); });
+      edge_plan = std::async(std::launch::async, [&]() { sym_.build_fronts(cp, 2, alive_plan, *ebuild); });
     }
     cell_step(cpp, Kar, cdesc_d, cdesc, lists_d);
     tr_.mark(level, "cell elimination");
@@ -682,17 +713,12 @@ void Builder<T>::run(const double* a_dev, const double* b_dev, double b_const) {
       face_plan.get();
       fplan = fbuild;
       tr_.mark(level, "face plan joined");
-      const int64_t dropped = skel_step(cp, 1, alive, Kar, cdesc_d, fplan);
+      const int64_t dropped = skel_step(cp, 1, alive, false, Kar, cdesc_d, fplan);
       tr_.mark(level, "faces");
       edge_plan.get();
       eplan = ebuild;
       start_stage_jobs();
       tr_.mark(level, "edge plan joined");
-      if (dropped) {
-        auto filtered = std::make_shared<SkelPlan>();
-        sym_.filter_rows(*eplan, alive, *filtered);
-        eplan = std::move(filtered);
-      }
       // the next level's cells, assuming the edges keep every DOF (they
       // usually do), are planned on a host thread while the edges run;
       // rebuilt at the next level if an edge lost DOFs
@@ -705,14 +731,15 @@ void Builder<T>::run(const double* a_dev, const double* b_dev, double b_const) {
         sym_.build_cells_from(level + 1, act, spec_cells_);
         sym_.merge_maps(cp, spec_cells_, spec_mapOff_, spec_map_);
       });
-      skel_step(cp, 2, alive, Kar, cdesc_d, eplan);
+      skel_step(cp, 2, alive, dropped > 0, Kar, cdesc_d, eplan);
       spec.get();
       have_spec_ = (alive == alive_faces);
       tr_.mark(level, "edges");
     } else {
       start_stage_jobs();
     }
-    check_flags("level factorization");
+    check_flags("level factorization");   // waits for st_, the row lists' reader
+    row_bufs_.clear();
     std::vector<int32_t> next;
     next.reserve(cp.active.size());
     for (int32_t g : cp.active)
@@ -878,25 +905,57 @@ void Builder<T>::upload_stages(bool all) {
 }
 
 template <typename T>
-int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>& alive,
+int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>& alive, bool filter,
                               DevBuf& Kar, DevBuf& cdesc_d, std::shared_ptr<const SkelPlan> plan) {
   const SkelPlan& sp = *plan;
   tr_.mark(level_, kind == 1 ? " symbolic faces" : " symbolic edges");
   const int nf = sp.nfront;
   if (nf == 0) return 0;
   const int ncp = sp.ncellPer;
+  // row lists: counts, then positions, on row_st_
+  std::vector<int> nR(nf);
+  std::vector<int64_t> rowOff(nf + 1, 0);
+  int32_t* rowpos = nullptr;
+  {
+    std::vector<RowFront> rf(nf);
+    for (int f = 0; f < nf; ++f) {
+      rf[f] = RowFront{{0, 0, 0, 0}, sp.sep[f], sp.nF[f]};
+      for (int i = 0; i < ncp; ++i) rf[f].cell[i] = sp.cells[(size_t)f * ncp + i];
+    }
+    RowFront* rf_d = static_cast<RowFront*>(row_alloc(sizeof(RowFront) * nf));
+    int* nR_d = static_cast<int*>(row_alloc(sizeof(int) * nf));
+    int64_t* off_d = static_cast<int64_t*>(row_alloc(sizeof(int64_t) * nf));
+    uint8_t* alive_d = nullptr;
+    if (filter) {
+      alive_d = static_cast<uint8_t*>(row_alloc(alive.size()));
+      HIF_CUDA_TRY(cudaMemcpyAsync(alive_d, alive.data(), alive.size(), cudaMemcpyHostToDevice, row_st_));
+    }
+    HIF_CUDA_TRY(cudaMemcpyAsync(rf_d, rf.data(), sizeof(RowFront) * nf, cudaMemcpyHostToDevice, row_st_));
+    const int mean = (int)(cp.dofs.size() / std::max(1, cp.ncell));
+    skel_rows(geo_, rf_d, nf, ncp, row_cells_, row_lists_, row_posb_, alive_d, mean, nR_d, nullptr,
+              nullptr, row_st_);
+    HIF_CUDA_TRY(cudaMemcpyAsync(nR.data(), nR_d, sizeof(int) * nf, cudaMemcpyDeviceToHost, row_st_));
+    HIF_CUDA_TRY(cudaStreamSynchronize(row_st_));
+    for (int f = 0; f < nf; ++f) rowOff[f + 1] = rowOff[f] + sp.nF[f] + nR[f];
+    HIF_CUDA_TRY(cudaMemcpyAsync(off_d, rowOff.data(), sizeof(int64_t) * nf, cudaMemcpyHostToDevice, row_st_));
+    rowpos = static_cast<int32_t*>(row_alloc(sizeof(int32_t) * rowOff[nf] * ncp));
+    skel_rows(geo_, rf_d, nf, ncp, row_cells_, row_lists_, row_posb_, alive_d, mean, nullptr, off_d,
+              rowpos, row_st_);
+    HIF_CUDA_TRY(cudaEventRecord(row_ev_, row_st_));
+    HIF_CUDA_TRY(cudaStreamWaitEvent(st_, row_ev_, 0));
+  }
   std::vector<SkelDesc> sd(nf);
   int64_t goff = 0, poff = 0, toff = 0;
   for (int f = 0; f < nf; ++f) {
     SkelDesc& d = sd[f];
     std::memset(&d, 0, sizeof(d));
     d.nF = sp.nF[f];
-    d.nR = sp.nR[f];
+    d.nR = nR[f];
     d.G = goff;
-    d.idoff = goff + sp.nF[f];
-    d.idm = sp.nR[f];
-    d.idld = sp.nF[f] + sp.nR[f];
-    d.rows = sp.rowOff[f] * ncp;
+    d.idoff = goff + d.nF;
+    d.idm = d.nR;
+    d.idld = d.nF + d.nR;
+    d.rows = rowOff[f] * ncp;
     d.perm = poff;
     d.Tm = toff;
     for (int i = 0; i < ncp; ++i) d.cell[i] = sp.cells[(size_t)f * ncp + i];
@@ -905,14 +964,13 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
     toff += (int64_t)(d.nF / 2) * (d.nF - d.nF / 2);
     F_.stats.flops += 2.0 * d.nR * (double)d.nF * d.nF;
   }
-  DevBuf rowpos_d, sd_d, G, perm_d, steps, tm;
-  upload_async(rowpos_d, sp.rowPos, &F_.mem, st_);
+  DevBuf sd_d, G, perm_d, steps, tm;
   upload_async(sd_d, sd, &F_.mem, st_);
   G.alloc_async(sizeof(T) * std::max<int64_t>(1, goff), &F_.mem, st_);
   perm_d.alloc_async(sizeof(int32_t) * poff, &F_.mem, st_);
   steps.alloc_async(sizeof(int32_t) * poff, &F_.mem, st_);
   tm.alloc(sizeof(T) * std::max<int64_t>(1, toff), &F_.mem);
-  skel_gather<T>(sd_d.as<SkelDesc>(), sd.data(), nf, ncp, rowpos_d.as<int32_t>(),
+  skel_gather<T>(sd_d.as<SkelDesc>(), sd.data(), nf, ncp, rowpos,
                  cdesc_d.as<CellDesc>(), Kar.as<T>(), G.as<T>(), st_);
   // fronts with many more coupled rows than DOFs: reduce the rows by an
   // unpivoted QR first; their ID then runs on the square triangular factor
@@ -1050,7 +1108,7 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
   int64_t dropped = 0;
   for (int f : act) {
     const int32_t* pm = &perm[sd[f].perm];
-    for (int i = sd[f].k; i < sd[f].nF; ++i) alive[sp.rowDof[sp.rowOff[f] + pm[i]]] = 0;
+    for (int i = sd[f].k; i < sd[f].nF; ++i) alive[sp.mem[sp.memOff[f] + pm[i]]] = 0;
     dropped += sd[f].nF - sd[f].k;
   }
   if (act.empty()) return 0;
@@ -1113,7 +1171,7 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
   partial_cholesky<T>(fr_d.as<DFront>(), frs.data(), (int)frs.size(), Z.as<T>(), s.panels.as<T>(),
                       flags_.as<int>(), F_.opt.tensor_cores != 0, st_, &retry_);
   tr_.mark(level_, " Z products + Cholesky queued");
-  skel_writeback<T>(sda_d.as<SkelDesc>(), sda.data(), (int)sda.size(), ncp, rowpos_d.as<int32_t>(),
+  skel_writeback<T>(sda_d.as<SkelDesc>(), sda.data(), (int)sda.size(), ncp, rowpos,
                     perm_d.as<int32_t>(), cdesc_d.as<CellDesc>(), Z.as<T>(), Kar.as<T>(), st_);
   // apply stage: the lists are built on a worker thread
   int64_t totalF = 0;
@@ -1123,8 +1181,8 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
   const size_t si = F_.stages.size();
   F_.stages.push_back(std::move(s));
   auto job = [sda, perm = std::move(perm), act, plan, totalF]() {
-    const auto& rowDof = plan->rowDof;
-    const auto& rowOff = plan->rowOff;
+    const auto& mem = plan->mem;
+    const auto& memOff = plan->memOff;
     StageHost h;
     int64_t vo = 0;
     for (const SkelDesc& d : sda) {
@@ -1132,8 +1190,8 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
       const int32_t* pm = &perm[d.perm];
       const int src = act[&d - sda.data()];
       const int64_t base = (int64_t)h.idx.size();
-      for (int i = 0; i < p; ++i) h.idx.push_back(rowDof[rowOff[src] + pm[k + i]]);
-      for (int i = 0; i < k; ++i) h.idx.push_back(rowDof[rowOff[src] + pm[i]]);
+      for (int i = 0; i < p; ++i) h.idx.push_back(mem[memOff[src] + pm[k + i]]);
+      for (int i = 0; i < k; ++i) h.idx.push_back(mem[memOff[src] + pm[i]]);
       const int64_t to = totalF + vo;
       // forward: v_c -= T^T v_h ; t_c = Linv v_c ; v_h -= X^T t_c
       if (k) h.fwd[0].push_back(GemvOp{d.Tm, vo + p, vo, k, p, k, 0, -1.0f, 1});

@@ -354,6 +354,63 @@ void Symbolic::merge_maps(const CellPlan& child, const CellPlan& parent,
   });
 }
 
+void Symbolic::build_fronts(const CellPlan& cp, int kind, const std::vector<uint8_t>& alive,
+                            SkelPlan& sp) const {
+  const int C = cp.C;
+  sp.kind = kind;
+  sp.ncellPer = kind == 1 ? 2 : 4;
+  // a front is the DOFs of one separator mask whose low cell is the cell: each
+  // cell owns up to three, found in its boundary list (ascending global ids)
+  static constexpr int mask_of[3][3] = {{0, 0, 0}, {1, 2, 4}, {3, 5, 6}};
+  const int* mask = mask_of[kind];
+  auto low_cell = [&](int64_t pk) {
+    return (int)(pk & 0xffff) + C * ((int)((pk >> 16) & 0xffff) + C * (int)((pk >> 32) & 0xffff));
+  };
+  auto for_members = [&](int c, auto&& f) {
+    for (int64_t t = cp.off[c] + cp.p[c]; t < cp.off[c + 1]; ++t) {
+      const int64_t pk = cp.dofPk[t];
+      const int sp_mask = (int)(pk >> 48);
+      if (popc3(sp_mask) != kind || low_cell(pk) != c || !alive[cp.dofs[t]]) continue;
+      f(sp_mask == mask[0] ? 0 : sp_mask == mask[1] ? 1 : 2, cp.dofs[t]);
+    }
+  };
+  std::vector<int32_t> cnt((size_t)cp.ncell * 3, 0);
+  // cells that hold some 4096 DOFs together
+  const int64_t grain =
+      std::max<int64_t>(1, (int64_t)4096 * cp.ncell / std::max<int64_t>(1, cp.off[cp.ncell]));
+  parallel_for(workers_, cp.ncell, grain, [&](int64_t c) {
+    for_members((int)c, [&](int m, int32_t) { cnt[c * 3 + m]++; });
+  });
+  std::vector<int32_t> id((size_t)cp.ncell * 3, -1);
+  sp.nfront = 0;
+  sp.sep.clear();
+  sp.nF.clear();
+  sp.cells.clear();
+  sp.memOff.assign(1, 0);
+  for (int c = 0; c < cp.ncell; ++c)
+    for (int m = 0; m < 3; ++m) {
+      if (!cnt[(size_t)c * 3 + m]) continue;
+      id[(size_t)c * 3 + m] = sp.nfront++;
+      sp.sep.push_back(mask[m]);
+      sp.nF.push_back(cnt[(size_t)c * 3 + m]);
+      sp.memOff.push_back(sp.memOff.back() + cnt[(size_t)c * 3 + m]);
+      const int lc[3] = {c % C, (c / C) % C, c / (C * C)};
+      for (int q = 0; q < 8; ++q) {   // the cells over its separator dimensions
+        if (q & ~mask[m]) continue;
+        const int c0 = (lc[0] + (q & 1)) % C, c1 = (lc[1] + ((q >> 1) & 1)) % C,
+                  c2 = (lc[2] + ((q >> 2) & 1)) % C;
+        sp.cells.push_back(c0 + C * (c1 + C * c2));
+      }
+    }
+  sp.mem.resize(sp.memOff.back());
+  parallel_for(workers_, cp.ncell, grain, [&](int64_t c) {
+    int64_t cur[3] = {0, 0, 0};
+    for_members((int)c, [&](int m, int32_t g) {
+      sp.mem[sp.memOff[id[c * 3 + m]] + cur[m]++] = g;
+    });
+  });
+}
+
 void Symbolic::build_skel(const CellPlan& cp, int kind, const std::vector<uint8_t>& alive,
                           SkelPlan& sp) const {
   const int C = cp.C;

@@ -106,6 +106,11 @@ struct SkelPlan {
   std::vector<int64_t> rowOff;   // per front offset into rowDof (nfront + 1)
   PlanVec32 rowDof;              // global ids: the front's DOFs first, then R
   PlanVec32 rowPos;              // per row, ncellPer boundary positions (-1 = absent)
+  // build_fronts: the fronts' DOFs alone (ascending global ids), in memOff order,
+  // and their separator masks (low cell: the first of `cells`)
+  std::vector<int32_t> sep;
+  std::vector<int64_t> memOff;   // nfront + 1
+  PlanVec32 mem;
 };
 
 class Symbolic {
@@ -123,7 +128,12 @@ class Symbolic {
   // major) giving the child's boundary position of the parent's DOF, or -1.
   void merge_maps(const CellPlan& child, const CellPlan& parent,
                   std::vector<int64_t>& mapOff, PlanVec32& map) const;
-  // Faces (kind 1) or edges (kind 2) of the level with their coupled rows.
+  // Faces (kind 1) or edges (kind 2) of the level: cells, nF, sep, memOff and mem.
+  // Their rows are listed on the device (skel_rows).
+  void build_fronts(const CellPlan& cp, int kind, const std::vector<uint8_t>& alive,
+                    SkelPlan& sp) const;
+  // The same with the coupled rows, on the host: what skel_rows lists, front by
+  // front, for checks of the plan's consistency.
   // `alive` marks DOFs still active (redundant DOFs of faces are dropped
   // before the edges are planned).
   void build_skel(const CellPlan& cp, int kind, const std::vector<uint8_t>& alive,
