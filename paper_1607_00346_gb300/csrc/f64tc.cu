@@ -29,7 +29,9 @@
 // row, k_f64_slice writes the slices in the layout the tensor core reads (64 rows
 // x 16 k per block, all eight slices together: 16 KB), k_gemm_f64tc copies blocks
 // to shared memory with bulk copies and multiplies.  An operand used on both
-// sides (A A^T) is split once.
+// sides (A A^T) is split once; if all products of a batch are such and have at most
+// 64 k (the Cholesky updates), k_f64_slice_rows finds s and writes the slices with
+// one read.
 //
 // Measured (all launches, FMA form in brackets): one 64^3 product 40 (66) us, 512
 // of them 125 (270) us, one 256^3 55 (280) us, one 1024^3 0.11 (2.1) ms, one 2048^3
@@ -43,7 +45,14 @@
 // thread issues 12 instructions (M 128, N 64 to 256, K 16: a slice of A times
 // up to four neighbouring slices of B, whose products go to neighbouring
 // accumulators), and a warp copies the block three ahead; per 128 k the warps
-// read the accumulators back.
+// read the accumulators back.  A small tile is a chain of latencies (table,
+// exponents, copies, products, C): with the exponents read while tensor memory is
+// allocated, C copied to shared memory during the last read-back, and 512 threads
+// of 16 columns each for the rounding instead of 256 of 32, one 64^3 tile takes
+// 17.5 instead of 22.3 us and 1520 of them 166 us; 256^3 29 (34) us, 1024^3 81 (84),
+// 2048^3 570 (586), where the copies from L2 (6.4 TB/s) are the bound.  With the
+// one-pass slices a 64^3 FP64 factorization and solve went from 203 to 194 ms, a
+// 32^3 periodic one from 45.3 to 42.5 ms.
 #include <stdint.h>
 
 #include <algorithm>
@@ -66,7 +75,8 @@ constexpr int TM = 128, TN = 64;           // output tile
 constexpr int NST = 4;                     // shared-memory stages
 constexpr int STAGE = 3 * BLK;             // two blocks of A, one of B
 constexpr int GROUP = 8;                   // blocks (128 k) per exact accumulation
-constexpr int THREADS = 256;
+constexpr int THREADS = 512;
+constexpr int CW = TN * 128 / THREADS;     // columns of a thread: four warps share a row of lanes
 constexpr int NOT_FINITE = INT32_MAX;      // exponent of a row with inf or NaN
 constexpr long long WAIT_LIMIT = 20000000;  // mbarrier polls before giving up
 constexpr size_t WORK_LIMIT = (size_t)1 << 30;   // slices held at once, if several products
@@ -191,7 +201,36 @@ __device__ __forceinline__ int64_t fixed62(double x, int s) {
   return (int64_t)u < 0 ? -(int64_t)v : (int64_t)v;
 }
 
-// One thread: eight consecutive k of one row -> 16 bytes of each slice.
+// Eight consecutive k (group g) of row r -> 16 bytes of each slice of a block.
+__device__ __forceinline__ void write_slices(const double (&x)[8], int s, const int (&t)[8],
+                                             unsigned char* blk, int r, int g) {
+  // adding 128 to every digit but the first makes the bytes of the sum the
+  // digits + 128; a byte put into the low mantissa of 2^23 and taken back
+  // gives the digit as a float, whose upper half is its BF16
+  uint32_t lo[8], hi[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint64_t y = (uint64_t)(s == NOT_FINITE ? 0 : fixed62(x[j], s - t[j])) + 0x8080808080808080ull;
+    lo[j] = (uint32_t)y;
+    hi[j] = (uint32_t)(y >> 32);
+  }
+  unsigned char* out = blk + (r / 8) * 256 + (g % 2) * 128 + (r % 8) * 16;
+#pragma unroll
+  for (int i = 0; i < NSL; ++i) {
+    const uint32_t sel = 0x7440u | (uint32_t)((NSL - 1 - i) & 3);
+    uint32_t d[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const uint32_t w0 = i < 4 ? hi[2 * h] : lo[2 * h], w1 = i < 4 ? hi[2 * h + 1] : lo[2 * h + 1];
+      const float f0 = __uint_as_float(__byte_perm(w0, 0x4b000000u, sel)) - 8388736.0f;
+      const float f1 = __uint_as_float(__byte_perm(w1, 0x4b000000u, sel)) - 8388736.0f;
+      d[h] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+    }
+    *reinterpret_cast<uint4*>(out + i * SLICE) = make_uint4(d[0], d[1], d[2], d[3]);
+  }
+}
+
+// One thread: eight consecutive k of one row at a time.
 template <typename S>
 __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ blks,
                                                    const S* __restrict__ Ab,
@@ -216,30 +255,43 @@ __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ 
                  ? (double)X[b.kcont ? (int64_t)r * b.ld + k : r + (int64_t)k * b.ld]
                  : 0.0;
     }
-    // adding 128 to every digit but the first makes the bytes of the sum the
-    // digits + 128; a byte put into the low mantissa of 2^23 and taken back
-    // gives the digit as a float, whose upper half is its BF16
-    uint32_t lo[8], hi[8];
+    write_slices(x, s, t, W + (b.dst + g / 2) * BLK, r, g);
+  }
+}
+
+// Exponents and slices in one pass, for products A A^T of up to ROW_K k: a thread
+// keeps its row's entries (two groups of 8 k) in registers, the four threads of a
+// row agree on its largest exponent.
+constexpr int ROW_K = 64;
+template <typename S>
+__global__ void __launch_bounds__(256) k_f64_slice_rows(const SliceBlk* __restrict__ blks,
+                                                        const S* __restrict__ Ab, int* exps,
+                                                        unsigned char* W) {
+  const SliceBlk b = blks[blockIdx.x];
+  const S* X = Ab + b.src;
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int r = warp * 8 + lane % 8, kg = lane / 8;
+  double x[2][8];
+  int m = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const uint64_t y = (uint64_t)(s == NOT_FINITE ? 0 : fixed62(x[j], s - t[j])) + 0x8080808080808080ull;
-      lo[j] = (uint32_t)y;
-      hi[j] = (uint32_t)(y >> 32);
+      const int k = (4 * h + kg) * 8 + j;
+      x[h][j] = (r < b.rows && k < b.k)
+                    ? (double)X[b.kcont ? (int64_t)r * b.ld + k : r + (int64_t)k * b.ld]
+                    : 0.0;
+      m = max(m, entry_exp(x[h][j], 0));
     }
-    unsigned char* out = W + (b.dst + g / 2) * BLK + (r / 8) * 256 + (g % 2) * 128 + (r % 8) * 16;
+  m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
+  m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+  if (kg == 0) exps[(int64_t)blockIdx.x * BR + r] = m;
+  const int s = row_exp(m);
+  const int t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
-    for (int i = 0; i < NSL; ++i) {
-      const uint32_t sel = 0x7440u | (uint32_t)((NSL - 1 - i) & 3);
-      uint32_t d[4];
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const uint32_t w0 = i < 4 ? hi[2 * h] : lo[2 * h], w1 = i < 4 ? hi[2 * h + 1] : lo[2 * h + 1];
-        const float f0 = __uint_as_float(__byte_perm(w0, 0x4b000000u, sel)) - 8388736.0f;
-        const float f1 = __uint_as_float(__byte_perm(w1, 0x4b000000u, sel)) - 8388736.0f;
-        d[h] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-      }
-      *reinterpret_cast<uint4*>(out + i * SLICE) = make_uint4(d[0], d[1], d[2], d[3]);
-    }
+  for (int h = 0; h < 2; ++h) {
+    const int g = 4 * h + kg;
+    if (g < (b.k + KC - 1) / KC * 2) write_slices(x[h], s, t, W + (b.dst + g / 2) * BLK, r, g);
   }
 }
 
@@ -302,8 +354,15 @@ __global__ void __launch_bounds__(THREADS, 1)
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[NST], done[NST], accf;
   __shared__ uint32_t s_tmem;
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_ea[TM], s_eb[TN];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  if (tid < TM + TN) {   // the tile's row and column exponents
+    const bool a = tid < TM;
+    const int i = a ? tid : tid - TM;
+    const int64_t at = (int64_t)(a ? tl.ablk : tl.bblk) * BR + i;
+    const bool have = a ? tl.rb + i < o.m : tl.cb + i < o.n;
+    (a ? s_ea : s_eb)[i] = have ? row_exp(exps[at]) : 0;
+  }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(
         tc5::smem_u32(&s_tmem)));
@@ -360,9 +419,16 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 1)
     for (; loaded < min(NST - 1, nc); ++loaded) load(loaded);
 
-  int64_t hi[TN / 2], lo[TN / 2];   // this thread's row, half of the columns
+  // this thread's entries of the tile: one row, a quarter of the columns; their sums and
+  // C go through the stages' shared memory at the end
+  const int cr = tl.rb + (warp % 4) * 32 + lane, cc = tl.cb + (warp / 4) * CW;
+  int64_t* sum = reinterpret_cast<int64_t*>(smem) + tid;
+  double* cst = reinterpret_cast<double*>(smem + sizeof(int64_t) * 2 * CW * THREADS) + tid;
+  static_assert(sizeof(int64_t) * 2 * CW * THREADS + sizeof(double) * CW * THREADS <= NST * STAGE,
+                "sums and C fit the stages");
+  int64_t hi[CW], lo[CW];
 #pragma unroll
-  for (int j = 0; j < TN / 2; ++j) hi[j] = lo[j] = 0;
+  for (int j = 0; j < CW; ++j) hi[j] = lo[j] = 0;
   bool ok = true;
   const int ngroup = (nc + GROUP - 1) / GROUP;
   for (int g = 0; g < ngroup; ++g) {
@@ -419,9 +485,21 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (!ok) break;
     seen = issued;
     asm volatile("tcgen05.fence::after_thread_sync;\n");
-    const uint32_t base = tmem + ((uint32_t)((warp % 4) * 32) << 16) + (uint32_t)(warp / 4) * (TN / 2);
+    if (g == ngroup - 1 && o.beta != 0.f) {
+      // every copy and product is done: C arrives in the free stages while the
+      // last accumulators are read back
+#pragma unroll 4
+      for (int j = 0; j < CW; ++j) {
+        const bool in = cr < o.m && cc + j < o.n;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(
+                         tc5::smem_u32(cst + j * THREADS)),
+                     "l"(in ? Cb + o.C + cr + (int64_t)(cc + j) * o.ldc : Cb), "r"(in ? 8 : 0)
+                     : "memory");
+      }
+    }
+    const uint32_t base = tmem + ((uint32_t)((warp % 4) * 32) << 16) + (uint32_t)(warp / 4) * CW;
 #pragma unroll
-    for (int c0 = 0; c0 < TN / 2; c0 += 4) {
+    for (int c0 = 0; c0 < CW; c0 += 4) {
       uint32_t d[NSL][4];
 #pragma unroll
       for (int t = 0; t < NSL; ++t) tmem_ld4(base + t * TN + c0, d[t]);
@@ -447,32 +525,30 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   }
   if (ok) {
-    // the sums go through shared memory (every copy and product is done), so
-    // that one short loop rounds them: unrolled over the registers it was 32
+    // one short loop rounds the sums: unrolled over the registers it was 32
     // copies of the rounding, and fetching them took 30 us
-    int64_t* sum = reinterpret_cast<int64_t*>(smem) + tid;
 #pragma unroll
-    for (int j = 0; j < TN / 2; ++j) {
+    for (int j = 0; j < CW; ++j) {
       sum[(2 * j) * THREADS] = hi[j];
       sum[(2 * j + 1) * THREADS] = lo[j];
     }
-    const int r = tl.rb + (warp % 4) * 32 + lane, cb = tl.cb + (warp / 4) * (TN / 2);
-    if (r < o.m) {
-      const int ea = row_exp(exps[(int64_t)tl.ablk * BR + r - tl.rb]);
-      double* C = Cb + o.C + r + (int64_t)cb * o.ldc;
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if (cr < o.m) {
+      const int ea = s_ea[cr - tl.rb];
+      double* C = Cb + o.C + cr + (int64_t)cc * o.ldc;
       const double al = (double)o.alpha;
-      const int nj = min(TN / 2, o.n - cb);
-      const int* ebp = exps + (int64_t)tl.bblk * BR + (cb - tl.cb);
-#pragma unroll 2
+      const int nj = min(CW, o.n - cc);
+      const int* ebp = s_eb + (cc - tl.cb);
+#pragma unroll 4
       for (int j = 0; j < nj; ++j) {
-        const int eb = row_exp(ebp[j]);
+        const int eb = ebp[j];
         // 2^(sA - 62) 2^(sB - 62) 256^7, the biased exponents' offset 2 * 1023 taken out
         const double v = ea == NOT_FINITE || eb == NOT_FINITE
                              ? __longlong_as_double(0x7ff8000000000000ll)
                              : to_double(sum[(2 * j) * THREADS], sum[(2 * j + 1) * THREADS],
                                          ea + eb - 2 * 1023 - 124 + 56);
-        double* cp = C + (int64_t)j * o.ldc;
-        *cp = o.beta != 0.f ? fma(al, v, *cp) : al * v;
+        C[(int64_t)j * o.ldc] = o.beta != 0.f ? fma(al, v, ngroup ? cst[j * THREADS] : C[(int64_t)j * o.ldc])
+                                              : al * v;
       }
     }
   }
@@ -551,16 +627,23 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
     HIF_CUDA_TRY(cudaMemcpyAsync(d_tab, tab.data(), bb + tb, cudaMemcpyHostToDevice, st));
     const SliceBlk* d_blks = reinterpret_cast<const SliceBlk*>(d_tab);
     const Tile* d_tiles = reinterpret_cast<const Tile*>(d_tab + bb);
-    HIF_CUDA_TRY(cudaMemsetAsync(d_exps, 0, eb, st));
     const int gy = std::max(1, std::min({ceil_div(kmax, 64), 64, ceil_div(4096, (int64_t)blks.size())}));
-    if (nkx) {
-      k_f64_kmax<S><<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx);
+    const bool rows = nkx == 0 && kmax <= ROW_K;   // every product of the batch is A A^T
+    if (rows) {
+      k_f64_slice_rows<S><<<(unsigned)blks.size(), 256, 0, st>>>(d_blks, Abase, d_exps, W);
+      HIF_CHECK_LAUNCH();
+    } else {
+      const dim3 grid((unsigned)blks.size(), gy);
+      HIF_CUDA_TRY(cudaMemsetAsync(d_exps, 0, eb, st));
+      if (nkx) {
+        k_f64_kmax<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx);
+        HIF_CHECK_LAUNCH();
+      }
+      k_f64_exps<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps);
+      HIF_CHECK_LAUNCH();
+      k_f64_slice<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps, W);
       HIF_CHECK_LAUNCH();
     }
-    k_f64_exps<S><<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps);
-    HIF_CHECK_LAUNCH();
-    k_f64_slice<S><<<dim3((unsigned)blks.size(), gy), 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps, W);
-    HIF_CHECK_LAUNCH();
     k_gemm_f64tc<<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(d_tiles, d_ops, d_blks, d_exps,
                                                                        W, Cbase, d_flags);
     HIF_CHECK_LAUNCH();
