@@ -67,6 +67,13 @@ namespace hif {
 namespace {
 
 constexpr int NSL = 8;             // slices per operand, and accumulators
+// slices multiplied: all for FP64 operands.  FP32 operands (24 bits an entry) leave out
+// the last slice of each and the products with t = 7: their rows are then rounded 54
+// bits below the largest entry, which is as far as an FP64 FMA loop carries the sum.
+// (28 instead of 36 products; Gram matrices of a 128^3 FP32 factorization 60.8 -> 56.0
+// ms, of 96^3 13.4 -> 12.4 ms.)
+template <typename S>
+constexpr int slices_used() { return sizeof(S) == 4 ? NSL - 1 : NSL; }
 constexpr int BR = 64;             // rows of a block of slices
 constexpr int KC = 16;             // k of a block
 constexpr int SLICE = BR * KC * 2;         // bytes of one slice of a block (2 KB)
@@ -345,6 +352,8 @@ __device__ __forceinline__ double to_double(int64_t hi, int64_t lo, int ex) {
   return neg ? -v : v;
 }
 
+// NS: slices of each operand that are multiplied
+template <int NS>
 __global__ void __launch_bounds__(THREADS, 1)
     k_gemm_f64tc(const Tile* __restrict__ tiles, const GemmOp* __restrict__ ops,
                  const SliceBlk* __restrict__ blks, const int* __restrict__ exps,
@@ -403,15 +412,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (lane == 0)
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(
                        tc5::smem_u32(&full[s])),
-                   "r"((two ? 3 : 2) * BLK)
+                   "r"((two ? 3 : 2) * NS * SLICE)
                    : "memory");
     __syncwarp();
     const int64_t off = (int64_t)c * BLK;
-    if (lane < 2 * NSL) {
+    if (lane < 2 * NS) {
       if (two || lane % 2 == 0)
         bulk_copy(st + lane * SLICE, (lane % 2 ? A1 : A0) + off + (lane / 2) * SLICE, SLICE, &full[s]);
-    } else if (lane == 2 * NSL) {
-      bulk_copy(st + 2 * BLK, B0 + off, BLK, &full[s]);
+    } else if (lane == 2 * NS) {
+      bulk_copy(st + 2 * BLK, B0 + off, NS * SLICE, &full[s]);
     }
   };
   int loaded = 0;               // warp 1: blocks loaded
@@ -447,10 +456,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint64_t da = tc5::sdesc(a, 128, 256), db = tc5::sdesc(b, 128, 256);
         const uint32_t more = c > g * GROUP ? 1u : 0u;
 #pragma unroll
-        for (int i = 0; i < NSL; ++i)
+        for (int i = 0; i < NS; ++i)
 #pragma unroll
-          for (int j = 0; i + j < NSL; j += 4) {
-            const int w = NSL - i - j < 4 ? NSL - i - j : 4;
+          for (int j = 0; i + j < NS; j += 4) {
+            const int w = NS - i - j < 4 ? NS - i - j : 4;
             tc5::mma_bf16(tmem + (i + j) * TN, da + (2 * i * SLICE >> 4), db + (j * SLICE >> 4),
                           tc5::idesc_bf16(TM, w * TN), i > 0 ? 1u : more);
           }
@@ -502,13 +511,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int c0 = 0; c0 < CW; c0 += 4) {
       uint32_t d[NSL][4];
 #pragma unroll
-      for (int t = 0; t < NSL; ++t) tmem_ld4(base + t * TN + c0, d[t]);
+      for (int t = 0; t < NS; ++t) tmem_ld4(base + t * TN + c0, d[t]);
       asm volatile("tcgen05.wait::ld.sync.aligned;\n");
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         auto v = [&](int t) { return (int64_t)__float2int_rz(__uint_as_float(d[t][j])); };
         hi[c0 + j] += (v(0) << 24) + (v(1) << 16) + (v(2) << 8) + v(3);
-        lo[c0 + j] += (v(4) << 24) + (v(5) << 16) + (v(6) << 8) + v(7);
+        lo[c0 + j] += (v(4) << 24) + (v(5) << 16) + (v(6) << 8) + (NS == NSL ? v(NSL - 1) : 0);
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
@@ -571,7 +580,7 @@ template <typename S>
 void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Abase, const S* Bbase,
                 double* Cbase, int* d_flags, cudaStream_t st, const char* name) {
   static const bool attr = [] {   // initialised once, also under concurrent factorizations
-    HIF_CUDA_TRY(cudaFuncSetAttribute(k_gemm_f64tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_gemm_f64tc<slices_used<S>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       NST * STAGE));
     return true;
   }();
@@ -644,8 +653,8 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
       k_f64_slice<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps, W);
       HIF_CHECK_LAUNCH();
     }
-    k_gemm_f64tc<<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(d_tiles, d_ops, d_blks, d_exps,
-                                                                       W, Cbase, d_flags);
+    k_gemm_f64tc<slices_used<S>()><<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(
+        d_tiles, d_ops, d_blks, d_exps, W, Cbase, d_flags);
     HIF_CHECK_LAUNCH();
     HIF_CUDA_TRY(cudaFreeAsync(d_exps, st));
     HIF_CUDA_TRY(cudaFreeAsync(W, st));
