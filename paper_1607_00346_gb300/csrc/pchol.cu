@@ -17,9 +17,11 @@
 // read once, by tensor-core products, and a pivot step reads one column of G: 64
 // steps per launch in k_pchol (a cluster per front, one column per thread), then
 // one product per front updates G.  128^3, FP32, eps 1e-6: row reduction and ID of
-// the three upper levels' faces 300 ms, here 115 ms (61 + 28 the products, 26 the
-// steps; 32 steps per launch: 61 + 53 + 18).
+// the three upper levels' faces 300 ms, here 89 ms (56 + 15 the products, 18 the
+// steps; 48 steps per launch: 19.5 + 21 instead of 15 + 26 before the comparisons
+// and reciprocal roots left the FP64 unit, 32 steps: 27.5 + 18).
 #include <algorithm>
+#include <climits>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -35,11 +37,14 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int PC_THREADS = 256;    // columns per CTA
-constexpr int PC_WARPS = PC_THREADS / 32;
 constexpr int PC_STEPS = 64;       // pivots per launch
-constexpr int PC_MAX_CS = 16;
-constexpr size_t PC_SMEM = sizeof(double) * PC_STEPS * PC_THREADS;
+// A CTA of 128 columns keeps 64 KB of the block's rows, so that three share an SM and
+// one's barriers overlap the others' sums; 256 columns (one per SM, 128 KB) for fronts
+// of more than 1024 columns, which 8 CTAs of 128 do not hold.  128^3, eps 1e-6: 18.4
+// against 19.7 ms with 256 throughout; eps 1e-3: 7.2 against 8.9; 96^3: 7.4 and 7.3.
+constexpr int PC_NARROW = 128, PC_NARROW_CS = 8;
+constexpr int PC_WIDE = 256, PC_WIDE_CS = 16;
+constexpr size_t pc_smem(int threads) { return sizeof(double) * PC_STEPS * threads; }
 
 struct PcDesc {
   int64_t G;       // n x n (lower triangle), in the Gram arena
@@ -65,18 +70,34 @@ __global__ void k_pchol_init(const PcDesc* __restrict__ ds, const double* __rest
   if (threadIdx.x == 0) stt[blockIdx.x] = PcState{0.0, 0, 0};
 }
 
-// PC_STEPS pivots of each listed front: column c belongs to thread c % 256 of CTA
-// c / 256 of its cluster, which keeps its remaining diagonal in a register and its
+// The larger of two diagonals, the lower column on ties.  Diagonals are compared as
+// integers: positive doubles are ordered like their bits and above all negative ones,
+// and a comparison on the FP64 unit (16 clocks a warp) costs as much as an FMA.
+__device__ __forceinline__ bool larger(long long& bd, int& bc, long long od, int oc) {
+  const bool take = od > bd || (od == bd && oc < bc);
+  if (take) {
+    bd = od;
+    bc = oc;
+  }
+  return take;
+}
+
+// PC_STEPS pivots of each listed front: column c belongs to thread c % PC_THREADS of
+// CTA c / PC_THREADS of its cluster, which keeps its remaining diagonal in a register and its
 // entries of the block's rows of R in shared memory.  Per step every CTA proposes
 // its largest diagonal, with that column's entries of the block so far, to all
 // CTAs of the cluster; after one cluster barrier all pick the same winner
 // (largest, lowest column on ties) and each thread forms its entry of the new row,
-// (G_cp - sum of the block's products) / R_pp.
+// (G_cp - sum of the block's products) / R_pp.  What bounds it is the FP64 unit (2 per
+// clock and SM): comparisons are on integers, and 1 / R_pp comes with the proposal
+// (128^3: 26.0 -> 18.4 ms, 96^3: 9.6 -> 7.4 ms, against both in every thread).
+template <int PC_THREADS, int PC_MAX_CS>
 __global__ void __launch_bounds__(PC_THREADS) k_pchol(const PcDesc* __restrict__ ds,
                                                      const int* __restrict__ list,
                                                      const double* __restrict__ Gar, double* Lar,
                                                      float* Rar, double* diag, int* step,
                                                      PcState* stt, double eps2) {
+  constexpr int PC_WARPS = PC_THREADS / 32;
   cg::cluster_group cl = cg::this_cluster();
   const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int f = list[blockIdx.x / CS];
@@ -86,31 +107,26 @@ __global__ void __launch_bounds__(PC_THREADS) k_pchol(const PcDesc* __restrict__
   const bool in = c < n;
   extern __shared__ __align__(16) unsigned char psm[];
   double(*Lb)[PC_THREADS] = reinterpret_cast<double(*)[PC_THREADS]>(psm);
-  __shared__ double s_bd[2][PC_MAX_CS], s_row[2][PC_MAX_CS][PC_STEPS];
+  __shared__ double s_binv[2][PC_MAX_CS], s_row[2][PC_MAX_CS][PC_STEPS];
+  __shared__ long long s_bd[2][PC_MAX_CS];
   __shared__ int s_bc[2][PC_MAX_CS];
-  __shared__ double w_d[PC_WARPS];
+  __shared__ long long w_d[PC_WARPS];
   __shared__ int w_c[PC_WARPS];
   const double* G = Gar + d.G;
   double dc = in ? diag[d.col + c] : 0.0;
   int tk = in ? step[d.col + c] : 0;
   const PcState s0 = stt[f];
-  double d1 = s0.d1;
+  double d1 = s0.d1, least = eps2 * d1;
   bool done = false;
   int j = 0;
   cl.sync();   // every CTA of the cluster runs before the first push
   for (; j < PC_STEPS; ++j) {
     const int par = j & 1;
-    double bd = tk < 0 ? dc : -1.0;
+    long long bd = tk < 0 ? __double_as_longlong(dc) : LLONG_MIN;
     int bc = c;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double od = __shfl_xor_sync(0xffffffffu, bd, o);
-      const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
-      if (od > bd || (od == bd && oc < bc)) {
-        bd = od;
-        bc = oc;
-      }
-    }
+    for (int o = 16; o > 0; o >>= 1) larger(bd, bc, __shfl_xor_sync(0xffffffffu, bd, o),
+                                            __shfl_xor_sync(0xffffffffu, bc, o));
     if (lane == 0) {
       w_d[warp] = bd;
       w_c[warp] = bc;
@@ -120,40 +136,36 @@ __global__ void __launch_bounds__(PC_THREADS) k_pchol(const PcDesc* __restrict__
       bd = w_d[lane % PC_WARPS];
       bc = w_c[lane % PC_WARPS];
 #pragma unroll
-      for (int o = PC_WARPS / 2; o > 0; o >>= 1) {
-        const double od = __shfl_xor_sync(0xffffffffu, bd, o);
-        const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
-        if (od > bd || (od == bd && oc < bc)) {
-          bd = od;
-          bc = oc;
-        }
-      }
+      for (int o = PC_WARPS / 2; o > 0; o >>= 1) larger(bd, bc, __shfl_xor_sync(0xffffffffu, bd, o),
+                                                        __shfl_xor_sync(0xffffffffu, bc, o));
+      const double binv = rsqrt(__longlong_as_double(bd));
       for (int q = 0; q < CS; ++q) {
         for (int t = lane; t < j; t += 32)
           *cl.map_shared_rank(&s_row[par][rank][t], q) = Lb[t][bc - rank * PC_THREADS];
         if (lane == 0) {
           *cl.map_shared_rank(&s_bd[par][rank], q) = bd;
+          *cl.map_shared_rank(&s_binv[par][rank], q) = binv;
           *cl.map_shared_rank(&s_bc[par][rank], q) = bc;
         }
       }
     }
     cl.sync();
-    double md = -1.0;
-    int mc = 0, mr = 0;
-    for (int q = 0; q < CS; ++q)
-      if (s_bd[par][q] > md || (s_bd[par][q] == md && s_bc[par][q] < mc)) {
-        md = s_bd[par][q];
-        mc = s_bc[par][q];
-        mr = q;
-      }
-    if (s0.k + j == 0) d1 = md;
-    if (!(md > 0.0) || !(md > eps2 * d1) || !isfinite(md)) {
+    long long mk = s_bd[par][0];
+    int mc = s_bc[par][0], mr = 0;
+    for (int q = 1; q < CS; ++q)
+      if (larger(mk, mc, s_bd[par][q], s_bc[par][q])) mr = q;
+    const double md = __longlong_as_double(mk);
+    if (s0.k + j == 0) {
+      d1 = md;
+      least = eps2 * d1;
+    }
+    if (mk <= 0 || mk <= __double_as_longlong(least) || mk >= 0x7ff0000000000000ll) {
       done = true;
       break;
     }
     double l = 0.0;
     if (tk < 0) {
-      const double inv = rsqrt(md);
+      const double inv = s_binv[par][mr];
       const double g = c >= mc ? G[c + (int64_t)mc * n] : G[mc + (int64_t)c * n];
       const double* row = s_row[par][mr];
       double t0 = g, t1 = 0.0, t2 = 0.0, t3 = 0.0;
@@ -187,17 +199,18 @@ __global__ void __launch_bounds__(PC_THREADS) k_pchol(const PcDesc* __restrict__
 }
 
 // the pivots in order, then the other columns in increasing order
-__global__ void __launch_bounds__(PC_THREADS) k_pchol_perm(const PcDesc* __restrict__ ds,
+constexpr int PERM_THREADS = 256;
+__global__ void __launch_bounds__(PERM_THREADS) k_pchol_perm(const PcDesc* __restrict__ ds,
                                                           const int* __restrict__ step,
                                                           const PcState* __restrict__ stt,
                                                           int32_t* perm, SkelDesc* fr) {
   const PcDesc d = ds[blockIdx.x];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   int32_t* pv = perm + d.perm;
-  __shared__ int s_cnt[PC_WARPS];
+  __shared__ int s_cnt[PERM_THREADS / 32];
   int base = stt[blockIdx.x].k;
   if (tid == 0) fr[d.front].k = base;
-  for (int c0 = 0; c0 < d.n; c0 += PC_THREADS) {
+  for (int c0 = 0; c0 < d.n; c0 += PERM_THREADS) {
     const int c = c0 + tid;
     const int t = c < d.n ? step[d.col + c] : 0;
     const bool left = c < d.n && t < 0;
@@ -205,7 +218,7 @@ __global__ void __launch_bounds__(PC_THREADS) k_pchol_perm(const PcDesc* __restr
     if (lane == 0) s_cnt[warp] = __popc(m);
     __syncthreads();
     int before = base, all = 0;
-    for (int w = 0; w < PC_WARPS; ++w) {
+    for (int w = 0; w < PERM_THREADS / 32; ++w) {
       before += w < warp ? s_cnt[w] : 0;
       all += s_cnt[w];
     }
@@ -231,19 +244,22 @@ struct Pooled {   // stream-ordered scratch
 
 }  // namespace
 
-bool gram_id_fits(int nFmax) {
-  const int cs = ceil_div(nFmax, PC_THREADS);
-  if (cs > PC_MAX_CS) return false;
+namespace {
+
+// Cluster sizes of k_pchol<THREADS, MAX_CS> that can be resident (index: size)
+template <int THREADS, int MAX_CS>
+const std::vector<int>& pchol_placeable() {
   static const std::vector<int> placeable = [] {
-    HIF_CUDA_TRY(cudaFuncSetAttribute(k_pchol, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    HIF_CUDA_TRY(cudaFuncSetAttribute(k_pchol, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)PC_SMEM));
-    std::vector<int> ok(PC_MAX_CS + 1, 0);
-    for (int s = 1; s <= PC_MAX_CS; ++s) {
+    auto* k = k_pchol<THREADS, MAX_CS>;
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)pc_smem(THREADS)));
+    std::vector<int> ok(MAX_CS + 1, 0);
+    for (int s = 1; s <= MAX_CS; ++s) {
       cudaLaunchConfig_t q = {};
       q.gridDim = dim3((unsigned)s);
-      q.blockDim = dim3(PC_THREADS);
-      q.dynamicSmemBytes = PC_SMEM;
+      q.blockDim = dim3(THREADS);
+      q.dynamicSmemBytes = pc_smem(THREADS);
       cudaLaunchAttribute qa[1];
       qa[0].id = cudaLaunchAttributeClusterDimension;
       qa[0].val.clusterDim.x = s;
@@ -252,12 +268,26 @@ bool gram_id_fits(int nFmax) {
       q.attrs = qa;
       q.numAttrs = 1;
       int ncl = 0;
-      ok[s] = cudaOccupancyMaxActiveClusters(&ncl, k_pchol, &q) == cudaSuccess && ncl > 0;
+      ok[s] = cudaOccupancyMaxActiveClusters(&ncl, k, &q) == cudaSuccess && ncl > 0;
       cudaGetLastError();
     }
     return ok;
   }();
-  return placeable[cs] != 0;
+  return placeable;
+}
+
+// CTAs of 128 columns for a batch whose largest front has n columns
+bool pchol_narrow(int n) {
+  const int cs = ceil_div(n, PC_NARROW);
+  return cs <= PC_NARROW_CS && pchol_placeable<PC_NARROW, PC_NARROW_CS>()[cs] != 0;
+}
+
+}  // namespace
+
+bool gram_id_fits(int nFmax) {
+  if (pchol_narrow(nFmax)) return true;
+  const int cs = ceil_div(nFmax, PC_WIDE);
+  return cs <= PC_WIDE_CS && pchol_placeable<PC_WIDE, PC_WIDE_CS>()[cs] != 0;
 }
 
 void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, float* Rout,
@@ -277,7 +307,8 @@ void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, fl
     ct += s.nF;
     nmax = std::max(nmax, s.nF);
   }
-  const int CS = ceil_div(nmax, PC_THREADS);
+  const bool narrow = pchol_narrow(nmax);
+  const int threads = narrow ? PC_NARROW : PC_WIDE, CS = ceil_div(nmax, threads);
   Pooled G(sizeof(double) * gt, st), L(sizeof(double) * lt, st), diag(sizeof(double) * ct, st),
       step(sizeof(int) * ct, st), stt(sizeof(PcState) * nf, st), dds(sizeof(PcDesc) * nf, st),
       dop(sizeof(GemmOp) * nf, st), lst(sizeof(int) * nf, st);
@@ -298,8 +329,8 @@ void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, fl
     HIF_CUDA_TRY(cudaMemcpyAsync(lst.p, act.data(), sizeof(int) * act.size(), cudaMemcpyHostToDevice, st));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(act.size() * CS));
-    cfg.blockDim = dim3(PC_THREADS);
-    cfg.dynamicSmemBytes = PC_SMEM;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = pc_smem(threads);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -310,7 +341,8 @@ void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, fl
     cfg.numAttrs = 1;
     {
       ProfScope ps("id_pchol", st);
-      HIF_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_pchol, (const PcDesc*)dds.as<PcDesc>(),
+      HIF_CUDA_TRY(cudaLaunchKernelEx(&cfg, narrow ? k_pchol<PC_NARROW, PC_NARROW_CS> : k_pchol<PC_WIDE, PC_WIDE_CS>,
+                                      (const PcDesc*)dds.as<PcDesc>(),
                                       (const int*)lst.as<int>(), (const double*)G.as<double>(),
                                       L.as<double>(), Rout, diag.as<double>(), step.as<int>(),
                                       stt.as<PcState>(), eps * eps));
@@ -333,7 +365,7 @@ void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, fl
     gemm_f64tc<double>(dop.as<GemmOp>(), up.data(), (int)up.size(), L.as<double>(), L.as<double>(),
                        G.as<double>(), d_flags, st, "id_pchol_update_f64tc");
   }
-  k_pchol_perm<<<nf, PC_THREADS, 0, st>>>(dds.as<PcDesc>(), step.as<int>(), stt.as<PcState>(), perm, d_f);
+  k_pchol_perm<<<nf, PERM_THREADS, 0, st>>>(dds.as<PcDesc>(), step.as<int>(), stt.as<PcState>(), perm, d_f);
   HIF_CHECK_LAUNCH();
 }
 

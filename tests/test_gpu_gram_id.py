@@ -45,3 +45,27 @@ def test_gram_and_qr_skeletons(n, m, eps):
     if eps >= 1e-6:   # at 1e-9 FP32 noise decides what is kept
         for l, k in enumerate(kept[0, True]):
             assert abs(kept[1, True][l] - k) <= 0.01 * k, kept
+
+
+def test_fronts_wider_than_1024_columns():
+    # 96^3: the faces of the last level have up to 1141 DOFs, clusters of 256-column
+    # CTAs (the levels below: 128-column CTAs); the bounds are those above
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_1607_00346_gb300 import hif
+    n = 96
+    a = inputs.coeff_log_uniform(n, -2.0, 2.0, 8300)
+    A = stencil.assemble(a, 0.1, n)
+    x = inputs.normal_rhs(n, 1, 8301)[0]
+    ax = torch.from_numpy(A @ x).cuda()
+    err, kept = {}, {}
+    for tc in (True, False):
+        u = torch.zeros_like(ax)
+        with hif.factor(n, 3, torch.from_numpy(a).cuda(), b_const=0.1, eps=1e-6, precision=1,
+                        tensor_cores=tc) as h:
+            h.apply(ax, u)
+            kept[tc] = h.stats()["active_after"]
+        err[tc] = np.linalg.norm(u.cpu().numpy() - x) / np.linalg.norm(x)
+    assert err[True] <= 16.0 * err[False], (err, kept)
+    for k, q in zip(kept[True], kept[False]):
+        assert abs(k - q) <= 0.01 * q, kept
