@@ -38,6 +38,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <climits>
 #include <map>
 #include <mutex>
 #include <vector>
@@ -58,6 +59,26 @@ constexpr int ID_WARPS = ID_THREADS / 32;
 constexpr int NBK = 16;   // steps per block of deferred updates
 constexpr int RC = 128;   // rows of V staged in shared memory by the block update
 constexpr int CPQR_SMEM_MAX = 200 * 1024;   // dynamic shared memory of k_cpqr, bytes
+// What bounds the ID kernels in FP64 is the FP64 unit (2 multiply-adds per clock and
+// SM: a warp instruction takes 16 clocks, a root or a quotient ten of them), so a
+// step's scalars are formed by one warp, comparisons are on integers, and the small
+// sums of a column share one reduction.  64^3, FP64, eps 1e-4, against roots, quotients
+// and comparisons in every thread: k_cpqr 28.6 -> 20.2 ms, k_cpqr_dsm 16.0 -> 13.8,
+// k_cpqr_smem 6.2 -> 2.9; 128^3, FP32: 8.6 -> 8.1, 13.1 -> 12.3, 3.1 -> 2.9.
+//
+// Squared norms compared without the FP64 unit: doubles by their bits, which order
+// as they do from 0 up (NaN below all, as it loses every comparison).
+__device__ __forceinline__ float norm_key(float x) { return x; }
+__device__ __forceinline__ long long norm_key(double x) {
+  const long long k = __double_as_longlong(x);
+  return (k & LLONG_MAX) > 0x7ff0000000000000ll ? LLONG_MIN : k;
+}
+// eps |R_11|, rounded down to T: for a value of T above it is above the product
+__device__ __forceinline__ float id_threshold(double eps, float r11) {
+  return __double2float_rd(eps * (double)r11);
+}
+__device__ __forceinline__ double id_threshold(double eps, double r11) { return eps * r11; }
+
 // Per-CTA state of its own columns, in dynamic shared memory (local index q
 // of column c = rank + CS q): the downdated squared norm and its reference
 // (double), the F row of the current block, and the step at which the column
@@ -127,7 +148,8 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
         const int q = (c - rank) / CS;
         if (stepq[q] >= 0) continue;
         const double v = nrm[q];
-        if (v > bv || (v == bv && c < bi)) {
+        const auto kv = norm_key(v), kb = norm_key(bv);
+        if (kv > kb || (kv == kb && c < bi)) {
           bv = v;
           bi = c;
         }
@@ -135,7 +157,8 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
       for (int o = 16; o > 0; o >>= 1) {
         const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > bv || (ov == bv && oi < bi)) {
+        const auto kb = norm_key(bv), ko = norm_key(ov);
+        if (ko > kb || (ko == kb && oi < bi)) {
           bv = ov;
           bi = oi;
         }
@@ -145,16 +168,22 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
         s_idx[warp] = bi;
       }
       __syncthreads();
-      if (tid == 0) {
-        double v = s_val[0];
-        int ix = s_idx[0];
-        for (int w = 1; w < ID_WARPS; ++w)
-          if (s_val[w] > v || (s_val[w] == v && s_idx[w] < ix)) {
-            v = s_val[w];
-            ix = s_idx[w];
+      if (warp == 0) {
+        double v = lane < ID_WARPS ? s_val[lane] : -1.0;
+        int ix = lane < ID_WARPS ? s_idx[lane] : nF;
+        for (int o = 16; o > 0; o >>= 1) {
+          const double ov = __shfl_xor_sync(0xffffffffu, v, o);
+          const int oi = __shfl_xor_sync(0xffffffffu, ix, o);
+          const auto kv = norm_key(v), ko = norm_key(ov);
+          if (ko > kv || (ko == kv && oi < ix)) {
+            v = ov;
+            ix = oi;
           }
-        s_cand_val = v;
-        s_cand_idx = ix;
+        }
+        if (lane == 0) {
+          s_cand_val = v;
+          s_cand_idx = ix;
+        }
       }
       cl.sync();
       if (warp == 0) {
@@ -168,7 +197,8 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
         for (int o = 16; o > 0; o >>= 1) {
           const double ov = __shfl_xor_sync(0xffffffffu, v, o);
           const int oi = __shfl_xor_sync(0xffffffffu, ix, o);
-          if (ov > v || (ov == v && oi < ix)) {
+          const auto kv = norm_key(v), ko = norm_key(ov);
+          if (ko > kv || (ko == kv && oi < ix)) {
             v = ov;
             ix = oi;
           }
@@ -214,19 +244,22 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) s_val[warp] = s;
         __syncthreads();
-        if (tid == 0) {
-          double tail = 0.0;
-          for (int w = 0; w < ID_WARPS; ++w) tail += s_val[w];
+        if (warp == 0) {
+          double tail = lane < ID_WARPS ? s_val[lane] : 0.0;
+          for (int o = 16; o > 0; o >>= 1) tail += __shfl_xor_sync(0xffffffffu, tail, o);
           const double x0 = (double)cp[i];
           const double nx = sqrt(x0 * x0 + tail);
           const double alpha = x0 >= 0.0 ? -nx : nx;
           const double v0 = x0 - alpha;
           const double vtv = v0 * v0 + tail;
-          s_tau_own = vtv > 0.0 ? 2.0 / vtv : 0.0;
-          s_v0_own = v0;
-          cp[i] = (T)alpha;    // R_ii; v0 lives in shared memory
-          pv[i] = piv;
-          stepq[qp] = i;
+          __syncwarp();
+          if (lane == 0) {
+            s_tau_own = vtv > 0.0 ? 2.0 / vtv : 0.0;
+            s_v0_own = v0;
+            cp[i] = (T)alpha;    // R_ii; v0 lives in shared memory
+            pv[i] = piv;
+            stepq[qp] = i;
+          }
         }
         __syncthreads();
         // g_l = v_l^T v_j over rows i..m-1 (v_l is nonzero there, v_j starts at row i)
@@ -242,7 +275,7 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
       // 3. every CTA: the step's reflector scalars, then its own columns
       if (tid == 0) {
         s_pl[j] = piv;
-        s_v0[j] = (T)*cl.map_shared_rank(&s_v0_own, owner);
+        s_v0[j] = s_vrow[j] = (T)*cl.map_shared_rank(&s_v0_own, owner);
         s_tau[j] = (T)*cl.map_shared_rank(&s_tau_own, owner);
       }
       if (tid < j) {
@@ -250,29 +283,29 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
         s_vrow[tid] = M[i + (int64_t)s_pl[tid] * ld];
       }
       __syncthreads();
-      if (tid == 0) s_vrow[j] = s_v0[j];
-      __syncthreads();
       const T v0 = s_v0[j], tau = s_tau[j];
       for (int c = rank + CS * warp; c < nF; c += CS * ID_WARPS) {
         const int q = (c - rank) / CS;
         if (stepq[q] >= 0) continue;
         T* cc = M + (int64_t)c * ld;
         T* Fc = Fm + (int64_t)q * NBK;
-        T fl[NBK];
-#pragma unroll
-        for (int l = 0; l < NBK; ++l) fl[l] = l < j ? Fc[l] : T(0);
+        // F(c, j) = tau (v^T a_c - sum_l g_l F(c, l)) and R_ic = a_ic - sum_l V(i, l)
+        // F(c, l): lane l forms its terms of both sums, and one reduction sums the
+        // first in the lower and the second in the upper half of the warp
         const T aci = cc[i];
-        T dot = warp_dot(cp, cc, i + 1, m, lane);
-        dot = fma(v0, aci, dot);
-        T corr = T(0), rv = aci;
-#pragma unroll
-        for (int l = 0; l < NBK; ++l) {
-          if (l < j) {
-            corr = fma(s_g[l], fl[l], corr);
-            rv = fma(-s_vrow[l], fl[l], rv);
-          }
+        T dot = lane_dot(cp, cc, i + 1, m, lane), dr = T(0);
+        if (lane < j) {
+          const T fl = Fc[lane];
+          dot = fma(-s_g[lane], fl, dot);
+          dr = s_vrow[lane] * fl;
         }
-        const T fcj = tau * (dot - corr);
+        const bool up = lane >= 16;
+        T both = (up ? dr : dot) + __shfl_xor_sync(0xffffffffu, up ? dot : dr, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) both += __shfl_xor_sync(0xffffffffu, both, o);
+        dot = fma(v0, aci, __shfl_sync(0xffffffffu, both, 0));
+        const T fcj = tau * dot;
+        T rv = aci - __shfl_sync(0xffffffffu, both, 16);
         rv = fma(-s_vrow[j], fcj, rv);
         __syncwarp();
         if (lane == 0) {
@@ -285,7 +318,7 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
           double s = 0.0;
           for (int r = i + 1 + lane; r < m; r += 32) {
             T a = cc[r];
-            for (int l = 0; l < j; ++l) a = fma(-M[r + (int64_t)s_pl[l] * ld], fl[l], a);
+            for (int l = 0; l < j; ++l) a = fma(-M[r + (int64_t)s_pl[l] * ld], Fc[l], a);
             a = fma(-cp[r], fcj, a);
             s += (double)a * (double)a;
           }
@@ -347,8 +380,8 @@ __global__ void __launch_bounds__(ID_THREADS, 2) k_cpqr(SkelDesc* fr, const int*
 // kernel).  The pass that applies step i's reflector to a column also
 // recomputes, from the updated entries, the column's norm below row i + 1
 // and its row i + 1 entry, and every warp keeps the best candidate among its
-// columns; so each step needs a single barrier, and the norms involve no
-// downdating (no cancellation), which lets them run in the factor precision
+// columns; so each step needs two barriers (around the one warp that picks the pivot
+// and forms its reflector's scalars), and the norms involve no downdating (no cancellation), which lets them run in the factor precision
 // (FP64 arithmetic is a small fraction of the FP32 rate on this part).
 constexpr int SMEM_ID_MAX = 220 * 1024;   // dynamic shared memory per CTA, bytes
 
@@ -373,10 +406,10 @@ __global__ void __launch_bounds__(1024) k_cpqr_smem(SkelDesc* fr, const int* __r
   T* rdiag = tail + nF;                        // R_ii
   int* done = reinterpret_cast<int*>(rdiag + nF);
   T* A = reinterpret_cast<T*>(sm + ((size_t)nF * (2 * sizeof(T) + 4) + 15) / 16 * 16);
-  // per-warp candidates for the next pivot, |a_c[i:]|^2 and the column;
-  // double-buffered by step parity so that one barrier per step suffices
-  __shared__ T s_cv[2][32];
-  __shared__ int s_ci[2][32];
+  // per-warp candidates for the next pivot, |a_c[i:]|^2 and the column; the pivot and
+  // its reflector's scalars
+  __shared__ T s_cv[32], s_v0, s_tau;
+  __shared__ int s_ci[32], s_piv;
   const int tid = threadIdx.x, nt = blockDim.x, warp = tid / 32, lane = tid % 32, nw = nt / 32;
 
   // copy, and the norms for step 0
@@ -400,51 +433,62 @@ __global__ void __launch_bounds__(1024) k_cpqr_smem(SkelDesc* fr, const int* __r
         tail[c] = s;
         done[c] = 0;
       }
-      if (full > bv) {
+      if (norm_key(full) > norm_key(bv)) {
         bv = full;
         bc = c;
       }
     }
     if (lane == 0) {
-      s_cv[0][warp] = bv;
-      s_ci[0][warp] = bc;
+      s_cv[warp] = bv;
+      s_ci[warp] = bc;
     }
   }
   __syncthreads();
   const int kmax = min(m, nF);
   int k = kmax;
-  T r11 = T(0);
+  T least = T(0);
   for (int i = 0; i < kmax; ++i) {
-    // pivot: the best of the warps' candidates (largest norm, lowest column)
-    const int cur = i & 1;
-    T bv = s_cv[cur][0];
-    int p = s_ci[cur][0];
-    for (int w = 1; w < nw; ++w) {
-      const T v = s_cv[cur][w];
-      const int c = s_ci[cur][w];
-      if (v > bv || (v == bv && c < p)) {
-        bv = v;
-        p = c;
+    // pivot: the best of the warps' candidates (largest norm, lowest column), and
+    // its reflector over rows i..m-1, v = (x0 - alpha, a_p[i+1:]): by one warp, as
+    // roots and quotients of all of them are FP64 work like the columns' own
+    if (warp == 0) {
+      T bv = lane < nw ? s_cv[lane] : T(-1);
+      int bc = lane < nw ? s_ci[lane] : nF;
+      for (int o = 16; o > 0; o >>= 1) {
+        const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
+        const auto kb = norm_key(bv), ko = norm_key(ov);
+        if (ko > kb || (ko == kb && oc < bc)) {
+          bv = ov;
+          bc = oc;
+        }
       }
+      // |a_p[i:]|^2 was formed from this head and tail
+      const T nv = sqrt(fmax(bv, T(0)));
+      if (i == 0) least = id_threshold(eps, nv);
+      const bool stop = bc >= nF || (i == 0 ? nv == T(0) : !(nv > least));
+      if (!stop) {
+        const T x0 = A[(size_t)bc * m + i], tl = tail[bc];
+        const T alpha = x0 >= T(0) ? -nv : nv;
+        const T v0 = x0 - alpha;
+        const T vtv = fma(v0, v0, tl);
+        if (lane == 0) {
+          s_v0 = v0;
+          s_tau = vtv > T(0) ? T(2) / vtv : T(0);
+          rdiag[i] = alpha;
+          pv[i] = bc;
+        }
+      }
+      if (lane == 0) s_piv = stop ? -1 : bc;
     }
-    const T nv = sqrt(fmax(bv, T(0)));
-    if (i == 0) r11 = nv;
-    if (p >= nF || (i == 0 ? nv == T(0) : !((double)nv > eps * (double)r11))) {
+    __syncthreads();
+    const int p = s_piv;
+    if (p < 0) {
       k = i;
       break;
     }
-    // reflector of column p over rows i..m-1: v = (x0 - alpha, a_p[i+1:])
     const T* ap = A + (int64_t)p * m;
-    const T x0 = ap[i], tl = tail[p];
-    const T nx = sqrt(fma(x0, x0, tl));
-    const T alpha = x0 >= T(0) ? -nx : nx;
-    const T v0 = x0 - alpha;
-    const T vtv = fma(v0, v0, tl);
-    const T tau = vtv > T(0) ? T(2) / vtv : T(0);
-    if (tid == 0) {
-      rdiag[i] = alpha;
-      pv[i] = p;
-    }
+    const T v0 = s_v0, tau = s_tau;
     // the other remaining columns: a_c -= tau v (v^T a_c)
     T cbv = T(-1);
     int cbc = nF;
@@ -477,14 +521,14 @@ __global__ void __launch_bounds__(1024) k_cpqr_smem(SkelDesc* fr, const int* __r
         ac[i] = fma(-v0, tw, ac[i]);   // R_ic
         tail[c] = s;
       }
-      if (full > cbv) {
+      if (norm_key(full) > norm_key(cbv)) {
         cbv = full;
         cbc = c;
       }
     }
     if (lane == 0) {
-      s_cv[cur ^ 1][warp] = cbv;
-      s_ci[cur ^ 1][warp] = cbc;
+      s_cv[warp] = cbv;
+      s_ci[warp] = cbc;
     }
     if (tid == 0) done[p] = 1;
     __syncthreads();
@@ -522,7 +566,7 @@ __global__ void __launch_bounds__(1024) k_cpqr_smem(SkelDesc* fr, const int* __r
 // entries in the factor precision (no downdating), and the pivot is the
 // largest norm, lowest column index on ties.  Each step:
 //   1. a cluster barrier makes the CTAs' proposals for this step (their best
-//      column with its norm, row-i entry and tail norm, pushed into every
+//      column with its norm and its reflector's scalars, pushed into every
 //      CTA's shared memory) and their column updates of the last step visible;
 //   2. every warp takes the winner among the CS proposals; every CTA copies
 //      the pivot column's rows below the step from its owner into a local
@@ -612,9 +656,11 @@ __global__ void __launch_bounds__(DSM_THREADS, 1) k_cpqr_dsm(SkelDesc* fr, const
   unsigned char* done = reinterpret_cast<unsigned char*>(lpos + ncq);   // per front column
   __shared__ T s_wv[DSM_WARPS], s_wh[DSM_WARPS], s_wt[DSM_WARPS];
   __shared__ int s_wc[DSM_WARPS];
-  // the CTAs' proposals, by step parity and CTA: norm, column, row-i entry,
-  // tail norm (each CTA writes its own slot in every CTA of the cluster)
-  __shared__ T s_qv[2][DSM_MAX_CS], s_qh[2][DSM_MAX_CS], s_qt[2][DSM_MAX_CS];
+  // the CTAs' proposals, by step parity and CTA: squared norm, its root, column, and
+  // its reflector's alpha, v0 and tau (each CTA writes its own slot in every CTA of
+  // the cluster)
+  __shared__ T s_qv[2][DSM_MAX_CS], s_qn[2][DSM_MAX_CS], s_qa[2][DSM_MAX_CS], s_q0[2][DSM_MAX_CS],
+      s_qt[2][DSM_MAX_CS];
   __shared__ int s_qc[2][DSM_MAX_CS];
   __shared__ int s_nrem;
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
@@ -644,18 +690,29 @@ __global__ void __launch_bounds__(DSM_THREADS, 1) k_cpqr_dsm(SkelDesc* fr, const
         const int oc = __shfl_xor_sync(0xffffffffu, c, o);
         const T oh = __shfl_xor_sync(0xffffffffu, h, o);
         const T ot = __shfl_xor_sync(0xffffffffu, t, o);
-        if (ov > v || (ov == v && oc < c)) {
+        const auto kv = norm_key(v), ko = norm_key(ov);
+        if (ko > kv || (ko == kv && oc < c)) {
           v = ov;
           c = oc;
           h = oh;
           t = ot;
         }
       }
+      // the reflector it would make, v = (h - alpha, a_c[i+1:]), with |v| = sqrt(h^2 +
+      // t): by this warp alone, as roots and quotients of all of them are FP64 work
+      // like the columns' own
+      const T nv = sqrt(fmax(v, T(0)));
+      const T alpha = h >= T(0) ? -nv : nv;
+      const T v0 = h - alpha;
+      const T vtv = fma(v0, v0, t);
+      const T tau = vtv > T(0) ? T(2) / vtv : T(0);
       if (lane < CS) {
         *cl.map_shared_rank(&s_qv[par][rank], lane) = v;
+        *cl.map_shared_rank(&s_qn[par][rank], lane) = nv;
         *cl.map_shared_rank(&s_qc[par][rank], lane) = c;
-        *cl.map_shared_rank(&s_qh[par][rank], lane) = h;
-        *cl.map_shared_rank(&s_qt[par][rank], lane) = t;
+        *cl.map_shared_rank(&s_qa[par][rank], lane) = alpha;
+        *cl.map_shared_rank(&s_q0[par][rank], lane) = v0;
+        *cl.map_shared_rank(&s_qt[par][rank], lane) = tau;
       }
     }
   };
@@ -686,7 +743,7 @@ __global__ void __launch_bounds__(DSM_THREADS, 1) k_cpqr_dsm(SkelDesc* fr, const
       head = __shfl_sync(0xffffffffu, head, 0);
       const T full = fma(head, head, s);
       if (lane == 0) tail[q] = s;
-      if (full > bv) {
+      if (norm_key(full) > norm_key(bv)) {
         bv = full;
         bc = c;
         bh = head;
@@ -698,43 +755,39 @@ __global__ void __launch_bounds__(DSM_THREADS, 1) k_cpqr_dsm(SkelDesc* fr, const
     propose(0, bv, bc, bh, bt);
   }
   int k = kmax;
-  T r11 = T(0);
+  T least = T(0);
   for (int i = 0; i < kmax; ++i) {
     const int cur = i & 1;
     cl.sync();
     // 2. the pivot: the best of the CTAs' proposals (every warp, same result)
-    T bv = T(-1), x0 = T(0), tl = T(0);
-    int p = nF;
+    T bv = T(-1);
+    int p = nF, at = 0;
     if (lane < CS) {
       bv = s_qv[cur][lane];
       p = s_qc[cur][lane];
-      x0 = s_qh[cur][lane];
-      tl = s_qt[cur][lane];
+      at = lane;
     }
-    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int o = DSM_MAX_CS / 2; o > 0; o >>= 1) {
       const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oc = __shfl_xor_sync(0xffffffffu, p, o);
-      const T oh = __shfl_xor_sync(0xffffffffu, x0, o);
-      const T ot = __shfl_xor_sync(0xffffffffu, tl, o);
-      if (ov > bv || (ov == bv && oc < p)) {
+      const int oc = __shfl_xor_sync(0xffffffffu, p, o), oa = __shfl_xor_sync(0xffffffffu, at, o);
+      const auto kb = norm_key(bv), ko = norm_key(ov);
+      if (ko > kb || (ko == kb && oc < p)) {
         bv = ov;
         p = oc;
-        x0 = oh;
-        tl = ot;
+        at = oa;
       }
     }
-    const T nv = sqrt(fmax(bv, T(0)));
-    if (i == 0) r11 = nv;
-    if (p >= nF || (i == 0 ? nv == T(0) : !((double)nv > eps * (double)r11))) {
+    p = __shfl_sync(0xffffffffu, p, 0);   // lanes from 16 on compared other proposals
+    at = __shfl_sync(0xffffffffu, at, 0);
+    const T nv = s_qn[cur][at];
+    if (i == 0) least = id_threshold(eps, nv);
+    if (p >= nF || (i == 0 ? nv == T(0) : !(nv > least))) {
       k = i;
       break;
     }
-    // reflector of column p over rows i..m-1: v = (x0 - alpha, a_p[i+1:])
-    const T nx = sqrt(fma(x0, x0, tl));
-    const T alpha = x0 >= T(0) ? -nx : nx;
-    const T v0 = x0 - alpha;
-    const T vtv = fma(v0, v0, tl);
-    const T tau = vtv > T(0) ? T(2) / vtv : T(0);
+    // reflector of column p over rows i..m-1: v = (v0, a_p[i+1:])
+    const T alpha = s_qa[cur][at], v0 = s_q0[cur][at], tau = s_qt[cur][at];
     const int owner = p % CS, qp = p / CS;
     {
       // whole 16-byte vectors from the one holding row i + 1 (rows above it
@@ -850,7 +903,8 @@ __global__ void __launch_bounds__(DSM_THREADS, 1) k_cpqr_dsm(SkelDesc* fr, const
         ac[i] = fma(-v0, tw, aci);   // R_ic
         tail[q] = s;
       }
-      if (full > cbv || (full == cbv && c < cbc)) {
+      const auto kf = norm_key(full), kb = norm_key(cbv);
+      if (kf > kb || (kf == kb && c < cbc)) {
         cbv = full;
         cbc = c;
         cbh = head;

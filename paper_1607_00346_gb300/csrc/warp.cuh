@@ -9,10 +9,12 @@ namespace hif {
 
 constexpr int UNR = 8;    // independent loads in flight per lane in the column passes
 
-// sum_{r in [r0, r1)} a[r] b[r] over one warp (result in every lane)
+// this lane's part of sum_{r in [r0, r1)} a[r] b[r]; half as many loads in flight in
+// double, whose buffers would not fit the registers (the same bytes)
 template <typename T>
-__device__ __forceinline__ T warp_dot(const T* __restrict__ a, const T* __restrict__ b, int r0,
+__device__ __forceinline__ T lane_dot(const T* __restrict__ a, const T* __restrict__ b, int r0,
                                       int r1, int lane) {
+  constexpr int UNR = hif::UNR * 4 / (int)sizeof(T);
   T acc[4] = {T(0), T(0), T(0), T(0)};
   int r = r0 + lane;
   if (r + 32 * (UNR - 1) < r1) {
@@ -44,7 +46,14 @@ __device__ __forceinline__ T warp_dot(const T* __restrict__ a, const T* __restri
     for (int u = 0; u < UNR; ++u) acc[u & 3] = fma(x[u], y[u], acc[u & 3]);
   }
   for (; r < r1; r += 32) acc[0] = fma(a[r], b[r], acc[0]);
-  T s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+}
+
+// the sum over one warp (result in every lane)
+template <typename T>
+__device__ __forceinline__ T warp_dot(const T* __restrict__ a, const T* __restrict__ b, int r0,
+                                      int r1, int lane) {
+  T s = lane_dot(a, b, r0, r1, lane);
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
 }
