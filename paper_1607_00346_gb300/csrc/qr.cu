@@ -25,7 +25,7 @@
 //     memory of a cluster (row slices, one exchange per column), k_qr_panel
 //     (one CTA per front, the panel in global memory, norms in double) takes
 //     panels too tall for 16 CTAs;
-//   * the columns right of the panel inside its 128-column block: W = T^T
+//   * the columns right of the panel inside its block: W = T^T
 //     V^T A and A -= V W, two kernels that stream those columns once each
 //     (k_qr_w1/k_qr_w2, k_qr_update);
 //   * after a block's last panel, the columns right of the block, once per
@@ -52,12 +52,17 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int QB = 32;          // panel width
-constexpr int QB2 = 128;        // block width: trailing columns are updated once per block
+// Block width: trailing columns are updated once per block.  In FP64 the updates
+// inside a block are bound by the FP64 unit while the block's products run on the
+// tensor cores, so its blocks are narrower: 64^3, eps 1e-4, widths 128, 64, 32:
+// inside 18.5, 9.7, 0 ms, block products 7.8, 13.0, 27.9 ms.
+template <typename T>
+__host__ __device__ constexpr int qr_block() { return sizeof(T) == 8 ? 64 : 128; }
 
 // Panel p (32 columns) of the block starting at p0 keeps its reflectors in
 // the block's V (rows relative to p0, ld = m): column p - p0 on, row p - p0 on,
 // so V(r, j) of the panel (r relative to p) sits at V + voff + r + j m; its T
-// is the ((p - p0) / 32)-th 32 x 32 matrix of the block's four.
+// is the ((p - p0) / 32)-th 32 x 32 matrix of the block's.
 __host__ __device__ inline int64_t qr_voff(int p, int p0, int m) { return (int64_t)(p - p0) * (m + 1); }
 __host__ __device__ inline int64_t qr_toff(int p, int p0) { return (int64_t)((p - p0) / QB) * QB * QB; }
 constexpr int QR_THREADS = 512;
@@ -474,6 +479,7 @@ template <typename T>
 __global__ void __launch_bounds__(W1_THREADS, sizeof(T) == 4 ? 2 : 1)
     k_qr_w1(const QRDesc* __restrict__ ds, const T* __restrict__ Gar, const T* __restrict__ Var,
             T* Wp, const int64_t* __restrict__ wpo, int p, int p0, int S) {
+  constexpr int QB2 = qr_block<T>();
   const QRDesc d = ds[blockIdx.y];
   if (p >= d.n) return;
   const int jb = min(QB, d.n - p);
@@ -570,6 +576,7 @@ __global__ void __launch_bounds__(128) k_qr_w2(const QRDesc* __restrict__ ds,
                                                const int64_t* __restrict__ wpo,
                                                const T* __restrict__ Tar, T* War, int p, int p0,
                                                int S) {
+  constexpr int QB2 = qr_block<T>();
   const QRDesc d = ds[blockIdx.y];
   if (p >= d.n) return;
   const int jb = min(QB, d.n - p);
@@ -603,6 +610,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_qr_update(const QRDesc* __restrict__ ds, T* Gar,
                                                    const T* __restrict__ Var,
                                                    const T* __restrict__ War, int p, int p0) {
+  constexpr int QB2 = qr_block<T>();
   const QRDesc d = ds[blockIdx.y];
   if (p >= d.n) return;
   const int jb = min(QB, d.n - p);
@@ -675,14 +683,15 @@ __global__ void __launch_bounds__(256) k_qr_update(const QRDesc* __restrict__ ds
 }
 
 
-// T of a 128-column block from the Gram matrix G = V^T V of its reflectors
-// (G[l + j 128]) and their tau (the diagonals of its four panel T's): T[j][j]
+// T of a block of QB2 columns from the Gram matrix G = V^T V of its reflectors
+// (G[l + j QB2]) and their tau (the diagonals of its panel T's): T[j][j]
 // = tau_j, T[0:j, j] = -tau_j T[0:j, 0:j] G[0:j, j], column by column; thread
 // i owns row i.  One CTA per front.
 template <typename T>
-__global__ void __launch_bounds__(QB2) k_qr_tblk(const QRDesc* __restrict__ ds,
+__global__ void __launch_bounds__(qr_block<T>()) k_qr_tblk(const QRDesc* __restrict__ ds,
                                                  const T* __restrict__ Gb,
                                                  const T* __restrict__ Tar, T* Tb) {
+  constexpr int QB2 = qr_block<T>();
   const QRDesc d = ds[blockIdx.x];
   const T* G = Gb + (int64_t)blockIdx.x * QB2 * QB2;
   const T* Tp = Tar + d.Tt;
@@ -787,6 +796,7 @@ template <typename T>
 void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garena, T* Rout,
                     const std::vector<int64_t>& rOff, int* d_flags, bool tensor_cores,
                     cudaStream_t st) {
+  constexpr int QB2 = qr_block<T>();
   const int nq = (int)which.size();
   if (nq == 0) return;
   // fronts sorted by n (largest first) so that the fronts still factoring a
@@ -811,7 +821,7 @@ void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garen
     d.pad = 0;
     voff += (int64_t)d.m * QB2;          // the block's reflectors
     woff += (int64_t)QB * d.n;
-    toff += (QB2 / QB) * QB * QB;         // the block's four panel T's
+    toff += (QB2 / QB) * QB * QB;         // the block's panel T's
     ro[i] = rOff[ord[i]];
   }
   T *Var = nullptr, *War = nullptr, *Tar = nullptr;
