@@ -59,15 +59,19 @@ struct TileAcc {
 //
 // k_chol_diag: one CTA per front factors the jb x jb diagonal block (jb <= 64) in
 // shared memory, 16 columns at a time: one warp factors the 16 x 16 block in
-// registers (rows across lanes, pivot column by shuffles), one thread per row
-// solves the rows below, all threads update the rest; three CTA barriers per 16
-// columns.  Then it inverts L in the same pass (16 x 16 blocks by substitution,
-// merged pairwise to 32 and 64) and leaves L^{-1} in the factor panel, zeros above
-// the diagonal: the panel below becomes a product, and the triangular inverse of
-// the whole front needs these blocks anyway.  64 columns, FP32 25 us, FP64 100 us:
-// with one column per barrier pair and no inverse 62 and 112 us; the panel below
-// 8 us (by substitution 30-37, FP64 117), the 64-deep update of one tile 11 us
-// (18, FP64 49), and the separate inverse took 25-95 us.
+// registers (rows across lanes, pivot column by shuffles), four threads per row solve
+// the rows below and, in the same pass, the block's own inverse, all threads update
+// the rest; three CTA barriers per 16 columns.  The inverses are merged pairwise to 32
+// and 64 and L^{-1} left in the factor panel, zeros above the diagonal: the panel below
+// becomes a product, and the triangular inverse of the whole front needs these blocks
+// anyway.  In FP64 an instruction of one warp takes 64 clocks (each quarter of an SM
+// has a quarter of its FP64 unit), masked or not: so every phase but the factoring
+// warp's spreads over all quarters, without masked multiply-adds.  Clocks of a block,
+// before and after that: factor 69 k -> 58 k, solve and 16-wide inverses 43 k -> 20 k,
+// update 39 k -> 21 k, merges 50 k -> 28 k (FP64; after: counted from the instructions).
+// 64 columns, FP32 25 us, FP64 100 -> 77 us: with one column per barrier pair and no
+// inverse 62 and 112 us; the panel below 8 us (by substitution 30-37, FP64 117), the
+// 64-deep update of one tile 11 us (18, FP64 49), and the separate inverse took 25-95 us.
 //
 // A non-positive or non-finite pivot flags the front and continues with 1.  With
 // growth > 0 (FP32 fronts that may be retried in FP64), the panel's diagonal
@@ -83,16 +87,47 @@ constexpr size_t chol_diag_smem() {
   return sizeof(T) * 2 * NB * DP;
 }
 
-// sqrt(d) and its reciprocal in one chain (a reciprocal square root and, in
-// FP32, one Newton step on it): every column of the block waits for it.
-__device__ __forceinline__ void sqrt_and_inverse(float d, float& piv, float& inv) {
+// 1 / sqrt(d) (in FP32 with one Newton step): every column of the block waits for it.
+__device__ __forceinline__ float inverse_root(float d) {
   const float y = rsqrtf(d);
-  inv = fmaf(0.5f * y, fmaf(-d * y, y, 1.0f), y);
-  piv = d * inv;
+  return fmaf(0.5f * y, fmaf(-d * y, y, 1.0f), y);
 }
-__device__ __forceinline__ void sqrt_and_inverse(double d, double& piv, double& inv) {
-  inv = rsqrt(d);
-  piv = d * inv;
+__device__ __forceinline__ double inverse_root(double d) { return rsqrt(d); }
+// d positive and finite (the double without the FP64 unit)
+__device__ __forceinline__ bool pivot_ok(float d) { return d > 0.f && isfinite(d); }
+__device__ __forceinline__ bool pivot_ok(double d) {
+  const long long b = __double_as_longlong(d);
+  return b > 0 && b < 0x7ff0000000000000ll;
+}
+
+// S(i, j) -= X_i X_j^T over the N blocks of 16 rows below the block at o.  The number
+// of blocks is a template argument: masked multiply-adds take their turn on the FP64
+// unit like the others.
+template <int N, typename T>
+__device__ __forceinline__ void chol_diag_update(T (*S)[DP], int o) {
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  T u[N * (N + 1) / 2];
+#pragma unroll
+  for (int i = 0; i < N * (N + 1) / 2; ++i) u[i] = T(0);
+#pragma unroll
+  for (int l = 0; l < CB; ++l) {
+    T xr[N], xc[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      xr[i] = S[o + CB + ty + 16 * i][o + l];
+      xc[i] = S[o + CB + tx + 16 * i][o + l];
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int j = 0; j <= i; ++j)
+        u[i * (i + 1) / 2 + j] = fma(xr[i], xc[j], u[i * (i + 1) / 2 + j]);
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int j = 0; j <= i; ++j)
+      S[o + CB + ty + 16 * i][o + CB + tx + 16 * j] -= u[i * (i + 1) / 2 + j];
 }
 
 template <typename T>
@@ -130,17 +165,17 @@ __global__ void __launch_bounds__(256) k_chol_diag(const DFront* __restrict__ fr
 #pragma unroll
       for (int c = 0; c < CB; ++c) {
         T dv = __shfl_sync(0xffffffffu, a[c / 2], c + (c % 2) * CB);
-        const bool ok = dv > T(0) && isfinite(dv);
+        const bool ok = pivot_ok(dv);
         if (o + c < jb) {
           bad = bad || !ok;
           if (growth > 0.f) weak = weak || !ok || dv * (T)growth < s_orig[o + c];
         }
         if (!ok) dv = T(1);
-        T piv, inv;
-        sqrt_and_inverse(dv, piv, inv);
+        const T inv = inverse_root(dv);
         // column c of L, in every lane of row r
-        const T ac = __shfl_sync(0xffffffffu, a[c / 2], r + (c % 2) * CB);
-        const T l = r > c ? ac * inv : (r == c ? piv : T(0));
+        T ac = __shfl_sync(0xffffffffu, a[c / 2], r + (c % 2) * CB);
+        if (r == c) ac = dv;
+        const T l = r >= c ? ac * inv : T(0);
         if (h == c % 2) a[c / 2] = l;
         if (r == c) myinv = inv;
 #pragma unroll
@@ -161,73 +196,51 @@ __global__ void __launch_bounds__(256) k_chol_diag(const DFront* __restrict__ fr
       }
     }
     __syncthreads();
+    // rows below: X L_oo^T = A; and 16 rows of the identity, which become L_oo^{-T}:
+    // four threads per row (thread t: columns t + 4 q), so that all four parts of the
+    // SM have a share
     const int below = je - o - CB;
-    if (below == 0) break;
-    if (tid < below) {
-      T x[CB];
-      T* row = &S[o + CB + tid][o];
+    if (tid / 4 < below + CB) {   // whole warps
+      const int rr = tid / 4, t = tid % 4, e = rr - below;
+      T x[CB / 4];
 #pragma unroll
-      for (int j = 0; j < CB; ++j) x[j] = row[j];
+      for (int q = 0; q < CB / 4; ++q)
+        x[q] = e >= 0 ? T(t + 4 * q == e ? 1 : 0) : S[o + CB + rr][o + t + 4 * q];
 #pragma unroll
       for (int c = 0; c < CB; ++c) {
-        x[c] *= s_inv[o + c];
+        const T xc = __shfl_sync(0xffffffffu, x[c / 4] * s_inv[o + c], (lane & 28) | (c % 4));
+        if (t == c % 4) x[c / 4] = xc;
 #pragma unroll
-        for (int j = c + 1; j < CB; ++j) x[j] = fma(-x[c], S[o + j][o + c], x[j]);
+        for (int q = c / 4 + (c % 4 == 3); q < CB / 4; ++q)
+          if (t + 4 * q > c) x[q] = fma(-xc, S[o + t + 4 * q][o + c], x[q]);
       }
 #pragma unroll
-      for (int j = 0; j < CB; ++j) row[j] = x[j];
+      for (int q = 0; q < CB / 4; ++q) {
+        if (e >= 0) V[o + t + 4 * q][o + e] = x[q];
+        else S[o + CB + rr][o + t + 4 * q] = x[q];
+      }
     }
     __syncthreads();
+    if (below == 0) break;
     // rank-16 update of the lower triangle of the rest: thread (ty, tx) of a
     // 16 x 16 grid takes one entry of each 16 x 16 block
-    const int tx = tid % 16, ty = tid / 16, nbl = below / CB;
-    T u[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-#pragma unroll
-    for (int l = 0; l < CB; ++l) {
-      T xr[3], xc[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        if (i < nbl) {
-          xr[i] = S[o + CB + ty + 16 * i][o + l];
-          xc[i] = S[o + CB + tx + 16 * i][o + l];
-        }
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j <= i; ++j)
-          if (i < nbl) u[i * (i + 1) / 2 + j] = fma(xr[i], xc[j], u[i * (i + 1) / 2 + j]);
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j <= i; ++j)
-        if (i < nbl) S[o + CB + ty + 16 * i][o + CB + tx + 16 * j] -= u[i * (i + 1) / 2 + j];
+    if (below == 3 * CB) chol_diag_update<3>(S, o);
+    else if (below == 2 * CB) chol_diag_update<2>(S, o);
+    else chol_diag_update<1>(S, o);
     __syncthreads();
   }
-  // inverses of the 16 x 16 diagonal blocks: one warp each, one lane per column
-  if (warp < nb16 && lane < CB) {
-    const int o = warp * CB, c = lane;
-    T z[CB];
-#pragma unroll
-    for (int r = 0; r < CB; ++r) {
-      T t = T(0);
-#pragma unroll
-      for (int l = 0; l < r; ++l) t = fma(S[o + r][o + l], z[l], t);
-      z[r] = r == c ? s_inv[o + r] : (r > c ? -t * s_inv[o + r] : T(0));
-    }
-#pragma unroll
-    for (int r = 0; r < CB; ++r) V[o + r][o + c] = z[r];
-  }
-  __syncthreads();
   // pairs of blocks of w: [A 0; B C]^-1 = [A^-1 0; -C^-1 B A^-1  C^-1].  B A^-1 is
   // kept transposed in the free block above the diagonal.
   for (int w = CB; w < je; w *= 2) {
     // 2 x 2 entries per thread: w = 16 has up to two pairs (128 threads), w = 32
     // one (256); rows past je (a shorter right block) are computed and unused
-    const int per = w * w / 4, q = tid / per, r = tid % per % (w / 2) * 2, c = tid % per / (w / 2) * 2;
-    const int o = 2 * w * q;
-    const bool in = o + w + r < je;
-    if (in) {
+    const int per = w * w / 4, q = tid / per, o = 2 * w * q;
+    // the depth goes with 2 g, down or up: equal g in a half warp, and the two warps
+    // of one part of the SM (warp and warp + 4) from opposite ends
+    const int l = tid % per % (w / 2);
+    const int g = w == 32 ? (warp < 4 ? warp : 11 - warp) * 2 + lane / 16 : tid % per / (w / 2);
+    int r = 2 * l, c = 2 * g;
+    if (o + w + r < je) {
       T t00 = T(0), t01 = T(0), t10 = T(0), t11 = T(0);
 #pragma unroll 8
       for (int k = c; k < w; ++k) {   // V[o + k][.] is zero for k < c
@@ -244,7 +257,9 @@ __global__ void __launch_bounds__(256) k_chol_diag(const DFront* __restrict__ fr
       V[o + c + 1][o + w + r + 1] = t11;
     }
     __syncthreads();
-    if (in) {
+    r = 2 * g;
+    c = 2 * l;
+    if (o + w + r < je) {
       T t00 = T(0), t01 = T(0), t10 = T(0), t11 = T(0);
 #pragma unroll 8
       for (int k = 0; k <= r + 1; ++k) {
