@@ -71,7 +71,7 @@ def field_desc(w: dict) -> str:
 KERNEL_BOUND = {
     "gemm_tc": "tensor", "chol_block_update_tc": "tensor", "trtri_merge_tc": "tensor",
     "chol_panel": "alu", "chol_trailing_update": "alu", "gemm_batched": "alu",
-    "trtri_merge": "alu", "trtri_diag": "alu", "id_cpqr": "alu", "id_cpqr_smem": "alu",
+    "trtri_merge": "alu", "id_pchol": "alu64", "id_cpqr": "alu", "id_cpqr_smem": "alu",
     "id_cpqr_dsm": "alu",
     "id_rowreduce_panel": "alu", "id_rowreduce_w1": "alu", "skel_z_products": "alu",
     "id_rowreduce_block_tc": "tensor", "id_rowreduce_block": "alu", "id_rowreduce_blockt": "alu",
@@ -83,16 +83,16 @@ KERNEL_BOUND = {
     "apply_gather": "hbm", "apply_scatter": "hbm", "apply_accumulate": "hbm",
     "convert": "hbm", "skel_gather": "hbm", "merge_children": "hbm", "spmv": "hbm",
     "residual": "hbm", "dots": "hbm", "axpy": "hbm", "id_rowreduce_update": "hbm",
-    "stencil_coefficients": "hbm",
+    "stencil_coefficients": "hbm", "row_lists": "hbm", "chol_retry_snapshot": "hbm",
+    "id_gram_f64tc": "sliced", "id_pchol_update_f64tc": "sliced",
 }
+# BF16 products per FP64 product of the sliced form: 28 for FP32 operands, else 36
+SLICED = {"id_gram_f64tc": 28}
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a
-# kernel label in the bench workload, from the ncu captures summarised in
-# profiles/ (absent where no capture of the current kernel exists):
-# gemm_tc: the 12 Schur-product launches of one 128^3 factorization move
-# 53.8 GB (profiles/gemm_tc_traffic_contrast128.md); id_cpqr: its 4 k_cpqr
-# launches move 78.7 GB (profiles/id_cpqr_traffic_contrast128.md).
-TRAFFIC_PER_LAUNCH = {"gemm_tc": 53.76e9 / 12, "id_cpqr": 78.73e9 / 4}
+# kernel label in the bench workload, from ncu captures of the current kernels
+# (none taken since the products leave out the zeros of triangular operands)
+TRAFFIC_PER_LAUNCH = {}
 
 
 def _hbm_peak():
@@ -469,8 +469,14 @@ def main():
             ach = k["flops"] / max(k["launches"], 1) / per_launch_s / 1e12
             src = "measured in this run: tcgen05 kind::tf32 loop (hif_measure_peaks)"
             unit = "TFLOP/s"
-        elif bound == "alu":
-            fp32 = prec == hif.PREC_FP32
+        elif bound == "sliced":
+            # FP64 products as exact sums of products of 8-bit slices
+            peak = peaks["bf16_mma_tflops"] / SLICED.get(k["name"], 36)
+            ach = k["flops"] / max(k["launches"], 1) / per_launch_s / 1e12
+            src = "measured in this run: tcgen05 kind::f16 loop (hif_measure_peaks) / slice products"
+            unit = "TFLOP/s"
+        elif bound in ("alu", "alu64"):
+            fp32 = prec == hif.PREC_FP32 and bound == "alu"
             peak = peaks["fp32_fma_tflops" if fp32 else "fp64_fma_tflops"]
             ach = k["flops"] / max(k["launches"], 1) / per_launch_s / 1e12
             src = (f"measured in this run: {'FP32' if fp32 else 'FP64'} FMA loop "

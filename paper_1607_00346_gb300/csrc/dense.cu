@@ -66,9 +66,9 @@ struct TileAcc {
 // becomes a product, and the triangular inverse of the whole front needs these blocks
 // anyway.  In FP64 an instruction of one warp takes 64 clocks (each quarter of an SM
 // has a quarter of its FP64 unit), masked or not: so every phase but the factoring
-// warp's spreads over all quarters, without masked multiply-adds.  Clocks of a block,
-// before and after that: factor 69 k -> 58 k, solve and 16-wide inverses 43 k -> 20 k,
-// update 39 k -> 21 k, merges 50 k -> 28 k (FP64; after: counted from the instructions).
+// warp's spreads over all quarters, without masked multiply-adds.  Clocks of a 64-column
+// block in FP64, before and after that: factor 69 k -> 63 k, solve and 16-wide inverses
+// 43 k -> 25 k, update 39 k -> 23 k, merges 50 k -> 41 k.
 // 64 columns, FP32 25 us, FP64 100 -> 77 us: with one column per barrier pair and no
 // inverse 62 and 112 us; the panel below 8 us (by substitution 30-37, FP64 117), the
 // 64-deep update of one tile 11 us (18, FP64 49), and the separate inverse took 25-95 us.
@@ -173,9 +173,10 @@ __global__ void __launch_bounds__(256) k_chol_diag(const DFront* __restrict__ fr
         if (!ok) dv = T(1);
         const T inv = inverse_root(dv);
         // column c of L, in every lane of row r
-        T ac = __shfl_sync(0xffffffffu, a[c / 2], r + (c % 2) * CB);
-        if (r == c) ac = dv;
-        const T l = r >= c ? ac * inv : T(0);
+        const T ac = __shfl_sync(0xffffffffu, a[c / 2], r + (c % 2) * CB);
+        T l;   // in FP64 one product fewer (64 clocks), in FP32 a shorter chain
+        if constexpr (sizeof(T) == 8) l = r >= c ? (r == c ? dv : ac) * inv : T(0);
+        else l = r > c ? ac * inv : (r == c ? dv * inv : T(0));
         if (h == c % 2) a[c / 2] = l;
         if (r == c) myinv = inv;
 #pragma unroll
@@ -243,9 +244,9 @@ __global__ void __launch_bounds__(256) k_chol_diag(const DFront* __restrict__ fr
     if (o + w + r < je) {
       T t00 = T(0), t01 = T(0), t10 = T(0), t11 = T(0);
 #pragma unroll 8
-      for (int k = c; k < w; ++k) {   // V[o + k][.] is zero for k < c
+      for (int k = c; k < w; ++k) {   // V[o + k][o + c] is zero for k < c
         const T s0 = S[o + w + r][o + k], s1 = S[o + w + r + 1][o + k];
-        const T v0 = V[o + k][o + c], v1 = k > c ? V[o + k][o + c + 1] : T(0);
+        const T v0 = V[o + k][o + c], v1 = V[o + k][o + c + 1];
         t00 = fma(s0, v0, t00);
         t01 = fma(s0, v1, t01);
         t10 = fma(s1, v0, t10);
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(256) k_chol_diag(const DFront* __restrict__ fr
       T t00 = T(0), t01 = T(0), t10 = T(0), t11 = T(0);
 #pragma unroll 8
       for (int k = 0; k <= r + 1; ++k) {
-        const T v0 = k <= r ? V[o + w + r][o + w + k] : T(0), v1 = V[o + w + r + 1][o + w + k];
+        const T v0 = V[o + w + r][o + w + k], v1 = V[o + w + r + 1][o + w + k];
         const T s0 = V[o + c][o + w + k], s1 = V[o + c + 1][o + w + k];
         t00 = fma(v0, s0, t00);
         t01 = fma(v0, s1, t01);

@@ -1081,8 +1081,8 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
       for (size_t j = 0; j < sel[g].size(); ++j) {
         const int f = sel[g][j], sm = route[g][j];
         const double k = sd[f].k, nF = sd[f].nF;
-        if (sm == ID_ROUTE_GRAM) {   // pivoted Cholesky: k nF (nF - k) + k^3 / 3 ..
-          fl[sm] += k * nF * (nF - k) + k * k * k / 3.0;
+        if (sm == ID_ROUTE_GRAM) {   // pivoted Cholesky of G
+          fl[sm] += 64.0 * k * nF;   // inside blocks of 64 pivots; the rest: id_pchol_update_f64tc
           by[sm] += 8.0 * 0.5 * nF * nF;
           continue;
         }
