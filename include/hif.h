@@ -192,7 +192,8 @@ hif_status hif_solve(hif_handle h, const double* f, double* u, int nrhs,
  * hif_apply(h[i], f[i], u[i], nrhs[i]) gives.
  *   h:     nh distinct handles of one precision, on the current device.
  *   f, u:  arrays of nh pointers; f[i], u[i] hold nrhs[i] * n_i^3 doubles
- *          (host or device, as for hif_apply).
+ *          (host or device, as for hif_apply).  Every f is read before any u
+ *          is written, so a u may be any system's f.
  * Errors: INVALID_ARG (nh < 1, NULL or repeated handles, mixed precision or
  * device, nrhs < 1), OOM, CUDA.
  */
@@ -202,9 +203,11 @@ hif_status hif_apply_batch(const hif_handle* h, int nh, const double* const* f,
 /*
  * hif_solve_batch -- hif_solve for nh factors at once: the conjugate
  * gradients of all the systems advance in lockstep, each on a stream of its
- * own, and share the host's wait once per iteration.  Each system's iteration is the one hif_solve runs (same
- * kernels, same scalar arithmetic, its own pcg_tol and max_iter), so its
- * u, iteration counts and residuals are bitwise those of hif_solve alone.
+ * own, and share the host's wait once per iteration.  Each system's iteration
+ * is the one hif_solve runs (same kernels, same scalar arithmetic, its own
+ * pcg_tol and max_iter), so its u, iteration counts and residuals are bitwise
+ * those of hif_solve alone.  The systems are taken up in order, each clearing
+ * its u and then reading its f, so an f may be the u of a later system.
  * iters and relres (host, optional) receive sum(nrhs) entries, the columns
  * of the systems in order.
  * Errors: as hif_apply_batch, and NO_CONVERGENCE if any column did not

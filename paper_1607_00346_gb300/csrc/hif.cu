@@ -231,7 +231,16 @@ struct FactorBase {
     if (side_ev) cudaEventDestroy(side_ev);
     if (pinned) cudaFreeHost(pinned);
   }
-  virtual void apply(const double* f_dev, double* u_dev, int nrhs, cudaStream_t st) = 0;
+  // The three parts of an apply: f into the factor's own vector, the sweeps on it,
+  // and that vector to u.
+  virtual void apply_in(const double* f_dev, int nrhs, cudaStream_t st) = 0;
+  virtual void apply_sweeps(int nrhs, cudaStream_t st) = 0;
+  virtual void apply_out(double* u_dev, int nrhs, cudaStream_t st) = 0;
+  void apply(const double* f_dev, double* u_dev, int nrhs, cudaStream_t st) {
+    apply_in(f_dev, nrhs, st);
+    apply_sweeps(nrhs, st);
+    apply_out(u_dev, nrhs, st);
+  }
   // Bytes of work space the sweeps need for nrhs right-hand sides, and the
   // sweeps run in caller-provided work space (nothing is allocated).
   virtual size_t sweep_scratch_bytes(int nrhs) const = 0;
@@ -377,14 +386,15 @@ struct Factor : FactorBase {
     }
   }
 
-  void apply(const double* f_dev, double* u_dev, int nrhs, cudaStream_t st) override {
-    const int64_t N = (int64_t)n * n * n;
+  void apply_in(const double* f_dev, int nrhs, cudaStream_t st) override {
     ensure_apply_buffers(nrhs);
-    T* yv = y.as<T>();
-    T* w = work.as<T>();
-    vec_convert_in<T>(f_dev, yv, N * nrhs, st);
-    sweeps_maybe_graph(yv, w, nrhs, st);
-    vec_convert_out<T>(yv, u_dev, N * nrhs, st);
+    vec_convert_in<T>(f_dev, y.as<T>(), (int64_t)n * n * n * nrhs, st);
+  }
+  void apply_sweeps(int nrhs, cudaStream_t st) override {
+    sweeps_maybe_graph(y.as<T>(), work.as<T>(), nrhs, st);
+  }
+  void apply_out(double* u_dev, int nrhs, cudaStream_t st) override {
+    vec_convert_out<T>(y.as<T>(), u_dev, (int64_t)n * n * n * nrhs, st);
   }
 
   static size_t round256(size_t b) { return (b + 255) / 256 * 256; }
@@ -411,6 +421,10 @@ struct Factor : FactorBase {
 // the caller's stream and a join back to it, so that the factors' small launches
 // overlap on the GPU; a factor alone stays on the caller's stream.  Every
 // factor's buffers are its own, so its result is bitwise that of its own call.
+// Between fork and join a factor's stream reads none of the batch's inputs and
+// writes no array that another system reads: an output may be another system's
+// input, so all inputs are read on the caller's stream before the fork (and the
+// outputs of an apply written on it after the join).
 // (The batch used to run in shared launches, stage by stage: at each stage the
 // small factors waited for the large one's, and the host assembled some 350
 // launches per apply.  Four operators of 32^3 to 96^3, five iterations: 26.9 ms;
@@ -1234,7 +1248,7 @@ struct PcgItem {
   double* u = nullptr;
   int nrhs = 0;
   cudaStream_t st = nullptr;
-  DevBuf work;                       // every vector and scalar, from the stream's pool
+  DevBuf work;                       // every vector and scalar, ordered on the caller's stream
   double *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr;
   PcgScalars s{};
   double *rr = nullptr, *ff = nullptr;   // ||r||^2 and ||f||^2 in pinned host memory
@@ -1250,20 +1264,15 @@ struct PcgItem {
 // its columns reached its pcg_tol or after its max_iter iterations.  Returns
 // HIF_OK if every column converged.
 hif_status pcg_many(std::vector<PcgItem>& items, cudaStream_t st) {
-  std::vector<FactorBase*> Fs;
-  for (PcgItem& I : items) Fs.push_back(I.F);
-  Fork fork(Fs, st);
   auto N_of = [](const PcgItem& I) { return (int64_t)I.F->n * I.F->n * I.F->n; };
-  // rr to the host, read after the next wait (pinned: a copy to pageable memory
-  // would wait here, before the next item's launches)
-  auto fetch = [&](PcgItem& I, double* out) {
-    HIF_CUDA_TRY(cudaMemcpyAsync(out, I.s.rr, sizeof(double) * I.nrhs, cudaMemcpyDeviceToHost, I.st));
-  };
+  // on the caller's stream, system by system: u = 0, r = f (an f may be the u of a
+  // later system)
+  std::vector<FactorBase*> Fs;
   for (PcgItem& I : items) {
-    I.st = fork.stream(I.F);
+    Fs.push_back(I.F);
     const int64_t N = N_of(I), V = N * I.nrhs;
     const int64_t np = pcg_part_elems(N, I.nrhs);
-    I.work.alloc_async(sizeof(double) * (4 * V + np + 5 * I.nrhs), &I.F->mem, I.st);
+    I.work.alloc_async(sizeof(double) * (4 * V + np + 5 * I.nrhs), &I.F->mem, st);
     I.r = I.work.as<double>();
     I.z = I.r + V;
     I.p = I.z + V;
@@ -1274,13 +1283,23 @@ hif_status pcg_many(std::vector<PcgItem>& items, cudaStream_t st) {
     I.s.be = I.s.al + I.nrhs;
     I.s.rr = I.s.be + I.nrhs;
     I.s.done = reinterpret_cast<int*>(I.s.rr + I.nrhs);
+    HIF_CUDA_TRY(cudaMemsetAsync(I.u, 0, sizeof(double) * V, st));
+    HIF_CUDA_TRY(cudaMemcpyAsync(I.r, I.f, sizeof(double) * V, cudaMemcpyDeviceToDevice, st));
+  }
+  Fork fork(Fs, st);   // joined on return, before the items' vectors are freed on st
+  // rr to the host, read after the next wait (pinned: a copy to pageable memory
+  // would wait here, before the next item's launches)
+  auto fetch = [&](PcgItem& I, double* out) {
+    HIF_CUDA_TRY(cudaMemcpyAsync(out, I.s.rr, sizeof(double) * I.nrhs, cudaMemcpyDeviceToHost, I.st));
+  };
+  for (PcgItem& I : items) {
+    I.st = fork.stream(I.F);
+    const int64_t N = N_of(I);
     for (auto* v : {&I.fn, &I.rel}) v->assign(I.nrhs, 0.0);
     I.rr = I.F->pinned_norms(I.nrhs);
     I.ff = I.rr + I.nrhs;
     I.it.assign(I.nrhs, 0);
     I.done.assign(I.nrhs, 0);
-    HIF_CUDA_TRY(cudaMemsetAsync(I.u, 0, sizeof(double) * V, I.st));
-    HIF_CUDA_TRY(cudaMemcpyAsync(I.r, I.f, sizeof(double) * V, cudaMemcpyDeviceToDevice, I.st));
     pcg_start(I.r, N, I.nrhs, I.s, I.st);
     fetch(I, I.ff);
     I.F->apply(I.r, I.z, I.nrhs, I.st);
@@ -1347,10 +1366,7 @@ hif_status pcg_many(std::vector<PcgItem>& items, cudaStream_t st) {
     norms();
   }
   bool ok = true;
-  for (PcgItem& I : items) {
-    ok = ok && I.all;
-    I.work.release();   // in the order of its stream, before the join
-  }
+  for (PcgItem& I : items) ok = ok && I.all;
   return ok ? HIF_OK : HIF_ERR_NO_CONVERGENCE;
 }
 
@@ -1943,9 +1959,11 @@ hif_status hif_apply_batch(const hif_handle* hs, int nh, const double* const* f,
     up[i] = uo[i].p;
   }
   {
+    for (int i = 0; i < nh; ++i) Fs[i]->apply_in(fp[i], nrhs[i], st);
     hif::Fork fork(Fs, st);
-    for (int i = 0; i < nh; ++i) Fs[i]->apply(fp[i], up[i], nrhs[i], fork.stream(Fs[i]));
+    for (int i = 0; i < nh; ++i) Fs[i]->apply_sweeps(nrhs[i], fork.stream(Fs[i]));
   }
+  for (int i = 0; i < nh; ++i) Fs[i]->apply_out(up[i], nrhs[i], st);
   bool staged = false;
   for (int i = 0; i < nh; ++i) {
     uo[i].finish(st);
