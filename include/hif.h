@@ -97,7 +97,10 @@ typedef struct {
                         cores.  HIF_PREC_FP32: TF32 with the 3xTF32 split,
                         FP32 accumulation.  HIF_PREC_FP64: operands split
                         into eight 8-bit slices, exact sums, one rounding
-                        per entry (less error than the FMA form).  0: every
+                        per entry, where the operator's largest diagonal
+                        entry is at most 10^4 times its least (the solve
+                        error of an exact factorization is that of the FMA
+                        form there); on the FMA units beyond that.  0: every
                         product on the FMA units of its precision. */
   double retry_growth; /* HIF_PREC_FP32 only: a front whose Cholesky (the
                         LDL^T of §2.2 / §2.3) meets a pivot d_j with

@@ -101,6 +101,10 @@ struct DFront {
 // (half of the product): KZ_B_UP op(B)[k][c] = 0 for k > c, KZ_B_LOW
 // op(B)[k][c] = 0 for k < c, KZ_A_LOW op(A)[r][k] = 0 for k > r.
 enum : int { KZ_NONE = 0, KZ_B_UP = 1, KZ_B_LOW = 2, KZ_A_LOW = 3 };
+// kbal: how gemm_f64tc balances the scales of k between the operands (f64tc.cu).
+// KB_MAX by their largest entries, KB_NONE not at all, KB_DOWN column k of op(A) times
+// 2^-e[ks + k] and row k of op(B) times 2^e[ks + k], KB_UP the other way round.
+enum : int { KB_MAX = 0, KB_NONE = 1, KB_DOWN = 2, KB_UP = 3 };
 struct GemmOp {
   int64_t A, B, C;   // element offsets from the A, B and C base pointers of the launch
   int m, n, k;
@@ -109,6 +113,8 @@ struct GemmOp {
   float alpha, beta;
   int lower;         // 1: C is symmetric, only tiles touching its lower triangle are computed
   int kzero;
+  int kbal;
+  int64_t ks;
 };
 
 // The tile a block computes (longest sums first: with a triangular operand the

@@ -474,6 +474,16 @@ __global__ void __launch_bounds__(256) k_retry_writeback(const RetryMap* __restr
   }
 }
 
+__global__ void __launch_bounds__(128) k_diag_exponents(const DFront* __restrict__ fr,
+                                                       const double* __restrict__ Kar, int* e,
+                                                       int stride) {
+  const DFront d = fr[blockIdx.x];
+  for (int i = threadIdx.x; i < d.n; i += 128) {
+    const double v = Kar[d.K + i + (int64_t)i * d.ld];
+    e[(int64_t)blockIdx.x * stride + i] = v > 0.0 && isfinite(v) ? ilogb(v) >> 1 : 0;
+  }
+}
+
 // ---- generic batched GEMM ------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemm(const GemmOp* __restrict__ ops, const T* Ab,
@@ -541,7 +551,8 @@ constexpr int TC_MIN_ROWS = 256;
 
 template <typename T>
 void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T* Karena,
-                   T* Parena, int* d_flags, bool tensor_cores, cudaStream_t st);
+                   T* Parena, int* d_flags, bool tensor_cores, cudaStream_t st, const int* d_kexp,
+                   int kstride);
 
 // Refactor the flagged FP32 fronts entirely in FP64 (from the snapshot of
 // their leading blocks and their untouched A_NI, A_NN) and store the results
@@ -644,6 +655,14 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
   constexpr int NB2 = 256;
   const bool f64tc = sizeof(T) == 8 && tensor_cores;
   const bool outer = pmax > NB2 && !f64tc;
+  int* d_kexp = nullptr;   // scales of the eliminated DOFs, for the products' k
+  const int kstride = f64tc ? pmax : 0;
+  if constexpr (sizeof(T) == 8) {
+    if (f64tc) {
+      HIF_CUDA_TRY(cudaMallocAsync(&d_kexp, sizeof(int) * std::max<int64_t>(1, (int64_t)nfront * kstride), st));
+      diag_exponents(d_lead, nfront, Karena, d_kexp, kstride, st);
+    }
+  }
   static const bool attr = [] {   // initialised once, also under concurrent factorizations
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_chol_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)chol_diag_smem<T>()));
@@ -697,7 +716,7 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
             const int ld = h.ld, r = h.p - j0 - NB;
             const int64_t a21 = h.K + j0 + NB + (int64_t)j0 * ld;
             po[f] = GemmOp{a21, h.P + j0 + (int64_t)j0 * ld, a21, r, NB, NB, ld, ld, ld, 0, 1, 1.f, 0.f,
-                           0, KZ_B_UP};
+                           0, KZ_B_UP, KB_DOWN, (int64_t)f * kstride + j0};
             uo[f] = GemmOp{a21, a21, a21 + (int64_t)NB * ld, r, r, NB, ld, ld, ld, 0, 1, -1.f, 1.f, 1, 0};
           }
           GemmOp* d_step = nullptr;
@@ -705,7 +724,8 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
           po.insert(po.end(), uo.begin(), uo.end());
           HIF_CUDA_TRY(cudaMemcpyAsync(d_step, po.data(), sizeof(GemmOp) * 2 * nbelow,
                                        cudaMemcpyHostToDevice, st));
-          gemm_f64tc<double>(d_step, po.data(), nbelow, Karena, Parena, Karena, d_flags, st, "chol_panel_f64tc");
+          gemm_f64tc<double>(d_step, po.data(), nbelow, Karena, Parena, Karena, d_flags, st, "chol_panel_f64tc",
+                             d_kexp);
           gemm_f64tc<double>(d_step + nbelow, uo.data(), nbelow, Karena, Karena, Karena, d_flags, st,
                      "chol_trailing_update_f64tc");
           HIF_CUDA_TRY(cudaFreeAsync(d_step, st));
@@ -769,7 +789,7 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
     }
     if (!bad.empty()) {
       if constexpr (std::is_same<T, float>::value)
-        retry_fronts_fp64(bad, h_fronts, soff, Karena, Parena, snap, d_flags, tensor_cores, st);
+        retry_fronts_fp64(bad, h_fronts, soff, Karena, Parena, snap, d_flags, retry->tensor_cores, st);
       if (retry->retried) *retry->retried += (int64_t)bad.size();
       if (!keep.empty()) {
         HIF_CUDA_TRY(cudaMallocAsync(&d_keep, sizeof(DFront) * keep.size(), st));
@@ -785,14 +805,17 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
     HIF_CUDA_TRY(cudaFreeAsync(d_fflag, st));
     if (nfront == 0) return;
   }
-  finish_fronts(d_fronts, h_fronts, nfront, Karena, Parena, d_flags, tensor_cores, st);
+  finish_fronts(d_fronts, h_fronts, nfront, Karena, Parena, d_flags, tensor_cores, st, d_kexp, kstride);
+  if (d_kexp) HIF_CUDA_TRY(cudaFreeAsync(d_kexp, st));
   if (d_keep) HIF_CUDA_TRY(cudaFreeAsync(d_keep, st));
 }
 
-// Steps 2-4 of the partial Cholesky once the leading blocks hold L.
+// Steps 2-4 of the partial Cholesky once the leading blocks hold L.  d_kexp: the
+// exponents of the eliminated DOFs' scales, kstride per front (FP64 on tensor cores).
 template <typename T>
 void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T* Karena,
-                   T* Parena, int* d_flags, bool tensor_cores, cudaStream_t st) {
+                   T* Parena, int* d_flags, bool tensor_cores, cudaStream_t st, const int* d_kexp,
+                   int kstride) {
   const int pmax = h_fronts[0].p;
   // 2. Linv = L^{-1}: the diagonal blocks are inverted already; merge
   //    neighbouring inverted blocks pairwise up a binary tree of widths
@@ -809,8 +832,10 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
         const int64_t boff = (i0 + s) + (int64_t)i0 * ld;
         const int64_t aoff = i0 + (int64_t)i0 * ld;
         const int64_t coff = (i0 + s) + (int64_t)(i0 + s) * ld;
-        tops.push_back(GemmOp{h.K + boff, h.P + aoff, scr, rs, s, s, ld, ld, rs, 0, 0, 1.f, 0.f, 0, KZ_B_LOW});
-        rops.push_back(GemmOp{h.P + coff, scr, h.P + boff, rs, s, rs, ld, rs, ld, 0, 0, -1.f, 0.f, 0, KZ_A_LOW});
+        tops.push_back(GemmOp{h.K + boff, h.P + aoff, scr, rs, s, s, ld, ld, rs, 0, 0, 1.f, 0.f, 0, KZ_B_LOW,
+                              KB_NONE, 0});
+        rops.push_back(GemmOp{h.P + coff, scr, h.P + boff, rs, s, rs, ld, rs, ld, 0, 0, -1.f, 0.f, 0, KZ_A_LOW,
+                              KB_UP, (int64_t)f * kstride + i0 + s});
         scr += (int64_t)rs * s;
       }
     }
@@ -831,7 +856,7 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
         }
       }
       gemm_fma_or_f64tc<T>(dop, hop, (int)cnt, Ab, Bb, Cb, d_flags, tensor_cores, st, "trtri_merge",
-                           "trtri_merge_f64tc");
+                           "trtri_merge_f64tc", d_kexp);
     };
     gemm(d_ops, tops.data(), Karena, Parena, d_scr);
     gemm(d_ops + cnt, rops.data(), Parena, d_scr, Parena);
@@ -847,7 +872,8 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
     const int nb = h.n - h.p;
     if (nb <= 0 || h.p <= 0) continue;
     const int ld = h.ld;
-    GemmOp x{h.K + h.p, h.P, h.P + h.p, nb, h.p, h.p, ld, ld, ld, 0, 1, 1.f, 0.f, 0, KZ_B_UP};
+    GemmOp x{h.K + h.p, h.P, h.P + h.p, nb, h.p, h.p, ld, ld, ld, 0, 1, 1.f, 0.f, 0, KZ_B_UP,
+             KB_DOWN, (int64_t)f * kstride};
     GemmOp s{h.P + h.p, h.P + h.p, h.K + h.p + (int64_t)h.p * ld, nb, nb, h.p, ld, ld, ld, 0, 1,
              -1.f, 1.f, 1, 0};
     xo.push_back(x);
@@ -869,12 +895,20 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
         }
       }
       gemm_fma_or_f64tc<T>(dop, hop, (int)cnt, Ab, Bb, Cb, d_flags, tensor_cores, st, "gemm_batched",
-                           "gemm_f64tc");
+                           "gemm_f64tc", d_kexp);
     };
     gemm(d_ops, xo.data(), Karena, Parena, Parena);
     gemm(d_ops + cnt, so.data(), Parena, Parena, Karena);
     HIF_CUDA_TRY(cudaFreeAsync(d_ops, st));
   }
+}
+
+void diag_exponents(const DFront* d_fronts, int nfront, const double* Karena, int* d_kexp, int stride,
+                    cudaStream_t st) {
+  if (nfront == 0) return;
+  ProfScope ps("diag_exponents", st);
+  k_diag_exponents<<<nfront, 128, 0, st>>>(d_fronts, Karena, d_kexp, stride);
+  HIF_CHECK_LAUNCH();
 }
 
 template <typename T>

@@ -14,17 +14,19 @@ constexpr int TILE = 64;    // output tile of the trailing update / batched GEMM
 // in double when the FP32 one breaks down): a front whose leading-block
 // Cholesky meets a pivot d_j with A_jj / d_j > growth (or d_j not positive)
 // is refactored entirely in FP64; growth = 0 turns this off (such a pivot
-// then fails the factorization with HIF_ERR_NOT_SPD).  *retried counts them.
+// then fails the factorization with HIF_ERR_NOT_SPD).  *retried counts them;
+// tensor_cores: the retry's products may be slices.
 struct RetryOpts {
   double growth;
   int64_t* retried;
+  bool tensor_cores;
 };
 
 // Partial Cholesky of a batch of fronts (§2.2 and §2.3: A_II = L L^T,
 // X = L^{-1} A_IN, A_NN -= X^T X).  Fronts must be sorted by p, largest first.
 // On return: trailing blocks of K hold the Schur complements, P holds
 // [Linv; X^T] (Linv = L^{-1}, lower triangular) for each front.  With
-// tensor_cores (FP32 only) the deep products run on gemm_tc.  With retry
+// tensor_cores the deep products run on gemm_tc (FP64: gemm_f64tc).  With retry
 // (FP32 only) the host waits once after the leading blocks are factored to
 // read the per-front flags.
 template <typename T>
@@ -40,10 +42,16 @@ void gemm_tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const float* Ab
              const char* name = "gemm_tc");
 
 // The same with an FP64 result of FP64 or FP32 operands: 8-bit slices on the
-// BF16 tensor cores, exact sums, one rounding per entry (f64tc.cu).
+// BF16 tensor cores, exact sums, one rounding per entry (f64tc.cu).  d_kexp: the
+// exponents that KB_DOWN and KB_UP products name.
 template <typename S>
 void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Abase, const S* Bbase,
-                double* Cbase, int* d_flags, cudaStream_t st, const char* name);
+                double* Cbase, int* d_flags, cudaStream_t st, const char* name,
+                const int* d_kexp = nullptr);
+// The exponents of the square roots of the fronts' diagonals, front f's from
+// f * stride on (0 where a diagonal entry is not positive and finite).
+void diag_exponents(const DFront* d_fronts, int nfront, const double* Karena, int* d_kexp, int stride,
+                    cudaStream_t st);
 
 // Autotuning of gemm_tc's tile shape: time the variants on the product
 // shapes recorded during a tuning factorization (tune.h).
@@ -60,10 +68,10 @@ bool f64tc_worth(const GemmOp* h_ops, int nops);
 template <typename T>
 void gemm_fma_or_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const T* Abase,
                        const T* Bbase, T* Cbase, int* d_flags, bool tensor_cores, cudaStream_t st,
-                       const char* name, const char* name_tc) {
+                       const char* name, const char* name_tc, const int* d_kexp = nullptr) {
   if constexpr (sizeof(T) == 8) {
     if (tensor_cores && f64tc_worth(h_ops, nops)) {
-      gemm_f64tc<double>(d_ops, h_ops, nops, Abase, Bbase, Cbase, d_flags, st, name_tc);
+      gemm_f64tc<double>(d_ops, h_ops, nops, Abase, Bbase, Cbase, d_flags, st, name_tc, d_kexp);
       return;
     }
   }

@@ -8,25 +8,33 @@
 // slices (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
 // Algorithms 59, 2012):
 //
-//   x = 2^(s - 62) X,  X = sum_{i < 8} a_i 256^(7 - i),  |a_i| <= 128,
+//   x = 2^(s - 63) X,  X = sum_{i < 8} a_i 256^(7 - i),  |a_i| <= 128,
 //
-// with s per row of op(A) and per column of op(B) such that |x| < 2^s: X is x in
-// fixed point, 62 bits below the largest entry of its row.  Before that, k is
-// balanced: column k of op(A) is scaled by 2^t_k and row k of op(B) by 2^-t_k, with
-// t_k half the difference of their largest exponents, so that neither hides the
-// other's entries (A_NI = D^ A D and L^-T = D^-1 L^ have opposite scales in k, as
-// have the factors of every product with an inverse or an interpolation matrix;
-// coefficients over eight decades lost two decimal digits without it).  The
-// product is
-// sum_t 256^(14 - t) D_t, D_t = sum_{i + j = t} sum_k a_i b_j; the 36 products
-// with t < 8 are formed (the others are below 2^-62 of row maximum times column
-// maximum) in eight FP32 accumulators.  |D_t| <= 8 * 128 * 2^14 = 2^24 over 128 k,
-// which FP32 holds exactly; then they are added to 128-bit integers (two 64-bit
-// halves per entry), and each entry is rounded to double once at the end.  An
-// FMA loop rounds at every k; this sum is exact up to the 2^-62 of the split.
+// with s per row of op(A) and per column of op(B) such that |x| < (1 - 2^-7) 2^s (room
+// for the carry into a_0): X is x in fixed point, 62 to 63 bits below the largest entry
+// of its row.  Before that, k is balanced: column k of op(A) is scaled by 2^t_k and row
+// k of op(B) by 2^-t_k, so that an operand's own scale in k hides none of its entries.
+// Write a front as D A^ D with D^2 its diagonal.  Then L = D L^ has no scale in its
+// columns; A_NI = D A^ D and L^-T = D^-1 L^^-T have opposite ones in k, as have C^-1
+// and T in the second product of a triangular merge and A_FF and T in the skeleton
+// products.  So t_k is the exponent of D_k there (KB_DOWN, KB_UP; diag_exponents) and 0
+// in the merges' first product (KB_NONE); only the products of the row reduction take
+// half the difference of the operands' largest exponents (KB_MAX).  That was the rule
+// of all products at first, but the largest entry of column k of A_NI says which DOFs
+// k is coupled to, not how large k is: coefficients over six decades in blocks, layers
+// or a ramp lost 30 to 200 times the FMA form's error (x of O(1) everywhere, 2-norm).
 //
-// Four launches per batch: k_f64_kmax finds t_k (not for A A^T), k_f64_exps s per
-// row, k_f64_slice writes the slices in the layout the tensor core reads (64 rows
+// The product is sum_t 256^(14 - t) D_t, D_t = sum_{i + j = t} sum_k a_i b_j; the 36
+// products with t < 8 are formed in eight FP32 accumulators.  (Left out are seven
+// products a_i b_j per k with t = 8, and smaller ones: at most 2^-61 of 2^s 2^s' per k,
+// 2^-64 in the mean square.  With X one bit lower in a_0 they were four times as large,
+// and holes of 10^3.5 doubled the FMA form's largest error.)  |D_t| <= 8 * 128 * 2^14 =
+// 2^24 over 128 k, which FP32 holds exactly; then they are added to 128-bit integers
+// (two 64-bit halves per entry), and each entry is rounded to double once at the end.
+// An FMA loop rounds at every k; this sum is exact up to the split.
+//
+// Three launches per batch (four with KB_MAX, whose t_k k_f64_kmax finds): k_f64_exps
+// finds s per row, k_f64_slice writes the slices in the layout the tensor core reads (64 rows
 // x 16 k per block, all eight slices together: 16 KB), k_gemm_f64tc copies blocks
 // to shared memory with bulk copies and multiplies.  An operand used on both
 // sides (A A^T) is split once; if all products of a batch are such and have at most
@@ -36,9 +44,8 @@
 // Measured (all launches, FMA form in brackets): one 64^3 product 40 (66) us, 512
 // of them 125 (270) us, one 256^3 55 (280) us, one 1024^3 0.11 (2.1) ms, one 2048^3
 // 0.65 (14.5) ms = 26 TFLOP/s.  Error against quad precision, entries over 2 to
-// 12 decades: 5e-17 to 7e-17 in norm (3e-16 to 1.5e-15).  Solve error of an exact
-// factorization, coefficients over 2, 4, 6, 8 decades: 1.0, 1.0, 0.9, 1.5 to 2 times
-// the FMA form's.
+// 12 decades: 5e-17 to 7e-17 in norm (3e-16 to 1.5e-15).  For the solve error of a
+// factorization see SLICE_SPAN in hif.cu.
 //
 // k_gemm_f64tc: one 128 x 64 tile per CTA; the eight accumulators fill the 512
 // columns of tensor memory, four stages of 48 KB the shared memory.  Per 16 k one
@@ -68,7 +75,7 @@ namespace {
 
 constexpr int NSL = 8;             // slices per operand, and accumulators
 // slices multiplied: all for FP64 operands.  FP32 operands (24 bits an entry) leave out
-// the last slice of each and the products with t = 7: their rows are then rounded 54
+// the last slice of each and the products with t = 7: their rows are then rounded 55
 // bits below the largest entry, which is as far as an FP64 FMA loop carries the sum.
 // (28 instead of 36 products; Gram matrices of a 128^3 FP32 factorization 60.8 -> 56.0
 // ms, of 96^3 13.4 -> 12.4 ms.)
@@ -93,11 +100,12 @@ constexpr size_t WORK_LIMIT = (size_t)1 << 30;   // slices held at once, if seve
 struct SliceBlk {
   int64_t src;
   int64_t dst;       // index of its first 16 KB block in the work space
-  int64_t kx;        // index of the largest magnitudes of its product's columns of
-                     // op(A), then rows of op(B) (k each); -1: not balanced
+  int64_t kx;        // KB_MAX: index of the largest magnitudes of its product's
+                     // columns of op(A), then rows of op(B) (k each); KB_DOWN and
+                     // KB_UP: index of its exponents (GemmOp::ks)
   int ld, rows, k;
   int kcont, isB;
-  int pad;
+  int kbal;
 };
 
 struct Tile {
@@ -112,7 +120,7 @@ __global__ void __launch_bounds__(256) k_f64_kmax(const SliceBlk* __restrict__ b
                                                   const S* __restrict__ Ab,
                                                   const S* __restrict__ Bb, int* kx) {
   const SliceBlk b = blks[blockIdx.x];
-  if (b.kx < 0) return;
+  if (b.kbal != KB_MAX) return;
   const S* X = (b.isB ? Bb : Ab) + b.src;
   int* out = kx + b.kx + (b.isB ? b.k : 0);
   const int k0 = (int)((int64_t)b.k * blockIdx.y / gridDim.y);
@@ -139,8 +147,13 @@ __global__ void __launch_bounds__(256) k_f64_kmax(const SliceBlk* __restrict__ b
 }
 
 // The exponent added to this operand's entries at k.
-__device__ __forceinline__ int balance(const SliceBlk& b, const int* kx, int k) {
-  if (b.kx < 0) return 0;
+__device__ __forceinline__ int balance(const SliceBlk& b, const int* kx,
+                                       const int* __restrict__ kexp, int k) {
+  if (b.kbal == KB_NONE) return 0;
+  if (b.kbal != KB_MAX) {
+    const int e = kexp[b.kx + k];
+    return (b.kbal == KB_UP) == (b.isB == 0) ? e : -e;
+  }
   const int ea = kx[b.kx + k] >> 20, eb = kx[b.kx + b.k + k] >> 20;
   if (ea == 0 || eb == 0 || ea == 0x7ff || eb == 0x7ff) return 0;
   const int t = (eb - ea) >> 1;
@@ -149,19 +162,21 @@ __device__ __forceinline__ int balance(const SliceBlk& b, const int* kx, int k) 
 
 // Largest balanced exponent of each row, biased by ROW_BIAS on top of the
 // double's own bias so that a zero row is 0 (exps zeroed before; gridDim.y CTAs
-// share the block's k).
+// share the block's k).  Entries within 2^-6 of the next power of two count as that.
 constexpr int ROW_BIAS = 4096;
+constexpr int ROUND_UP = 1 << 14;   // 2^-6 of the upper word's mantissa
 __device__ __forceinline__ int entry_exp(double x, int t) {
   const int h = __double2hiint(x) & 0x7fffffff, e = h >> 20;
   if (e == 0x7ff) return NOT_FINITE;
   if (h == 0 && __double2loint(x) == 0) return 0;
-  return max(e, 1) + t + ROW_BIAS;
+  return max((h + ROUND_UP) >> 20, 1) + t + ROW_BIAS;
 }
 template <typename S>
 __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ blks,
                                                   const S* __restrict__ Ab,
                                                   const S* __restrict__ Bb,
-                                                  const int* __restrict__ kx, int* exps) {
+                                                  const int* __restrict__ kx,
+                                                  const int* __restrict__ kexp, int* exps) {
   const SliceBlk b = blks[blockIdx.x];
   const S* X = (b.isB ? Bb : Ab) + b.src;
   const int k0 = (int)((int64_t)b.k * blockIdx.y / gridDim.y);
@@ -174,7 +189,7 @@ __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ b
       int m = 0;
 #pragma unroll 4
       for (int k = k0 + lane; k < k1; k += 32)
-        m = max(m, entry_exp(X[(int64_t)r * b.ld + k], balance(b, kx, k)));
+        m = max(m, entry_exp(X[(int64_t)r * b.ld + k], balance(b, kx, kexp, k)));
       m = __reduce_max_sync(0xffffffffu, m);
       if (lane == 0) atomicMax(&out[r], m);
     }
@@ -184,23 +199,23 @@ __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ b
     int m = 0;
 #pragma unroll 8
     for (int k = k0 + threadIdx.x / BR; k < k1; k += 256 / BR)
-      m = max(m, entry_exp(X[r + (int64_t)k * b.ld], balance(b, kx, k)));
+      m = max(m, entry_exp(X[r + (int64_t)k * b.ld], balance(b, kx, kexp, k)));
     atomicMax(&out[r], m);
   }
 }
 
-// s of a row, as a biased exponent: |x| < 2^(s - 1023) for all its entries
+// s of a row, as a biased exponent: |x| < (1 - 2^-7) 2^(s - 1023) for all its entries
 __device__ __forceinline__ int row_exp(int v) {
   return v == NOT_FINITE ? NOT_FINITE : v == 0 ? 1 : v - ROW_BIAS + 1;
 }
 
-// x in fixed point, 62 bits below 2^s (s: biased exponent + 1 of the row)
-__device__ __forceinline__ int64_t fixed62(double x, int s) {
+// x in fixed point, 63 bits below 2^s (s: row_exp)
+__device__ __forceinline__ int64_t fixed63(double x, int s) {
   const uint64_t u = (uint64_t)__double_as_longlong(x);
   const int e = (int)(u >> 52) & 0x7ff;
   uint64_t m = u & 0xfffffffffffffull;
   if (e) m |= 1ull << 52;
-  const int sh = (e ? e : 1) - s + 10;   // at most 9
+  const int sh = (e ? e : 1) - s + 11;   // at most 10
   uint64_t v;
   if (sh >= 0) v = m << sh;
   else if (sh > -55) v = (m + (1ull << (-sh - 1))) >> -sh;
@@ -217,7 +232,7 @@ __device__ __forceinline__ void write_slices(const double (&x)[8], int s, const 
   uint32_t lo[8], hi[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const uint64_t y = (uint64_t)(s == NOT_FINITE ? 0 : fixed62(x[j], s - t[j])) + 0x8080808080808080ull;
+    const uint64_t y = (uint64_t)(s == NOT_FINITE ? 0 : fixed63(x[j], s - t[j])) + 0x8080808080808080ull;
     lo[j] = (uint32_t)y;
     hi[j] = (uint32_t)(y >> 32);
   }
@@ -243,6 +258,7 @@ __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ 
                                                    const S* __restrict__ Ab,
                                                    const S* __restrict__ Bb,
                                                    const int* __restrict__ kx,
+                                                   const int* __restrict__ kexp,
                                                    const int* __restrict__ exps, unsigned char* W) {
   const SliceBlk b = blks[blockIdx.x];
   const S* X = (b.isB ? Bb : Ab) + b.src;
@@ -257,7 +273,7 @@ __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ 
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int k = g * 8 + j;
-      t[j] = k < b.k ? balance(b, kx, k) : 0;
+      t[j] = k < b.k ? balance(b, kx, kexp, k) : 0;
       x[j] = (r < b.rows && k < b.k)
                  ? (double)X[b.kcont ? (int64_t)r * b.ld + k : r + (int64_t)k * b.ld]
                  : 0.0;
@@ -551,11 +567,11 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll 4
       for (int j = 0; j < nj; ++j) {
         const int eb = ebp[j];
-        // 2^(sA - 62) 2^(sB - 62) 256^7, the biased exponents' offset 2 * 1023 taken out
+        // 2^(sA - 63) 2^(sB - 63) 256^7, the biased exponents' offset 2 * 1023 taken out
         const double v = ea == NOT_FINITE || eb == NOT_FINITE
                              ? __longlong_as_double(0x7ff8000000000000ll)
                              : to_double(sum[(2 * j) * THREADS], sum[(2 * j + 1) * THREADS],
-                                         ea + eb - 2 * 1023 - 124 + 56);
+                                         ea + eb - 2 * 1023 - 126 + 56);
         C[(int64_t)j * o.ldc] = o.beta != 0.f ? fma(al, v, ngroup ? cst[j * THREADS] : C[(int64_t)j * o.ldc])
                                               : al * v;
       }
@@ -578,7 +594,7 @@ bool f64tc_worth(const GemmOp* h_ops, int nops) {
 
 template <typename S>
 void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Abase, const S* Bbase,
-                double* Cbase, int* d_flags, cudaStream_t st, const char* name) {
+                double* Cbase, int* d_flags, cudaStream_t st, const char* name, const int* d_kexp) {
   static const bool attr = [] {   // initialised once, also under concurrent factorizations
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_gemm_f64tc<slices_used<S>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       NST * STAGE));
@@ -592,6 +608,7 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
     int64_t nblk = 0, nkx = 0;
     double fl = 0;
     int f = f0, kmax = 0;
+    bool all_same = true;   // every product of the batch is A A^T
     for (; f < nops; ++f) {
       const GemmOp& o = h_ops[f];
       const int nk = ceil_div(o.k, KC);
@@ -599,18 +616,20 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
       const int na = ceil_div(o.m, BR), nb = ceil_div(o.n, BR);
       const int64_t need = (int64_t)(same ? std::max(na, nb) : na + nb) * nk;
       if (f > f0 && (size_t)(nblk + need) * BLK > WORK_LIMIT) break;
+      const int kbal = same ? KB_NONE : o.kbal;
+      all_same = all_same && same;
       auto add = [&](int64_t src, int rows, int ld, bool kcont, bool isB) {
         const int first = (int)blks.size();
         for (int r0 = 0; r0 < rows; r0 += BR) {
-          blks.push_back(SliceBlk{src + (kcont ? (int64_t)r0 * ld : r0), nblk, same ? -1 : nkx, ld,
-                                  std::min(BR, rows - r0), o.k, kcont ? 1 : 0, isB ? 1 : 0, 0});
+          blks.push_back(SliceBlk{src + (kcont ? (int64_t)r0 * ld : r0), nblk, kbal == KB_MAX ? nkx : o.ks, ld,
+                                  std::min(BR, rows - r0), o.k, kcont ? 1 : 0, isB ? 1 : 0, kbal});
           nblk += nk;
         }
         return first;
       };
       const int fa = add(o.A, same ? std::max(o.m, o.n) : o.m, o.lda, o.transA != 0, false);
       const int fb = same ? fa : add(o.B, o.n, o.ldb, o.transB == 0, true);
-      if (!same) nkx += 2 * (int64_t)o.k;
+      if (kbal == KB_MAX) nkx += 2 * (int64_t)o.k;
       const int tm = ceil_div(o.m, TM), tn = ceil_div(o.n, TN);
       for (int t = 0; t < tm * tn; ++t) {
         const int q = gemm_tile(o, t, tm * tn);
@@ -637,7 +656,7 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
     const SliceBlk* d_blks = reinterpret_cast<const SliceBlk*>(d_tab);
     const Tile* d_tiles = reinterpret_cast<const Tile*>(d_tab + bb);
     const int gy = std::max(1, std::min({ceil_div(kmax, 64), 64, ceil_div(4096, (int64_t)blks.size())}));
-    const bool rows = nkx == 0 && kmax <= ROW_K;   // every product of the batch is A A^T
+    const bool rows = all_same && kmax <= ROW_K;
     if (rows) {
       k_f64_slice_rows<S><<<(unsigned)blks.size(), 256, 0, st>>>(d_blks, Abase, d_exps, W);
       HIF_CHECK_LAUNCH();
@@ -648,9 +667,9 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
         k_f64_kmax<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx);
         HIF_CHECK_LAUNCH();
       }
-      k_f64_exps<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps);
+      k_f64_exps<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_kexp, d_exps);
       HIF_CHECK_LAUNCH();
-      k_f64_slice<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_exps, W);
+      k_f64_slice<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_kexp, d_exps, W);
       HIF_CHECK_LAUNCH();
     }
     k_gemm_f64tc<slices_used<S>()><<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(
@@ -664,8 +683,8 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
 }
 
 template void gemm_f64tc<double>(const GemmOp*, const GemmOp*, int, const double*, const double*,
-                                 double*, int*, cudaStream_t, const char*);
+                                 double*, int*, cudaStream_t, const char*, const int*);
 template void gemm_f64tc<float>(const GemmOp*, const GemmOp*, int, const float*, const float*,
-                                double*, int*, cudaStream_t, const char*);
+                                double*, int*, cudaStream_t, const char*, const int*);
 
 }  // namespace hif

@@ -53,6 +53,25 @@ __global__ void k_stencil(const double* __restrict__ a, const double* __restrict
   diag[j] = s * ih2 + bj;
 }
 
+// Positive doubles are ordered like their bits.
+__global__ void __launch_bounds__(256) k_value_range(const double* __restrict__ a, int64_t cnt,
+                                                     unsigned long long* range) {
+  unsigned long long lo = ~0ull, hi = 0;
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * 256) {
+    const unsigned long long v = (unsigned long long)__double_as_longlong(a[i]);
+    lo = min(lo, v);
+    hi = max(hi, v);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (threadIdx.x % 32 == 0) {
+    atomicMin(&range[0], lo);
+    atomicMax(&range[1], hi);
+  }
+}
+
 // The cell (coordinate along one dimension) that owns point x at cell side
 // s: a separator plane belongs to the cell below it (wrapping to the last
 // cell on the periodic grid, where plane 0 is a separator too).
@@ -454,6 +473,12 @@ void stencil_coefficients(const double* a, const double* b, double b_const, int 
   const int64_t N = (int64_t)n * n * n;
   ProfScope ps("stencil_coefficients", st, 0.0, 8.0 * N * (b ? 6.0 : 5.0));
   k_stencil<<<ceil_div(N, 256), 256, 0, st>>>(a, b, b_const, n, periodic, cpl, diag, d_bad);
+  HIF_CHECK_LAUNCH();
+}
+
+void value_range(const double* a, int64_t cnt, unsigned long long* range, cudaStream_t st) {
+  ProfScope ps("stencil_coefficients", st, 0.0, 8.0 * cnt);
+  k_value_range<<<(int)std::min<int64_t>(304, (cnt + 255) / 256), 256, 0, st>>>(a, cnt, range);
   HIF_CHECK_LAUNCH();
 }
 

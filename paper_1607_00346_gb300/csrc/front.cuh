@@ -20,6 +20,10 @@ struct CellDesc {
 void stencil_coefficients(const double* a, const double* b, double b_const, int n, int periodic,
                           double* cpl, double* diag, int* d_bad, cudaStream_t st);
 
+// range[0], range[1]: bits of the least and the largest of cnt positive doubles
+// (range[0] set to all ones and range[1] to zero before).
+void value_range(const double* a, int64_t cnt, unsigned long long* range, cudaStream_t st);
+
 // Level-0 frontal matrices from the stencil (each coupling counted in exactly
 // one cell: the lowest cell whose closure holds both points).
 template <typename T>

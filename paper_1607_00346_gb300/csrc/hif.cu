@@ -469,6 +469,18 @@ class Fork {
 
 // ---- the factorization ---------------------------------------------------------
 
+// FP64 products are split into slices (gemm_f64tc) up to this ratio of the operator's
+// largest diagonal entry to its least, and stay on the FMA units beyond it.  A slice
+// holds an entry below the largest of its row, so what soft and stiff DOFs, scaled by
+// the diagonal, couple by (the inverse root of the ratio) loses as many of 62 bits,
+// where FMA keeps 53 of every entry.  Error of an exact factorization's solution against
+// extended precision, as multiples of that of the FMA form with the panels solved by
+// substitution, x of O(1) everywhere (ten coefficient fields: boards, layers, holes, a
+// cube, a ramp, smooth, point by point; 20^3 to 32^3; 2-norm, max-norm): contrast 10^3
+// 0.4 to 0.8 and 0.5 to 0.8; 10^4 0.4 to 0.8 and 0.4 to 0.9; 10^6 0.5 to 1.5 and 0.4 to
+// 5.6; 10^8 0.3 to 8.5 and 0.4 to 23.
+constexpr double SLICE_SPAN = 1e4;
+
 template <typename T>
 class Builder {
  public:
@@ -555,6 +567,7 @@ class Builder {
   Factor<T>& F_;
   cudaStream_t st_;
   RetryOpts retry_{};
+  bool tc_ = false;   // products on the tensor cores
   Symbolic sym_;
   DevBuf flags_;
   int level_ = 0;
@@ -600,17 +613,28 @@ void Builder<T>::run(const double* a_dev, const double* b_dev, double b_const) {
   }
   F_.cpl.alloc(sizeof(double) * 3 * N, &F_.mem);
   F_.diag.alloc(sizeof(double) * N, &F_.mem);
-  DevBuf bad;
-  bad.alloc_async(sizeof(int), &F_.mem, st_);
-  HIF_CUDA_TRY(cudaMemsetAsync(bad.as<int>(), 0, sizeof(int), st_));
+  // one word that an invalid coefficient sets, and the range of the diagonal
+  unsigned long long h[3] = {0, 0, 0};
+  DevBuf check;
+  check.alloc_async(sizeof(h), &F_.mem, st_);
+  unsigned long long* range = check.as<unsigned long long>() + 1;
+  HIF_CUDA_TRY(cudaMemsetAsync(check.as<void>(), 0, sizeof(h), st_));
+  HIF_CUDA_TRY(cudaMemsetAsync(range, 0xff, sizeof(h[1]), st_));
   stencil_coefficients(a_dev, b_dev, b_const, n, F_.bc, F_.cpl.template as<double>(), F_.diag.template as<double>(),
-                       bad.as<int>(), st_);
-  int hbad = 0;
-  HIF_CUDA_TRY(cudaMemcpyAsync(&hbad, bad.as<int>(), sizeof(int), cudaMemcpyDeviceToHost, st_));
+                       check.as<int>(), st_);
+  // FP64 products, of an FP64 factor or of a retried front
+  const bool f64_tc = F_.opt.tensor_cores && (sizeof(T) == 8 || retry_.growth > 0.0);
+  if (f64_tc) value_range(F_.diag.template as<double>(), N, range, st_);
+  HIF_CUDA_TRY(cudaMemcpyAsync(h, check.as<void>(), sizeof(h), cudaMemcpyDeviceToHost, st_));
   HIF_CUDA_TRY(cudaStreamSynchronize(st_));
-  if (hbad)
+  if (h[0])
     throw Error{HIF_ERR_INVALID_ARG, F_.bc ? "a must be finite and > 0, b finite and > 0 (periodic grid)"
                                            : "a must be finite and > 0, b finite and >= 0"};
+  double least = 0.0, largest = 0.0;
+  std::memcpy(&least, &h[1], sizeof(double));
+  std::memcpy(&largest, &h[2], sizeof(double));
+  retry_.tensor_cores = f64_tc && largest <= SLICE_SPAN * least;
+  tc_ = F_.opt.tensor_cores && (sizeof(T) == 4 || retry_.tensor_cores);
   flags_.alloc_async(sizeof(int) * FLAG_COUNT, &F_.mem, st_);
   HIF_CUDA_TRY(cudaMemsetAsync(flags_.as<int>(), 0xff, sizeof(int) * FLAG_COUNT, st_));
 
@@ -804,7 +828,7 @@ void Builder<T>::cell_step(std::shared_ptr<const CellPlan> cpp, DevBuf& Kar, Dev
   DevBuf fr_d;
   upload_async(fr_d, fr, &F_.mem, st_);
   partial_cholesky<T>(fr_d.as<DFront>(), fr.data(), (int)fr.size(), Kar.as<T>(), s.panels.as<T>(),
-                      flags_.as<int>(), F_.opt.tensor_cores != 0, st_, &retry_);
+                      flags_.as<int>(), tc_, st_, &retry_);
   tr_.mark(level_, " cells: partial Cholesky queued");
   // apply stage: gather the whole frontal list of every cell (already on
   // the device); the rest is built on a worker thread
@@ -1003,10 +1027,10 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
       nFmax = std::max(nFmax, sd[sel[1][i]].nF);
     }
     Rbuf.alloc_async(sizeof(T) * rtot, &F_.mem, st_);
-    gram = std::is_same<T, float>::value && F_.opt.tensor_cores && gram_id_fits(nFmax);
+    gram = std::is_same<T, float>::value && tc_ && gram_id_fits(nFmax);
     if (!gram)
       reduce_rows_qr<T>(sd.data(), sel[1], G.as<T>(), Rbuf.as<T>(), roff, flags_.as<int>(),
-                        F_.opt.tensor_cores != 0, st_);
+                        tc_, st_);
     for (size_t i = 0; i < sel[1].size(); ++i) {
       SkelDesc& d = sd[sel[1][i]];
       d.idoff = roff[i];
@@ -1151,27 +1175,42 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
   skel_permute<T>(sda_d.as<SkelDesc>(), sda.data(), (int)sda.size(), perm_d.as<int32_t>(),
                   G.as<T>(), Z.as<T>(), st_);
   // B_{F^F~} = A_{F^F~} - A_{F^F^} T ;  B_{F~F~} = A_{F~F~} - A_{F~F^} T - T^T B_{F^F~}
+  // (FP64 on the tensor cores: k is balanced by the scales of the skeleton DOFs, in
+  // A_FF as they are, in T inverse)
+  const bool zscale = sizeof(T) == 8 && tc_;
+  DevBuf zexp, zfr_d;
+  int zstride = 0;
+  if constexpr (sizeof(T) == 8) {
+    if (zscale) {
+      for (const DFront& d : fr) zstride = std::max(zstride, d.n);
+      upload_async(zfr_d, fr, &F_.mem, st_);
+      zexp.alloc_async(sizeof(int) * fr.size() * zstride, &F_.mem, st_);
+      diag_exponents(zfr_d.as<DFront>(), (int)fr.size(), Z.as<T>(), zexp.as<int>(), zstride, st_);
+    }
+  }
   std::vector<GemmOp> g1, g2, g3;
-  for (const SkelDesc& d : sda) {
+  for (size_t i = 0; i < sda.size(); ++i) {
+    const SkelDesc& d = sda[i];
     const int k = d.k, p = d.nF - k, nF = d.nF;
     if (k == 0) continue;
-    g1.push_back(GemmOp{d.Z + p + (int64_t)p * nF, d.Tm, d.Z + p, k, p, k, nF, k, nF, 0, 0, -1.f, 1.f, 0, 0});
-    g2.push_back(GemmOp{d.Z + (int64_t)p * nF, d.Tm, d.Z, p, p, k, nF, k, nF, 0, 0, -1.f, 1.f, 0, 0});
-    g3.push_back(GemmOp{d.Tm, d.Z + p, d.Z, p, p, k, k, nF, nF, 1, 0, -1.f, 1.f, 0, 0});
+    const int64_t ks = (int64_t)i * zstride + p;
+    g1.push_back(GemmOp{d.Z + p + (int64_t)p * nF, d.Tm, d.Z + p, k, p, k, nF, k, nF, 0, 0, -1.f, 1.f, 0, 0, KB_DOWN, ks});
+    g2.push_back(GemmOp{d.Z + (int64_t)p * nF, d.Tm, d.Z, p, p, k, nF, k, nF, 0, 0, -1.f, 1.f, 0, 0, KB_DOWN, ks});
+    g3.push_back(GemmOp{d.Tm, d.Z + p, d.Z, p, p, k, k, nF, nF, 1, 0, -1.f, 1.f, 0, 0, KB_UP, ks});
   }
   DevBuf g1d, g2d, g3d;
   upload_async(g1d, g1, &F_.mem, st_);
   upload_async(g2d, g2, &F_.mem, st_);
   upload_async(g3d, g3, &F_.mem, st_);
   gemm_fma_or_f64tc<T>(g1d.as<GemmOp>(), g1.data(), (int)g1.size(), Z.as<T>(), tm.as<T>(), Z.as<T>(),
-                       flags_.as<int>(), F_.opt.tensor_cores != 0, st_, "skel_z_products",
-                       "skel_z_products_f64tc");
+                       flags_.as<int>(), tc_, st_, "skel_z_products",
+                       "skel_z_products_f64tc", zexp.as<int>());
   gemm_fma_or_f64tc<T>(g2d.as<GemmOp>(), g2.data(), (int)g2.size(), Z.as<T>(), tm.as<T>(), Z.as<T>(),
-                       flags_.as<int>(), F_.opt.tensor_cores != 0, st_, "skel_z_products",
-                       "skel_z_products_f64tc");
+                       flags_.as<int>(), tc_, st_, "skel_z_products",
+                       "skel_z_products_f64tc", zexp.as<int>());
   gemm_fma_or_f64tc<T>(g3d.as<GemmOp>(), g3.data(), (int)g3.size(), tm.as<T>(), Z.as<T>(), Z.as<T>(),
-                       flags_.as<int>(), F_.opt.tensor_cores != 0, st_, "skel_z_products",
-                       "skel_z_products_f64tc");
+                       flags_.as<int>(), tc_, st_, "skel_z_products",
+                       "skel_z_products_f64tc", zexp.as<int>());
   // partial Cholesky of Z: eliminate the redundant DOFs
   Stage s;
   s.kind = 1;
@@ -1183,7 +1222,7 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
   DevBuf fr_d;
   upload_async(fr_d, frs, &F_.mem, st_);
   partial_cholesky<T>(fr_d.as<DFront>(), frs.data(), (int)frs.size(), Z.as<T>(), s.panels.as<T>(),
-                      flags_.as<int>(), F_.opt.tensor_cores != 0, st_, &retry_);
+                      flags_.as<int>(), tc_, st_, &retry_);
   tr_.mark(level_, " Z products + Cholesky queued");
   skel_writeback<T>(sda_d.as<SkelDesc>(), sda.data(), (int)sda.size(), ncp, rowpos,
                     perm_d.as<int32_t>(), cdesc_d.as<CellDesc>(), Z.as<T>(), Kar.as<T>(), st_);
