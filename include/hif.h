@@ -255,9 +255,11 @@ hif_status hif_query_active(hif_handle h, int level, int32_t* out, int64_t cap,
 /*
  * hif_predict_bytes -- device bytes hif_factor is expected to need at its
  * peak for this grid and options (used for admission control): an upper
- * estimate fitted to measured peaks (within ~25-60% above them at eps 1e-6
- * to 1e-4 for n = 64 ... 256); it depends on n, the precision and eps, not
- * on the coefficients.  0 for an invalid grid.
+ * estimate fitted to measured peaks, work space included (2% to 50% above
+ * them for n = 64 ... 256, m = 3 to 5, coefficients over two decades, eps 0
+ * to 1e-3; more above smaller or smoother problems and without tensor cores);
+ * it depends on n, m, the boundary, the precision and eps, not on the
+ * coefficients.  0 for an invalid grid.
  */
 size_t hif_predict_bytes(const hif_grid* grid, const hif_options* opt);
 

@@ -4,7 +4,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
+#include <utility>
 
 #include "../../include/hif.h"
 
@@ -73,6 +75,100 @@ class ProfSuspend {
     ++::hif::launch_counter();             \
     HIF_CUDA_TRY(cudaGetLastError());      \
   } while (0)
+
+// ---- device memory --------------------------------------------------------------
+
+// Device bytes of a factor and its factorization: now, and the most so far.
+struct MemStats {
+  size_t cur = 0, peak = 0;
+  void add(size_t bytes) {
+    cur += bytes;
+    peak = std::max(peak, cur);
+  }
+};
+
+// Where this thread's factorization counts its kernels' work space (null: nowhere).
+inline MemStats*& scratch_stats() {
+  static thread_local MemStats* ms = nullptr;
+  return ms;
+}
+class ScratchScope {
+ public:
+  explicit ScratchScope(MemStats* ms) : prev_(scratch_stats()) { scratch_stats() = ms; }
+  ~ScratchScope() { scratch_stats() = prev_; }
+  ScratchScope(const ScratchScope&) = delete;
+  ScratchScope& operator=(const ScratchScope&) = delete;
+
+ private:
+  MemStats* prev_;
+};
+
+class DevBuf {
+ public:
+  DevBuf() = default;
+  DevBuf(const DevBuf&) = delete;
+  DevBuf& operator=(const DevBuf&) = delete;
+  DevBuf(DevBuf&& o) noexcept { swap(o); }
+  DevBuf& operator=(DevBuf&& o) noexcept {
+    release();
+    swap(o);
+    return *this;
+  }
+  ~DevBuf() { release(); }
+  void alloc(size_t bytes, MemStats* ms) {
+    release();
+    ms_ = ms;
+    if (bytes == 0) return;
+    HIF_CUDA_TRY(cudaMalloc(&p_, bytes));
+    bytes_ = bytes;
+    if (ms_) ms_->add(bytes);
+  }
+  // Stream-ordered: allocated and later freed in order on `st` (no device
+  // synchronisation); for the temporaries of one factorization.
+  void alloc_async(size_t bytes, MemStats* ms, cudaStream_t st) {
+    release();
+    ms_ = ms;
+    if (bytes == 0) return;
+    HIF_CUDA_TRY(cudaMallocAsync(&p_, bytes, st));
+    st_ = st;
+    async_ = true;
+    bytes_ = bytes;
+    if (ms_) ms_->add(bytes);
+  }
+  // Work space of a kernel: alloc_async counted in scratch_stats().
+  template <typename U>
+  U* scratch(size_t count, cudaStream_t st) {
+    alloc_async(sizeof(U) * std::max<size_t>(1, count), scratch_stats(), st);
+    return as<U>();
+  }
+  void release() {
+    if (p_) {
+      if (async_) cudaFreeAsync(p_, st_);
+      else cudaFree(p_);
+      if (ms_) ms_->cur -= bytes_;
+    }
+    p_ = nullptr;
+    bytes_ = 0;
+    async_ = false;
+  }
+  template <typename U>
+  U* as() const { return static_cast<U*>(p_); }
+  size_t bytes() const { return bytes_; }
+
+ private:
+  void swap(DevBuf& o) {
+    std::swap(p_, o.p_);
+    std::swap(bytes_, o.bytes_);
+    std::swap(ms_, o.ms_);
+    std::swap(st_, o.st_);
+    std::swap(async_, o.async_);
+  }
+  void* p_ = nullptr;
+  size_t bytes_ = 0;
+  MemStats* ms_ = nullptr;
+  cudaStream_t st_ = nullptr;
+  bool async_ = false;
+};
 
 // ---- device-side error flags -------------------------------------------------
 // Kernels never trap.  A failed Cholesky pivot (not positive or not finite)

@@ -572,14 +572,11 @@ static void retry_fronts_fp64(const std::vector<int>& bad, const DFront* h_front
     pt += (int64_t)h.ld * h.p;
     mx = std::max<int64_t>(mx, (int64_t)h.ld * h.ld);
   }
-  double* Kd = nullptr;
-  double* Pd = nullptr;
-  RetryMap* d_maps = nullptr;
-  DFront* d_dl = nullptr;
-  HIF_CUDA_TRY(cudaMallocAsync(&Kd, sizeof(double) * kt, st));
-  HIF_CUDA_TRY(cudaMallocAsync(&Pd, sizeof(double) * std::max<int64_t>(1, pt), st));
-  HIF_CUDA_TRY(cudaMallocAsync(&d_maps, sizeof(RetryMap) * nb, st));
-  HIF_CUDA_TRY(cudaMallocAsync(&d_dl, sizeof(DFront) * nb, st));
+  DevBuf Kb, Pb, maps_b, dl_b;
+  double* Kd = Kb.scratch<double>(kt, st);
+  double* Pd = Pb.scratch<double>(pt, st);
+  RetryMap* d_maps = maps_b.scratch<RetryMap>(nb, st);
+  DFront* d_dl = dl_b.scratch<DFront>(nb, st);
   HIF_CUDA_TRY(cudaMemsetAsync(Pd, 0, sizeof(double) * std::max<int64_t>(1, pt), st));
   HIF_CUDA_TRY(cudaMemcpyAsync(d_maps, maps.data(), sizeof(RetryMap) * nb, cudaMemcpyHostToDevice, st));
   HIF_CUDA_TRY(cudaMemcpyAsync(d_dl, dl.data(), sizeof(DFront) * nb, cudaMemcpyHostToDevice, st));
@@ -597,10 +594,6 @@ static void retry_fronts_fp64(const std::vector<int>& bad, const DFront* h_front
     k_retry_writeback<<<dim3(gx, c), 256, 0, st>>>(d_maps + f0, Kd, Pd, Karena, Parena);
     HIF_CHECK_LAUNCH();
   }
-  HIF_CUDA_TRY(cudaFreeAsync(d_dl, st));
-  HIF_CUDA_TRY(cudaFreeAsync(d_maps, st));
-  HIF_CUDA_TRY(cudaFreeAsync(Pd, st));
-  HIF_CUDA_TRY(cudaFreeAsync(Kd, st));
 }
 
 template <typename T>
@@ -613,6 +606,7 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
   // original diagonal in the panel, one flag per front
   const bool growth_on = std::is_same<T, float>::value && retry && retry->growth > 0.0;
   int* d_fflag = nullptr;
+  DevBuf snap_b;
   T* snap = nullptr;
   int64_t* d_soff = nullptr;
   std::vector<int64_t> soff;
@@ -625,7 +619,7 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
       mx = std::max<int64_t>(mx, (int64_t)h_fronts[f].p * h_fronts[f].p);
     }
     HIF_CUDA_TRY(cudaMallocAsync(&d_fflag, sizeof(int) * nfront, st));
-    HIF_CUDA_TRY(cudaMallocAsync(&snap, sizeof(T) * std::max<int64_t>(1, tot), st));
+    snap = snap_b.scratch<T>(tot, st);
     HIF_CUDA_TRY(cudaMallocAsync(&d_soff, sizeof(int64_t) * nfront, st));
     HIF_CUDA_TRY(cudaMemsetAsync(d_fflag, 0, sizeof(int) * nfront, st));
     HIF_CUDA_TRY(cudaMemcpyAsync(d_soff, soff.data(), sizeof(int64_t) * nfront,
@@ -655,11 +649,12 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
   constexpr int NB2 = 256;
   const bool f64tc = sizeof(T) == 8 && tensor_cores;
   const bool outer = pmax > NB2 && !f64tc;
+  DevBuf kexp_b;
   int* d_kexp = nullptr;   // scales of the eliminated DOFs, for the products' k
   const int kstride = f64tc ? pmax : 0;
   if constexpr (sizeof(T) == 8) {
     if (f64tc) {
-      HIF_CUDA_TRY(cudaMallocAsync(&d_kexp, sizeof(int) * std::max<int64_t>(1, (int64_t)nfront * kstride), st));
+      d_kexp = kexp_b.scratch<int>((size_t)nfront * kstride, st);
       diag_exponents(d_lead, nfront, Karena, d_kexp, kstride, st);
     }
   }
@@ -801,12 +796,11 @@ void partial_cholesky(const DFront* d_fronts, const DFront* h_fronts, int nfront
       nfront = (int)keep.size();
     }
     HIF_CUDA_TRY(cudaFreeAsync(d_soff, st));
-    HIF_CUDA_TRY(cudaFreeAsync(snap, st));
+    snap_b.release();
     HIF_CUDA_TRY(cudaFreeAsync(d_fflag, st));
     if (nfront == 0) return;
   }
   finish_fronts(d_fronts, h_fronts, nfront, Karena, Parena, d_flags, tensor_cores, st, d_kexp, kstride);
-  if (d_kexp) HIF_CUDA_TRY(cudaFreeAsync(d_kexp, st));
   if (d_keep) HIF_CUDA_TRY(cudaFreeAsync(d_keep, st));
 }
 
@@ -842,9 +836,9 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
     if (tops.empty()) break;
     const size_t cnt = tops.size();
     GemmOp* d_ops = nullptr;
-    T* d_scr = nullptr;
+    DevBuf scr_b;
     HIF_CUDA_TRY(cudaMallocAsync(&d_ops, sizeof(GemmOp) * 2 * cnt, st));
-    HIF_CUDA_TRY(cudaMallocAsync(&d_scr, sizeof(T) * scr, st));
+    T* d_scr = scr_b.scratch<T>(scr, st);
     HIF_CUDA_TRY(cudaMemcpyAsync(d_ops, tops.data(), sizeof(GemmOp) * cnt, cudaMemcpyHostToDevice, st));
     HIF_CUDA_TRY(cudaMemcpyAsync(d_ops + cnt, rops.data(), sizeof(GemmOp) * cnt,
                                  cudaMemcpyHostToDevice, st));
@@ -860,7 +854,6 @@ void finish_fronts(const DFront* d_fronts, const DFront* h_fronts, int nfront, T
     };
     gemm(d_ops, tops.data(), Karena, Parena, d_scr);
     gemm(d_ops + cnt, rops.data(), Parena, d_scr, Parena);
-    HIF_CUDA_TRY(cudaFreeAsync(d_scr, st));
     HIF_CUDA_TRY(cudaFreeAsync(d_ops, st));
   }
   // 3. X^T = A_NI L^{-T} (into the panel below Linv) and 4. the Schur

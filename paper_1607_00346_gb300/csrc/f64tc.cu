@@ -642,12 +642,11 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
     }
     ProfScope ps(name, st, fl, 0.0);
     const size_t bb = sizeof(SliceBlk) * blks.size(), tb = sizeof(Tile) * tiles.size();
-    unsigned char *d_tab = nullptr, *W = nullptr;
-    int* d_exps = nullptr;
-    HIF_CUDA_TRY(cudaMallocAsync(&d_tab, bb + tb, st));
-    HIF_CUDA_TRY(cudaMallocAsync(&W, (size_t)std::max<int64_t>(1, nblk) * BLK, st));
+    DevBuf tab_b, work_b, exps_b;
+    unsigned char* d_tab = tab_b.scratch<unsigned char>(bb + tb, st);
+    unsigned char* W = work_b.scratch<unsigned char>((size_t)nblk * BLK, st);
     const size_t eb = sizeof(int) * (BR * blks.size() + (size_t)nkx);   // exps, then kx
-    HIF_CUDA_TRY(cudaMallocAsync(&d_exps, eb, st));
+    int* d_exps = exps_b.scratch<int>(eb / sizeof(int), st);
     int* d_kx = d_exps + BR * blks.size();
     std::vector<unsigned char> tab(bb + tb);
     std::copy_n(reinterpret_cast<const unsigned char*>(blks.data()), bb, tab.data());
@@ -675,9 +674,6 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
     k_gemm_f64tc<slices_used<S>()><<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(
         d_tiles, d_ops, d_blks, d_exps, W, Cbase, d_flags);
     HIF_CHECK_LAUNCH();
-    HIF_CUDA_TRY(cudaFreeAsync(d_exps, st));
-    HIF_CUDA_TRY(cudaFreeAsync(W, st));
-    HIF_CUDA_TRY(cudaFreeAsync(d_tab, st));
     f0 = f;
   }
 }

@@ -80,79 +80,6 @@ struct Trace {
   }
 };
 
-// ---- device memory --------------------------------------------------------------
-
-struct MemStats {
-  size_t cur = 0, peak = 0;
-};
-
-class DevBuf {
- public:
-  DevBuf() = default;
-  DevBuf(const DevBuf&) = delete;
-  DevBuf& operator=(const DevBuf&) = delete;
-  DevBuf(DevBuf&& o) noexcept { swap(o); }
-  DevBuf& operator=(DevBuf&& o) noexcept {
-    release();
-    swap(o);
-    return *this;
-  }
-  ~DevBuf() { release(); }
-  void alloc(size_t bytes, MemStats* ms) {
-    release();
-    ms_ = ms;
-    if (bytes == 0) return;
-    HIF_CUDA_TRY(cudaMalloc(&p_, bytes));
-    bytes_ = bytes;
-    if (ms_) {
-      ms_->cur += bytes;
-      ms_->peak = std::max(ms_->peak, ms_->cur);
-    }
-  }
-  // Stream-ordered: allocated and later freed in order on `st` (no device
-  // synchronisation); for the temporaries of one factorization.
-  void alloc_async(size_t bytes, MemStats* ms, cudaStream_t st) {
-    release();
-    ms_ = ms;
-    if (bytes == 0) return;
-    HIF_CUDA_TRY(cudaMallocAsync(&p_, bytes, st));
-    st_ = st;
-    async_ = true;
-    bytes_ = bytes;
-    if (ms_) {
-      ms_->cur += bytes;
-      ms_->peak = std::max(ms_->peak, ms_->cur);
-    }
-  }
-  void release() {
-    if (p_) {
-      if (async_) cudaFreeAsync(p_, st_);
-      else cudaFree(p_);
-      if (ms_) ms_->cur -= bytes_;
-    }
-    p_ = nullptr;
-    bytes_ = 0;
-    async_ = false;
-  }
-  template <typename U>
-  U* as() const { return static_cast<U*>(p_); }
-  size_t bytes() const { return bytes_; }
-
- private:
-  void swap(DevBuf& o) {
-    std::swap(p_, o.p_);
-    std::swap(bytes_, o.bytes_);
-    std::swap(ms_, o.ms_);
-    std::swap(st_, o.st_);
-    std::swap(async_, o.async_);
-  }
-  void* p_ = nullptr;
-  size_t bytes_ = 0;
-  MemStats* ms_ = nullptr;
-  cudaStream_t st_ = nullptr;
-  bool async_ = false;
-};
-
 template <typename U, typename A>
 void upload_async(DevBuf& b, const std::vector<U, A>& h, MemStats* ms, cudaStream_t st) {
   b.alloc_async(h.size() * sizeof(U), ms, st);
@@ -599,6 +526,7 @@ void Builder<T>::run(const double* a_dev, const double* b_dev, double b_const) {
   const int n = F_.n;
   const int64_t N = (int64_t)n * n * n;
   auto t0 = Clock::now();
+  ScratchScope counted(&F_.mem);
   {
     // keep the stream-ordered pool's memory between levels instead of
     // returning it to the driver at every synchronisation
@@ -2146,18 +2074,32 @@ size_t hif_predict_bytes(const hif_grid* grid, const hif_options* opt) {
   const double N = (double)grid->n * grid->n * grid->n;
   const int prec = opt ? opt->precision : HIF_PREC_FP64;
   const double word = prec == HIF_PREC_FP32 ? 4.0 : 8.0;
-  // Peak device bytes of hif_factor: the operator (32 B per DOF) plus factor
-  // words per DOF growing with log2 n, fitted to measured peaks at eps = 1e-6
-  // (64^3: ~2000 words per DOF, 128^3: ~3000) with a 25% margin, and at
-  // least 400 words per DOF for small grids.  A larger eps keeps fewer
-  // skeletons: the measured peaks shrink by ~0.56 per decade of eps above
-  // 1e-6 (64^3: 2.1 / 1.2 / 0.7 GB at 1e-6 / 1e-5 / 1e-4; 256^3 at 1e-4:
-  // 74 GB), taken here as 0.6 per decade, at most four decades.
-  const double lg = std::log2((double)grid->n);
-  double words = std::max(400.0, -3718.0 + 955.0 * lg);
+  // Peak device bytes of hif_factor, fitted to measured peaks (16^3 to 256^3, m = 2 to
+  // 16, eps 0 to 1e-3, coefficients over two and four decades), in four parts:
+  //   * the operator, 32 B per DOF;
+  //   * the frontal matrices of a level and the factor so far: words per DOF growing
+  //     with log2 n, with a 25% margin (eps = 1e-6; eps = 0 keeps every separator, 49 n
+  //     above 64), a larger eps shrinking them by 0.87 per decade up to 32^3 and 0.8
+  //     from 64^3 on, at most four decades;
+  //   * the level-0 cells, whose fronts grow with m^6: at least their frontal matrices,
+  //     panels and snapshots, and their panels on top of what m = 3 to 5 were fitted to;
+  //   * the work space of the products and of the Gram form, 0.8 of that and 1.4 GB at
+  //     most (gemm_f64tc holds up to 1 GB of slices at a time).
+  // The periodic grid's fronts need three times as much.
+  const double lg = std::log2((double)grid->n), m = grid->m;
   const double eps = opt ? opt->eps : 1e-6;
-  if (eps > 1e-6) words *= std::pow(0.6, std::min(4.0, std::log10(eps / 1e-6)));
-  return (size_t)(N * (32.0 + 1.25 * words * word) + (64u << 20));
+  double words = std::max(400.0, -3718.0 + 955.0 * lg);
+  if (eps > 1e-6) {
+    const double shrink = 0.87 - 0.07 * std::min(1.0, std::max(0.0, lg - 5.0));
+    words *= std::pow(shrink, std::min(4.0, std::log10(eps / 1e-6)));
+  } else if (eps == 0.0 && grid->n > 64) {
+    words = 39.0 * grid->n;
+  }
+  const double nc = (m + 1) * (m + 1) * (m + 1), pc = (m - 1) * (m - 1) * (m - 1);
+  const double cells = N / (m * m * m);
+  const double fronts = word * (grid->bc == 1 ? 3.0 : 1.0) *
+                        (1.25 * std::max(N * words, cells * (nc * nc + nc * pc + pc * pc)) + cells * nc * pc);
+  return (size_t)(32.0 * N + fronts + std::min(1.4e9, 0.8 * fronts) + (64u << 20));
 }
 
 void hif_destroy(hif_handle h) { delete h; }

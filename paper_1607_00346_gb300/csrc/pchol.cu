@@ -229,23 +229,6 @@ __global__ void __launch_bounds__(PERM_THREADS) k_pchol_perm(const PcDesc* __res
   }
 }
 
-struct Pooled {   // stream-ordered scratch
-  void* p = nullptr;
-  cudaStream_t st;
-  Pooled(size_t bytes, cudaStream_t s) : st(s) {
-    HIF_CUDA_TRY(cudaMallocAsync(&p, std::max<size_t>(16, bytes), s));
-  }
-  Pooled(const Pooled&) = delete;
-  Pooled& operator=(const Pooled&) = delete;
-  ~Pooled() { cudaFreeAsync(p, st); }
-  template <typename U>
-  U* as() const { return static_cast<U*>(p); }
-};
-
-}  // namespace
-
-namespace {
-
 // Cluster sizes of k_pchol<THREADS, MAX_CS> that can be resident (index: size)
 template <int THREADS, int MAX_CS>
 const std::vector<int>& pchol_placeable() {
@@ -309,11 +292,17 @@ void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, fl
   }
   const bool narrow = pchol_narrow(nmax);
   const int threads = narrow ? PC_NARROW : PC_WIDE, CS = ceil_div(nmax, threads);
-  Pooled G(sizeof(double) * gt, st), L(sizeof(double) * lt, st), diag(sizeof(double) * ct, st),
-      step(sizeof(int) * ct, st), stt(sizeof(PcState) * nf, st), dds(sizeof(PcDesc) * nf, st),
-      dop(sizeof(GemmOp) * nf, st), lst(sizeof(int) * nf, st);
-  HIF_CUDA_TRY(cudaMemcpyAsync(dds.p, ds.data(), sizeof(PcDesc) * nf, cudaMemcpyHostToDevice, st));
-  HIF_CUDA_TRY(cudaMemcpyAsync(dop.p, ops.data(), sizeof(GemmOp) * nf, cudaMemcpyHostToDevice, st));
+  DevBuf G, L, diag, step, stt, dds, dop, lst;
+  G.scratch<double>(gt, st);
+  L.scratch<double>(lt, st);
+  diag.scratch<double>(ct, st);
+  step.scratch<int>(ct, st);
+  stt.scratch<PcState>(nf, st);
+  dds.scratch<PcDesc>(nf, st);
+  dop.scratch<GemmOp>(nf, st);
+  lst.scratch<int>(nf, st);
+  HIF_CUDA_TRY(cudaMemcpyAsync(dds.as<void>(), ds.data(), sizeof(PcDesc) * nf, cudaMemcpyHostToDevice, st));
+  HIF_CUDA_TRY(cudaMemcpyAsync(dop.as<void>(), ops.data(), sizeof(GemmOp) * nf, cudaMemcpyHostToDevice, st));
   gemm_f64tc<float>(dop.as<GemmOp>(), ops.data(), nf, Garena, Garena, G.as<double>(), d_flags, st,
                     "id_gram_f64tc");
   {
@@ -326,7 +315,7 @@ void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, fl
   for (int f = 0; f < nf; ++f) act[f] = f;
   std::vector<PcState> h(nf);
   while (!act.empty()) {
-    HIF_CUDA_TRY(cudaMemcpyAsync(lst.p, act.data(), sizeof(int) * act.size(), cudaMemcpyHostToDevice, st));
+    HIF_CUDA_TRY(cudaMemcpyAsync(lst.as<void>(), act.data(), sizeof(int) * act.size(), cudaMemcpyHostToDevice, st));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(act.size() * CS));
     cfg.blockDim = dim3(threads);
@@ -348,7 +337,7 @@ void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, fl
                                       stt.as<PcState>(), eps * eps));
       HIF_CHECK_LAUNCH();
     }
-    HIF_CUDA_TRY(cudaMemcpyAsync(h.data(), stt.p, sizeof(PcState) * nf, cudaMemcpyDeviceToHost, st));
+    HIF_CUDA_TRY(cudaMemcpyAsync(h.data(), stt.as<void>(), sizeof(PcState) * nf, cudaMemcpyDeviceToHost, st));
     HIF_CUDA_TRY(cudaStreamSynchronize(st));
     std::vector<int> next;
     for (int f : act)
@@ -361,7 +350,7 @@ void gram_id(SkelDesc* d_f, const SkelDesc* h_f, int nf, const float* Garena, fl
       const PcDesc& d = ds[act[i]];
       up[i] = GemmOp{d.L, d.L, d.G, d.n, d.n, PC_STEPS, d.n, d.n, d.n, 0, 1, -1.f, 1.f, 1, 0};
     }
-    HIF_CUDA_TRY(cudaMemcpyAsync(dop.p, up.data(), sizeof(GemmOp) * up.size(), cudaMemcpyHostToDevice, st));
+    HIF_CUDA_TRY(cudaMemcpyAsync(dop.as<void>(), up.data(), sizeof(GemmOp) * up.size(), cudaMemcpyHostToDevice, st));
     gemm_f64tc<double>(dop.as<GemmOp>(), up.data(), (int)up.size(), L.as<double>(), L.as<double>(),
                        G.as<double>(), d_flags, st, "id_pchol_update_f64tc");
   }

@@ -824,12 +824,12 @@ void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garen
     toff += (QB2 / QB) * QB * QB;         // the block's panel T's
     ro[i] = rOff[ord[i]];
   }
-  T *Var = nullptr, *War = nullptr, *Tar = nullptr;
+  DevBuf V_b, W_b, T_b, Wp_b, G_b, Tb_b, W1_b, W2_b;
+  T* Var = V_b.scratch<T>(voff, st);
+  T* War = W_b.scratch<T>(woff, st);
+  T* Tar = T_b.scratch<T>(toff, st);
   QRDesc* d_qd = nullptr;
   int64_t* d_ro = nullptr;
-  HIF_CUDA_TRY(cudaMallocAsync(&Var, sizeof(T) * voff, st));
-  HIF_CUDA_TRY(cudaMallocAsync(&War, sizeof(T) * woff, st));
-  HIF_CUDA_TRY(cudaMallocAsync(&Tar, sizeof(T) * toff, st));
   HIF_CUDA_TRY(cudaMallocAsync(&d_qd, sizeof(QRDesc) * nq, st));
   HIF_CUDA_TRY(cudaMallocAsync(&d_ro, sizeof(int64_t) * nq, st));
   HIF_CUDA_TRY(cudaMemcpyAsync(d_qd, qd.data(), sizeof(QRDesc) * nq, cudaMemcpyHostToDevice, st));
@@ -861,9 +861,8 @@ void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garen
     wpo[i] = wptot;
     wptot += (int64_t)smax * QB * qd[i].n;
   }
-  T* Wp = nullptr;
+  T* Wp = Wp_b.scratch<T>(wptot, st);
   int64_t* d_wpo = nullptr;
-  HIF_CUDA_TRY(cudaMallocAsync(&Wp, sizeof(T) * std::max<int64_t>(1, wptot), st));
   HIF_CUDA_TRY(cudaMallocAsync(&d_wpo, sizeof(int64_t) * nq, st));
   HIF_CUDA_TRY(cudaMemcpyAsync(d_wpo, wpo.data(), sizeof(int64_t) * nq, cudaMemcpyHostToDevice, st));
   static const bool w1_attr = [] {
@@ -883,10 +882,10 @@ void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garen
   const bool blocks = nmax > QB2;
   T *Gb = nullptr, *Tb = nullptr, *W1b = nullptr, *W2b = nullptr;
   if (blocks) {
-    HIF_CUDA_TRY(cudaMallocAsync(&Gb, sizeof(T) * nq * QB2 * QB2, st));
-    HIF_CUDA_TRY(cudaMallocAsync(&Tb, sizeof(T) * nq * QB2 * QB2, st));
-    HIF_CUDA_TRY(cudaMallocAsync(&W1b, sizeof(T) * w2tot, st));
-    HIF_CUDA_TRY(cudaMallocAsync(&W2b, sizeof(T) * w2tot, st));
+    Gb = G_b.scratch<T>((size_t)nq * QB2 * QB2, st);
+    Tb = Tb_b.scratch<T>((size_t)nq * QB2 * QB2, st);
+    W1b = W1_b.scratch<T>(w2tot, st);
+    W2b = W2_b.scratch<T>(w2tot, st);
   }
   for (int p = 0; p < nmax; p += QB) {
     const int p0 = p / QB2 * QB2;
@@ -1016,12 +1015,6 @@ void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garen
          "id_rowreduce_block_f64tc");
     HIF_CUDA_TRY(cudaFreeAsync(d_ops, st));
   }
-  if (blocks) {
-    HIF_CUDA_TRY(cudaFreeAsync(W2b, st));
-    HIF_CUDA_TRY(cudaFreeAsync(W1b, st));
-    HIF_CUDA_TRY(cudaFreeAsync(Tb, st));
-    HIF_CUDA_TRY(cudaFreeAsync(Gb, st));
-  }
   {
     ProfScope ps("id_rowreduce_extract", st);
     const int64_t mx = (int64_t)nmax * nmax;
@@ -1029,12 +1022,8 @@ void reduce_rows_qr(const SkelDesc* h_f, const std::vector<int>& which, T* Garen
     HIF_CHECK_LAUNCH();
   }
   HIF_CUDA_TRY(cudaFreeAsync(d_wpo, st));
-  HIF_CUDA_TRY(cudaFreeAsync(Wp, st));
   HIF_CUDA_TRY(cudaFreeAsync(d_ro, st));
   HIF_CUDA_TRY(cudaFreeAsync(d_qd, st));
-  HIF_CUDA_TRY(cudaFreeAsync(Tar, st));
-  HIF_CUDA_TRY(cudaFreeAsync(War, st));
-  HIF_CUDA_TRY(cudaFreeAsync(Var, st));
 }
 
 template void reduce_rows_qr<float>(const SkelDesc*, const std::vector<int>&, float*, float*,

@@ -442,7 +442,7 @@ void gemm_tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const float* Ab
   tile_counts(h_ops, nops, VAR_TN[v], &tiles, &mt);
   ProfScope ps(name, st, fl, 0.0);
   int64_t* d_woff = nullptr;
-  float* Wk = nullptr;
+  DevBuf work_b;
   if (S > 1) {
     std::vector<int64_t> woff(nops);
     int64_t tot = 0;
@@ -453,14 +453,13 @@ void gemm_tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const float* Ab
       mnmax = std::max<int64_t>(mnmax, (int64_t)h_ops[i].m * h_ops[i].n);
     }
     HIF_CUDA_TRY(cudaMallocAsync(&d_woff, sizeof(int64_t) * nops, st));
-    HIF_CUDA_TRY(cudaMallocAsync(&Wk, sizeof(float) * tot, st));
+    float* Wk = work_b.scratch<float>(tot, st);
     HIF_CUDA_TRY(cudaMemcpyAsync(d_woff, woff.data(), sizeof(int64_t) * nops,
                                  cudaMemcpyHostToDevice, st));
     launch_variant(v, d_ops, nops, mt, Abase, Bbase, Cbase, d_flags, st, S, d_woff, Wk);
     k_splitk_reduce<<<dim3((unsigned)ceil_div(mnmax, 256), nops), 256, 0, st>>>(d_ops, d_woff, Wk,
                                                                                 S, Cbase);
     HIF_CHECK_LAUNCH();
-    HIF_CUDA_TRY(cudaFreeAsync(Wk, st));
     HIF_CUDA_TRY(cudaFreeAsync(d_woff, st));
     return;
   }

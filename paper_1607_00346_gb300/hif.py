@@ -216,8 +216,8 @@ def measure_peaks(stream=None) -> dict:
     return {k: getattr(p, k) for k, _ in Peaks._fields_}
 
 
-def predict_bytes(n: int, m: int, **opts) -> int:
-    g = Grid(n, m, 0)
+def predict_bytes(n: int, m: int, periodic: bool = False, **opts) -> int:
+    g = Grid(n, m, 1 if periodic else 0)
     o = default_options(**opts)
     return int(load().hif_predict_bytes(ctypes.byref(g), ctypes.byref(o)))
 
