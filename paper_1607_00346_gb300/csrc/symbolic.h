@@ -132,8 +132,9 @@ class Symbolic {
   // Their rows are listed on the device (skel_rows).
   void build_fronts(const CellPlan& cp, int kind, const std::vector<uint8_t>& alive,
                     SkelPlan& sp) const;
-  // The same with the coupled rows, on the host: what skel_rows lists, front by
-  // front, for checks of the plan's consistency.
+  // The same with the coupled rows, on the host, the fronts in order of their lowest
+  // DOF: what the checks compare build_fronts and the device's row lists (skel_rows)
+  // with.  A factorization calls neither this nor filter_rows.
   // `alive` marks DOFs still active (redundant DOFs of faces are dropped
   // before the edges are planned).
   void build_skel(const CellPlan& cp, int kind, const std::vector<uint8_t>& alive,
