@@ -2099,7 +2099,7 @@ size_t hif_predict_bytes(const hif_grid* grid, const hif_options* opt) {
   const double cells = N / (m * m * m);
   const double fronts = word * (grid->bc == 1 ? 3.0 : 1.0) *
                         (1.25 * std::max(N * words, cells * (nc * nc + nc * pc + pc * pc)) + cells * nc * pc);
-  return (size_t)(32.0 * N + fronts + std::min(1.4e9, 0.8 * fronts) + (64u << 20));
+  return (size_t)(32.0 * N + fronts + std::min(1.4e9, 0.8 * fronts) + (56u << 20));
 }
 
 void hif_destroy(hif_handle h) { delete h; }
