@@ -41,11 +41,11 @@
 // 64 k (the Cholesky updates), k_f64_slice_rows finds s and writes the slices with
 // one read.
 //
-// Measured (all launches, FMA form in brackets): one 64^3 product 40 (66) us, 512
-// of them 125 (270) us, one 256^3 55 (280) us, one 1024^3 0.11 (2.1) ms, one 2048^3
-// 0.65 (14.5) ms = 26 TFLOP/s.  Error against quad precision, entries over 2 to
-// 12 decades: 5e-17 to 7e-17 in norm (3e-16 to 1.5e-15).  For the solve error of a
-// factorization see SLICE_SPAN in hif.cu.
+// Measured (all launches, FMA form in brackets): one 64^3 product 34 (76) us, 512 of
+// them 108 (274) us, A A^T 28 (74) and 81 (270) us; one 256^3 48 (287) us, one 1024^3
+// 0.106 (2.14) ms, one 2048^3 0.63 (14.5) ms = 27 TFLOP/s (by maxima, four launches,
+// 0.66 ms).  Error against extended precision: 2e-17 to 6e-17 in norm.  For the solve
+// error of a factorization see SLICE_SPAN in hif.cu.
 //
 // k_gemm_f64tc: one 128 x 64 tile per CTA; the eight accumulators fill the 512
 // columns of tensor memory, four stages of 48 KB the shared memory.  Per 16 k one
@@ -53,13 +53,13 @@
 // up to four neighbouring slices of B, whose products go to neighbouring
 // accumulators), and a warp copies the block three ahead; per 128 k the warps
 // read the accumulators back.  A small tile is a chain of latencies (table,
-// exponents, copies, products, C): with the exponents read while tensor memory is
-// allocated, C copied to shared memory during the last read-back, and 512 threads
-// of 16 columns each for the rounding instead of 256 of 32, one 64^3 tile takes
-// 17.5 instead of 22.3 us and 1520 of them 166 us; 256^3 29 (34) us, 1024^3 81 (84),
-// 2048^3 570 (586), where the copies from L2 (6.4 TB/s) are the bound.  With the
-// one-pass slices a 64^3 FP64 factorization and solve went from 203 to 194 ms, a
-// 32^3 periodic one from 45.3 to 42.5 ms.
+// exponents, copies, products, C): exponents are read while tensor memory is
+// allocated, C is copied to shared memory during the last read-back, and 512 threads of
+// 16 columns each round the sums (256 of 32: 22.3 instead of 17.5 us for one 64^3
+// tile; large products 3% slower).  This kernel alone: 1520 tiles of 64 k 166 us, 256^3
+// 29 us, 1024^3 81, 2048^3 570, where the copies from L2 (6.4 TB/s) are the bound.
+// With that and the one-pass slices a 64^3 FP64 factorization and solve went from 203 to
+// 194 ms, a 32^3 periodic one from 45.3 to 42.5 ms.
 #include <stdint.h>
 
 #include <algorithm>
@@ -146,10 +146,12 @@ __global__ void __launch_bounds__(256) k_f64_kmax(const SliceBlk* __restrict__ b
   }
 }
 
-// The exponent added to this operand's entries at k.
+// The exponent added to this operand's entries at k.  (BAL: some product of the batch is
+// balanced; the loads and branches cost the Gram matrices, which are not, 3%.)
+template <bool BAL>
 __device__ __forceinline__ int balance(const SliceBlk& b, const int* kx,
                                        const int* __restrict__ kexp, int k) {
-  if (b.kbal == KB_NONE) return 0;
+  if (!BAL || b.kbal == KB_NONE) return 0;
   if (b.kbal != KB_MAX) {
     const int e = kexp[b.kx + k];
     return (b.kbal == KB_UP) == (b.isB == 0) ? e : -e;
@@ -171,7 +173,7 @@ __device__ __forceinline__ int entry_exp(double x, int t) {
   if (h == 0 && __double2loint(x) == 0) return 0;
   return max((h + ROUND_UP) >> 20, 1) + t + ROW_BIAS;
 }
-template <typename S>
+template <typename S, bool BAL>
 __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ blks,
                                                   const S* __restrict__ Ab,
                                                   const S* __restrict__ Bb,
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ b
       int m = 0;
 #pragma unroll 4
       for (int k = k0 + lane; k < k1; k += 32)
-        m = max(m, entry_exp(X[(int64_t)r * b.ld + k], balance(b, kx, kexp, k)));
+        m = max(m, entry_exp(X[(int64_t)r * b.ld + k], balance<BAL>(b, kx, kexp, k)));
       m = __reduce_max_sync(0xffffffffu, m);
       if (lane == 0) atomicMax(&out[r], m);
     }
@@ -199,7 +201,7 @@ __global__ void __launch_bounds__(256) k_f64_exps(const SliceBlk* __restrict__ b
     int m = 0;
 #pragma unroll 8
     for (int k = k0 + threadIdx.x / BR; k < k1; k += 256 / BR)
-      m = max(m, entry_exp(X[r + (int64_t)k * b.ld], balance(b, kx, kexp, k)));
+      m = max(m, entry_exp(X[r + (int64_t)k * b.ld], balance<BAL>(b, kx, kexp, k)));
     atomicMax(&out[r], m);
   }
 }
@@ -253,7 +255,7 @@ __device__ __forceinline__ void write_slices(const double (&x)[8], int s, const 
 }
 
 // One thread: eight consecutive k of one row at a time.
-template <typename S>
+template <typename S, bool BAL>
 __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ blks,
                                                    const S* __restrict__ Ab,
                                                    const S* __restrict__ Bb,
@@ -273,7 +275,7 @@ __global__ void __launch_bounds__(256) k_f64_slice(const SliceBlk* __restrict__ 
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int k = g * 8 + j;
-      t[j] = k < b.k ? balance(b, kx, kexp, k) : 0;
+      t[j] = k < b.k ? balance<BAL>(b, kx, kexp, k) : 0;
       x[j] = (r < b.rows && k < b.k)
                  ? (double)X[b.kcont ? (int64_t)r * b.ld + k : r + (int64_t)k * b.ld]
                  : 0.0;
@@ -584,8 +586,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 }  // namespace
 
-// One 64 x 64 tile of the FMA form takes 1.2 us per k on its SM; the four
-// launches and one tile here take about 40 us, whatever the k up to 100.
+// One 64 x 64 tile of the FMA form takes 1.2 us per k on its SM; the launches and one
+// tile here take 28 to 34 us, whatever the k up to 100.
 bool f64tc_worth(const GemmOp* h_ops, int nops) {
   for (int i = 0; i < nops; ++i)
     if (h_ops[i].k >= 24 && (int64_t)h_ops[i].m * h_ops[i].n >= 1024) return true;
@@ -608,7 +610,7 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
     int64_t nblk = 0, nkx = 0;
     double fl = 0;
     int f = f0, kmax = 0;
-    bool all_same = true;   // every product of the batch is A A^T
+    bool all_same = true, balanced = false;
     for (; f < nops; ++f) {
       const GemmOp& o = h_ops[f];
       const int nk = ceil_div(o.k, KC);
@@ -618,6 +620,7 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
       if (f > f0 && (size_t)(nblk + need) * BLK > WORK_LIMIT) break;
       const int kbal = same ? KB_NONE : o.kbal;
       all_same = all_same && same;
+      balanced = balanced || kbal != KB_NONE;
       auto add = [&](int64_t src, int rows, int ld, bool kcont, bool isB) {
         const int first = (int)blks.size();
         for (int r0 = 0; r0 < rows; r0 += BR) {
@@ -666,9 +669,11 @@ void gemm_f64tc(const GemmOp* d_ops, const GemmOp* h_ops, int nops, const S* Aba
         k_f64_kmax<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx);
         HIF_CHECK_LAUNCH();
       }
-      k_f64_exps<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_kexp, d_exps);
+      (balanced ? k_f64_exps<S, true> : k_f64_exps<S, false>)<<<grid, 256, 0, st>>>(
+          d_blks, Abase, Bbase, d_kx, d_kexp, d_exps);
       HIF_CHECK_LAUNCH();
-      k_f64_slice<S><<<grid, 256, 0, st>>>(d_blks, Abase, Bbase, d_kx, d_kexp, d_exps, W);
+      (balanced ? k_f64_slice<S, true> : k_f64_slice<S, false>)<<<grid, 256, 0, st>>>(
+          d_blks, Abase, Bbase, d_kx, d_kexp, d_exps, W);
       HIF_CHECK_LAUNCH();
     }
     k_gemm_f64tc<slices_used<S>()><<<(unsigned)tiles.size(), THREADS, NST * STAGE, st>>>(
