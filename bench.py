@@ -91,8 +91,8 @@ SLICED = {"id_gram_f64tc": 28}
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a
 # kernel label in the bench workload, from ncu captures of the current kernels
-# (none taken since the products leave out the zeros of triangular operands)
-TRAFFIC_PER_LAUNCH = {}
+# (profiles/gemm_tc_traffic_contrast128.md)
+TRAFFIC_PER_LAUNCH = {"gemm_tc": 3.67e9}
 
 
 def _hbm_peak():
@@ -461,7 +461,8 @@ def main():
 
     def roofline(k):
         per_launch_s = k["seconds"] / max(k["launches"], 1)
-        bound = KERNEL_BOUND.get(k["name"], "alu" if k["flops"] > 0 else "hbm")
+        bound = KERNEL_BOUND.get(k["name"], "sliced" if k["name"].endswith("_f64tc")
+                                 else "alu" if k["flops"] > 0 else "hbm")
         if bound == "tensor":
             # algorithmic flops 2mnk of the products (the 3xTF32 split issues
             # three TF32 products per algorithmic one; that cost is the kernel's)
@@ -488,7 +489,9 @@ def main():
             src = hbm_src
             unit = "GB/s"
         return {"bound": bound, "achieved": ach, "peak": peak, "unit": unit, "frac": ach / peak,
-                "traffic": TRAFFIC_PER_LAUNCH.get(k["name"]), "kernel": k["name"],
+                "traffic": (TRAFFIC_PER_LAUNCH.get(k["name"])
+                            if args.workload == "contrast128" and args.precision == "fp32" else None),
+                "kernel": k["name"],
                 "peak_source": src, "share": k["seconds"] / total_prof_s,
                 "launches_per_step": k["launches"] / args.steps}
 

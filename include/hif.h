@@ -270,7 +270,8 @@ size_t hif_predict_bytes(const hif_grid* grid, const hif_options* opt);
  * cap per-kernel aggregates (*count receives the number available).  flops
  * and bytes are the algorithmic counts of the launches (0 where not defined).
  * An apply whose sweeps replay a CUDA graph is timed as one launch named
- * "apply_sweeps_graph" (its kernels are not timed one by one).
+ * "apply_sweeps_graph" (its kernels are not timed one by one).  The factors of
+ * a batch run side by side: their times overlap, and the record adds them up.
  * Process-wide; meant for benchmarking, not for concurrent use.
  */
 typedef struct {

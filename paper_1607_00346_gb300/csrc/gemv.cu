@@ -27,8 +27,8 @@
 // the mat-vecs of one apply: 1 column 3.9 ms (5.9 TB/s), 4 columns 5.0 ms, 16
 // columns 8.7 ms; with one CTA per 128 rows or 8 columns and x read from L1 by
 // every warp (blocks 16, 8, 4, 2, 1) they took 6.5 ms for 1 column and 37 ms
-// for 16.  On a 64^3 FP64 factor 8 columns take 8.7 ms, 7.2 ms of which are the
-// multiply-adds at the FP64 rate.
+// for 16.  On a 64^3 FP64 factor an apply of 8 columns takes 7.7 ms, 7.2 ms of which
+// are the multiply-adds at the FP64 rate.
 #include <algorithm>
 #include <vector>
 

@@ -6,10 +6,10 @@
 // of the pivoted Cholesky factorization G = A_RF^T A_RF = P R^T R P^T: each step
 // takes the column with the largest remaining diagonal entry, |R_ii|^2, and
 // subtracts the outer product of its row of R.  Squaring the matrix squares its
-// condition number, so G needs twice the digits: it is formed from the FP32
-// entries with exact sums (f64tc.cu, 2^-62 below column maximum times column
-// maximum) and factored in FP64, which leaves R_ii an error of 1e-8 |R_11| at the
-// worst, where Householder QR in FP32 leaves 6e-8.
+// condition number, so G needs twice the digits: it is formed from the FP32 entries,
+// cut 55 bits below the largest of their column, with sums off by less than 2^-50 of the
+// two columns' largest entries per row (f64tc.cu: seven slices), and factored in FP64,
+// which leaves R_ii an error of 1e-8 |R_11|, where Householder QR in FP32 leaves 6e-8.
 //
 // What it replaces is bound by chains: the unpivoted QR of the tall A_RF column by
 // column (two barriers and a pass over a 32-column panel each), then pivoted QR of

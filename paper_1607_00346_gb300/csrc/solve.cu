@@ -91,7 +91,7 @@ __device__ __forceinline__ double stencil_apply(const StencilRow& r, const doubl
 }
 
 // r = f - A u, one point of every column per thread.  Bound by the FP64 unit, 8
-// operations per point and column (128^3, 3 columns: 84 us; HBM 32 us).
+// operations per point and column (128^3, 3 columns: 95 us of 115; HBM 32 us).
 __global__ void __launch_bounds__(VT) k_residual(const double* __restrict__ cpl,
                                                  const double* __restrict__ diag, int n,
                                                  int periodic, const double* __restrict__ f,
