@@ -955,7 +955,7 @@ int64_t Builder<T>::skel_step(const CellPlan& cp, int kind, std::vector<uint8_t>
       nFmax = std::max(nFmax, sd[sel[1][i]].nF);
     }
     Rbuf.alloc_async(sizeof(T) * rtot, &F_.mem, st_);
-    gram = std::is_same<T, float>::value && tc_ && gram_id_fits(nFmax);
+    gram = std::is_same<T, float>::value && tc_ && gram_id_fits(nFmax, F_.eps);
     if (!gram)
       reduce_rows_qr<T>(sd.data(), sel[1], G.as<T>(), Rbuf.as<T>(), roff, flags_.as<int>(),
                         tc_, st_);

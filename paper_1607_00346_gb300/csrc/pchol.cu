@@ -10,6 +10,11 @@
 // cut 55 bits below the largest of their column, with sums off by less than 2^-50 of the
 // two columns' largest entries per row (f64tc.cu: seven slices), and factored in FP64,
 // which leaves R_ii an error of 1e-8 |R_11|, where Householder QR in FP32 leaves 6e-8.
+// Pivots below that are noise whose rows of R need not be bounded by them (QR's are), so
+// fronts with a smaller eps than GRAM_EPS stay with the row reduction and QR: FP32 at
+// eps 1e-12, a = 10^U(-2,2), the Gram form lost 250 times the solve error at 48^3 and
+// failed at 64^3; at 1e-10 it kept 3% fewer skeletons; at 1e-7 and above it keeps the
+// same ones.
 //
 // What it replaces is bound by chains: the unpivoted QR of the tall A_RF column by
 // column (two barriers and a pass over a 32-column panel each), then pivoted QR of
@@ -37,6 +42,7 @@ namespace cg = cooperative_groups;
 
 namespace {
 
+constexpr double GRAM_EPS = 1e-7;  // the least eps whose pivots G resolves
 constexpr int PC_STEPS = 64;       // pivots per launch
 // A CTA of 128 columns keeps 64 KB of the block's rows, so that three share an SM and
 // one's barriers overlap the others' sums; 256 columns (one per SM, 128 KB) for fronts
@@ -267,7 +273,8 @@ bool pchol_narrow(int n) {
 
 }  // namespace
 
-bool gram_id_fits(int nFmax) {
+bool gram_id_fits(int nFmax, double eps) {
+  if (eps < GRAM_EPS) return false;
   if (pchol_narrow(nFmax)) return true;
   const int cs = ceil_div(nFmax, PC_WIDE);
   return cs <= PC_WIDE_CS && pchol_placeable<PC_WIDE, PC_WIDE_CS>()[cs] != 0;

@@ -7,8 +7,8 @@
 namespace hif {
 
 // Whether fronts of up to nFmax DOFs fit one cluster (one column per thread, 16
-// CTAs of 256).
-bool gram_id_fits(int nFmax);
+// CTAs of 256) and G resolves pivots down to eps.
+bool gram_id_fits(int nFmax, double eps);
 // Column-pivoted R factor of the fronts' gathered rows (nR x nF blocks of the
 // gather arena below the nF x nF ones), stopped at |R_ii| <= eps |R_11|: R (row l of
 // column c, leading dimension nF) to Rout + idoff, the permutation and the rank
